@@ -80,7 +80,10 @@ gemm_simt_kernel(const T* __restrict__ A, long a_rs, long a_cs, const T* __restr
 void gemm(const Ctx& c, const void* A, long a_rs, long a_cs, const void* B, long b_rs, long b_cs, void* C,
           int out_is_float, int m, int n, int k, const GemmEpilogue& e) {
   if (m <= 0 || n <= 0) return;
-  if (c.dtype == 1 && c.use_tc && gemm_tc_supported(m, n, k)) {
+  // The tensor-core kernels take any reduction length: what TMA wants aligned is the row pitch of each operand (checked
+  // there), and slabs past the end arrive as zeros.  Weight gradients reduce over batch x tokens rows, which an odd batch
+  // leaves odd: at batch 45 of ViT-B they took 515 us a launch on the FP32-FMA kernel below, 18 us on the tensor cores.
+  if (c.dtype == 1 && c.use_tc && (n % 8) == 0) {
     if (c.use_tc >= 2 && m > 128 &&
         gemm_tc2_strided(c, A, a_rs, a_cs, B, b_rs, b_cs, C, out_is_float, m, n, k, e, c.split_ws, c.split_ws_floats) == 0) return;
     if (gemm_tc_strided(c, A, a_rs, a_cs, B, b_rs, b_cs, C, out_is_float, m, n, k, e, c.split_ws, c.split_ws_floats) == 0) return;
