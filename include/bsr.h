@@ -364,8 +364,9 @@ int32_t bsr_attention_forward(const void* qkv_dev, int32_t dtype, int32_t batch,
  * attention map is recomputed from qkv_dev and lse_dev (as written by bsr_attention_forward).  score_grad_dev optional
  * [batch, t-1] float32: a gradient arriving at the head-mean classification scores of Eq. 6 (from the fused token);
  * every head's classification row receives 1/heads of it.  delta_scratch_dev: batch*heads*t floats of caller-owned
- * scratch (used by the kernels without tensor cores; may be null when use_tensor_cores != 0).  use_tensor_cores != 0
- * selects the tcgen05 kernels (bf16, d = 64, t <= 256) and fails with BSR_ERR_UNSUPPORTED outside their range. */
+ * scratch (used by the kernels without tensor cores and beyond 256 tokens; may be null when use_tensor_cores != 0 and
+ * t <= 256).  use_tensor_cores != 0 selects the tcgen05 kernels (bf16, d = 64; without the scratch t <= 256) and fails
+ * with BSR_ERR_UNSUPPORTED outside their range. */
 int32_t bsr_attention_backward(const void* qkv_dev, const void* dout_dev, const float* lse_dev, const float* score_grad_dev,
                                int32_t dtype, int32_t batch, int32_t t, int32_t heads, int32_t d, void* dqkv_dev_out,
                                float* delta_scratch_dev, int32_t use_tensor_cores, void* stream);

@@ -1601,8 +1601,8 @@ int32_t bsr_attention_backward(const void* qkv, const void* dout, const float* l
   if (batch < 1 || t < 1 || heads < 1 || d < 8 || d > 64 || d % 8 != 0) return set_err(g_error, BSR_ERR_INVALID_ARG, "bad shape: head dimension must be a multiple of 8, at most 64");
   Ctx c = bare_ctx(dtype, stream);
   if (use_tensor_cores) {
-    if (attention_bwd_tc(c, qkv, dout, lse, score_grad, dqkv, batch, t, heads, d) != 0)
-      return set_err(g_error, BSR_ERR_UNSUPPORTED, "the tcgen05 attention backward needs bf16, head dimension 64 and at most 256 tokens");
+    if (attention_bwd_tc(c, qkv, dout, lse, score_grad, delta_scratch, dqkv, batch, t, heads, d) != 0)
+      return set_err(g_error, BSR_ERR_UNSUPPORTED, "the tcgen05 attention backward needs bf16, head dimension 64 and, beyond 256 tokens, delta_scratch_dev");
     return check_cuda(nullptr, "bsr_attention_backward");
   }
   if (delta_scratch == nullptr) return set_err(g_error, BSR_ERR_INVALID_ARG, "delta_scratch_dev is required without tensor cores");

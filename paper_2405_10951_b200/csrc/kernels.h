@@ -172,8 +172,9 @@ void wait_expiry_selftest(const Ctx& c, unsigned long long limit_ns);
 // scaled scores; cls_prob (optional) [B, H, T-1].
 // tcgen05 kernels (bf16, head dimension 64); return non-zero when they do not take the problem.
 int attention_fwd_tc(const Ctx& c, const void* qkv, void* out, float* lse, float* cls_prob, int B, int T, int H, int d);
-int attention_bwd_tc(const Ctx& c, const void* qkv, const void* dout, const float* lse, const float* cls_extra, void* dqkv,
-                     int B, int T, int H, int d);
+// delta: scratch [B, H, T], needed beyond 256 tokens only.
+int attention_bwd_tc(const Ctx& c, const void* qkv, const void* dout, const float* lse, const float* cls_extra, float* delta,
+                     void* dqkv, int B, int T, int H, int d);
 int attention_fwd(const Ctx& c, const void* qkv, void* out, float* lse, float* cls_prob, int B, int T, int H, int d);
 // dqkv from dout; delta scratch [B, H, T]; cls_extra (optional) [B, T-1]: gradient arriving at the head-mean
 // score of each non-classification token (zero for kept tokens); cls_prob needed with it.

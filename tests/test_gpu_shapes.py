@@ -19,3 +19,44 @@ def test_bf16_step_with_odd_row_counts(batch):
     images, labels, task_ids, params = synth.make_workload(cfg, peaked=False)
     gpu = P.run_gpu_step(cfg, images, labels, task_ids, params)
     P.compare_step(cfg, images, labels, task_ids, params, gpu, P.BF16_TOL, P.BF16_EXACT_MARGIN, P.BF16_SCORE_TOL)
+
+
+@pytest.mark.parametrize("with_score_grad", [False, True])
+@pytest.mark.parametrize("B,T,H", [(1, 257, 1), (2, 290, 3), (1, 384, 2), (1, 385, 1), (2, 577, 2), (1, 1025, 1)])
+def test_attention_backward_beyond_256_tokens(B, T, H, with_score_grad):
+    """dQ, dK, dV of the kernel pair that walks the other side in blocks of 64, last blocks of 1 to 64 columns and last
+    row tiles of 1 to 128 rows; same bf16 inputs and tolerance as the shorter kernels."""
+    import ctypes as C
+
+    import torch
+    from oracle import bsr_oracle as O
+    from paper_2405_10951_b200 import binding as Bd
+    d = 64
+    rng = np.random.default_rng(T * 7 + B)
+    qkv = synth.round_to_bf16(rng.standard_normal((B, T, 3, H, d)))
+    do = synth.round_to_bf16(rng.standard_normal((B, T, H * d)))
+    sg = rng.standard_normal((B, T - 1)) * 3.0 if with_score_grad else None
+    q, k, v = (qkv[:, :, i].transpose(0, 2, 1, 3) for i in range(3))
+
+    class Cfg:
+        heads = H
+        dim = H * d
+    _, A = O.attention_fwd(Cfg, q, k, v)
+    dA_cls = None
+    if sg is not None:
+        dA_cls = np.zeros((B, T))
+        dA_cls[:, 1:] = sg / H
+    want = np.stack(O.attention_bwd(Cfg, A, q, k, v, do.reshape(B, T, H, d).transpose(0, 2, 1, 3), dA_cls), axis=0).transpose(1, 3, 0, 2, 4)
+    dev = torch.as_tensor(qkv.astype(np.float32)).cuda().bfloat16()
+    dod = torch.as_tensor(do.astype(np.float32)).cuda().bfloat16()
+    sgd = None if sg is None else torch.as_tensor(sg.astype(np.float32)).cuda()
+    _, _, lse = Bd.bsr_attention_forward(dev, H, use_tensor_cores=True, want_lse=True)
+    out, delta = torch.empty_like(dev), torch.empty(B * H * T, device="cuda")
+    p = lambda t: None if t is None else C.c_void_p(t.data_ptr())
+    rc = Bd.lib().bsr_attention_backward(p(dev), p(dod), p(lse), p(sgd), Bd.DTYPE_BF16, B, T, H, d, p(out), p(delta), 1,
+                                         C.c_void_p(torch.cuda.current_stream().cuda_stream))
+    assert rc == Bd.BSR_OK
+    torch.cuda.synchronize()
+    got = out.float().cpu().numpy().astype(np.float64)
+    for i, name in enumerate(("dq", "dk", "dv")):
+        assert P.rel_err(got[:, :, i], want[:, :, i]) < 8e-3, name
