@@ -73,6 +73,7 @@ template <typename T>
 __global__ void __launch_bounds__(AT_WARPS * 32)
 attn_fwd_kernel(const T* __restrict__ qkv, T* __restrict__ out, float* __restrict__ lse, float* __restrict__ cls_prob,
                 int B, int T_, int H, int d, int qsplit) {
+  dependent_sync();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   int rs = Row<T>::stride(d);
   T* Ks = reinterpret_cast<T*>(smem_raw);
@@ -140,6 +141,7 @@ __global__ void __launch_bounds__(AT_WARPS * 32)
 attn_bwd_dq_kernel(const T* __restrict__ qkv, const T* __restrict__ dout, const float* __restrict__ lse,
                    float* __restrict__ delta, const float* __restrict__ cls_extra, T* __restrict__ dqkv,
                    int B, int T_, int H, int d, int qsplit) {
+  dependent_sync();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   int rs = Row<T>::stride(d);
   T* Ks = reinterpret_cast<T*>(smem_raw);
@@ -206,6 +208,7 @@ __global__ void __launch_bounds__(AT_WARPS * 32)
 attn_bwd_dkv_kernel(const T* __restrict__ qkv, const T* __restrict__ dout, const float* __restrict__ lse,
                     const float* __restrict__ delta, const float* __restrict__ cls_extra, T* __restrict__ dqkv,
                     int B, int T_, int H, int d, int ksplit) {
+  dependent_sync();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   int rs = Row<T>::stride(d);
   T* Qs = reinterpret_cast<T*>(smem_raw);
@@ -280,7 +283,7 @@ static int launch_fwd(const Ctx& c, const void* qkv, void* out, float* lse, floa
   int qs = split_for(c, B * H, T_);
   dim3 grid(B * H, qs);
   note_launch(1);
-  attn_fwd_kernel<T><<<grid, AT_WARPS * 32, smem, c.stream>>>((const T*)qkv, (T*)out, lse, cls_prob, B, T_, H, d, qs);
+  launch_k(attn_fwd_kernel<T>, grid, AT_WARPS * 32, smem, c.stream, (const T*)qkv, (T*)out, lse, cls_prob, B, T_, H, d, qs);
   return 0;
 }
 
@@ -303,8 +306,8 @@ static int launch_bwd(const Ctx& c, const void* qkv, const void* dout, const flo
   int qs = split_for(c, B * H, T_);
   dim3 grid(B * H, qs);
   note_launch(2);
-  attn_bwd_dq_kernel<T><<<grid, AT_WARPS * 32, smem1, c.stream>>>((const T*)qkv, (const T*)dout, lse, delta, cls_extra, (T*)dqkv, B, T_, H, d, qs);
-  attn_bwd_dkv_kernel<T><<<grid, AT_WARPS * 32, smem2, c.stream>>>((const T*)qkv, (const T*)dout, lse, delta, cls_extra, (T*)dqkv, B, T_, H, d, qs);
+  launch_k(attn_bwd_dq_kernel<T>, grid, AT_WARPS * 32, smem1, c.stream, (const T*)qkv, (const T*)dout, lse, delta, cls_extra, (T*)dqkv, B, T_, H, d, qs);
+  launch_k(attn_bwd_dkv_kernel<T>, grid, AT_WARPS * 32, smem2, c.stream, (const T*)qkv, (const T*)dout, lse, delta, cls_extra, (T*)dqkv, B, T_, H, d, qs);
   return 0;
 }
 
@@ -403,6 +406,7 @@ __device__ __forceinline__ void cls_row_probs(const T* kbase, long row_stride, c
 template <typename T>
 __global__ void __launch_bounds__(ATC_THREADS)
 attn_cls_fwd_kernel(const T* __restrict__ qkv, T* __restrict__ out_cls, int B, int T_, int H, int d) {
+  dependent_sync();
   __shared__ __align__(16) float qs[AT_MAXD];
   __shared__ float part[ATC_WARPS][AT_MAXD];
   __shared__ float red[ATC_WARPS];
@@ -442,6 +446,7 @@ attn_cls_fwd_kernel(const T* __restrict__ qkv, T* __restrict__ out_cls, int B, i
 template <typename T>
 __global__ void __launch_bounds__(ATC_THREADS)
 attn_cls_bwd_kernel(const T* __restrict__ qkv, const T* __restrict__ dout_cls, T* __restrict__ dqkv, int B, int T_, int H, int d) {
+  dependent_sync();
   __shared__ __align__(16) float qs[AT_MAXD];
   __shared__ __align__(16) float gs[AT_MAXD];
   __shared__ float part[ATC_WARPS][AT_MAXD];
@@ -507,8 +512,8 @@ static int launch_cls(const Ctx& c, bool bwd, const void* qkv, const void* io_cl
   if (d > AT_MAXD || (d % 8) != 0 || T_ < 1 || T_ > ATC_MAXKEYS) return -2;
   int blocks = B * H;
   note_launch(1);
-  if (bwd) attn_cls_bwd_kernel<T><<<blocks, ATC_THREADS, 0, c.stream>>>((const T*)qkv, (const T*)io_cls, (T*)dqkv, B, T_, H, d);
-  else attn_cls_fwd_kernel<T><<<blocks, ATC_THREADS, 0, c.stream>>>((const T*)qkv, (T*)const_cast<void*>(io_cls), B, T_, H, d);
+  if (bwd) launch_k(attn_cls_bwd_kernel<T>, blocks, ATC_THREADS, 0, c.stream, (const T*)qkv, (const T*)io_cls, (T*)dqkv, B, T_, H, d);
+  else launch_k(attn_cls_fwd_kernel<T>, blocks, ATC_THREADS, 0, c.stream, (const T*)qkv, (T*)const_cast<void*>(io_cls), B, T_, H, d);
   return 0;
 }
 

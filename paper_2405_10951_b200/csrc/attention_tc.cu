@@ -124,6 +124,8 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = tmem_slot;
+  if (leaves_sms_idle()) release_dependents();
+  await_inputs();
   volatile int* abortp = &abort_flag;
 
   if (warp == LOADER) {
@@ -383,6 +385,8 @@ attn_fwd_tc_long_kernel(const __grid_constant__ CUtensorMap map_qkv, bf16* __res
   __syncthreads();
   tc_fence_after();
   uint32_t tmem = tmem_slot;
+  if (leaves_sms_idle()) release_dependents();
+  await_inputs();
   constexpr uint32_t C_O = KB;
   volatile int* abortp = &abort_flag;
   const float c = 0.125f * 1.4426950408889634f;
@@ -602,6 +606,8 @@ attn_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_qkv, const __grid_con
   __syncthreads();
   tc_fence_after();
   uint32_t tmem = tmem_slot;
+  if (leaves_sms_idle()) release_dependents();
+  await_inputs();
   // dQ, dK, dV reuse the columns of S and dP, which are dead once P and dS sit in shared memory
   constexpr uint32_t C_S = 0, C_DP = 128, C_DQ = 0, C_DK = 64, C_DV = 128;
   volatile int* abortp = &abort_flag;
@@ -815,6 +821,8 @@ attn_bwd_tc256_kernel(const __grid_constant__ CUtensorMap map_qkv, const __grid_
   __syncthreads();
   tc_fence_after();
   uint32_t tmem = tmem_slot;
+  if (leaves_sms_idle()) release_dependents();
+  await_inputs();
   constexpr uint32_t C_S = 0, C_DP = 128, C_DQ = 256, C_DK = 384, C_DV = 448;
   volatile int* abortp = &abort_flag;
   const int tpad = (T + 15) & ~15;
@@ -1090,6 +1098,8 @@ attn_bwd_long_kernel(const __grid_constant__ CUtensorMap map_qkv, const __grid_c
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = tmem_slot;
+  if (leaves_sms_idle()) release_dependents();
+  await_inputs();
   constexpr uint32_t C_S = 0, C_DP = 64, C_A1 = 128, C_A2 = 192;          // A1: dQ or dK, A2: dV
   volatile int* abortp = &abort_flag;
   const uint32_t trow = tmem + ((uint32_t)((warp & 3) * 32) << 16);
@@ -1278,7 +1288,7 @@ int attention_fwd_tc(const Ctx& c, const void* qkv, void* out, float* lse, float
     if (!ensure_smem(lim_l, attn_fwd_tc_long_kernel, smem_l)) return -3;
     dim3 grid_l((T + AT_QROWS - 1) / AT_QROWS, B * H);
     note_launch(1);
-    attn_fwd_tc_long_kernel<<<grid_l, 128, smem_l, c.stream>>>(map, (bf16*)out, lse, cls_prob, B, T, H, c.status);
+    launch_k(attn_fwd_tc_long_kernel, grid_l, 128, smem_l, c.stream, map, (bf16*)out, lse, cls_prob, B, T, H, c.status);
     return 0;
   }
   int tpad = (T + 15) & ~15;
@@ -1298,7 +1308,7 @@ int attention_fwd_tc(const Ctx& c, const void* qkv, void* out, float* lse, float
   auto launch = [&](auto kern, int threads) -> int {
     if (!ensure_smem(lim[nbuf], kern, smem)) return -3;
     note_launch(1);
-    kern<<<grid, threads, smem, c.stream>>>(map_q, map_kv, (bf16*)out, lse, cls_prob, B, T, H, kvslots, c.status);
+    launch_k(kern, grid, threads, smem, c.stream, map_q, map_kv, (bf16*)out, lse, cls_prob, B, T, H, kvslots, c.status);
     return 0;
   };
   if (nbuf == 4) return launch(attn_fwd_ws_kernel<4>, 19 * 32);
@@ -1326,8 +1336,8 @@ int attention_bwd_tc(const Ctx& c, const void* qkv, const void* dout, const floa
     if (!ensure_smem(lim_q, attn_bwd_long_kernel<false>, smem_l) || !ensure_smem(lim_kv, attn_bwd_long_kernel<true>, smem_l)) return -3;
     dim3 grid((T + AT_QROWS - 1) / AT_QROWS, B * H);
     note_launch(2);
-    attn_bwd_long_kernel<false><<<grid, 256, smem_l, c.stream>>>(mq, mg, lse, delta, cls_extra, (bf16*)dqkv, B, T, H, c.status);
-    attn_bwd_long_kernel<true><<<grid, 256, smem_l, c.stream>>>(mq, mg, lse, delta, cls_extra, (bf16*)dqkv, B, T, H, c.status);
+    launch_k(attn_bwd_long_kernel<false>, grid, 256, smem_l, c.stream, mq, mg, lse, delta, cls_extra, (bf16*)dqkv, B, T, H, c.status);
+    launch_k(attn_bwd_long_kernel<true>, grid, 256, smem_l, c.stream, mq, mg, lse, delta, cls_extra, (bf16*)dqkv, B, T, H, c.status);
     return 0;
   }
   if (T > AT_QROWS) {                      // two tiles of queries and keys
@@ -1335,7 +1345,7 @@ int attention_bwd_tc(const Ctx& c, const void* qkv, const void* dout, const floa
     static SmemLimit lim2;
     if (!ensure_smem(lim2, attn_bwd_tc256_kernel, smem2)) return -3;
     note_launch(1);
-    attn_bwd_tc256_kernel<<<B * H, 256, smem2, c.stream>>>(mq, mg, lse, cls_extra, (bf16*)dqkv, B, T, H, c.status);
+    launch_k(attn_bwd_tc256_kernel, B * H, 256, smem2, c.stream, mq, mg, lse, cls_extra, (bf16*)dqkv, B, T, H, c.status);
     return 0;
   }
   size_t tile = 2 * (size_t)AT_BOX_BYTES, ch = (size_t)((T + 15) & ~15) * 128;
@@ -1343,7 +1353,7 @@ int attention_bwd_tc(const Ctx& c, const void* qkv, const void* dout, const floa
   static SmemLimit lim;
   if (!ensure_smem(lim, attn_bwd_tc_kernel, smem)) return -3;
   note_launch(1);
-  attn_bwd_tc_kernel<<<B * H, 256, smem, c.stream>>>(mq, mg, lse, cls_extra, (bf16*)dqkv, B, T, H, c.status);
+  launch_k(attn_bwd_tc_kernel, B * H, 256, smem, c.stream, mq, mg, lse, cls_extra, (bf16*)dqkv, B, T, H, c.status);
   return 0;
 }
 

@@ -13,6 +13,7 @@ __global__ void __launch_bounds__(SG_THREADS)
 gemm_simt_kernel(const T* __restrict__ A, long a_rs, long a_cs, const T* __restrict__ B, long b_rs, long b_cs,
                  TC* __restrict__ C, int M, int N, int K, const float* __restrict__ bias, const TC* __restrict__ residual,
                  int act, TC* __restrict__ aux_out, const T* __restrict__ aux_in) {
+  dependent_sync();
   __shared__ float As[SG_BK][SG_BM + 4];
   __shared__ float Bs[SG_BK][SG_BN + 4];
   int tid = threadIdx.x;
@@ -91,15 +92,15 @@ void gemm(const Ctx& c, const void* A, long a_rs, long a_cs, const void* B, long
   dim3 grid(ceil_div(n, SG_BN), ceil_div(m, SG_BM));
   note_launch(1);
   if (c.dtype == 0) {
-    gemm_simt_kernel<float, float><<<grid, SG_THREADS, 0, c.stream>>>(
+    launch_k(gemm_simt_kernel<float, float>, grid, SG_THREADS, 0, c.stream, 
         (const float*)A, a_rs, a_cs, (const float*)B, b_rs, b_cs, (float*)C, m, n, k, e.bias, (const float*)e.residual,
         e.act, (float*)e.aux_out, (const float*)e.aux_in);
   } else if (out_is_float) {
-    gemm_simt_kernel<bf16, float><<<grid, SG_THREADS, 0, c.stream>>>(
+    launch_k(gemm_simt_kernel<bf16, float>, grid, SG_THREADS, 0, c.stream, 
         (const bf16*)A, a_rs, a_cs, (const bf16*)B, b_rs, b_cs, (float*)C, m, n, k, e.bias, (const float*)e.residual,
         e.act, (float*)e.aux_out, (const bf16*)e.aux_in);
   } else {
-    gemm_simt_kernel<bf16, bf16><<<grid, SG_THREADS, 0, c.stream>>>(
+    launch_k(gemm_simt_kernel<bf16, bf16>, grid, SG_THREADS, 0, c.stream, 
         (const bf16*)A, a_rs, a_cs, (const bf16*)B, b_rs, b_cs, (bf16*)C, m, n, k, e.bias, (const bf16*)e.residual,
         e.act, (bf16*)e.aux_out, (const bf16*)e.aux_in);
   }

@@ -115,6 +115,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   __syncthreads();
   tc_fence_after();
   uint32_t tmem_base = tmem_base_slot;
+  if (leaves_sms_idle()) release_dependents();
+  await_inputs();
   volatile int* abortp = &abort_flag;
 
   if (warp == 0) {
@@ -297,6 +299,7 @@ __global__ void wait_expiry_kernel(int* status, unsigned long long limit_ns) {
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  dependent_sync();
   if (threadIdx.x == 0) mbar_wait_ns(bar, 0, &abort_flag, limit_ns);
   tc_fence_before();
   __syncthreads();
@@ -307,6 +310,7 @@ __global__ void wait_expiry_kernel(int* status, unsigned long long limit_ns) {
 
 // out[i] = sum over splits of partial[s][i], ascending s.
 __global__ void splitk_reduce_kernel(const float* __restrict__ partial, float* __restrict__ out, size_t n, int splits) {
+  dependent_sync();
   size_t i = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) * 4;
   if (i >= n) return;
   float4 acc = *reinterpret_cast<const float4*>(partial + i);
@@ -321,6 +325,7 @@ __global__ void splitk_reduce_kernel(const float* __restrict__ partial, float* _
 // pre-activation, GELU derivative of a stored pre-activation, residual), for products whose few tiles are split along k.
 template <typename TOut>
 __global__ void splitk_reduce_epi_kernel(const float* __restrict__ partial, TOut* __restrict__ out, int m, int n, int splits, Epi ep) {
+  dependent_sync();
   size_t total = (size_t)m * n;
   size_t i = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) * 4;
   if (i >= total) return;
@@ -405,7 +410,7 @@ static int launch(const Ctx& c, const CUtensorMap& ma, const CUtensorMap& mb, vo
   int sms = c.sm_count > 0 ? c.sm_count : 148;
   int grid = work < sms ? work : sms;
   note_launch(1);
-  kern<<<grid, THREADS, SMEM_BYTES, c.stream>>>(ma, mb, (TOut*)C, m, n, k, ep, tiles_m, tiles_n, splits, kb_per_split, grp, c.status);
+  launch_k(kern, grid, THREADS, SMEM_BYTES, c.stream, ma, mb, (TOut*)C, m, n, k, ep, tiles_m, tiles_n, splits, kb_per_split, grp, c.status);
   return 0;
 }
 
@@ -413,12 +418,12 @@ static int launch(const Ctx& c, const CUtensorMap& ma, const CUtensorMap& mb, vo
 
 void wait_expiry_selftest(const Ctx& c, unsigned long long limit_ns) {
   note_launch(1);
-  tc::wait_expiry_kernel<<<1, 32, 0, c.stream>>>(c.status, limit_ns);
+  launch_k(tc::wait_expiry_kernel, 1, 32, 0, c.stream, c.status, limit_ns);
 }
 
 void splitk_reduce(cudaStream_t s, const float* partial, float* out, size_t n, int splits) {
   note_launch(1);
-  tc::splitk_reduce_kernel<<<ceil_div((long)(n / 4), 256), 256, 0, s>>>(partial, out, n, splits);
+  launch_k(tc::splitk_reduce_kernel, ceil_div((long)(n / 4), 256), 256, 0, s, partial, out, n, splits);
 }
 
 bool gemm_tc_supported(int m, int n, int k) { return m >= 1 && n >= 8 && k >= 8 && (n % 8) == 0 && (k % 8) == 0; }
@@ -499,8 +504,8 @@ int gemm_tc_strided(const Ctx& c, const void* A, long a_rs, long a_cs, const voi
     } else {
       note_launch(1);
       int blocks = ceil_div((long)(total / 4), 256);
-      if (final_is_float) splitk_reduce_epi_kernel<float><<<blocks, 256, 0, c.stream>>>(split_ws, (float*)C, m, n, splits, ep_full);
-      else splitk_reduce_epi_kernel<bf16><<<blocks, 256, 0, c.stream>>>(split_ws, (bf16*)C, m, n, splits, ep_full);
+      if (final_is_float) launch_k(splitk_reduce_epi_kernel<float>, blocks, 256, 0, c.stream, split_ws, (float*)C, m, n, splits, ep_full);
+      else launch_k(splitk_reduce_epi_kernel<bf16>, blocks, 256, 0, c.stream, split_ws, (bf16*)C, m, n, splits, ep_full);
     }
   }
   if (c.prof != nullptr && c.prof->on) c.prof->end(c.stream);

@@ -15,6 +15,7 @@ long g_kernel_launches = 0;
 template <typename T>
 __global__ void patchify_kernel(const T* __restrict__ img, T* __restrict__ out, int B, int C, int S, int P, long total,
                                 const long long* __restrict__ img_offset) {
+  dependent_sync();
   long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= total) return;
   if (img_offset != nullptr) img += *img_offset;
@@ -32,6 +33,7 @@ __global__ void patchify_kernel(const T* __restrict__ img, T* __restrict__ out, 
 template <typename T>
 __global__ void patchify_vec_kernel(const T* __restrict__ img, T* __restrict__ out, int B, int C, int S, int P, long units,
                                     const long long* __restrict__ img_offset) {
+  dependent_sync();
   constexpr int E = 16 / sizeof(T);
   long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= units) return;
@@ -59,15 +61,15 @@ void patchify(const Ctx& c, const void* images, void* patches, int B, int C, int
   if (vec) {
     long units = total * (long)es / 16;
     int blocks = ceil_div(units, threads);
-    if (c.dtype == 0) patchify_vec_kernel<float><<<blocks, threads, 0, c.stream>>>((const float*)images, (float*)patches, B, C, S, P, units, img_offset);
-    else patchify_vec_kernel<bf16><<<blocks, threads, 0, c.stream>>>((const bf16*)images, (bf16*)patches, B, C, S, P, units, img_offset);
+    if (c.dtype == 0) launch_k(patchify_vec_kernel<float>, blocks, threads, 0, c.stream, (const float*)images, (float*)patches, B, C, S, P, units, img_offset);
+    else launch_k(patchify_vec_kernel<bf16>, blocks, threads, 0, c.stream, (const bf16*)images, (bf16*)patches, B, C, S, P, units, img_offset);
     return;
   }
   int blocks = ceil_div(total, threads);
   if (c.dtype == 0)
-    patchify_kernel<float><<<blocks, threads, 0, c.stream>>>((const float*)images, (float*)patches, B, C, S, P, total, img_offset);
+    launch_k(patchify_kernel<float>, blocks, threads, 0, c.stream, (const float*)images, (float*)patches, B, C, S, P, total, img_offset);
   else
-    patchify_kernel<bf16><<<blocks, threads, 0, c.stream>>>((const bf16*)images, (bf16*)patches, B, C, S, P, total, img_offset);
+    launch_k(patchify_kernel<bf16>, blocks, threads, 0, c.stream, (const bf16*)images, (bf16*)patches, B, C, S, P, total, img_offset);
 }
 
 // x[b, 0] = cls + pos[0];  x[b, 1 + n] = emb[b, n] + pos[1 + n]   (classification token and positional embedding);
@@ -75,6 +77,7 @@ void patchify(const Ctx& c, const void* images, void* patches, int B, int C, int
 template <typename T>
 __global__ void assemble_kernel(const T* __restrict__ emb, const float* __restrict__ cls, const float* __restrict__ pos,
                                 float* __restrict__ x, int B, int N, int D, long total4) {
+  dependent_sync();
   long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= total4) return;
   int d4 = D / 4;
@@ -95,9 +98,9 @@ void assemble_tokens(const Ctx& c, const void* emb, const float* cls, const floa
   long total4 = (long)B * (N + 1) * D / 4;
   int threads = 256, blocks = ceil_div(total4, threads);
   if (c.dtype == 0)
-    assemble_kernel<float><<<blocks, threads, 0, c.stream>>>((const float*)emb, cls, pos, x, B, N, D, total4);
+    launch_k(assemble_kernel<float>, blocks, threads, 0, c.stream, (const float*)emb, cls, pos, x, B, N, D, total4);
   else
-    assemble_kernel<bf16><<<blocks, threads, 0, c.stream>>>((const bf16*)emb, cls, pos, x, B, N, D, total4);
+    launch_k(assemble_kernel<bf16>, blocks, threads, 0, c.stream, (const bf16*)emb, cls, pos, x, B, N, D, total4);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -111,6 +114,7 @@ template <typename TY, int NCH>
 __global__ void layernorm_fwd_kernel(const float* __restrict__ x, long x_stride, const float* __restrict__ g,
                                      const float* __restrict__ b, TY* __restrict__ y, float* __restrict__ mean,
                                      float* __restrict__ rstd, int rows, int D, float eps) {
+  dependent_sync();
   int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   int lane = threadIdx.x & 31;
   if (warp >= rows) return;
@@ -164,7 +168,7 @@ static void launch_ln_fwd(const Ctx& c, const float* x, long x_stride, const flo
   int threads = 256;
   int blocks = ceil_div((long)rows * 32, threads);
   int nch = ceil_div(D, 128);
-#define BSR_LN_FWD(N) layernorm_fwd_kernel<TY, N><<<blocks, threads, 0, c.stream>>>(x, x_stride, g, b, y, mean, rstd, rows, D, eps)
+#define BSR_LN_FWD(N) launch_k(layernorm_fwd_kernel<TY, N>, blocks, threads, 0, c.stream, x, x_stride, g, b, y, mean, rstd, rows, D, eps)
   if (nch <= 2) BSR_LN_FWD(2); else if (nch == 3) BSR_LN_FWD(3); else if (nch == 4) BSR_LN_FWD(4); else if (nch <= 6) BSR_LN_FWD(6); else BSR_LN_FWD(8);
 #undef BSR_LN_FWD
 }
@@ -192,6 +196,7 @@ __device__ __forceinline__ float e4m3_scale(float amax) { return amax > 0.f ? __
 
 // One warp per row (cols % 4 == 0): scale = max|row| / 448, q = round(x / scale).
 __global__ void quantize_rows_e4m3_kernel(const bf16* __restrict__ x, int rows, int cols, uint8_t* __restrict__ q, float* __restrict__ scale) {
+  dependent_sync();
   int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (warp >= rows) return;
   const bf16* xr = x + (size_t)warp * cols;
@@ -214,7 +219,7 @@ __global__ void quantize_rows_e4m3_kernel(const bf16* __restrict__ x, int rows, 
 }
 void quantize_rows_e4m3(const Ctx& c, const void* x, int rows, int cols, void* q, float* scale) {
   note_launch(1);
-  quantize_rows_e4m3_kernel<<<ceil_div((long)rows * 32, 256), 256, 0, c.stream>>>((const bf16*)x, rows, cols, (uint8_t*)q, scale);
+  launch_k(quantize_rows_e4m3_kernel, ceil_div((long)rows * 32, 256), 256, 0, c.stream, (const bf16*)x, rows, cols, (uint8_t*)q, scale);
 }
 
 // E4M3 byte to float: sign, exponent (bias 7) and mantissa unpacked by hand (subnormals: exponent field 0).
@@ -225,13 +230,14 @@ __device__ __forceinline__ float from_e4m3(uint8_t b) {
 }
 __global__ void dequantize_rows_e4m3_kernel(const uint8_t* __restrict__ q, const float* __restrict__ scale, int rows, int cols,
                                             float* __restrict__ out) {
+  dependent_sync();
   size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= (size_t)rows * cols) return;
   out[i] = from_e4m3(q[i]) * scale[i / cols];
 }
 void dequantize_rows_e4m3(const Ctx& c, const void* q, const float* scale, int rows, int cols, float* out) {
   note_launch(1);
-  dequantize_rows_e4m3_kernel<<<ceil_div((long)rows * cols, 256), 256, 0, c.stream>>>((const uint8_t*)q, scale, rows, cols, out);
+  launch_k(dequantize_rows_e4m3_kernel, ceil_div((long)rows * cols, 256), 256, 0, c.stream, (const uint8_t*)q, scale, rows, cols, out);
 }
 
 // LayerNorm forward whose output row goes out as E4M3 with scale max|y| / 448: the row is already in the warp's
@@ -240,6 +246,7 @@ template <int NCH>
 __global__ void layernorm_fwd_e4m3_kernel(const float* __restrict__ x, long x_stride, const float* __restrict__ g,
                                           const float* __restrict__ b, uint8_t* __restrict__ yq, float* __restrict__ y_scale,
                                           int rows, int D, float eps) {
+  dependent_sync();
   int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   int lane = threadIdx.x & 31;
   if (warp >= rows) return;
@@ -297,7 +304,7 @@ void layernorm_fwd_e4m3(const Ctx& c, const float* x, long x_stride, const float
   int threads = 256;
   int blocks = ceil_div((long)rows * 32, threads);
   int nch = ceil_div(D, 128);
-#define BSR_LN_Q(N) layernorm_fwd_e4m3_kernel<N><<<blocks, threads, 0, c.stream>>>(x, x_stride, g, b, (uint8_t*)yq, y_scale, rows, D, eps)
+#define BSR_LN_Q(N) launch_k(layernorm_fwd_e4m3_kernel<N>, blocks, threads, 0, c.stream, x, x_stride, g, b, (uint8_t*)yq, y_scale, rows, D, eps)
   if (nch <= 2) BSR_LN_Q(2); else if (nch == 3) BSR_LN_Q(3); else if (nch == 4) BSR_LN_Q(4); else if (nch <= 6) BSR_LN_Q(6); else BSR_LN_Q(8);
 #undef BSR_LN_Q
 }
@@ -314,6 +321,7 @@ __global__ void __launch_bounds__(256, 2) layernorm_bwd_kernel(const TDY* __rest
                                      const float* __restrict__ mean, const float* __restrict__ rstd,
                                      const float* __restrict__ g, const float* __restrict__ dres, float* __restrict__ dx,
                                      long dx_stride, TC* __restrict__ dx_copy, float* __restrict__ partials, int rows, int D, int nsum) {
+  dependent_sync();
   extern __shared__ float sm[];   // [LNB_WARPS][nsum][D]: dgamma, dbeta and (nsum == 3) the column sums of dx
   int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int chunks = D / 4;
@@ -407,7 +415,8 @@ __global__ void __launch_bounds__(256, 2) layernorm_bwd_kernel(const TDY* __rest
 // out_y[col] = sum over groups of partials[y][group][col] for y = blockIdx.y (one or two outputs per launch).
 // 16 lanes stride the groups and are combined through shared memory in lane order: the result is deterministic.
 __global__ void reduce_partials_kernel(const float* __restrict__ partials, int groups, int cols, float* __restrict__ out0,
-                                       float* __restrict__ out1, float* __restrict__ out2 = nullptr) {
+                                       float* __restrict__ out1, float* __restrict__ out2) {
+  dependent_sync();
   __shared__ float sm[16][17];
   int cx = threadIdx.x & 15, gy = threadIdx.x >> 4;
   int col = blockIdx.x * 16 + cx;
@@ -441,7 +450,7 @@ static void launch_ln_bwd(const Ctx& c, int groups, size_t smem, const void* dy,
   do {                                                                                                                  \
     static SmemLimit lim;                                                                                               \
     ensure_smem(lim, layernorm_bwd_kernel<TDY, TC, N>, smem);                                                           \
-    layernorm_bwd_kernel<TDY, TC, N><<<groups, LNB_WARPS * 32, smem, c.stream>>>((const TDY*)dy, x, x_stride, mean, rstd, g, dres, \
+    launch_k(layernorm_bwd_kernel<TDY, TC, N>, groups, LNB_WARPS * 32, smem, c.stream, (const TDY*)dy, x, x_stride, mean, rstd, g, dres, \
                                                                                  dx, dx_stride, (TC*)dx_copy, partials, rows, D, nsum); \
   } while (0)
   if (nch <= 2) BSR_LN_BWD(2); else if (nch == 3) BSR_LN_BWD(3); else if (nch == 4) BSR_LN_BWD(4); else if (nch <= 6) BSR_LN_BWD(6); else BSR_LN_BWD(8);
@@ -465,7 +474,7 @@ void layernorm_bwd(const Ctx& c, const void* dy, int dy_is_float, const float* x
   if (dgamma == nullptr && nsum == 2) return;                          // a frozen block in the gradient path: only dx is wanted
   dim3 grid(ceil_div(D, 16), nsum);
   cudaStream_t rs = side_begin(c);                                     // only the optimiser reads these sums
-  reduce_partials_kernel<<<grid, 256, 0, rs>>>(partials, groups, D, dgamma, dbeta, nsum == 3 ? dx_colsum : nullptr);
+  launch_k(reduce_partials_kernel, grid, 256, 0, rs, partials, groups, D, dgamma, dbeta, nsum == 3 ? dx_colsum : nullptr);
   side_end(c, 0);
 }
 
@@ -477,6 +486,7 @@ constexpr int CS_GROUPS = 64;
 
 template <typename T>
 __global__ void colsum_kernel(const T* __restrict__ x, int rows, int cols, float* __restrict__ partials) {
+  dependent_sync();
   constexpr int N = Pack<T>::N;
   __shared__ float sm[CS_ROWLANES][32 * N];
   int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
@@ -531,13 +541,13 @@ void colsum(const Ctx& c, const void* x, int rows, int cols, float* partials, fl
   side_join(c, 1);
   if (c.dtype == 0) {
     dim3 grid(ceil_div(cols, 32 * 4), groups);
-    colsum_kernel<float><<<grid, threads, 0, c.stream>>>((const float*)x, rows, cols, partials);
+    launch_k(colsum_kernel<float>, grid, threads, 0, c.stream, (const float*)x, rows, cols, partials);
   } else {
     dim3 grid(ceil_div(cols, 32 * 8), groups);
-    colsum_kernel<bf16><<<grid, threads, 0, c.stream>>>((const bf16*)x, rows, cols, partials);
+    launch_k(colsum_kernel<bf16>, grid, threads, 0, c.stream, (const bf16*)x, rows, cols, partials);
   }
   cudaStream_t rs = side_begin(c);
-  reduce_partials_kernel<<<dim3(ceil_div(cols, 16), 1), 256, 0, rs>>>(partials, groups, cols, out, out);
+  launch_k(reduce_partials_kernel, dim3(ceil_div(cols, 16), 1), 256, 0, rs, partials, groups, cols, out, out, nullptr);
   side_end(c, 1);
 }
 
@@ -556,6 +566,7 @@ struct HeadDev {
 template <typename T>
 __global__ void head_fwd_kernel(HeadDev h, const float* __restrict__ xn, const int* __restrict__ task_ids,
                                 float* __restrict__ logits, int B) {
+  dependent_sync();
   int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (warp >= B * h.cmax) return;
   int b = warp / h.cmax, cls = warp % h.cmax;
@@ -582,14 +593,15 @@ static HeadDev to_dev(const HeadDesc& h) {
 void head_fwd(const Ctx& c, const HeadDesc& h, const float* xn, const int* task_ids, float* logits, int B) {
   note_launch(1);
   int threads = 256, blocks = ceil_div((long)B * h.cmax * 32, threads);
-  if (c.dtype == 0) head_fwd_kernel<float><<<blocks, threads, 0, c.stream>>>(to_dev(h), xn, task_ids, logits, B);
-  else head_fwd_kernel<bf16><<<blocks, threads, 0, c.stream>>>(to_dev(h), xn, task_ids, logits, B);
+  if (c.dtype == 0) launch_k(head_fwd_kernel<float>, blocks, threads, 0, c.stream, to_dev(h), xn, task_ids, logits, B);
+  else launch_k(head_fwd_kernel<bf16>, blocks, threads, 0, c.stream, to_dev(h), xn, task_ids, logits, B);
 }
 
 // One warp per image: loss_b = logsumexp(logits) - logits[label]; dlogits = (softmax - onehot) / B.
 __global__ void cross_entropy_kernel(HeadDev h, const float* __restrict__ logits, const int* __restrict__ labels,
                                      const int* __restrict__ task_ids, float* __restrict__ per_image,
                                      float* __restrict__ dlogits, int B, int* status) {
+  dependent_sync();
   int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (warp >= B) return;
   int t = task_ids ? task_ids[warp] : 0;
@@ -623,6 +635,7 @@ __global__ void cross_entropy_kernel(HeadDev h, const float* __restrict__ logits
 
 // Single warp: mean of the per-image losses, lanes stride the images, fixed order.
 __global__ void loss_reduce_kernel(const float* __restrict__ per_image, int B, float* __restrict__ loss, int* status) {
+  dependent_sync();
   int lane = threadIdx.x;
   float s = 0.f;
   for (int i = lane; i < B; i += 32) s += per_image[i];
@@ -638,13 +651,14 @@ void cross_entropy(const Ctx& c, const HeadDesc& h, const float* logits, const i
                    float* per_image, float* dlogits, float* loss, int B) {
   note_launch(2);
   int threads = 128, blocks = ceil_div((long)B * 32, threads);
-  cross_entropy_kernel<<<blocks, threads, 0, c.stream>>>(to_dev(h), logits, labels, task_ids, per_image, dlogits, B, c.status);
-  loss_reduce_kernel<<<1, 32, 0, c.stream>>>(per_image, B, loss, c.status);
+  launch_k(cross_entropy_kernel, blocks, threads, 0, c.stream, to_dev(h), logits, labels, task_ids, per_image, dlogits, B, c.status);
+  launch_k(loss_reduce_kernel, 1, 32, 0, c.stream, per_image, B, loss, c.status);
 }
 
 // dW_t[c, d] = sum_b [task(b) = t] dlogits[b, c] xn[b, d];  db_t[c] = sum_b [..] dlogits[b, c]
 __global__ void head_wgrad_kernel(HeadDev h, const float* __restrict__ xn, const float* __restrict__ dlogits,
                                   const int* __restrict__ task_ids, int B, int t) {
+  dependent_sync();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   int n = h.ncls[t];
   if (i >= n * (h.D + 1)) return;
@@ -665,6 +679,7 @@ __global__ void head_wgrad_kernel(HeadDev h, const float* __restrict__ xn, const
 template <typename T>
 __global__ void head_dgrad_kernel(HeadDev h, const float* __restrict__ dlogits, const int* __restrict__ task_ids,
                                   float* __restrict__ dxn, int B) {
+  dependent_sync();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= B * h.D) return;
   int b = i / h.D, d = i % h.D;
@@ -680,11 +695,11 @@ void head_bwd(const Ctx& c, const HeadDesc& h, const float* xn, const float* dlo
   HeadDev hd = to_dev(h);
   for (int t = 0; t < h.num_tasks; ++t) {
     int total = h.ncls[t] * (h.D + 1);
-    head_wgrad_kernel<<<ceil_div(total, 128), 128, 0, c.stream>>>(hd, xn, dlogits, task_ids, B, t);
+    launch_k(head_wgrad_kernel, ceil_div(total, 128), 128, 0, c.stream, hd, xn, dlogits, task_ids, B, t);
   }
   int total = B * h.D;
-  if (c.dtype == 0) head_dgrad_kernel<float><<<ceil_div(total, 128), 128, 0, c.stream>>>(hd, dlogits, task_ids, dxn, B);
-  else head_dgrad_kernel<bf16><<<ceil_div(total, 128), 128, 0, c.stream>>>(hd, dlogits, task_ids, dxn, B);
+  if (c.dtype == 0) launch_k(head_dgrad_kernel<float>, ceil_div(total, 128), 128, 0, c.stream, hd, dlogits, task_ids, dxn, B);
+  else launch_k(head_dgrad_kernel<bf16>, ceil_div(total, 128), 128, 0, c.stream, hd, dlogits, task_ids, dxn, B);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -697,6 +712,7 @@ __global__ void adamw_kernel(const AdamChunk* __restrict__ chunks, float* __rest
                              const float* __restrict__ grad, float* __restrict__ m, float* __restrict__ v,
                              T* __restrict__ shadow_base, const float* __restrict__ scalars, float b1, float b2, float eps,
                              float wd) {
+  dependent_sync();
   // step-dependent scalars live in device memory so that a captured graph of the step stays valid: lr, 1-b1^t, 1-b2^t
   float lr = scalars[0], bc1 = scalars[1], bc2 = scalars[2];
   AdamChunk ch = chunks[blockIdx.x];
@@ -720,6 +736,7 @@ template <typename T>
 __global__ void sgd_kernel(const AdamChunk* __restrict__ chunks, float* __restrict__ master, const float* __restrict__ grad,
                            float* __restrict__ buf, T* __restrict__ shadow_base, const float* __restrict__ scalars, float mu,
                            float wd) {
+  dependent_sync();
   float lr = scalars[0];
   AdamChunk ch = chunks[blockIdx.x];
   float decay = ch.decay ? wd : 0.f;
@@ -739,9 +756,9 @@ void sgd_momentum(const Ctx& c, const AdamChunk* chunks, int nchunks, float* mas
   if (nchunks <= 0) return;
   note_launch(1);
   if (c.dtype == 0)
-    sgd_kernel<float><<<nchunks, 256, 0, c.stream>>>(chunks, master, grad, buf, (float*)shadow_base, scalars, mu, wd);
+    launch_k(sgd_kernel<float>, nchunks, 256, 0, c.stream, chunks, master, grad, buf, (float*)shadow_base, scalars, mu, wd);
   else
-    sgd_kernel<bf16><<<nchunks, 256, 0, c.stream>>>(chunks, master, grad, buf, (bf16*)shadow_base, scalars, mu, wd);
+    launch_k(sgd_kernel<bf16>, nchunks, 256, 0, c.stream, chunks, master, grad, buf, (bf16*)shadow_base, scalars, mu, wd);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -751,11 +768,13 @@ void sgd_momentum(const Ctx& c, const AdamChunk* chunks, int nchunks, float* mas
 // ------------------------------------------------------------------------------------------------
 __global__ void loop_init_kernel(LoopState* st, long long step_done, long long total, long long image_stride, float lr_max,
                                  float lr_min, float b1, float b2, int n) {
+  dependent_sync();
   st->step_done = step_done; st->total_steps = total; st->image_stride = image_stride; st->image_offset = 0;
   st->lr_max = lr_max; st->lr_min = lr_min; st->beta1 = b1; st->beta2 = b2; st->i = 0; st->n = n;
 }
 __global__ void loop_begin_kernel(LoopState* st, float* scalars, const int* __restrict__ labels, const int* __restrict__ tasks,
                                   int* __restrict__ lab_stage, int* __restrict__ task_stage, int batch) {
+  dependent_sync();
   int i = st->i;
   for (int j = threadIdx.x; j < batch; j += blockDim.x) {
     lab_stage[j] = labels[(long)i * batch + j];
@@ -772,6 +791,7 @@ __global__ void loop_begin_kernel(LoopState* st, float* scalars, const int* __re
   }
 }
 __global__ void loop_end_kernel(LoopState* st, const float* __restrict__ loss, float* __restrict__ loss_out) {
+  dependent_sync();
   loss_out[st->i] = *loss;
   st->i += 1;
   st->step_done += 1;
@@ -779,19 +799,20 @@ __global__ void loop_end_kernel(LoopState* st, const float* __restrict__ loss, f
 void loop_init(cudaStream_t s, LoopState* st, long long step_done, long long total, long long image_stride, float lr_max, float lr_min,
                float b1, float b2, int n) {
   note_launch(1);
-  loop_init_kernel<<<1, 1, 0, s>>>(st, step_done, total, image_stride, lr_max, lr_min, b1, b2, n);
+  launch_k(loop_init_kernel, 1, 1, 0, s, st, step_done, total, image_stride, lr_max, lr_min, b1, b2, n);
 }
 void loop_begin(cudaStream_t s, LoopState* st, float* scalars, const int* labels, const int* tasks, int* lab_stage, int* task_stage, int batch) {
   note_launch(1);
-  loop_begin_kernel<<<1, 256, 0, s>>>(st, scalars, labels, tasks, lab_stage, task_stage, batch);
+  launch_k(loop_begin_kernel, 1, 256, 0, s, st, scalars, labels, tasks, lab_stage, task_stage, batch);
 }
 void loop_end(cudaStream_t s, LoopState* st, const float* loss, float* loss_out) {
   note_launch(1);
-  loop_end_kernel<<<1, 1, 0, s>>>(st, loss, loss_out);
+  launch_k(loop_end_kernel, 1, 1, 0, s, st, loss, loss_out);
 }
 
 // Guard words after every workspace slice: one warp per guard.
 __global__ void guards_write_kernel(char* base, const unsigned long long* __restrict__ table, int n, int words, uint32_t word) {
+  dependent_sync();
   int g = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (g >= n) return;
   uint32_t* p = reinterpret_cast<uint32_t*>(base + table[g]);
@@ -799,6 +820,7 @@ __global__ void guards_write_kernel(char* base, const unsigned long long* __rest
 }
 __global__ void guards_check_kernel(const char* base, const unsigned long long* __restrict__ table, int n, int words, uint32_t word,
                                     int* status) {
+  dependent_sync();
   int g = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (g >= n) return;
   const uint32_t* p = reinterpret_cast<const uint32_t*>(base + table[g]);
@@ -808,19 +830,20 @@ __global__ void guards_check_kernel(const char* base, const unsigned long long* 
 }
 void guards_write(cudaStream_t s, char* base, const unsigned long long* table, int n, int words, uint32_t word) {
   note_launch(1);
-  guards_write_kernel<<<ceil_div((long)n * 32, 256), 256, 0, s>>>(base, table, n, words, word);
+  launch_k(guards_write_kernel, ceil_div((long)n * 32, 256), 256, 0, s, base, table, n, words, word);
 }
 void guards_check(cudaStream_t s, const char* base, const unsigned long long* table, int n, int words, uint32_t word, int* status) {
   note_launch(1);
-  guards_check_kernel<<<ceil_div((long)n * 32, 256), 256, 0, s>>>(base, table, n, words, word, status);
+  launch_k(guards_check_kernel, ceil_div((long)n * 32, 256), 256, 0, s, base, table, n, words, word, status);
 }
 
 __global__ void set_scalars_kernel(float* dst, float a, float b, float c3) {
+  dependent_sync();
   dst[0] = a; dst[1] = b; dst[2] = c3;
 }
 void set_scalars(cudaStream_t s, float* dst, float a, float b, float c3) {
   note_launch(1);
-  set_scalars_kernel<<<1, 1, 0, s>>>(dst, a, b, c3);
+  launch_k(set_scalars_kernel, 1, 1, 0, s, dst, a, b, c3);
 }
 
 void adamw(const Ctx& c, const AdamChunk* chunks, int nchunks, float* master, const float* grad, float* m, float* v,
@@ -828,9 +851,9 @@ void adamw(const Ctx& c, const AdamChunk* chunks, int nchunks, float* master, co
   if (nchunks <= 0) return;
   note_launch(1);
   if (c.dtype == 0)
-    adamw_kernel<float><<<nchunks, 256, 0, c.stream>>>(chunks, master, grad, m, v, (float*)shadow_base, scalars, b1, b2, eps, wd);
+    launch_k(adamw_kernel<float>, nchunks, 256, 0, c.stream, chunks, master, grad, m, v, (float*)shadow_base, scalars, b1, b2, eps, wd);
   else
-    adamw_kernel<bf16><<<nchunks, 256, 0, c.stream>>>(chunks, master, grad, m, v, (bf16*)shadow_base, scalars, b1, b2, eps, wd);
+    launch_k(adamw_kernel<bf16>, nchunks, 256, 0, c.stream, chunks, master, grad, m, v, (bf16*)shadow_base, scalars, b1, b2, eps, wd);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -839,6 +862,7 @@ void adamw(const Ctx& c, const AdamChunk* chunks, int nchunks, float* master, co
 // ------------------------------------------------------------------------------------------------
 __global__ void copy_rows_kernel(const char* __restrict__ src, long src_pitch, char* __restrict__ dst, long dst_pitch, int rows,
                                  int units) {
+  dependent_sync();
   long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= (long)rows * units) return;
   int r = (int)(i / units), u = (int)(i % units);
@@ -849,7 +873,7 @@ void copy_rows(cudaStream_t st, const void* src, long src_pitch_bytes, void* dst
   note_launch(1);
   int units = row_bytes / 16;
   long total = (long)rows * units;
-  copy_rows_kernel<<<ceil_div(total, 256), 256, 0, st>>>((const char*)src, src_pitch_bytes, (char*)dst, dst_pitch_bytes, rows, units);
+  launch_k(copy_rows_kernel, ceil_div(total, 256), 256, 0, st, (const char*)src, src_pitch_bytes, (char*)dst, dst_pitch_bytes, rows, units);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -857,15 +881,18 @@ void copy_rows(cudaStream_t st, const void* src, long src_pitch_bytes, void* dst
 // ------------------------------------------------------------------------------------------------
 template <typename T>
 __global__ void from_float_kernel(const float* __restrict__ s, T* __restrict__ d, size_t n) {
+  dependent_sync();
   size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) d[i] = from_f<T>(s[i]);
 }
 template <typename T>
 __global__ void to_float_kernel(const T* __restrict__ s, float* __restrict__ d, size_t n) {
+  dependent_sync();
   size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) d[i] = to_f(s[i]);
 }
 __global__ void fill_kernel(float* d, float v, size_t n) {
+  dependent_sync();
   size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) d[i] = v;
 }
@@ -874,29 +901,30 @@ void convert_from_float(const Ctx& c, const float* src, void* dst, size_t n) {
   note_launch(1);
   if (n == 0) return;
   int blocks = ceil_div((long)n, 256);
-  if (c.dtype == 0) from_float_kernel<float><<<blocks, 256, 0, c.stream>>>(src, (float*)dst, n);
-  else from_float_kernel<bf16><<<blocks, 256, 0, c.stream>>>(src, (bf16*)dst, n);
+  if (c.dtype == 0) launch_k(from_float_kernel<float>, blocks, 256, 0, c.stream, src, (float*)dst, n);
+  else launch_k(from_float_kernel<bf16>, blocks, 256, 0, c.stream, src, (bf16*)dst, n);
 }
 void convert_to_float(const Ctx& c, const void* src, float* dst, size_t n) {
   note_launch(1);
   if (n == 0) return;
   int blocks = ceil_div((long)n, 256);
-  if (c.dtype == 0) to_float_kernel<float><<<blocks, 256, 0, c.stream>>>((const float*)src, dst, n);
-  else to_float_kernel<bf16><<<blocks, 256, 0, c.stream>>>((const bf16*)src, dst, n);
+  if (c.dtype == 0) launch_k(to_float_kernel<float>, blocks, 256, 0, c.stream, (const float*)src, dst, n);
+  else launch_k(to_float_kernel<bf16>, blocks, 256, 0, c.stream, (const bf16*)src, dst, n);
 }
 __global__ void int_to_float_kernel(const int* s, float* d, size_t n) {
+  dependent_sync();
   size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) d[i] = (float)s[i];
 }
 void convert_int_to_float(cudaStream_t st, const int* src, float* dst, size_t n) {
   if (n == 0) return;
   note_launch(1);
-  int_to_float_kernel<<<ceil_div((long)n, 256), 256, 0, st>>>(src, dst, n);
+  launch_k(int_to_float_kernel, ceil_div((long)n, 256), 256, 0, st, src, dst, n);
 }
 void fill_float(cudaStream_t s, float* dst, float v, size_t n) {
   note_launch(1);
   if (n == 0) return;
-  fill_kernel<<<ceil_div((long)n, 256), 256, 0, s>>>(dst, v, n);
+  launch_k(fill_kernel, ceil_div((long)n, 256), 256, 0, s, dst, v, n);
 }
 
 }  // namespace bsr

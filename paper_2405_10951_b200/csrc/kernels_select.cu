@@ -17,6 +17,7 @@ constexpr int SEL_WARPS = 4;
 
 __global__ void token_select_kernel(const float* __restrict__ p, int B, int H, int M, int k,
                                     float* __restrict__ scores, int* __restrict__ kept, int* __restrict__ dropped) {
+  dependent_sync();
   extern __shared__ uint32_t keys_all[];
   int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int b = blockIdx.x * SEL_WARPS + warp;
@@ -70,6 +71,7 @@ template <int IPL>
 __global__ void __launch_bounds__(SEL_WARPS * 32)
 token_select_reg_kernel(const float* __restrict__ p, int B, int H, int M, int k, float* __restrict__ scores,
                         int* __restrict__ kept, int* __restrict__ dropped) {
+  dependent_sync();
   int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int b = blockIdx.x * SEL_WARPS + warp;
   if (b >= B) return;
@@ -151,11 +153,11 @@ token_select_reg_kernel(const float* __restrict__ p, int B, int H, int M, int k,
 void token_select(cudaStream_t s, const float* p, int B, int H, int M, int k, float* scores, int* kept, int* dropped) {
   note_launch(1);
   int blocks = ceil_div(B, SEL_WARPS), threads = SEL_WARPS * 32;
-  if (M <= 256) { token_select_reg_kernel<8><<<blocks, threads, 0, s>>>(p, B, H, M, k, scores, kept, dropped); return; }
-  if (M <= 640) { token_select_reg_kernel<20><<<blocks, threads, 0, s>>>(p, B, H, M, k, scores, kept, dropped); return; }
+  if (M <= 256) { launch_k(token_select_reg_kernel<8>, blocks, threads, 0, s, p, B, H, M, k, scores, kept, dropped); return; }
+  if (M <= 640) { launch_k(token_select_reg_kernel<20>, blocks, threads, 0, s, p, B, H, M, k, scores, kept, dropped); return; }
   size_t smem = (size_t)SEL_WARPS * M * sizeof(uint32_t);
   if (smem > 48 * 1024) cudaFuncSetAttribute(token_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  token_select_kernel<<<blocks, threads, smem, s>>>(p, B, H, M, k, scores, kept, dropped);
+  launch_k(token_select_kernel, blocks, threads, smem, s, p, B, H, M, k, scores, kept, dropped);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -172,6 +174,7 @@ template <typename T>
 __global__ void gather_fuse_kernel(const T* __restrict__ x, int M, int D, int k, const int* __restrict__ kept,
                                    const int* __restrict__ dropped, const float* __restrict__ scores, int fuse,
                                    T* __restrict__ out, int copy_splits, int* status) {
+  dependent_sync();
   constexpr int N = Pack<T>::N;
   int b = blockIdx.x;
   int chunks = D / N;
@@ -247,9 +250,9 @@ void gather_fuse(const Ctx& c, const void* x, int B, int M, int D, int k, const 
   if (copy_splits > 1 + k) copy_splits = 1 + k;
   dim3 grid(B, copy_splits + fuse_slices);
   if (c.dtype == 0)
-    gather_fuse_kernel<float><<<grid, GF_THREADS, 0, c.stream>>>((const float*)x, M, D, k, kept, dropped, scores, do_fuse, (float*)out, copy_splits, c.status);
+    launch_k(gather_fuse_kernel<float>, grid, GF_THREADS, 0, c.stream, (const float*)x, M, D, k, kept, dropped, scores, do_fuse, (float*)out, copy_splits, c.status);
   else
-    gather_fuse_kernel<bf16><<<grid, GF_THREADS, 0, c.stream>>>((const bf16*)x, M, D, k, kept, dropped, scores, do_fuse, (bf16*)out, copy_splits, c.status);
+    launch_k(gather_fuse_kernel<bf16>, grid, GF_THREADS, 0, c.stream, (const bf16*)x, M, D, k, kept, dropped, scores, do_fuse, (bf16*)out, copy_splits, c.status);
 }
 
 // Backward of the compaction, one warp per input row (the index sets are constants, the fusion weights are
@@ -262,6 +265,7 @@ __global__ void gather_fuse_bwd_kernel(const float* __restrict__ dout, const flo
                                        const float* __restrict__ scores, int fuse, float* __restrict__ dx,
                                        bf16* __restrict__ dx_copy, float* __restrict__ escore, const float* __restrict__ fwd_out,
                                        int* status) {
+  dependent_sync();
   int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (warp >= B * (1 + M)) return;
   int b = warp / (1 + M), e = warp % (1 + M);
@@ -328,7 +332,7 @@ void gather_fuse_bwd(const Ctx& c, const void* dout, const void* x, int B, int M
   note_launch(1);
   int do_fuse = ((fuse == 1 || fuse == 2) && k < M) ? fuse : 0;
   int threads = 256, blocks = ceil_div((long)B * (1 + M) * 32, threads);
-  gather_fuse_bwd_kernel<<<blocks, threads, 0, c.stream>>>((const float*)dout, (const float*)x, B, M, D, k, kept, dropped, scores,
+  launch_k(gather_fuse_bwd_kernel, blocks, threads, 0, c.stream, (const float*)dout, (const float*)x, B, M, D, k, kept, dropped, scores,
                                                            do_fuse, (float*)dx, (bf16*)dx_copy, escore, (const float*)fwd_out, c.status);
 }
 

@@ -24,6 +24,7 @@ __global__ void __launch_bounds__(MOE_ROUTE_WARPS * 32)
 moe_route_kernel(const T* __restrict__ y, const T* __restrict__ wg, const float* __restrict__ logits, int logit_stride,
                  const int* __restrict__ task_ids, int tokens_per_image, int M, int D, int E, int K, int gate_elems_in_smem,
                  int* __restrict__ eidx, float* __restrict__ ew, int* __restrict__ blk_counts) {
+  dependent_sync();
   // A block takes MOE_ROUTE_TOKENS consecutive tokens (a divisor of MOE_BLOCK_TOKENS, so all of them fall into one
   // counting group), a warp one token at a time.  Expert by expert the lanes multiply 16-byte pieces of the token's row
   // of y (coalesced; from L1 after the first expert) with the same pieces of the gate row -- the gate matrices of all
@@ -116,6 +117,7 @@ __global__ void __launch_bounds__(256)
 moe_assign_kernel(const int* __restrict__ eidx, const float* __restrict__ ew, const int* __restrict__ blk_counts, int nblk,
                   int tiles_cap, int M, int E, int K, int* __restrict__ seg_start, int* __restrict__ tile_expert,
                   int* __restrict__ pos, int* __restrict__ row_token, float* __restrict__ row_w) {
+  dependent_sync();
   __shared__ int total[MOE_MAX_E];
   __shared__ int before[MOE_MAX_E];
   __shared__ int start[MOE_MAX_E + 1];
@@ -175,6 +177,7 @@ moe_assign_kernel(const int* __restrict__ eidx, const float* __restrict__ ew, co
 template <typename T>
 __global__ void moe_gather_kernel(const T* __restrict__ y, const int* __restrict__ row_token, const int* __restrict__ seg_start,
                                   int E, int D, T* __restrict__ xg, int rows_cap, int M, int* status) {
+  dependent_sync();
   constexpr int N = Pack<T>::N;
   int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (warp >= rows_cap || warp >= seg_start[E]) return;
@@ -190,6 +193,7 @@ __global__ void moe_gather_kernel(const T* __restrict__ y, const int* __restrict
 // ---- combine: out[t] = res[t] + sum_slot w_slot * og[pos(t, slot)]  (float residual stream) ------------------------
 __global__ void moe_combine_kernel(const float* __restrict__ og, const int* __restrict__ pos, const float* __restrict__ ew,
                                    const float* __restrict__ res, float* __restrict__ out, int M, int D, int K) {
+  dependent_sync();
   int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (warp >= M) return;
   for (int ch = lane; ch < D / 4; ch += 32) {
@@ -211,6 +215,7 @@ template <typename T>
 __global__ void moe_combine_bwd_kernel(const float* __restrict__ dout, const float* __restrict__ og, const int* __restrict__ row_token,
                                        const float* __restrict__ row_w, const int* __restrict__ seg_start, int E, int D,
                                        T* __restrict__ dog, float* __restrict__ dw, int rows_cap) {
+  dependent_sync();
   int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (warp >= rows_cap || warp >= seg_start[E]) return;
   int tok = row_token[warp];
@@ -236,6 +241,7 @@ __global__ void moe_combine_bwd_kernel(const float* __restrict__ dout, const flo
 template <typename T>
 __global__ void __launch_bounds__(256)
 moe_seg_colsum_kernel(const T* __restrict__ x, const int* __restrict__ seg_start, int cols, float* __restrict__ out) {
+  dependent_sync();
   constexpr int N = Pack<T>::N;
   __shared__ float sm[8][32 * N];
   int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
@@ -273,6 +279,7 @@ __global__ void moe_gate_bwd_kernel(const T* __restrict__ dxg, const float* __re
                                     const int* __restrict__ eidx, const float* __restrict__ ew, const T* __restrict__ wg,
                                     const int* __restrict__ task_ids, int tokens_per_image, int M, int D, int E, int K,
                                     T* __restrict__ dy, float* __restrict__ dsel_row) {
+  dependent_sync();
   int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (warp >= M) return;
   int task = task_ids ? task_ids[warp / tokens_per_image] : 0;
@@ -309,6 +316,7 @@ __global__ void __launch_bounds__(256)
 moe_gate_wgrad_kernel(const T* __restrict__ xg, const float* __restrict__ dsel_row, const int* __restrict__ row_token,
                       const int* __restrict__ seg_start, const int* __restrict__ task_ids, int tokens_per_image, int D, int E,
                       float* __restrict__ dwg) {
+  dependent_sync();
   constexpr int N = Pack<T>::N;
   __shared__ float sm[8][32 * N];
   int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
@@ -364,25 +372,25 @@ void moe_route(const Ctx& c, const MoeBufs& b, const void* y, const void* wg, co
   cudaMemsetAsync(b.blk_counts, 0, (size_t)nblk * E * sizeof(int), c.stream);
   if (c.dtype == 0) {
     ensure_smem(lim[0], moe_route_kernel<float>, smem);
-    moe_route_kernel<float><<<rblk, MOE_ROUTE_WARPS * 32, smem, c.stream>>>((const float*)y, (const float*)wg, logits, logit_stride, task_ids, tokens_per_image, M, D, E, K,
+    launch_k(moe_route_kernel<float>, rblk, MOE_ROUTE_WARPS * 32, smem, c.stream, (const float*)y, (const float*)wg, logits, logit_stride, task_ids, tokens_per_image, M, D, E, K,
                                                                         (int)gate_elems, b.eidx, b.ew, b.blk_counts);
   } else {
     ensure_smem(lim[1], moe_route_kernel<bf16>, smem);
-    moe_route_kernel<bf16><<<rblk, MOE_ROUTE_WARPS * 32, smem, c.stream>>>((const bf16*)y, (const bf16*)wg, logits, logit_stride, task_ids, tokens_per_image, M, D, E, K,
+    launch_k(moe_route_kernel<bf16>, rblk, MOE_ROUTE_WARPS * 32, smem, c.stream, (const bf16*)y, (const bf16*)wg, logits, logit_stride, task_ids, tokens_per_image, M, D, E, K,
                                                                        (int)gate_elems, b.eidx, b.ew, b.blk_counts);
   }
   cudaMemsetAsync(b.row_token, 0xFF, (size_t)rows_cap * sizeof(int), c.stream);
-  moe_assign_kernel<<<nblk, 256, 0, c.stream>>>(b.eidx, b.ew, b.blk_counts, nblk, rows_cap / 128, M, E, K, b.seg_start, b.tile_expert,
+  launch_k(moe_assign_kernel, nblk, 256, 0, c.stream, b.eidx, b.ew, b.blk_counts, nblk, rows_cap / 128, M, E, K, b.seg_start, b.tile_expert,
                                                 b.pos, b.row_token, b.row_w);
   int blocks = ceil_div((long)rows_cap * 32, 256);
-  if (c.dtype == 0) moe_gather_kernel<float><<<blocks, 256, 0, c.stream>>>((const float*)y, b.row_token, b.seg_start, E, D, (float*)b.xg, rows_cap, M, c.status);
-  else moe_gather_kernel<bf16><<<blocks, 256, 0, c.stream>>>((const bf16*)y, b.row_token, b.seg_start, E, D, (bf16*)b.xg, rows_cap, M, c.status);
+  if (c.dtype == 0) launch_k(moe_gather_kernel<float>, blocks, 256, 0, c.stream, (const float*)y, b.row_token, b.seg_start, E, D, (float*)b.xg, rows_cap, M, c.status);
+  else launch_k(moe_gather_kernel<bf16>, blocks, 256, 0, c.stream, (const bf16*)y, b.row_token, b.seg_start, E, D, (bf16*)b.xg, rows_cap, M, c.status);
 }
 
 void moe_combine(const Ctx& c, const MoeBufs& b, const float* res, float* out, int M, int D, int K) {
   note_launch(1);
   int blocks = ceil_div((long)M * 32, 256);
-  moe_combine_kernel<<<blocks, 256, 0, c.stream>>>(b.og, b.pos, b.ew, res, out, M, D, K);
+  launch_k(moe_combine_kernel, blocks, 256, 0, c.stream, b.og, b.pos, b.ew, res, out, M, D, K);
 }
 
 void moe_combine_bwd(const Ctx& c, const MoeBufs& b, const float* dout, void* dog, float* dw, int M, int D, int E, int K) {
@@ -390,15 +398,15 @@ void moe_combine_bwd(const Ctx& c, const MoeBufs& b, const float* dout, void* do
   int rows_cap = moe_rows_cap(M, E, K);
   int blocks = ceil_div((long)rows_cap * 32, 256);
   if (c.dtype == 0)
-    moe_combine_bwd_kernel<float><<<blocks, 256, 0, c.stream>>>(dout, b.og, b.row_token, b.row_w, b.seg_start, E, D, (float*)dog, dw, rows_cap);
+    launch_k(moe_combine_bwd_kernel<float>, blocks, 256, 0, c.stream, dout, b.og, b.row_token, b.row_w, b.seg_start, E, D, (float*)dog, dw, rows_cap);
   else
-    moe_combine_bwd_kernel<bf16><<<blocks, 256, 0, c.stream>>>(dout, b.og, b.row_token, b.row_w, b.seg_start, E, D, (bf16*)dog, dw, rows_cap);
+    launch_k(moe_combine_bwd_kernel<bf16>, blocks, 256, 0, c.stream, dout, b.og, b.row_token, b.row_w, b.seg_start, E, D, (bf16*)dog, dw, rows_cap);
 }
 
 void moe_seg_colsum(const Ctx& c, const MoeBufs& b, const void* x, int cols, int E, float* out) {
   note_launch(1);
-  if (c.dtype == 0) moe_seg_colsum_kernel<float><<<dim3(ceil_div(cols, 128), E), 256, 0, c.stream>>>((const float*)x, b.seg_start, cols, out);
-  else moe_seg_colsum_kernel<bf16><<<dim3(ceil_div(cols, 256), E), 256, 0, c.stream>>>((const bf16*)x, b.seg_start, cols, out);
+  if (c.dtype == 0) launch_k(moe_seg_colsum_kernel<float>, dim3(ceil_div(cols, 128), E), 256, 0, c.stream, (const float*)x, b.seg_start, cols, out);
+  else launch_k(moe_seg_colsum_kernel<bf16>, dim3(ceil_div(cols, 256), E), 256, 0, c.stream, (const bf16*)x, b.seg_start, cols, out);
 }
 
 void moe_gate_bwd(const Ctx& c, const MoeBufs& b, const void* dxg, const float* dw, const void* wg, const int* task_ids,
@@ -406,11 +414,11 @@ void moe_gate_bwd(const Ctx& c, const MoeBufs& b, const void* dxg, const float* 
   note_launch(2);
   int blocks = ceil_div((long)M * 32, 256);
   if (c.dtype == 0) {
-    moe_gate_bwd_kernel<float><<<blocks, 256, 0, c.stream>>>((const float*)dxg, dw, b.pos, b.eidx, b.ew, (const float*)wg, task_ids, tokens_per_image, M, D, E, K, (float*)dy, dsel_row);
-    if (dwg != nullptr) moe_gate_wgrad_kernel<float><<<dim3(ceil_div(D, 128), E, tasks), 256, 0, c.stream>>>((const float*)b.xg, dsel_row, b.row_token, b.seg_start, task_ids, tokens_per_image, D, E, dwg);
+    launch_k(moe_gate_bwd_kernel<float>, blocks, 256, 0, c.stream, (const float*)dxg, dw, b.pos, b.eidx, b.ew, (const float*)wg, task_ids, tokens_per_image, M, D, E, K, (float*)dy, dsel_row);
+    if (dwg != nullptr) launch_k(moe_gate_wgrad_kernel<float>, dim3(ceil_div(D, 128), E, tasks), 256, 0, c.stream, (const float*)b.xg, dsel_row, b.row_token, b.seg_start, task_ids, tokens_per_image, D, E, dwg);
   } else {
-    moe_gate_bwd_kernel<bf16><<<blocks, 256, 0, c.stream>>>((const bf16*)dxg, dw, b.pos, b.eidx, b.ew, (const bf16*)wg, task_ids, tokens_per_image, M, D, E, K, (bf16*)dy, dsel_row);
-    if (dwg != nullptr) moe_gate_wgrad_kernel<bf16><<<dim3(ceil_div(D, 256), E, tasks), 256, 0, c.stream>>>((const bf16*)b.xg, dsel_row, b.row_token, b.seg_start, task_ids, tokens_per_image, D, E, dwg);
+    launch_k(moe_gate_bwd_kernel<bf16>, blocks, 256, 0, c.stream, (const bf16*)dxg, dw, b.pos, b.eidx, b.ew, (const bf16*)wg, task_ids, tokens_per_image, M, D, E, K, (bf16*)dy, dsel_row);
+    if (dwg != nullptr) launch_k(moe_gate_wgrad_kernel<bf16>, dim3(ceil_div(D, 256), E, tasks), 256, 0, c.stream, (const bf16*)b.xg, dsel_row, b.row_token, b.seg_start, task_ids, tokens_per_image, D, E, dwg);
   }
 }
 
