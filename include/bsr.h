@@ -253,13 +253,13 @@ int32_t bsr_selftest_wait_expiry(bsr_handle* h, uint64_t limit_ns, void* stream)
  * tile (the default), 2 = as 1 but GEMMs with more than 128 rows run on CTA pairs (cta_group::2). */
 int32_t bsr_set_gemm_mode(bsr_handle* h, int32_t mode);
 
-/* bsr_train_step replays a captured CUDA graph of its ~200 launches when `stream` can be captured (any stream but
- * the legacy default stream, and not one the caller is capturing) -- the first call with a given set of pointers
- * and batch captures it, later calls with the same arguments replay it.  The key of a captured graph is (images,
- * labels, task ids, loss and kept-index pointers, batch, kernel mode); the handle keeps the eight most recently
- * used graphs, so an input pipeline should rotate through at most eight sets of buffers (bsr_profile.graph_captures
- * counts captures: it stops growing once a pipeline fits).  on = 0 turns this off (every call enqueues its kernels
- * one by one); the results are identical.  No counterpart in the paper. */
+/* bsr_train_step replays a captured CUDA graph of its ~200 launches (unless the caller is capturing `stream`): the first
+ * call with a given set of pointers and batch enqueues its kernels one by one, the second captures them, later calls
+ * with the same arguments replay the graph.  The key of a captured graph is (images, labels, task ids, loss and
+ * kept-index pointers, batch, kernel mode); the handle keeps the eight most recently used graphs, so an input pipeline
+ * should rotate through at most eight sets of buffers (bsr_profile.graph_captures counts captures: it stops growing once
+ * a pipeline fits).  bsr_eval_forward does the same with a graph per batch size, whatever the pointers.  on = 0 turns this
+ * off (every call enqueues its kernels one by one); the results are identical.  No counterpart in the paper. */
 int32_t bsr_set_graph_mode(bsr_handle* h, int32_t on);
 
 /* Measurement support (no counterpart in the paper).  bsr_profile_enable resets the counters; with

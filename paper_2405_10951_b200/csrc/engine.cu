@@ -177,13 +177,18 @@ struct bsr_handle {
   std::vector<size_t> score_rec;       // per drop location's block: head-mean scores [max_batch, M] of the last step
   size_t off_m_dog = 0, off_m_dzg = 0, off_m_dxg = 0, off_m_dw = 0, off_m_dsel = 0;
   GemmProfile prof;
-  // Captured graphs of the training step.  The key is everything a captured launch has baked in: the caller's
-  // pointers, the batch, the kernel mode and whether the step reads its inputs through the multi-step loop state.
-  // Up to GRAPH_CACHE graphs are kept; the least recently used one is dropped.
+  // Captured graphs.  The key is everything a captured launch has baked in: the caller's pointers, the batch, the kernel
+  // mode and which path it is (a training step, a step of the multi-step loop, forward and backward alone; inference bakes
+  // in no caller's pointer: those go through EvalIo).  Up to GRAPH_CACHE graphs of either kind are kept; the least
+  // recently used one is dropped.  A key is captured when it comes round the second time (`seen`): a first pass, or an input
+  // pipeline that never returns to a buffer, does not pay for a graph it will not replay (a first DeiT-S step at batch 64
+  // took 2.93 ms with the capture in it).
   struct StepGraph { const void* images; const void* labels; const void* tasks; void* loss; void* kept; int batch; int mode; int loop;
                      cudaGraphExec_t exec; long launches; uint64_t last_use; };
   static constexpr size_t GRAPH_CACHE = 8;
-  std::vector<StepGraph> graphs;
+  std::vector<StepGraph> graphs, eval_graphs;
+  std::vector<StepGraph> seen;
+  cudaStream_t capture_stream = nullptr;   // graphs are captured here, whatever stream they are replayed on
   uint64_t graph_clock = 0;
   uint64_t graph_captures = 0;        // how many times a step was captured (a pipeline that cycles through more buffers than the cache holds re-captures every step)
   int use_graph = 1;
@@ -963,6 +968,8 @@ int32_t bsr_destroy(bsr_handle* h) {
   if (h != nullptr) {
     for (cudaEvent_t ev : h->prof.events) cudaEventDestroy(ev);
     for (auto& g : h->graphs) cudaGraphExecDestroy(g.exec);
+    for (auto& g : h->eval_graphs) cudaGraphExecDestroy(g.exec);
+    if (h->capture_stream) cudaStreamDestroy(h->capture_stream);
     for (int i = 0; i < 2; ++i) {
       if (h->ev_copied[i]) cudaEventDestroy(h->ev_copied[i]);
       if (h->ev_done[i]) cudaEventDestroy(h->ev_done[i]);
@@ -1160,35 +1167,54 @@ static void enqueue_optimizer(bsr_handle* h, const Ctx& c) {
 
 }  // extern "C"
 
-// Runs `enqueue` (which puts one step's kernels on `st`) either directly or, when the stream allows capture (any
-// stream but the legacy default one, not one the caller is capturing, no per-launch events asked for), as a CUDA graph
-// captured on first use and replayed afterwards.
+// Runs `enqueue(stream)` (which puts one step's kernels on a stream) either directly or, when the caller's stream is not
+// itself being captured and no per-launch events are asked for, as a CUDA graph that is captured the second time its key
+// comes round and replayed from then on.  at_once: the caller knows that the key will come round again.
 template <typename Enqueue>
-static int run_step_graphed(bsr_handle* h, cudaStream_t st, const bsr_handle::StepGraph& key, Enqueue enqueue) {
+static int run_graphed(bsr_handle* h, cudaStream_t st, std::vector<bsr_handle::StepGraph>& cache, const bsr_handle::StepGraph& key, bool at_once,
+                       uint64_t* captures, Enqueue enqueue) {
   int rc;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  bool can_graph = h->use_graph && st != nullptr && st != cudaStreamLegacy && !h->prof.on &&
-                   cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+  const bool legacy = st == nullptr || st == cudaStreamLegacy;
+  bool can_graph = h->use_graph && !h->prof.on && (legacy || (cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone));
   auto direct = [&]() -> int {
     cudaGetLastError();
-    int r = enqueue();
-    return r != BSR_OK ? r : check_cuda(h, "training step");
+    int r = enqueue(st);
+    return r != BSR_OK ? r : check_cuda(h, "step");
+  };
+  auto same = [&](const bsr_handle::StepGraph& g) {
+    return g.images == key.images && g.labels == key.labels && g.tasks == key.tasks && g.loss == key.loss && g.kept == key.kept &&
+           g.batch == key.batch && g.mode == key.mode && g.loop == key.loop;
+  };
+  auto replay = [&](const bsr_handle::StepGraph& g) -> int {
+    if (cudaGraphLaunch(g.exec, st) != cudaSuccess) return set_err(h->err, BSR_ERR_CUDA, "graph launch failed: %s", cudaGetErrorString(cudaGetLastError()));
+    return BSR_OK;
   };
   if (!can_graph) return direct();
-  for (auto& g : h->graphs) {
-    if (g.images == key.images && g.labels == key.labels && g.tasks == key.tasks && g.loss == key.loss && g.kept == key.kept &&
-        g.batch == key.batch && g.mode == key.mode && g.loop == key.loop) {
+  for (auto& g : cache)
+    if (same(g)) {
       g_kernel_launches += g.launches;
       g.last_use = ++h->graph_clock;
-      if (cudaGraphLaunch(g.exec, st) != cudaSuccess) return set_err(h->err, BSR_ERR_CUDA, "graph launch failed: %s", cudaGetErrorString(cudaGetLastError()));
-      return BSR_OK;
+      return replay(g);
+    }
+  if (!at_once) {
+    bool known = false;
+    for (auto& g : h->seen) known = known || same(g);
+    if (!known) {
+      if (h->seen.size() >= 4 * bsr_handle::GRAPH_CACHE) h->seen.erase(h->seen.begin());
+      h->seen.push_back(key);
+      return direct();
     }
   }
+  if (h->capture_stream == nullptr && cudaStreamCreateWithFlags(&h->capture_stream, cudaStreamNonBlocking) != cudaSuccess) {
+    h->capture_stream = nullptr;
+    return direct();
+  }
   long before = g_kernel_launches;
-  if (cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return direct();
-  rc = enqueue();
+  if (cudaStreamBeginCapture(h->capture_stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return direct();
+  rc = enqueue(h->capture_stream);
   cudaGraph_t graph = nullptr;
-  cudaError_t ce = cudaStreamEndCapture(st, &graph);
+  cudaError_t ce = cudaStreamEndCapture(h->capture_stream, &graph);
   if (rc != BSR_OK) {
     if (graph) cudaGraphDestroy(graph);
     return rc;
@@ -1200,17 +1226,21 @@ static int run_step_graphed(bsr_handle* h, cudaStream_t st, const bsr_handle::St
     return direct();                                     // nothing ran during the capture
   }
   cudaGraphDestroy(graph);
-  ++h->graph_captures;
-  if (h->graphs.size() >= bsr_handle::GRAPH_CACHE) {     // drop the least recently used graph
+  if (captures != nullptr) ++*captures;
+  if (cache.size() >= bsr_handle::GRAPH_CACHE) {         // drop the least recently used graph
     size_t lru = 0;
-    for (size_t i = 1; i < h->graphs.size(); ++i)
-      if (h->graphs[i].last_use < h->graphs[lru].last_use) lru = i;
-    cudaGraphExecDestroy(h->graphs[lru].exec);
-    h->graphs.erase(h->graphs.begin() + lru);
+    for (size_t i = 1; i < cache.size(); ++i)
+      if (cache[i].last_use < cache[lru].last_use) lru = i;
+    cudaGraphExecDestroy(cache[lru].exec);
+    cache.erase(cache.begin() + lru);
   }
-  h->graphs.push_back(sg);
-  if (cudaGraphLaunch(sg.exec, st) != cudaSuccess) return set_err(h->err, BSR_ERR_CUDA, "graph launch failed: %s", cudaGetErrorString(cudaGetLastError()));
-  return BSR_OK;
+  cache.push_back(sg);
+  return replay(sg);
+}
+
+static bsr_handle::StepGraph graph_key(const bsr_handle* h, const void* images, const void* labels, const void* tasks, void* loss,
+                                       void* kept, int batch, int loop) {
+  return {images, labels, tasks, loss, kept, batch, h->use_tc, loop, nullptr, 0, 0};
 }
 
 extern "C" {
@@ -1227,10 +1257,9 @@ int32_t bsr_train_step(bsr_handle* h, const void* images, const int32_t* labels,
   double bc1 = 1.0 - std::pow((double)h->cfg.beta1, (double)step_next);
   double bc2 = 1.0 - std::pow((double)h->cfg.beta2, (double)step_next);
   set_scalars(st, h->at<float>(h->off_status + 128), h->lr, (float)bc1, (float)bc2);
-  bsr_handle::StepGraph key;
-  key.images = images; key.labels = labels; key.tasks = task_ids; key.loss = loss_out; key.kept = kept_out; key.batch = batch;
-  key.mode = h->use_tc; key.loop = 0; key.exec = nullptr; key.launches = 0; key.last_use = 0;
-  rc = run_step_graphed(h, st, key, [&]() { return enqueue_train_step(h, images, labels, task_ids, batch, stream, loss_out, kept_out); });
+  auto key = graph_key(h, images, labels, task_ids, loss_out, kept_out, batch, 0);
+  rc = run_graphed(h, st, h->graphs, key, false, &h->graph_captures,
+                   [&](cudaStream_t s) { return enqueue_train_step(h, images, labels, task_ids, batch, s, loss_out, kept_out); });
   if (rc == BSR_OK) h->step = step_next;
   return rc;
 }
@@ -1241,11 +1270,9 @@ int32_t bsr_forward_backward(bsr_handle* h, const void* images, const int32_t* l
   if (rc != BSR_OK) return rc;
   if (labels == nullptr || loss_out == nullptr) return set_err(h->err, BSR_ERR_INVALID_ARG, "labels_dev and loss_dev_out must not be null");
   if (h->cfg.dims.num_tasks > 1 && task_ids == nullptr) return set_err(h->err, BSR_ERR_INVALID_ARG, "task_ids_dev is required with several tasks");
-  bsr_handle::StepGraph key;
-  key.images = images; key.labels = labels; key.tasks = task_ids; key.loss = loss_out; key.kept = kept_out; key.batch = batch;
-  key.mode = h->use_tc; key.loop = 2; key.exec = nullptr; key.launches = 0; key.last_use = 0;
-  return run_step_graphed(h, (cudaStream_t)stream, key, [&]() {
-    return enqueue_train_step(h, images, labels, task_ids, batch, stream, loss_out, kept_out, nullptr, false);
+  auto key = graph_key(h, images, labels, task_ids, loss_out, kept_out, batch, 2);
+  return run_graphed(h, (cudaStream_t)stream, h->graphs, key, false, &h->graph_captures, [&](cudaStream_t s) {
+    return enqueue_train_step(h, images, labels, task_ids, batch, s, loss_out, kept_out, nullptr, false);
   });
 }
 
@@ -1288,14 +1315,12 @@ int32_t bsr_train_steps(bsr_handle* h, const void* images, const int32_t* labels
   int* lab_stage = h->at<int>(h->off_lab_stage);
   int* task_stage = task_ids != nullptr ? h->at<int>(h->off_task_stage) : nullptr;
   float* scalars = h->at<float>(h->off_status + 128);
-  bsr_handle::StepGraph key;
-  key.images = images; key.labels = labels; key.tasks = task_ids; key.loss = loss_out; key.kept = kept_out; key.batch = batch;
-  key.mode = h->use_tc; key.loop = 1; key.exec = nullptr; key.launches = 0; key.last_use = 0;
+  auto key = graph_key(h, images, labels, task_ids, loss_out, kept_out, batch, 1);
   for (int i = 0; i < n_steps; ++i) {
-    rc = run_step_graphed(h, st, key, [&]() {
-      loop_begin(st, ls, scalars, labels, task_ids, lab_stage, task_stage, batch);
-      int r = enqueue_train_step(h, images, lab_stage, task_stage, batch, stream, nullptr, kept_out, &ls->image_offset);
-      loop_end(st, ls, h->at<float>(h->off_loss), loss_out);
+    rc = run_graphed(h, st, h->graphs, key, n_steps > 2, &h->graph_captures, [&](cudaStream_t s) {
+      loop_begin(s, ls, scalars, labels, task_ids, lab_stage, task_stage, batch);
+      int r = enqueue_train_step(h, images, lab_stage, task_stage, batch, s, nullptr, kept_out, &ls->image_offset);
+      loop_end(s, ls, h->at<float>(h->off_loss), loss_out);
       return r;
     });
     if (rc != BSR_OK) return rc;
@@ -1353,21 +1378,38 @@ int32_t bsr_eval_forward(bsr_handle* h, const void* images, const int32_t* task_
   if (rc != BSR_OK) return rc;
   if (logits_out == nullptr) return set_err(h->err, BSR_ERR_INVALID_ARG, "logits_dev_out is null");
   if (h->cfg.dims.num_tasks > 1 && task_ids == nullptr) return set_err(h->err, BSR_ERR_INVALID_ARG, "task_ids_dev is required with several tasks");
+  // Everything the kernels read or write of the caller's goes through EvalIo and the task staging area, so that one graph
+  // per batch size serves every call: 99 to 111 launches of 3 to 6 us of host time each against a replay.
   const bsr_dims& d = h->cfg.dims;
-  Ctx c = make_ctx(h, stream);
-  size_t x_last = 0;
-  rc = forward_all(h, c, images, batch, false, &x_last, task_ids);
-  if (rc != BSR_OK) return rc;
-  int Tl = cls_tail(h, d.depth - 1) ? 1 : h->sched.tf[d.depth - 1];   // rows per image in the last block's output
-  HeadDesc hd = head_desc(h);
-  float* xn = h->at<float>(h->off_xn);
-  layernorm_fwd(c, h->at<float>(x_last), (long)Tl * d.dim, (const float*)h->w("norm.weight"), (const float*)h->w("norm.bias"), xn, 1,
-                nullptr, nullptr, batch, d.dim, d.ln_eps);
-  head_fwd(c, hd, xn, task_ids, h->at<float>(h->off_logits), batch);
-  cudaMemcpyAsync(logits_out, h->at<float>(h->off_logits), (size_t)batch * hd.cmax * 4, cudaMemcpyDeviceToDevice, c.stream);
-  if (kept_out != nullptr && kept_total(h, batch) > 0)
-    cudaMemcpyAsync(kept_out, h->base + h->off_kept_all, kept_total(h, batch) * 4, cudaMemcpyDeviceToDevice, c.stream);
-  return check_cuda(h, "bsr_eval_forward");
+  cudaStream_t st = (cudaStream_t)stream;
+  const size_t es = dtype_size(d.dtype);
+  EvalIo* io = h->at<EvalIo>(h->off_status + 192);
+  EvalIo value;
+  value.image_offset = (long long)((intptr_t)images - (intptr_t)h->base) / (long long)es;
+  value.logits = logits_out;
+  value.kept = kept_out;
+  int32_t* tasks = task_ids != nullptr ? h->at<int32_t>(h->off_task_stage) : nullptr;
+  const bool relative = (uintptr_t)images % 16 == 0;       // the vectorised patch kernel counts on it
+  auto key = graph_key(h, nullptr, nullptr, tasks, nullptr, nullptr, batch, 3);
+  auto enqueue = [&](cudaStream_t s) -> int {
+    Ctx c = make_ctx(h, s);
+    size_t x_last = 0;
+    int r = relative ? forward_all(h, c, h->base, batch, false, &x_last, tasks, &io->image_offset) : forward_all(h, c, images, batch, false, &x_last, tasks);
+    if (r != BSR_OK) return r;
+    int Tl = cls_tail(h, d.depth - 1) ? 1 : h->sched.tf[d.depth - 1];   // rows per image in the last block's output
+    HeadDesc hd = head_desc(h);
+    float* xn = h->at<float>(h->off_xn);
+    layernorm_fwd(c, h->at<float>(x_last), (long)Tl * d.dim, (const float*)h->w("norm.weight"), (const float*)h->w("norm.bias"), xn, 1,
+                  nullptr, nullptr, batch, d.dim, d.ln_eps);
+    head_fwd(c, hd, xn, tasks, h->at<float>(h->off_logits), batch);
+    eval_end(c.stream, io, h->at<float>(h->off_logits), (size_t)batch * hd.cmax, h->at<int>(h->off_kept_all), kept_total(h, batch));
+    return BSR_OK;
+  };
+  cudaGetLastError();
+  eval_begin(st, io, value, task_ids, tasks, batch);
+  if (relative) return run_graphed(h, st, h->eval_graphs, key, false, nullptr, enqueue);
+  rc = enqueue(st);
+  return rc != BSR_OK ? rc : check_cuda(h, "bsr_eval_forward");
 }
 
 int32_t bsr_get_footprint(const bsr_handle* h, bsr_footprint* out) {

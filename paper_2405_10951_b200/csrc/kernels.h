@@ -239,6 +239,15 @@ void loop_begin(cudaStream_t s, LoopState* st, float* scalars, const int* labels
 // End of a step: loss_out[i] = loss, counters advance.
 void loop_end(cudaStream_t s, LoopState* st, const float* loss, float* loss_out);
 
+// Inference replayed from a graph: what differs from call to call lives in device memory, written before the replay.
+struct EvalIo {
+  long long image_offset;    // elements from the base the captured patch kernel reads from to this call's images
+  float* logits;             // where this call wants its logits ...
+  int* kept;                 // ... and the kept positions (may be null)
+};
+void eval_begin(cudaStream_t s, EvalIo* io, const EvalIo& value, const int* tasks, int* task_stage, int batch);
+void eval_end(cudaStream_t s, const EvalIo* io, const float* logits, size_t n_logits, const int* kept, size_t n_kept);
+
 // dst row r = src row r (row_bytes a multiple of 16), independent pitches: gathers / scatters token rows.
 void copy_rows(cudaStream_t s, const void* src, long src_pitch_bytes, void* dst, long dst_pitch_bytes, int rows, int row_bytes);
 

@@ -810,6 +810,31 @@ void loop_end(cudaStream_t s, LoopState* st, const float* loss, float* loss_out)
   launch_k(loop_end_kernel, 1, 1, 0, s, st, loss, loss_out);
 }
 
+__global__ void eval_begin_kernel(EvalIo* io, EvalIo value, const int* __restrict__ tasks, int* __restrict__ task_stage, int batch) {
+  dependent_sync();
+  if (threadIdx.x == 0) *io = value;
+  if (tasks != nullptr)
+    for (int j = threadIdx.x; j < batch; j += blockDim.x) task_stage[j] = tasks[j];
+}
+__global__ void eval_end_kernel(const EvalIo* io, const float* __restrict__ logits, size_t n_logits, const int* __restrict__ kept, size_t n_kept) {
+  dependent_sync();
+  EvalIo out = *io;
+  size_t step = (size_t)gridDim.x * blockDim.x, i0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  for (size_t i = i0; i < n_logits; i += step) out.logits[i] = logits[i];
+  if (out.kept != nullptr)
+    for (size_t i = i0; i < n_kept; i += step) out.kept[i] = kept[i];
+}
+void eval_begin(cudaStream_t s, EvalIo* io, const EvalIo& value, const int* tasks, int* task_stage, int batch) {
+  note_launch(1);
+  launch_k(eval_begin_kernel, 1, 128, 0, s, io, value, tasks, task_stage, batch);
+}
+void eval_end(cudaStream_t s, const EvalIo* io, const float* logits, size_t n_logits, const int* kept, size_t n_kept) {
+  note_launch(1);
+  size_t n = n_logits > n_kept ? n_logits : n_kept;
+  int blocks = ceil_div((long)n, 256);
+  launch_k(eval_end_kernel, blocks < 64 ? blocks : 64, 256, 0, s, io, logits, n_logits, kept, n_kept);
+}
+
 // Guard words after every workspace slice: one warp per guard.
 __global__ void guards_write_kernel(char* base, const unsigned long long* __restrict__ table, int n, int words, uint32_t word) {
   dependent_sync();
