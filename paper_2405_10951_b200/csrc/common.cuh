@@ -130,20 +130,26 @@ static inline void note_launch(int n = 1) { g_kernel_launches += n; }
 // the SMs whose CTA leaves first instead of spreading over all of them (ViT-B at batch 128: 5336 us without, 5341 us so,
 // 5534 us with a release at their start).  On at most half of the SMs they do: the next kernel finds the others idle.
 constexpr int B200_SMS = 148;
-__device__ __forceinline__ bool leaves_sms_idle() { return 2u * gridDim.x * gridDim.y <= (unsigned)B200_SMS; }
+__device__ __forceinline__ bool leaves_sms_idle() { return 2u * gridDim.x * gridDim.y * gridDim.z <= (unsigned)B200_SMS; }
 __device__ __forceinline__ void release_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void await_inputs() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void dependent_sync() { release_dependents(); await_inputs(); }
 
 template <typename... KArgs, typename... Args>
-static inline void launch_k(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, Args&&... args) {
+static inline void launch_cluster(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, dim3 cluster, Args&&... args) {
   cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = cluster.x; attr[1].val.clusterDim.y = cluster.y; attr[1].val.clusterDim.z = cluster.z;
   cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = stream;
-  cfg.attrs = attr; cfg.numAttrs = 1;
+  cfg.attrs = attr; cfg.numAttrs = cluster.x * cluster.y * cluster.z > 1 ? 2 : 1;
   cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
+}
+template <typename... KArgs, typename... Args>
+static inline void launch_k(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, Args&&... args) {
+  launch_cluster(kern, grid, block, smem, stream, dim3(1, 1, 1), std::forward<Args>(args)...);
 }
 
 // The dynamic shared-memory limit of a kernel is an attribute of the (kernel, device) pair, so the largest value set so

@@ -1,69 +1,80 @@
 // FP32-FMA dense contraction with arbitrary operand strides.  It is the contraction of the fp32
 // configuration (TF32 tensor-core math cannot hold a 1e-4 relative tolerance) and the fall-back for
 // bf16 problems the tcgen05 kernel does not take (tiny or unaligned shapes).
+#include <cooperative_groups.h>
+
 #include "common.cuh"
 #include "kernels.h"
 
 namespace bsr {
 
-constexpr int SG_BM = 64, SG_BN = 64, SG_BK = 16, SG_THREADS = 256;
+namespace cg = cooperative_groups;
+
+// A CTA of 128 threads forms a 64 x 64 tile, 8 x 4 outputs per thread: per k step a warp reads 2 + 1 wavefronts of shared
+// memory for 1024 multiply-adds, so the FMA pipe is the limit.  Slabs of 32 along k go through registers into two shared
+// buffers, the loads of the next slab in flight during the arithmetic of this one.  The products of this configuration are
+// small (520 x 576 x 192: 81 tiles on 148 SMs), so a tile's k range is split over the CTAs of a cluster (up to 8), whose
+// partial tiles are summed through distributed shared memory in rank order before the epilogue: no second kernel, no
+// workspace, the result does not depend on scheduling.  The step of the fp32 configuration at batch 8 (41 products) took
+// 1310 us with 4 x 4 outputs per thread, no split and no loads in flight, 800 us so.
+constexpr int SG_BM = 64, SG_BN = 64, SG_BK = 32, SG_THREADS = 128, SG_LD = SG_BM + 4, SG_MAXSPLIT = 8;
+
+// One thread's share (16 values) of a 64 x 32 operand slab: contiguous along k (row r = t % 64, 16 k values) or along its
+// own index (four k rows, 4 consecutive values each).  VEC: rows are aligned for four-element accesses.
+template <typename T>
+__device__ __forceinline__ void slab_load(const T* __restrict__ P, long ld, bool kmajor, bool vec, int r0, int k0, int R, int K, float* v) {
+  const int t = threadIdx.x;
+  if (kmajor) {
+    const int r = r0 + (t & 63), k = k0 + (t >> 6) * 16;
+    const T* src = P + (long)r * ld + k;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if (vec && r < R && k + q * 4 + 3 < K) load4(src + q * 4, v + q * 4);
+      else
+#pragma unroll
+        for (int j = 0; j < 4; ++j) v[q * 4 + j] = (r < R && k + q * 4 + j < K) ? to_f(src[q * 4 + j]) : 0.f;
+    }
+  } else {
+    const int r = r0 + (t & 15) * 4;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int k = k0 + (t >> 4) + q * 8;
+      const T* src = P + (long)k * ld + r;
+      if (vec && k < K && r + 3 < R) load4(src, v + q * 4);
+      else
+#pragma unroll
+        for (int j = 0; j < 4; ++j) v[q * 4 + j] = (k < K && r + j < R) ? to_f(src[j]) : 0.f;
+    }
+  }
+}
+__device__ __forceinline__ void slab_store(float (*S)[SG_LD], bool kmajor, const float* v) {
+  const int t = threadIdx.x;
+  if (kmajor) {
+#pragma unroll
+    for (int i = 0; i < 16; ++i) S[(t >> 6) * 16 + i][t & 63] = v[i];
+  } else {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) *reinterpret_cast<float4*>(&S[(t >> 4) + q * 8][(t & 15) * 4]) = make_float4(v[q * 4], v[q * 4 + 1], v[q * 4 + 2], v[q * 4 + 3]);
+  }
+}
 
 template <typename T, typename TC>
-__global__ void __launch_bounds__(SG_THREADS)
-gemm_simt_kernel(const T* __restrict__ A, long a_rs, long a_cs, const T* __restrict__ B, long b_rs, long b_cs,
-                 TC* __restrict__ C, int M, int N, int K, const float* __restrict__ bias, const TC* __restrict__ residual,
-                 int act, TC* __restrict__ aux_out, const T* __restrict__ aux_in) {
-  dependent_sync();
-  __shared__ float As[SG_BK][SG_BM + 4];
-  __shared__ float Bs[SG_BK][SG_BN + 4];
-  int tid = threadIdx.x;
-  int m0 = blockIdx.y * SG_BM, n0 = blockIdx.x * SG_BN;
-  int tx = tid % 16, ty = tid / 16;
-  float acc[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-  bool a_kmajor = (a_cs == 1), b_kmajor = (b_cs == 1);
-  for (int k0 = 0; k0 < K; k0 += SG_BK) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      int idx = tid + i * SG_THREADS;
-      int r, kk;
-      if (a_kmajor) { r = idx / SG_BK; kk = idx % SG_BK; } else { r = idx % SG_BM; kk = idx / SG_BM; }
-      int gm = m0 + r, gk = k0 + kk;
-      As[kk][r] = (gm < M && gk < K) ? to_f(A[(long)gm * a_rs + (long)gk * a_cs]) : 0.f;
-      if (b_kmajor) { r = idx / SG_BK; kk = idx % SG_BK; } else { r = idx % SG_BN; kk = idx / SG_BN; }
-      int gn = n0 + r;
-      gk = k0 + kk;
-      Bs[kk][r] = (gn < N && gk < K) ? to_f(B[(long)gn * b_rs + (long)gk * b_cs]) : 0.f;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < SG_BK; ++kk) {
-      float a[4], b[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[kk][ty * 4 + i];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx * 4 + j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    int gm = m0 + ty * 4 + i;
-    if (gm >= M) continue;
+struct SimtEpi {
+  TC* C;
+  const float* bias;
+  const TC* residual;
+  TC* aux_out;
+  const T* aux_in;
+  int M, N, act;
+  // four consecutive columns of one row
+  __device__ __forceinline__ void operator()(int gm, int gn, const float* acc) const {
+    if (gm >= M) return;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      int gn = n0 + tx * 4 + j;
-      if (gn >= N) continue;
-      size_t o = (size_t)gm * N + gn;
-      float v = acc[i][j];
-      if (bias != nullptr) v += bias[gn];
+      if (gn + j >= N) continue;
+      size_t o = (size_t)gm * N + gn + j;
+      float v = acc[j];
+      if (bias != nullptr) v += bias[gn + j];
       if (act == 1) {
         if (aux_out != nullptr) aux_out[o] = from_f<TC>(v);
         v = gelu_f(v);
@@ -76,34 +87,125 @@ gemm_simt_kernel(const T* __restrict__ A, long a_rs, long a_cs, const T* __restr
       C[o] = from_f<TC>(v);
     }
   }
+};
+
+template <typename T, typename TC>
+__global__ void __launch_bounds__(SG_THREADS)
+gemm_simt_kernel(const T* __restrict__ A, long lda, int a_kmajor, int a_vec, const T* __restrict__ B, long ldb, int b_kmajor, int b_vec,
+                 int K, int k_per_split, SimtEpi<T, TC> epi) {
+  __shared__ __align__(16) float As[2][SG_BK][SG_LD];
+  __shared__ __align__(16) float Bs[2][SG_BK][SG_LD];
+  if (leaves_sms_idle()) release_dependents();
+  await_inputs();
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const int m0 = blockIdx.y * SG_BM, n0 = blockIdx.x * SG_BN;
+  const int splits = gridDim.z, rank = blockIdx.z;
+  const int kb = rank * k_per_split, ke = min(K, kb + k_per_split);
+  float acc[8][4];
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+  float va[16], vb[16];
+  if (kb < ke) {
+    slab_load(A, lda, a_kmajor, a_vec, m0, kb, epi.M, ke, va);
+    slab_load(B, ldb, b_kmajor, b_vec, n0, kb, epi.N, ke, vb);
+    slab_store(As[0], a_kmajor, va);
+    slab_store(Bs[0], b_kmajor, vb);
+  }
+  __syncthreads();
+  int buf = 0;
+  for (int k0 = kb; k0 < ke; k0 += SG_BK) {
+    const bool more = k0 + SG_BK < ke;
+    if (more) {
+      slab_load(A, lda, a_kmajor, a_vec, m0, k0 + SG_BK, epi.M, ke, va);
+      slab_load(B, ldb, b_kmajor, b_vec, n0, k0 + SG_BK, epi.N, ke, vb);
+    }
+#pragma unroll 8
+    for (int kk = 0; kk < SG_BK; ++kk) {
+      float a[8], b[4];
+      load16(&As[buf][kk][ty * 8], a);
+      load16(&As[buf][kk][ty * 8 + 4], a + 4);
+      load16(&Bs[buf][kk][tx * 4], b);
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+    }
+    if (more) {
+      slab_store(As[buf ^ 1], a_kmajor, va);
+      slab_store(Bs[buf ^ 1], b_kmajor, vb);
+    }
+    __syncthreads();
+    buf ^= 1;
+  }
+  if (splits == 1) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) epi(m0 + ty * 8 + i, n0 + tx * 4, acc[i]);
+    return;
+  }
+  // partial tile [64][64] over the operand buffers; every rank sums and finishes its share of the tile
+  float* part = &As[0][0][0];
+  static_assert(sizeof(As) >= SG_BM * SG_BN * sizeof(float), "a partial tile fits the operand buffer");
+  cg::cluster_group cluster = cg::this_cluster();
+#pragma unroll
+  for (int i = 0; i < 8; ++i) store16(part + (ty * 8 + i) * SG_BN + tx * 4, acc[i]);
+  cluster.sync();
+  constexpr int UNITS = SG_BM * SG_BN / 4;
+  const int u1 = UNITS * (rank + 1) / splits;
+  for (int u = UNITS * rank / splits + tid; u < u1; u += SG_THREADS) {
+    float4 v[SG_MAXSPLIT];
+#pragma unroll
+    for (int s = 0; s < SG_MAXSPLIT; ++s)
+      if (s < splits) v[s] = *reinterpret_cast<const float4*>(cluster.map_shared_rank(part, s) + u * 4);
+    float4 t = v[0];
+#pragma unroll
+    for (int s = 1; s < SG_MAXSPLIT; ++s)
+      if (s < splits) { t.x += v[s].x; t.y += v[s].y; t.z += v[s].z; t.w += v[s].w; }
+    float o[4] = {t.x, t.y, t.z, t.w};
+    epi(m0 + u / (SG_BN / 4), n0 + (u % (SG_BN / 4)) * 4, o);
+  }
+  cluster.sync();                          // no CTA leaves while another may still read its partial tile
 }
 
+template <typename T, typename TC>
+static void launch_simt(const Ctx& c, const void* A, long a_rs, long a_cs, const void* B, long b_rs, long b_cs, void* C, int m, int n, int k,
+                        const GemmEpilogue& e) {
+  const int tiles_n = ceil_div(n, SG_BN), tiles = tiles_n * ceil_div(m, SG_BM);
+  // Splits: the SM with the most CTAs sets the time, each CTA costing its k range plus about 32 k steps of prologue and
+  // reduction; more than two CTAs per SM gain nothing.
+  const int sms = c.sm_count > 0 ? c.sm_count : B200_SMS;
+  int splits = 1, best = ceil_div(tiles, sms) * (k + 32);
+  for (int s = 2; s <= SG_MAXSPLIT && k >= s * 2 * SG_BK; ++s) {
+    int cost = ceil_div((long)tiles * s, sms) * (ceil_div(k, s) + 64);
+    if (cost < best) { best = cost; splits = s; }
+  }
+  const int per = ceil_div(ceil_div(k, splits), SG_BK) * SG_BK;
+  splits = ceil_div(k, per) < 1 ? 1 : ceil_div(k, per);
+  const bool ak = a_cs == 1, bk = b_cs == 1;
+  const long lda = ak ? a_rs : a_cs, ldb = bk ? b_rs : b_cs;
+  const size_t quad = 4 * sizeof(T);
+  SimtEpi<T, TC> epi = {(TC*)C, e.bias, (const TC*)e.residual, (TC*)e.aux_out, (const T*)e.aux_in, m, n, e.act};
+  launch_cluster(gemm_simt_kernel<T, TC>, dim3(tiles_n, ceil_div(m, SG_BM), splits), SG_THREADS, 0, c.stream, dim3(1, 1, splits), (const T*)A, lda, (int)ak,
+                 (int)(lda % 4 == 0 && (uintptr_t)A % quad == 0), (const T*)B, ldb, (int)bk, (int)(ldb % 4 == 0 && (uintptr_t)B % quad == 0), k, per, epi);
+}
+
+// Strides: A(m, k) = A[m * a_rs + k * a_cs], B alike; one stride of each operand is 1.
 void gemm(const Ctx& c, const void* A, long a_rs, long a_cs, const void* B, long b_rs, long b_cs, void* C,
           int out_is_float, int m, int n, int k, const GemmEpilogue& e) {
   if (m <= 0 || n <= 0) return;
   // The tensor-core kernels take any reduction length: what TMA wants aligned is the row pitch of each operand (checked
   // there), and slabs past the end arrive as zeros.  Weight gradients reduce over batch x tokens rows, which an odd batch
-  // leaves odd: at batch 45 of ViT-B they took 515 us a launch on the FP32-FMA kernel below, 18 us on the tensor cores.
+  // leaves odd: at batch 45 of ViT-B they took 515 us a launch on FP32 FMAs, 18 us on the tensor cores.
   if (c.dtype == 1 && c.use_tc && (n % 8) == 0) {
     if (c.use_tc >= 2 && m > 128 &&
         gemm_tc2_strided(c, A, a_rs, a_cs, B, b_rs, b_cs, C, out_is_float, m, n, k, e, c.split_ws, c.split_ws_floats) == 0) return;
     if (gemm_tc_strided(c, A, a_rs, a_cs, B, b_rs, b_cs, C, out_is_float, m, n, k, e, c.split_ws, c.split_ws_floats) == 0) return;
   }
-  dim3 grid(ceil_div(n, SG_BN), ceil_div(m, SG_BM));
   note_launch(1);
-  if (c.dtype == 0) {
-    launch_k(gemm_simt_kernel<float, float>, grid, SG_THREADS, 0, c.stream, 
-        (const float*)A, a_rs, a_cs, (const float*)B, b_rs, b_cs, (float*)C, m, n, k, e.bias, (const float*)e.residual,
-        e.act, (float*)e.aux_out, (const float*)e.aux_in);
-  } else if (out_is_float) {
-    launch_k(gemm_simt_kernel<bf16, float>, grid, SG_THREADS, 0, c.stream, 
-        (const bf16*)A, a_rs, a_cs, (const bf16*)B, b_rs, b_cs, (float*)C, m, n, k, e.bias, (const float*)e.residual,
-        e.act, (float*)e.aux_out, (const bf16*)e.aux_in);
-  } else {
-    launch_k(gemm_simt_kernel<bf16, bf16>, grid, SG_THREADS, 0, c.stream, 
-        (const bf16*)A, a_rs, a_cs, (const bf16*)B, b_rs, b_cs, (bf16*)C, m, n, k, e.bias, (const bf16*)e.residual,
-        e.act, (bf16*)e.aux_out, (const bf16*)e.aux_in);
-  }
+  if (c.dtype == 0) launch_simt<float, float>(c, A, a_rs, a_cs, B, b_rs, b_cs, C, m, n, k, e);
+  else if (out_is_float) launch_simt<bf16, float>(c, A, a_rs, a_cs, B, b_rs, b_cs, C, m, n, k, e);
+  else launch_simt<bf16, bf16>(c, A, a_rs, a_cs, B, b_rs, b_cs, C, m, n, k, e);
 }
 
 }  // namespace bsr

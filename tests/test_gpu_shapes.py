@@ -86,3 +86,21 @@ def test_eval_replay_equals_launch_by_launch(shift):
                 assert torch.equal(l0, l1) and all(torch.equal(a, b) for a, b in zip(k0, k1))
             assert not torch.equal(runs[0][0][0], runs[0][1][0])
     eng.close()
+
+
+@pytest.mark.parametrize("dtype,tol", [("fp32", 2e-6), ("bf16", 4e-3)])
+@pytest.mark.parametrize("m,n,k", [(1, 8, 8), (64, 64, 64), (65, 60, 63), (520, 192, 768), (33, 30, 1030), (2080, 576, 40)])
+def test_fma_contraction_forward_and_backward(m, n, k, dtype, tol):
+    """The FP32-FMA contraction at tile remainders and at one to eight splits of the reduction over a cluster, all three operand
+    orders: y = x W^T, dx = dy W, dW = dy^T x.  Tolerance: fp32 sums of up to 2080 products, or one bf16 rounding."""
+    import torch
+    from paper_2405_10951_b200 import binding as Bd
+    rng = np.random.default_rng(m + n + k)
+    mk = lambda *s: synth.round_to_bf16(rng.standard_normal(s)) if dtype == "bf16" else rng.standard_normal(s).astype(np.float32).astype(np.float64)
+    x, w, dy = mk(m, k), mk(n, k), mk(m, n)
+    dev = lambda a: torch.as_tensor(a.astype(np.float32)).cuda().to(torch.bfloat16 if dtype == "bf16" else torch.float32)
+    y = Bd.bsr_linear_forward(dev(x), dev(w))
+    dx, dw = Bd.bsr_linear_backward(dev(x), dev(w), dev(dy))
+    torch.cuda.synchronize()
+    for got, want in ((y, x @ w.T), (dx, dy @ w), (dw, dy.T @ x)):
+        assert P.rel_err(got.float().cpu().numpy(), want) < tol
