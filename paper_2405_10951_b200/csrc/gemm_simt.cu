@@ -172,17 +172,25 @@ template <typename T, typename TC>
 static void launch_simt(const Ctx& c, const void* A, long a_rs, long a_cs, const void* B, long b_rs, long b_cs, void* C, int m, int n, int k,
                         const GemmEpilogue& e) {
   const int tiles_n = ceil_div(n, SG_BN), tiles = tiles_n * ceil_div(m, SG_BM);
-  // Splits: the SM with the most CTAs sets the time, each CTA costing its k range plus about 32 k steps of prologue and
-  // reduction; more than two CTAs per SM gain nothing.
-  const int sms = c.sm_count > 0 ? c.sm_count : B200_SMS;
-  int splits = 1, best = ceil_div(tiles, sms) * (k + 32);
-  for (int s = 2; s <= SG_MAXSPLIT && k >= s * 2 * SG_BK; ++s) {
-    int cost = ceil_div((long)tiles * s, sms) * (ceil_div(k, s) + 64);
-    if (cost < best) { best = cost; splits = s; }
+  const bool ak = a_cs == 1, bk = b_cs == 1;
+  int splits;
+  if (ak) {
+    // A layer's output or input gradient: by the reduction length alone, so that an image's result does not depend on
+    // how many others are in the batch.
+    splits = ceil_div(k, 128) < SG_MAXSPLIT ? ceil_div(k, 128) : SG_MAXSPLIT;
+  } else {
+    // A weight gradient, reduced over the rows of the batch: the SM with the most CTAs sets the time, each CTA costing its
+    // k range plus about 32 k steps of prologue and as much for the reduction.
+    const int sms = c.sm_count > 0 ? c.sm_count : B200_SMS;
+    int best = ceil_div(tiles, sms) * (k + 32);
+    splits = 1;
+    for (int s = 2; s <= SG_MAXSPLIT && k >= s * 2 * SG_BK; ++s) {
+      int cost = ceil_div((long)tiles * s, sms) * (ceil_div(k, s) + 64);
+      if (cost < best) { best = cost; splits = s; }
+    }
   }
   const int per = ceil_div(ceil_div(k, splits), SG_BK) * SG_BK;
   splits = ceil_div(k, per) < 1 ? 1 : ceil_div(k, per);
-  const bool ak = a_cs == 1, bk = b_cs == 1;
   const long lda = ak ? a_rs : a_cs, ldb = bk ? b_rs : b_cs;
   const size_t quad = 4 * sizeof(T);
   SimtEpi<T, TC> epi = {(TC*)C, e.bias, (const TC*)e.residual, (TC*)e.aux_out, (const T*)e.aux_in, m, n, e.act};
