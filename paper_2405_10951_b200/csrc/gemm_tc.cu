@@ -204,6 +204,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     int quarter = warp & 3;                 // TMEM lanes 32*quarter .. 32*quarter+31 (fixed by the warp's rank)
     int chalf = ew >> 2;                    // which half of the tile's columns
     unsigned char* st = smem_dyn + (staging0 - smem_u32(smem_dyn)) + ew * STAGING_BYTES;
+    float* sbias = reinterpret_cast<float*>(st + 2048);      // behind the 32 rows of 64 bytes a bf16 chunk takes: bias, column scales
     int local = 0;
     bool ok = true;
     for (int w = blockIdx.x; w < work_items && ok; w += gridDim.x) {
@@ -216,25 +217,45 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       bool empty = wk.kb0 >= wk.kb1;          // an expert without tokens: its gradient tile is zero
       int row0 = mt * BM + quarter * 32;
       TOut* Cs = C + wk.c_off;
-      // float outputs without activation take the single-transposition path; their residual is fetched a chunk ahead
-      const bool f32_path = sizeof(TOut) == 4 && epw.act == 0 && epw.aux_out == nullptr;
+      // float outputs (never with an activation) are transposed once; their residual is fetched a chunk ahead
+      constexpr bool f32_path = sizeof(TOut) == 4;
       const bool has_res = f32_path && epw.residual != nullptr;
       // the stored pre-activation of the GELU derivative is fetched a chunk ahead as well
       const bool pre_z = sizeof(TOut) == 2 && epw.act == 2;       // (bf16 outputs: dz of the FFN backward)
       uint4 xn[8];
+      // Bias (and the column scales of 8-bit operands) of the tile are fetched before its accumulators are complete: read where
+      // they were added, they came from L2 (the operand ring leaves hardly any L1) and took 900 of the 1700 clocks of a chunk.
+      const int cb = nt * BN + chalf * HALF_CHUNKS * 32;
+      auto bias4 = [&](int cc) {               // a float output's four columns of chunk cc
+        const int col = cb + cc * 32 + (lane % 8) * 4;
+        return epw.bias != nullptr && col < N ? __ldg(reinterpret_cast<const float4*>(epw.bias + col)) : make_float4(0.f, 0.f, 0.f, 0.f);
+      };
+      float4 bn;
+      if (f32_path) {
+        bn = bias4(0);
+      } else if (lane < HALF_CHUNKS * 8) {
+        const int col = cb + lane * 4;
+        float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (epw.bias != nullptr) *reinterpret_cast<float4*>(sbias + lane * 4) = col < N ? __ldg(reinterpret_cast<const float4*>(epw.bias + col)) : z4;
+        if (FP8) *reinterpret_cast<float4*>(sbias + 128 + lane * 4) = col < N ? __ldg(reinterpret_cast<const float4*>(epw.col_scale + col)) : z4;
+      }
+      const float rs = FP8 && row0 + lane < M ? __ldg(epw.row_scale + row0 + lane) : 0.f;
       if (has_res) chunk_issue((const float*)epw.residual, N, row0, nt * BN + chalf * HALF_CHUNKS * 32, M, N, lane, xn);
       if (pre_z) chunk_issue((const bf16*)epw.aux_in, N, row0, nt * BN + chalf * HALF_CHUNKS * 32, M, N, lane, xn);
       ok = mbar_wait(tfull_bar(buf), (local >> 1) & 1, abortp);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
+      __syncwarp();
       tc_fence_after();
-      if (f32_path) {
+      if constexpr (f32_path) {
 #pragma unroll
         for (int cc = 0; cc < HALF_CHUNKS; ++cc) {
           int cchunk = chalf * HALF_CHUNKS + cc;
           uint4 xc[8];
 #pragma unroll
           for (int i = 0; i < 8; ++i) xc[i] = xn[i];
+          const float4 bb = bn;
+          if (cc + 1 < HALF_CHUNKS) bn = bias4(cc + 1);
           if (has_res && cc + 1 < HALF_CHUNKS) chunk_issue((const float*)epw.residual, N, row0, nt * BN + (cchunk + 1) * 32, M, N, lane, xn);
           uint32_t r[32];
           uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * BN + cchunk * 32);
@@ -244,7 +265,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
 #pragma unroll
             for (int j = 0; j < 32; ++j) r[j] = 0u;
           }
-          epilogue_chunk_f32(r, epw.bias, (float*)Cs, M, N, row0, nt * BN + cchunk * 32, st, lane, xc, has_res);
+          epilogue_chunk_f32(r, bb, (float*)Cs, M, N, row0, nt * BN + cchunk * 32, st, lane, xc, has_res);
         }
       } else {
 #pragma unroll 1
@@ -263,7 +284,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
 #pragma unroll
           for (int j = 0; j < 32; ++j) r[j] = 0u;
         }
-        epilogue_chunk<TOut>(r, epw, Cs, M, N, row0, nt * BN + cchunk * 32, st, lane, pre_z ? z : nullptr);
+        epilogue_chunk<TOut>(r, epw, epw.bias != nullptr ? sbias + cc * 32 : nullptr, FP8 ? sbias + 128 + cc * 32 : nullptr, rs, Cs, M, N, row0,
+                             nt * BN + cchunk * 32, st, lane, pre_z ? z : nullptr);
       }
       }
       tc_fence_before();
@@ -440,6 +462,7 @@ int gemm_tc_strided(const Ctx& c, const void* A, long a_rs, long a_cs, const voi
   if ((n % 8) != 0) return -1;
   if (a_mn && (m % 8) != 0) return -1;
   if (a_mn && !b_mn) return -1;                 // combination not instantiated
+  if (out_is_float && e.act != 0) return -1;    // activations belong to bf16 outputs
   CUtensorMap ma, mb;
   bool ok = a_mn ? make_map(&ma, A, (uint64_t)m, (uint64_t)k, (uint64_t)lda, BK) : make_map(&ma, A, (uint64_t)k, (uint64_t)m, (uint64_t)lda, BM);
   int sms = c.sm_count > 0 ? c.sm_count : 148;
@@ -517,6 +540,7 @@ int gemm_tc_grouped_rows(const Ctx& c, const void* A, const void* Bst, int b_mn,
                          int experts, const int* tile_expert, const GemmEpilogue& e) {
   using namespace tc;
   if ((n % 8) || (k % 8) || (rows_cap % BM) || ((uintptr_t)A & 15) || ((uintptr_t)Bst & 15) || ((uintptr_t)C & 15)) return -1;
+  if (out_is_float && e.act != 0) return -1;
   if (b_mn && (k % BK)) return -1;             // a k-slab must not straddle two experts' weights
   CUtensorMap ma, mb;
   bool ok = make_map(&ma, A, (uint64_t)k, (uint64_t)rows_cap, (uint64_t)k, BM);

@@ -113,7 +113,11 @@ struct ChunkIO {
   static constexpr int E = 16 / sizeof(T);          // elements per 16-byte unit
   static constexpr int UNITS = 32 / E;               // units per chunk row: 4 (bf16) or 8 (float)
   static constexpr int ROWS_PER_PASS = 32 / UNITS;
-  __device__ static uint32_t slot(int r, int u) { return (uint32_t)(r * 128 + ((u ^ (r & 7)) << 4)); }
+  // rows of 128 bytes (float) or 64 bytes (bf16); the order of a row's units depends on the row so that neither direction
+  // has bank conflicts
+  __device__ static uint32_t slot(int r, int u) {
+    return sizeof(T) == 4 ? (uint32_t)(r * 128 + ((u ^ (r & 7)) << 4)) : (uint32_t)(r * 64 + ((u ^ ((r >> 1) & 3)) << 4));
+  }
 
   // All global loads are issued before the first shared-memory store: the staging pointer may alias anything as
   // far as the compiler knows, so a load placed after a store could not be moved ahead of it.
@@ -181,30 +185,26 @@ template <> __device__ __forceinline__ uint4 ChunkIO<bf16>::pack(const float* f)
 
 // v[j]: accumulator of (row0 + lane, col0 + j).  All lanes of the warp take part (row0, col0 are warp-uniform).
 // zpre: the chunk of the stored pre-activation for act == 2, already in this lane's row order (or null: loaded here).
+// sbias, scol: the chunk's 32 bias values and column scales in shared memory (null: none), rs: this lane's row scale.
 template <typename TOut>
-__device__ __forceinline__ void epilogue_chunk(const uint32_t* r, const Epi& ep, TOut* Cs, int M, int N, int row0, int col0,
-                                               unsigned char* st, int lane, const float* zpre = nullptr) {
+__device__ __forceinline__ void epilogue_chunk(const uint32_t* r, const Epi& ep, const float* sbias, const float* scol, float rs, TOut* Cs, int M,
+                                               int N, int row0, int col0, unsigned char* st, int lane, const float* zpre = nullptr) {
   if (row0 < M && col0 < N) {
     float v[32];
 #pragma unroll
     for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
-    if (ep.row_scale != nullptr) {
-      float rs = row0 + lane < M ? __ldg(ep.row_scale + row0 + lane) : 0.f;
+    if (scol != nullptr) {
 #pragma unroll
       for (int g = 0; g < 8; ++g) {
-        if (col0 + g * 4 < N) {
-          float4 cs = __ldg(reinterpret_cast<const float4*>(ep.col_scale + col0 + g * 4));
-          v[g * 4 + 0] *= rs * cs.x; v[g * 4 + 1] *= rs * cs.y; v[g * 4 + 2] *= rs * cs.z; v[g * 4 + 3] *= rs * cs.w;
-        }
+        float4 cs = *reinterpret_cast<const float4*>(scol + g * 4);
+        v[g * 4 + 0] *= rs * cs.x; v[g * 4 + 1] *= rs * cs.y; v[g * 4 + 2] *= rs * cs.z; v[g * 4 + 3] *= rs * cs.w;
       }
     }
-    if (ep.bias != nullptr) {
+    if (sbias != nullptr) {
 #pragma unroll
       for (int g = 0; g < 8; ++g) {
-        if (col0 + g * 4 < N) {
-          float4 bb = __ldg(reinterpret_cast<const float4*>(ep.bias + col0 + g * 4));
-          v[g * 4 + 0] += bb.x; v[g * 4 + 1] += bb.y; v[g * 4 + 2] += bb.z; v[g * 4 + 3] += bb.w;
-        }
+        float4 bb = *reinterpret_cast<const float4*>(sbias + g * 4);
+        v[g * 4 + 0] += bb.x; v[g * 4 + 1] += bb.y; v[g * 4 + 2] += bb.z; v[g * 4 + 3] += bb.w;
       }
     }
     if (ep.act == 1) {
@@ -252,7 +252,8 @@ __device__ __forceinline__ void chunk_issue(const float* g, int ld, int row0, in
     if (row0 + r < M && col < N) x[i] = ld_stream(g + (size_t)(row0 + r) * ld + col);
   }
 }
-__device__ __forceinline__ void epilogue_chunk_f32(const uint32_t* r, const float* bias, float* Cs, int M, int N, int row0, int col0,
+// bb: bias of columns col0 + 4 (lane % 8) .. + 3.
+__device__ __forceinline__ void epilogue_chunk_f32(const uint32_t* r, float4 bb, float* Cs, int M, int N, int row0, int col0,
                                                    unsigned char* st, int lane, const uint4* xres, bool has_res) {
   if (row0 < M && col0 < N) {
     using IO = ChunkIO<float>;
@@ -261,8 +262,6 @@ __device__ __forceinline__ void epilogue_chunk_f32(const uint32_t* r, const floa
       *reinterpret_cast<uint4*>(st + IO::slot(lane, u)) = make_uint4(r[4 * u], r[4 * u + 1], r[4 * u + 2], r[4 * u + 3]);
     __syncwarp();
     int u = lane % 8, col = col0 + u * 4;
-    float4 bb = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (bias != nullptr && col < N) bb = __ldg(reinterpret_cast<const float4*>(bias + col));
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       int rr = i * 4 + lane / 8;
