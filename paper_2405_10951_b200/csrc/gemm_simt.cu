@@ -206,8 +206,11 @@ void gemm(const Ctx& c, const void* A, long a_rs, long a_cs, const void* B, long
   // there), and slabs past the end arrive as zeros.  Weight gradients reduce over batch x tokens rows, which an odd batch
   // leaves odd: at batch 45 of ViT-B they took 515 us a launch on FP32 FMAs, 18 us on the tensor cores.
   if (c.dtype == 1 && c.use_tc && (n % 8) == 0) {
-    if (c.use_tc >= 2 && m > 128 &&
-        gemm_tc2_strided(c, A, a_rs, a_cs, B, b_rs, b_cs, C, out_is_float, m, n, k, e, c.split_ws, c.split_ws_floats) == 0) return;
+    // CTA pairs where a wide output over many rows keeps all of them busy (QKV and first FFN layer of ViT-B from batch 61):
+    // 25216 x 2304 x 768 73.1 -> 71.4 us, and less power, which is what limits a long run (ViT-B step at batch 128 5.81 -> 5.72 ms,
+    // inference 3.93 -> 3.86 ms).  Narrower outputs lose (25216 x 768 x 3072: 92 -> 107 us; B read across k: 159 -> 166 us).
+    const bool pairs = c.use_tc >= 2 ? m > 128 : (m >= 12000 && n >= 2048 && a_cs == 1 && b_cs == 1);
+    if (pairs && gemm_tc2_strided(c, A, a_rs, a_cs, B, b_rs, b_cs, C, out_is_float, m, n, k, e) == 0) return;
     if (gemm_tc_strided(c, A, a_rs, a_cs, B, b_rs, b_cs, C, out_is_float, m, n, k, e, c.split_ws, c.split_ws_floats) == 0) return;
   }
   note_launch(1);

@@ -204,7 +204,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     int quarter = warp & 3;                 // TMEM lanes 32*quarter .. 32*quarter+31 (fixed by the warp's rank)
     int chalf = ew >> 2;                    // which half of the tile's columns
     unsigned char* st = smem_dyn + (staging0 - smem_u32(smem_dyn)) + ew * STAGING_BYTES;
-    float* sbias = reinterpret_cast<float*>(st + 2048);      // behind the 32 rows of 64 bytes a bf16 chunk takes: bias, column scales
     int local = 0;
     bool ok = true;
     for (int w = blockIdx.x; w < work_items && ok; w += gridDim.x) {
@@ -212,82 +211,16 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       if (!wk.active) continue;
       int nt = wk.nt, mt = wk.mt;
       int buf = local & 1;
-      Epi epw = ep;
-      if (epw.bias != nullptr) epw.bias += wk.bias_off;
-      bool empty = wk.kb0 >= wk.kb1;          // an expert without tokens: its gradient tile is zero
-      int row0 = mt * BM + quarter * 32;
-      TOut* Cs = C + wk.c_off;
-      // float outputs (never with an activation) are transposed once; their residual is fetched a chunk ahead
-      constexpr bool f32_path = sizeof(TOut) == 4;
-      const bool has_res = f32_path && epw.residual != nullptr;
-      // the stored pre-activation of the GELU derivative is fetched a chunk ahead as well
-      const bool pre_z = sizeof(TOut) == 2 && epw.act == 2;       // (bf16 outputs: dz of the FFN backward)
-      uint4 xn[8];
-      // Bias (and the column scales of 8-bit operands) of the tile are fetched before its accumulators are complete: read where
-      // they were added, they came from L2 (the operand ring leaves hardly any L1) and took 900 of the 1700 clocks of a chunk.
-      const int cb = nt * BN + chalf * HALF_CHUNKS * 32;
-      auto bias4 = [&](int cc) {               // a float output's four columns of chunk cc
-        const int col = cb + cc * 32 + (lane % 8) * 4;
-        return epw.bias != nullptr && col < N ? __ldg(reinterpret_cast<const float4*>(epw.bias + col)) : make_float4(0.f, 0.f, 0.f, 0.f);
+      auto ready = [&]() {
+        bool w = mbar_wait(tfull_bar(buf), (local >> 1) & 1, abortp);
+        w = __all_sync(0xffffffffu, w);
+        tc_fence_after();
+        return w;
       };
-      float4 bn;
-      if (f32_path) {
-        bn = bias4(0);
-      } else if (lane < HALF_CHUNKS * 8) {
-        const int col = cb + lane * 4;
-        float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (epw.bias != nullptr) *reinterpret_cast<float4*>(sbias + lane * 4) = col < N ? __ldg(reinterpret_cast<const float4*>(epw.bias + col)) : z4;
-        if (FP8) *reinterpret_cast<float4*>(sbias + 128 + lane * 4) = col < N ? __ldg(reinterpret_cast<const float4*>(epw.col_scale + col)) : z4;
-      }
-      const float rs = FP8 && row0 + lane < M ? __ldg(epw.row_scale + row0 + lane) : 0.f;
-      if (has_res) chunk_issue((const float*)epw.residual, N, row0, nt * BN + chalf * HALF_CHUNKS * 32, M, N, lane, xn);
-      if (pre_z) chunk_issue((const bf16*)epw.aux_in, N, row0, nt * BN + chalf * HALF_CHUNKS * 32, M, N, lane, xn);
-      ok = mbar_wait(tfull_bar(buf), (local >> 1) & 1, abortp);
-      ok = __all_sync(0xffffffffu, ok);
+      ok = epilogue_tile<TOut, FP8>(ready, ep, wk.bias_off, C + wk.c_off, M, N, mt * BM + quarter * 32, nt * BN + chalf * HALF_CHUNKS * 32, HALF_CHUNKS,
+                                    tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * BN + chalf * HALF_CHUNKS * 32),
+                                    wk.kb0 >= wk.kb1, st, lane);
       if (!ok) break;
-      __syncwarp();
-      tc_fence_after();
-      if constexpr (f32_path) {
-#pragma unroll
-        for (int cc = 0; cc < HALF_CHUNKS; ++cc) {
-          int cchunk = chalf * HALF_CHUNKS + cc;
-          uint4 xc[8];
-#pragma unroll
-          for (int i = 0; i < 8; ++i) xc[i] = xn[i];
-          const float4 bb = bn;
-          if (cc + 1 < HALF_CHUNKS) bn = bias4(cc + 1);
-          if (has_res && cc + 1 < HALF_CHUNKS) chunk_issue((const float*)epw.residual, N, row0, nt * BN + (cchunk + 1) * 32, M, N, lane, xn);
-          uint32_t r[32];
-          uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * BN + cchunk * 32);
-          tmem_ld32(taddr, r);
-          tmem_ld_wait();
-          if (empty) {
-#pragma unroll
-            for (int j = 0; j < 32; ++j) r[j] = 0u;
-          }
-          epilogue_chunk_f32(r, bb, (float*)Cs, M, N, row0, nt * BN + cchunk * 32, st, lane, xc, has_res);
-        }
-      } else {
-#pragma unroll 1
-      for (int cc = 0; cc < HALF_CHUNKS; ++cc) {
-        int cchunk = chalf * HALF_CHUNKS + cc;
-        float z[sizeof(TOut) == 2 ? 32 : 1];
-        if (sizeof(TOut) == 2 && pre_z) {
-          chunk_land_bf16(xn, st, lane, z);
-          if (cc + 1 < HALF_CHUNKS) chunk_issue((const bf16*)epw.aux_in, N, row0, nt * BN + (cchunk + 1) * 32, M, N, lane, xn);
-        }
-        uint32_t r[32];
-        uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * BN + cchunk * 32);
-        tmem_ld32(taddr, r);
-        tmem_ld_wait();
-        if (empty) {
-#pragma unroll
-          for (int j = 0; j < 32; ++j) r[j] = 0u;
-        }
-        epilogue_chunk<TOut>(r, epw, epw.bias != nullptr ? sbias + cc * 32 : nullptr, FP8 ? sbias + 128 + cc * 32 : nullptr, rs, Cs, M, N, row0,
-                             nt * BN + cchunk * 32, st, lane, pre_z ? z : nullptr);
-      }
-      }
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(tempty_bar(buf));
@@ -408,6 +341,17 @@ bool make_map(CUtensorMap* map, const void* ptr, uint64_t inner, uint64_t outer,
   cuuint32_t box[2] = {64, box_outer};
   cuuint32_t estr[2] = {1, 1};
   return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(ptr), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+            CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+bool make_map_chunks(CUtensorMap* map, const void* ptr, uint64_t extent, uint64_t outer, uint64_t ld, uint32_t box_chunks) {
+  EncodeFn fn = encode_fn();
+  if (fn == nullptr) return false;
+  cuuint64_t dims[3] = {64, outer, extent / 64};
+  cuuint64_t strides[2] = {ld * 2, 128};
+  cuuint32_t box[3] = {64, 64, box_chunks};
+  cuuint32_t estr[3] = {1, 1, 1};
+  return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 

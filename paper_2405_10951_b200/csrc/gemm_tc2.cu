@@ -1,13 +1,14 @@
 // bf16 GEMM on CTA pairs: tcgen05.mma cta_group::2 with a 256 x 256 accumulator tile spread over the tensor
-// memory of two SMs.  Same contract as the single-CTA kernel (operand majors, epilogues, split-k), but each SM
-// stages only its own 128 rows of A and its own 128 columns' worth of B per k-slab (32 KB instead of 48 KB
-// for the same number of multiply-accumulates), which is what the per-SM shared-memory fill rate limits.
+// memory of two SMs.  Same contract as the single-CTA kernel for an operand A read along k, but each SM stages only its
+// own 128 rows of A and its own half of the columns of B per k-slab: 32 KB instead of 48 KB for the same number of
+// multiply-accumulates.  That is what bounds the single-CTA kernel's main loop: four slabs of 48 KB in flight cover less
+// than the 2000-odd clocks a slab takes to arrive; six slabs of 32 KB fit here.
 //
 // Cluster of two CTAs, persistent, one cluster per SM pair:
 //   warp 0 (both CTAs) : TMA producer; every copy signals the full barrier of the leader CTA (rank 0)
 //   warp 1 (leader)    : issues the MMAs; its commits arrive on the empty / accumulator-full barriers of both CTAs
 //   warps 2..9 (both)  : epilogue of the CTA's own 128 rows; they release the accumulator on the leader's barrier
-// Five-stage ring of 32 KB per CTA; the epilogue prefetches residual / pre-activation chunks with cp.async.  Waits are bounded as in the single-CTA kernel.
+// Waits are bounded as in the single-CTA kernel.
 #include <cuda.h>
 
 #include "common.cuh"
@@ -23,13 +24,13 @@ using namespace tc;
 constexpr int BM = 128;                   // rows per CTA (256 per pair)
 constexpr int BN = 256;                   // columns per pair tile; each CTA stages BN/2 of B
 constexpr int BK = 64;
-constexpr int STAGES = 5;
+constexpr int STAGES = 6;
 constexpr int UMMA_K = 16;
 constexpr int A_BYTES = BM * BK * 2, B_BYTES = (BN / 2) * BK * 2;
 constexpr int STAGE_BYTES = A_BYTES + B_BYTES;      // 32 KB
 constexpr int EPI_WARPS = 8;
 constexpr int STAGING_BYTES = 32 * 128;
-constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 2 * EPI_WARPS * STAGING_BYTES + 1024 + 256;
+constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + EPI_WARPS * STAGING_BYTES + 1024 + 256;
 constexpr int THREADS = 64 + EPI_WARPS * 32;
 constexpr uint32_t TMEM_COLS = 512;
 constexpr uint32_t PEER_MASK = 0xFEFFFFFFu;         // clears the CTA-rank bit of a shared address: the even CTA of the pair
@@ -79,26 +80,71 @@ __device__ __forceinline__ void mbar_arrive_leader(uint32_t bar) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(remote) : "memory");
 }
 
-template <bool A_MN, bool B_MN, typename TOut>
+
+// The tiles of one pair.  Whole tiles go round in as many full waves as there are; the tiles of a last wave that would leave
+// pairs idle are cut along n into as many parts as there are pairs for them (25216 rows are 98.5 tiles of 256: at 768 columns
+// 297 tiles on 74 pairs, the last wave a single tile).  Parts are multiples of UNIT columns: 64, or 128 where B is read
+// across k (64-column chunks for each CTA).  Stepping to the next whole tile takes no division.
+struct Tile {
+  int mt, n0, width;
+};
+template <int UNIT>
+struct Walk {
+  static constexpr int UNITS = BN / UNIT;
+  int i, row, nt, step, full, items, parts, workers;
+  __device__ __forceinline__ static int part_units(int parts) { return (UNITS + parts - 1) / parts; }
+  __device__ __forceinline__ Walk(int tiles_m, int tiles_n, int worker, int workers_) {
+    const int total = tiles_m * tiles_n;
+    workers = workers_;
+    full = total - total % workers;
+    const int rem = total - full;
+    parts = rem > 0 ? min(UNITS, workers / rem) : 1;
+    parts = (UNITS + part_units(parts) - 1) / part_units(parts);
+    items = full + rem * parts;
+    i = worker;
+    row = i / tiles_n;
+    nt = i - row * tiles_n;
+    step = (workers / tiles_n) << 16 | (workers % tiles_n);
+  }
+  __device__ __forceinline__ bool next(int N, int tiles_n, Tile& t) {
+    if (i >= items) return false;
+    int off = 0, r = row, c = nt;
+    t.width = BN;
+    if (i >= full && parts > 1) {            // each pair comes here once at most
+      const int j = i - full, q = j / parts, pu = part_units(parts), tile = full + q;
+      r = tile / tiles_n;
+      c = tile - r * tiles_n;
+      off = (j - q * parts) * pu;
+      t.width = min(pu, UNITS - off) * UNIT;
+    }
+    i += workers;
+    row += step >> 16;
+    nt += step & 0xffff;
+    if (nt >= tiles_n) { nt -= tiles_n; ++row; }
+    t.mt = r;
+    t.n0 = c * BN + off * UNIT;
+    return t.n0 < N;                         // false: a part past the last column, the last of this pair's items
+  }
+};
+
+template <bool B_MN, typename TOut>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
-gemm_tc2_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, TOut* __restrict__ C,
-                int M, int N, int K, Epi ep, int pairs_m, int tiles_n, int splits, int kb_per_split, int* status) {
+gemm_tc2_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, const __grid_constant__ CUtensorMap map_part,
+                int wide, TOut* __restrict__ C, int M, int N, int K, Epi ep, int tiles_m, int tiles_n, int* status) {
   extern __shared__ unsigned char smem_dyn[];
   uint32_t base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
   uint32_t staging0 = base + STAGES * STAGE_BYTES;
-  uint32_t bars = staging0 + 2 * EPI_WARPS * STAGING_BYTES;   // full[STAGES], empty[STAGES], tfull[2], tempty[2]
+  uint32_t bars = staging0 + EPI_WARPS * STAGING_BYTES;   // full[STAGES], empty[STAGES], tfull[2], tempty[2]
   auto full_bar = [&](int s) { return bars + 8u * s; };
   auto empty_bar = [&](int s) { return bars + 8u * (STAGES + s); };
   auto tfull_bar = [&](int b) { return bars + 8u * (2 * STAGES + b); };
   auto tempty_bar = [&](int b) { return bars + 8u * (2 * STAGES + 2 + b); };
   __shared__ uint32_t tmem_base_slot;
   __shared__ int abort_flag;
-  int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  uint32_t rank = cluster_rank();
-  bool leader = rank == 0;
-  int cluster_id = blockIdx.x >> 1, n_clusters = gridDim.x >> 1;
-  int total_kb = (K + BK - 1) / BK;
-  int work_items = pairs_m * tiles_n * splits;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t rank = cluster_rank();
+  const bool leader = rank == 0;
+  const int total_kb = (K + BK - 1) / BK;
 
   if (threadIdx.x == 0) {
     abort_flag = 0;
@@ -114,7 +160,10 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
   cluster_sync_all();                       // barriers of both CTAs exist before anyone signals them
   tc_fence_after();
   uint32_t tmem_base = tmem_base_slot;
+  await_inputs();                           // (fills the SMs: see release_dependents)
   volatile int* abortp = &abort_flag;
+  Walk<B_MN ? 128 : 64> walk(tiles_m, tiles_n, blockIdx.x >> 1, gridDim.x >> 1);
+  Tile t;
 
   if (warp == 0) {
     // ------------------------------- TMA producer (both CTAs) -------------------------------
@@ -123,27 +172,25 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
       uint32_t phase = 0;
       int armed = 0;
       bool ok = true;
-      for (int w = cluster_id; w < work_items && ok; w += n_clusters) {
-        int nt = w % tiles_n, pm = (w / tiles_n) % pairs_m, sp = w / (pairs_m * tiles_n);
-        int kb0 = sp * kb_per_split, kb1 = min(total_kb, kb0 + kb_per_split);
-        int m0 = pm * (2 * BM) + (int)rank * BM;          // this CTA's rows of A
-        int n0 = nt * BN + (int)rank * (BN / 2);          // this CTA's share of B
-        for (int kb = kb0; kb < kb1; ++kb) {
+      while (ok && walk.next(N, tiles_n, t)) {
+        const int m0 = t.mt * (2 * BM) + (int)rank * BM;        // this CTA's rows of A
+        const int cols = t.width >> 1, n0 = t.n0 + (int)rank * cols;   // this CTA's share of B
+        const bool whole = t.width == BN && wide;
+        const uint32_t bytes = 2u * (uint32_t)(A_BYTES + cols * (BK * 2));
+        for (int kb = 0; kb < total_kb; ++kb) {
           if (!mbar_wait(empty_bar(stage), phase ^ 1u, abortp)) { ok = false; break; }
-          uint32_t fb = full_bar(stage) & PEER_MASK;      // the leader's barrier collects both CTAs' bytes
-          if (leader) mbar_expect_tx(full_bar(stage), 2 * STAGE_BYTES);
-          uint32_t sa = base + stage * STAGE_BYTES, sb = sa + A_BYTES;
-          if (!A_MN) {
-            tma_load_2d_pair(sa, &map_a, fb, kb * BK, m0);
+          const uint32_t fb = full_bar(stage) & PEER_MASK;      // the leader's barrier collects both CTAs' bytes
+          if (leader) mbar_expect_tx(full_bar(stage), bytes);
+          const uint32_t sa = base + stage * STAGE_BYTES, sb = sa + A_BYTES;
+          tma_load_2d_pair(sa, &map_a, fb, kb * BK, m0);
+          if (whole) {
+            if (!B_MN) tma_load_2d_pair(sb, &map_b, fb, kb * BK, n0);
+            else tma_load_3d_pair(sb, &map_b, fb, 0, kb * BK, n0 >> 6);
           } else {
-#pragma unroll
-            for (int j = 0; j < BM / 64; ++j) tma_load_2d_pair(sa + j * (BK * 128), &map_a, fb, m0 + j * 64, kb * BK);
-          }
-          if (!B_MN) {
-            tma_load_2d_pair(sb, &map_b, fb, kb * BK, n0);
-          } else {
-#pragma unroll
-            for (int j = 0; j < BN / 128; ++j) tma_load_2d_pair(sb + j * (BK * 128), &map_b, fb, n0 + j * 64, kb * BK);
+            for (int j = 0; j < cols; j += B_MN ? 64 : 32) {
+              if (!B_MN) tma_load_2d_pair(sb + j * 128, &map_part, fb, kb * BK, n0 + j);
+              else tma_load_2d_pair(sb + j * (BK * 2), &map_part, fb, n0 + j, kb * BK);
+            }
           }
           ++armed;
           if (++stage == STAGES) { stage = 0; phase ^= 1u; }
@@ -157,28 +204,27 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
   } else if (warp == 1) {
     // ------------------------------- MMA issuer (leader CTA only) ---------------------------
     if (lane == 0 && leader) {
-      constexpr uint32_t idesc = make_idesc_mn(2 * BM, BN, A_MN, B_MN);
+      constexpr uint32_t idesc0 = make_idesc_mn(2 * BM, 0, false, B_MN);
+      constexpr uint32_t A_KSTEP = (UMMA_K * 2) >> 4, B_KSTEP = (B_MN ? UMMA_K * 128 : UMMA_K * 2) >> 4;
+      const uint64_t desc_a0 = make_desc(base, 16, 1024);
+      const uint64_t desc_b0 = B_MN ? make_desc(base + A_BYTES, BK * 128, 1024) : make_desc(base + A_BYTES, 16, 1024);
       int stage = 0;
       uint32_t phase = 0;
       int local = 0;
       bool ok = true;
-      for (int w = cluster_id; w < work_items && ok; w += n_clusters, ++local) {
-        int sp = w / (pairs_m * tiles_n);
-        int kb0 = sp * kb_per_split, kb1 = min(total_kb, kb0 + kb_per_split);
-        int buf = local & 1;
+      for (; ok && walk.next(N, tiles_n, t); ++local) {
+        const int buf = local & 1;
+        const uint32_t idesc = idesc0 | ((uint32_t)(t.width >> 3) << 17);
         if (!mbar_wait(tempty_bar(buf), ((local >> 1) & 1) ^ 1u, abortp)) { ok = false; break; }
         tc_fence_after();
-        uint32_t d_tmem = tmem_base + buf * BN;
-        for (int kb = kb0; kb < kb1; ++kb) {
+        const uint32_t d_tmem = tmem_base + buf * BN;
+        for (int kb = 0; kb < total_kb; ++kb) {
           if (!mbar_wait(full_bar(stage), phase, abortp)) { ok = false; break; }
           tc_fence_after();
-          uint32_t sa = base + stage * STAGE_BYTES, sb = sa + A_BYTES;
+          const uint64_t off = (uint64_t)((stage * STAGE_BYTES) >> 4);
 #pragma unroll
-          for (int k = 0; k < BK / UMMA_K; ++k) {
-            uint64_t da = A_MN ? make_desc(sa + k * (UMMA_K * 128), BK * 128, 1024) : make_desc(sa + k * (UMMA_K * 2), 16, 1024);
-            uint64_t db = B_MN ? make_desc(sb + k * (UMMA_K * 128), BK * 128, 1024) : make_desc(sb + k * (UMMA_K * 2), 16, 1024);
-            umma_bf16_pair(d_tmem, da, db, idesc, (kb > kb0 || k > 0) ? 1u : 0u);
-          }
+          for (int k = 0; k < BK / UMMA_K; ++k)
+            umma_bf16_pair(d_tmem, desc_a0 + off + (uint64_t)(k * A_KSTEP), desc_b0 + off + (uint64_t)(k * B_KSTEP), idesc, (kb > 0 || k > 0) ? 1u : 0u);
           umma_commit_pair(empty_bar(stage));
           if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
@@ -187,32 +233,24 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     }
   } else {
     // ------------------------------- epilogue (both CTAs, own rows) --------------------------
-    int ew = warp - 2;
-    int quarter = warp & 3;
-    int chalf = ew >> 2;
-    uint32_t st_in_addr = staging0 + (2 * ew) * STAGING_BYTES;
-    unsigned char* st_in = smem_dyn + (st_in_addr - smem_u32(smem_dyn));
-    unsigned char* st_out = st_in + STAGING_BYTES;
+    const int ew = warp - 2, quarter = warp & 3, chalf = ew >> 2;
+    unsigned char* st = smem_dyn + (staging0 - smem_u32(smem_dyn)) + ew * STAGING_BYTES;
     int local = 0;
-    bool ok = true;
-    for (int w = cluster_id; w < work_items && ok; w += n_clusters, ++local) {
-      int nt = w % tiles_n, pm = (w / tiles_n) % pairs_m, sp = w / (pairs_m * tiles_n);
-      int buf = local & 1;
-      ok = mbar_wait(tfull_bar(buf), (local >> 1) & 1, abortp);
-      ok = __all_sync(0xffffffffu, ok);
-      if (!ok) break;
-      tc_fence_after();
-      int row0 = pm * (2 * BM) + (int)rank * BM + quarter * 32;
-      TOut* Cs = C + (size_t)sp * M * N;
-      uint32_t taddr0 = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * BN + chalf * 128);
-      auto load_tmem = [&](int cc, uint32_t* r) {
-        tmem_ld32(taddr0 + cc * 32, r);
-        tmem_ld_wait();
+    while (walk.next(N, tiles_n, t)) {
+      const int buf = local & 1, nc = t.width >> 6;      // chunks of 32 columns for each half of the warps
+      auto ready = [&]() {
+        bool w = mbar_wait(tfull_bar(buf), (local >> 1) & 1, abortp);
+        w = __all_sync(0xffffffffu, w);
+        tc_fence_after();
+        return w;
       };
-      epilogue_warp_tile<TOut>(load_tmem, ep, Cs, M, N, row0, nt * BN + chalf * 128, 4, st_in, st_in_addr, st_out, lane, false);
+      if (!epilogue_tile<TOut, false>(ready, ep, 0, C, M, N, t.mt * (2 * BM) + (int)rank * BM + quarter * 32, t.n0 + chalf * nc * 32, nc,
+                                      tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * BN + chalf * nc * 32), false, st, lane))
+        break;
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive_leader(tempty_bar(buf));
+      ++local;
     }
   }
   tc_fence_before();
@@ -225,73 +263,52 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
   if (threadIdx.x == 0 && abort_flag && status != nullptr) atomicOr(status, STATUS_TIMEOUT);
 }
 
-template <bool A_MN, bool B_MN, typename TOut>
-static int launch(const Ctx& c, const CUtensorMap& ma, const CUtensorMap& mb, void* C, int m, int n, int k, const Epi& ep,
-                  int pairs_m, int tiles_n, int splits, int kb_per_split) {
-  auto kern = gemm_tc2_kernel<A_MN, B_MN, TOut>;
+template <bool B_MN, typename TOut>
+static int launch(const Ctx& c, const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorMap& mp, int wide, void* C, int m, int n, int k,
+                  const Epi& ep, int tiles_m, int tiles_n) {
+  auto kern = gemm_tc2_kernel<B_MN, TOut>;
   static SmemLimit lim;
   if (!ensure_smem(lim, kern, SMEM_BYTES)) return -3;
-  int work = pairs_m * tiles_n * splits;
-  int sms = c.sm_count > 0 ? c.sm_count : 148;
-  int clusters = work < sms / 2 ? work : sms / 2;
+  const long work = (long)tiles_m * tiles_n * (BN / (B_MN ? 128 : 64));
+  const int pairs = (c.sm_count > 0 ? c.sm_count : B200_SMS) / 2;
   note_launch(1);
-  kern<<<2 * clusters, THREADS, SMEM_BYTES, c.stream>>>(ma, mb, (TOut*)C, m, n, k, ep, pairs_m, tiles_n, splits, kb_per_split, c.status);
+  launch_k(kern, 2 * (int)(work < pairs ? work : pairs), THREADS, SMEM_BYTES, c.stream, ma, mb, mp, wide, (TOut*)C, m, n, k, ep, tiles_m, tiles_n, c.status);
   return 0;
 }
 
 }  // namespace tc2
 
-// Same contract as gemm_tc_strided, on CTA pairs.  Returns non-zero when the problem is not taken.
+// Same contract as gemm_tc_strided without splits, on CTA pairs; A contiguous along k.  Returns non-zero when the problem is
+// not taken.
 int gemm_tc2_strided(const Ctx& c, const void* A, long a_rs, long a_cs, const void* B, long b_rs, long b_cs, void* C,
-                     int out_is_float, int m, int n, int k, const GemmEpilogue& e, float* split_ws, size_t split_ws_floats) {
+                     int out_is_float, int m, int n, int k, const GemmEpilogue& e) {
   using namespace tc2;
-  bool a_mn = (a_cs != 1), b_mn = (b_cs != 1);
-  if (a_mn && a_rs != 1) return -1;
-  if (b_mn && b_rs != 1) return -1;
-  long lda = a_mn ? a_cs : a_rs, ldb = b_mn ? b_cs : b_rs;
+  const bool b_mn = b_cs != 1;
+  if (a_cs != 1 || (b_mn && b_rs != 1)) return -1;
+  const long lda = a_rs, ldb = b_mn ? b_cs : b_rs;
   if ((lda % 8) != 0 || (ldb % 8) != 0 || ((uintptr_t)A & 15) || ((uintptr_t)B & 15) || ((uintptr_t)C & 15)) return -1;
   if ((n % 8) != 0) return -1;
-  if (a_mn && (m % 8) != 0) return -1;
-  if (a_mn && !b_mn) return -1;
-  CUtensorMap ma, mb;
-  bool ok = a_mn ? tc::make_map(&ma, A, (uint64_t)m, (uint64_t)k, (uint64_t)lda, BK) : tc::make_map(&ma, A, (uint64_t)k, (uint64_t)m, (uint64_t)lda, BM);
-  ok = ok && (b_mn ? tc::make_map(&mb, B, (uint64_t)n, (uint64_t)k, (uint64_t)ldb, BK) : tc::make_map(&mb, B, (uint64_t)k, (uint64_t)n, (uint64_t)ldb, BN / 2));
-  if (!ok) return -2;
-  int pairs_m = ceil_div(m, 2 * BM), tiles_n = ceil_div(n, BN);
-  int total_kb = ceil_div(k, BK);
-  int splits = 1;
-  bool plain = e.bias == nullptr && e.residual == nullptr && e.act == 0;
-  int clusters = (c.sm_count > 0 ? c.sm_count : 148) / 2;
-  if (out_is_float && plain && split_ws != nullptr && pairs_m * tiles_n * 2 <= clusters && total_kb >= 8) {
-    splits = clusters / (pairs_m * tiles_n);
-    if (splits > total_kb / 4) splits = total_kb / 4;
-    if (splits > 16) splits = 16;
-    while (splits > 1 && (size_t)splits * m * n > split_ws_floats) --splits;
-    if (splits < 1) splits = 1;
+  if (out_is_float && e.act != 0) return -1;
+  CUtensorMap ma, mb, mp;
+  bool ok = tc::make_map(&ma, A, (uint64_t)k, (uint64_t)m, (uint64_t)lda, BM);
+  const int wide = !b_mn || n % 64 == 0;       // whole tiles of B in one copy
+  if (!b_mn) {
+    ok = ok && tc::make_map(&mb, B, (uint64_t)k, (uint64_t)n, (uint64_t)ldb, BN / 2) && tc::make_map(&mp, B, (uint64_t)k, (uint64_t)n, (uint64_t)ldb, 32);
+  } else {
+    ok = ok && tc::make_map(&mp, B, (uint64_t)n, (uint64_t)k, (uint64_t)ldb, BK);
+    if (ok && wide) ok = tc::make_map_chunks(&mb, B, (uint64_t)n, (uint64_t)k, (uint64_t)ldb, BN / 128);
+    else mb = mp;
   }
-  int kb_per_split = ceil_div(total_kb, splits);
-  splits = ceil_div(total_kb, kb_per_split);
+  if (!ok) return -2;
+  const int tiles_m = ceil_div(m, 2 * BM), tiles_n = ceil_div(n, BN);
   tc::Epi ep;
   ep.bias = e.bias; ep.residual = e.residual; ep.aux_out = e.aux_out; ep.aux_in = e.aux_in; ep.act = e.act;
-  void* dst = (splits > 1) ? (void*)split_ws : C;
   if (c.prof != nullptr && c.prof->on) c.prof->begin(c.stream, 2.0 * m * n * (double)k);
   int rc;
-  if (out_is_float) {
-    if (a_mn) rc = launch<true, true, float>(c, ma, mb, dst, m, n, k, ep, pairs_m, tiles_n, splits, kb_per_split);
-    else if (b_mn) rc = launch<false, true, float>(c, ma, mb, dst, m, n, k, ep, pairs_m, tiles_n, splits, kb_per_split);
-    else rc = launch<false, false, float>(c, ma, mb, dst, m, n, k, ep, pairs_m, tiles_n, splits, kb_per_split);
-  } else {
-    if (a_mn) rc = launch<true, true, bf16>(c, ma, mb, dst, m, n, k, ep, pairs_m, tiles_n, splits, kb_per_split);
-    else if (b_mn) rc = launch<false, true, bf16>(c, ma, mb, dst, m, n, k, ep, pairs_m, tiles_n, splits, kb_per_split);
-    else rc = launch<false, false, bf16>(c, ma, mb, dst, m, n, k, ep, pairs_m, tiles_n, splits, kb_per_split);
-  }
-  if (rc != 0) return rc;
-  if (splits > 1) {
-    size_t total = (size_t)m * n;
-    splitk_reduce(c.stream, split_ws, (float*)C, total, splits);
-  }
+  if (out_is_float) rc = b_mn ? launch<true, float>(c, ma, mb, mp, wide, C, m, n, k, ep, tiles_m, tiles_n) : launch<false, float>(c, ma, mb, mp, wide, C, m, n, k, ep, tiles_m, tiles_n);
+  else rc = b_mn ? launch<true, bf16>(c, ma, mb, mp, wide, C, m, n, k, ep, tiles_m, tiles_n) : launch<false, bf16>(c, ma, mb, mp, wide, C, m, n, k, ep, tiles_m, tiles_n);
   if (c.prof != nullptr && c.prof->on) c.prof->end(c.stream);
-  return 0;
+  return rc;
 }
 
 }  // namespace bsr

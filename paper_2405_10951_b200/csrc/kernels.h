@@ -160,9 +160,9 @@ int gemm_tc_grouped_rows(const Ctx& c, const void* A, const void* Bst, int b_mn,
 // dW[e][m, n] = sum over rows r of expert e's segment of dY[r, m] * X[r, n]  (float out).
 int gemm_tc_grouped_wgrad(const Ctx& c, const void* dY, const void* X, float* dW, int rows_cap, int m, int n, int experts,
                           const int* seg_start);
-// The same on CTA pairs (tcgen05 cta_group::2, 256 x 256 tiles); preferred when m > 128.
+// The same on CTA pairs (tcgen05 cta_group::2, 256 x 256 tiles): A contiguous along k, no split.
 int gemm_tc2_strided(const Ctx& c, const void* A, long a_rs, long a_cs, const void* B, long b_rs, long b_cs, void* C,
-                     int out_is_float, int m, int n, int k, const GemmEpilogue& e, float* split_ws, size_t split_ws_floats);
+                     int out_is_float, int m, int n, int k, const GemmEpilogue& e);
 void splitk_reduce(cudaStream_t s, const float* partial, float* out, size_t n, int splits);
 // Diagnostic: one CTA whose bounded wait expires after limit_ns and which then tears down as the GEMM kernels do.
 void wait_expiry_selftest(const Ctx& c, unsigned long long limit_ns);

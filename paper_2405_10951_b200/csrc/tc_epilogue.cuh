@@ -4,6 +4,7 @@
 #pragma once
 
 #include "common.cuh"
+#include "tc_ptx.cuh"
 
 namespace bsr {
 namespace tc {
@@ -184,11 +185,11 @@ template <> __device__ __forceinline__ uint4 ChunkIO<bf16>::pack(const float* f)
 }
 
 // v[j]: accumulator of (row0 + lane, col0 + j).  All lanes of the warp take part (row0, col0 are warp-uniform).
-// zpre: the chunk of the stored pre-activation for act == 2, already in this lane's row order (or null: loaded here).
+// z: the chunk of the stored pre-activation for act == 2, already in this lane's row order (overwritten).
 // sbias, scol: the chunk's 32 bias values and column scales in shared memory (null: none), rs: this lane's row scale.
 template <typename TOut>
 __device__ __forceinline__ void epilogue_chunk(const uint32_t* r, const Epi& ep, const float* sbias, const float* scol, float rs, TOut* Cs, int M,
-                                               int N, int row0, int col0, unsigned char* st, int lane, const float* zpre = nullptr) {
+                                               int N, int row0, int col0, unsigned char* st, int lane, float* z) {
   if (row0 < M && col0 < N) {
     float v[32];
 #pragma unroll
@@ -212,13 +213,6 @@ __device__ __forceinline__ void epilogue_chunk(const uint32_t* r, const Epi& ep,
 #pragma unroll
       for (int j = 0; j < 32; j += 2) gelu_fast2(v[j], v[j + 1]);
     } else if (ep.act == 2) {
-      float z[32];
-      if (zpre != nullptr) {
-#pragma unroll
-        for (int j = 0; j < 32; ++j) z[j] = zpre[j];
-      } else {
-        ChunkIO<bf16>::load((const bf16*)ep.aux_in, N, row0, col0, M, N, st, lane, z);
-      }
       if (ep.aux_out != nullptr) {          // GELU(z) recomputed for the weight gradient of the second FFN layer
 #pragma unroll
         for (int j = 0; j < 32; j += 2) gelu_grad_mul2h(v[j], v[j + 1], z[j], z[j + 1], z[j], z[j + 1]);
@@ -299,98 +293,72 @@ __device__ __forceinline__ void chunk_land_bf16(const uint4* x, unsigned char* s
   __syncwarp();
 }
 
-// ---- the same with the auxiliary input (residual, or the stored pre-activation) prefetched one chunk ahead ----
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, uint32_t src_bytes) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
-
-// Starts the copy of a 32 x 32 chunk of g into the staging buffer `st` (shared address `st_addr`); out-of-range
-// units are zero-filled.
-template <typename T>
-__device__ __forceinline__ void chunk_prefetch(const T* g, int ld, int row0, int col0, int M, int N, uint32_t st_addr, int lane) {
-  using IO = ChunkIO<T>;
+// A warp's share of a tile: `nc` (at most four) chunks of 32 columns from column cb of 32 rows, accumulators at taddr.  ready()
+// waits for the accumulators; what does not depend on them is fetched before: bias and column scales (read where they
+// are added, they came from L2 -- the operand ring leaves hardly any L1 -- and took 900 of the 1700 clocks of a chunk) and
+// the first chunk of the residual or of the stored pre-activation, whose next chunk is always on its way.
+// empty: no products were accumulated (an expert without tokens): the result is zero.  st: this warp's staging buffer, 4 KB.
+template <typename TOut, bool FP8, typename Ready>
+__device__ __forceinline__ bool epilogue_tile(Ready ready, const Epi& ep, int bias_off, TOut* Cs, int M, int N, int row0, int cb, int nc, uint32_t taddr,
+                                              bool empty, unsigned char* st, int lane) {
+  const float* bias = ep.bias == nullptr ? nullptr : ep.bias + bias_off;
+  uint4 xn[8];
+  if constexpr (sizeof(TOut) == 4) {           // float outputs (never with an activation) are transposed once
+    const bool has_res = ep.residual != nullptr;
+    auto bias4 = [&](int cc) {
+      const int col = cb + cc * 32 + (lane % 8) * 4;
+      return bias != nullptr && col < N ? __ldg(reinterpret_cast<const float4*>(bias + col)) : make_float4(0.f, 0.f, 0.f, 0.f);
+    };
+    float4 bn = bias4(0);
+    if (has_res) chunk_issue((const float*)ep.residual, N, row0, cb, M, N, lane, xn);
+    if (!ready()) return false;
+#pragma unroll 1
+    for (int cc = 0; cc < nc; ++cc) {
+      uint4 xc[8];
 #pragma unroll
-  for (int i = 0; i < IO::UNITS; ++i) {
-    int r = i * IO::ROWS_PER_PASS + lane / IO::UNITS, u = lane % IO::UNITS;
-    int col = col0 + u * IO::E;
-    bool in = row0 + r < M && col < N;
-    const T* src = in ? g + (size_t)(row0 + r) * ld + col : g;
-    cp_async16(st_addr + IO::slot(r, u), src, in ? 16u : 0u);
-  }
-  cp_async_commit();
-}
-template <typename T>
-__device__ __forceinline__ void chunk_take(unsigned char* st, int lane, float* v) {
-  using IO = ChunkIO<T>;
-  cp_async_wait_all();
-  __syncwarp();
-#pragma unroll
-  for (int u = 0; u < IO::UNITS; ++u) {
-    uint4 x = *reinterpret_cast<const uint4*>(st + IO::slot(lane, u));
-    IO::unpack(x, v + u * IO::E);
-  }
-  __syncwarp();
-}
-
-// One warp's share of a tile: `nchunks` chunks of 32 columns starting at column colbase, accumulators at
-// taddr0 + 32 * chunk.  st_in / st_out: two staging buffers of this warp.
-template <typename TOut, typename LoadTmem>
-__device__ __forceinline__ void epilogue_warp_tile(LoadTmem load_tmem, const Epi& ep, TOut* Cs, int M, int N, int row0, int colbase,
-                                                   int nchunks, unsigned char* st_in, uint32_t st_in_addr, unsigned char* st_out,
-                                                   int lane, bool prefetched_first) {
-  bool pre_res = ep.residual != nullptr;
-  bool pre_aux = !pre_res && ep.act == 2;
-  for (int cc = 0; cc < nchunks; ++cc) {
-    int col0 = colbase + cc * 32;
-    uint32_t r[32];
-    load_tmem(cc, r);
-    bool live = row0 < M && col0 < N;                       // warp-uniform
-    if (!live) continue;
-    if (cc == 0 && !prefetched_first) {
-      if (pre_res) chunk_prefetch<TOut>((const TOut*)ep.residual, N, row0, col0, M, N, st_in_addr, lane);
-      else if (pre_aux) chunk_prefetch<bf16>((const bf16*)ep.aux_in, N, row0, col0, M, N, st_in_addr, lane);
-    }
-    float v[32], a[32];
-    if (pre_res) chunk_take<TOut>(st_in, lane, a);
-    else if (pre_aux) chunk_take<bf16>(st_in, lane, a);
-    if (cc + 1 < nchunks && col0 + 32 < N) {                // next chunk's auxiliary input, overlapped with this chunk's work
-      if (pre_res) chunk_prefetch<TOut>((const TOut*)ep.residual, N, row0, col0 + 32, M, N, st_in_addr, lane);
-      else if (pre_aux) chunk_prefetch<bf16>((const bf16*)ep.aux_in, N, row0, col0 + 32, M, N, st_in_addr, lane);
-    }
-#pragma unroll
-    for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
-    if (ep.bias != nullptr) {
-#pragma unroll
-      for (int g = 0; g < 8; ++g) {
-        if (col0 + g * 4 < N) {
-          float4 bb = __ldg(reinterpret_cast<const float4*>(ep.bias + col0 + g * 4));
-          v[g * 4 + 0] += bb.x; v[g * 4 + 1] += bb.y; v[g * 4 + 2] += bb.z; v[g * 4 + 3] += bb.w;
-        }
+      for (int i = 0; i < 8; ++i) xc[i] = xn[i];
+      const float4 bb = bn;
+      if (cc + 1 < nc) {
+        bn = bias4(cc + 1);
+        if (has_res) chunk_issue((const float*)ep.residual, N, row0, cb + (cc + 1) * 32, M, N, lane, xn);
       }
-    }
-    if (ep.act == 1) {
-      if (ep.aux_out != nullptr) ChunkIO<TOut>::store((TOut*)ep.aux_out, N, row0, col0, M, N, st_out, lane, v);
+      uint32_t r[32];
+      tmem_ld32(taddr + cc * 32, r);
+      tmem_ld_wait();
+      if (empty) {
 #pragma unroll
-      for (int j = 0; j < 32; j += 2) gelu_fast2(v[j], v[j + 1]);
-    } else if (ep.act == 2) {
-      if (!pre_aux) ChunkIO<bf16>::load((const bf16*)ep.aux_in, N, row0, col0, M, N, st_out, lane, a);
-      if (ep.aux_out != nullptr) {
-#pragma unroll
-        for (int j = 0; j < 32; j += 2) gelu_grad_mul2h(v[j], v[j + 1], a[j], a[j + 1], a[j], a[j + 1]);
-        ChunkIO<bf16>::store((bf16*)ep.aux_out, N, row0, col0, M, N, st_out, lane, a);
-      } else {
-#pragma unroll
-        for (int j = 0; j < 32; j += 2) gelu_grad_mul2(v[j], v[j + 1], a[j], a[j + 1]);
+        for (int j = 0; j < 32; ++j) r[j] = 0u;
       }
+      epilogue_chunk_f32(r, bb, (float*)Cs, M, N, row0, cb + cc * 32, st, lane, xc, has_res);
     }
-    if (pre_res) {
-#pragma unroll
-      for (int j = 0; j < 32; ++j) v[j] += a[j];
+  } else {
+    float* sbias = reinterpret_cast<float*>(st + 2048);      // behind the 32 rows of 64 bytes a chunk takes: bias, column scales
+    if (lane < nc * 8) {
+      const int col = cb + lane * 4;
+      const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (bias != nullptr) *reinterpret_cast<float4*>(sbias + lane * 4) = col < N ? __ldg(reinterpret_cast<const float4*>(bias + col)) : z4;
+      if (FP8) *reinterpret_cast<float4*>(sbias + 128 + lane * 4) = col < N ? __ldg(reinterpret_cast<const float4*>(ep.col_scale + col)) : z4;
     }
-    ChunkIO<TOut>::store(Cs, N, row0, col0, M, N, st_out, lane, v);
+    const float rs = FP8 && row0 + lane < M ? __ldg(ep.row_scale + row0 + lane) : 0.f;
+    const bool pre_z = ep.act == 2;            // dz of the FFN backward
+    if (pre_z) chunk_issue((const bf16*)ep.aux_in, N, row0, cb, M, N, lane, xn);
+    if (!ready()) return false;
+    __syncwarp();
+#pragma unroll 1
+    for (int cc = 0; cc < nc; ++cc) {
+      float z[32];
+      if (pre_z) {
+        chunk_land_bf16(xn, st, lane, z);
+        if (cc + 1 < nc) chunk_issue((const bf16*)ep.aux_in, N, row0, cb + (cc + 1) * 32, M, N, lane, xn);
+      }
+      uint32_t r[32];
+      tmem_ld32(taddr + cc * 32, r);
+      tmem_ld_wait();
+      epilogue_chunk<TOut>(r, ep, bias != nullptr ? sbias + cc * 32 : nullptr, FP8 ? sbias + 128 + cc * 32 : nullptr, rs, Cs, M, N, row0, cb + cc * 32, st,
+                           lane, z);
+    }
   }
+  return true;
 }
 
 }  // namespace tc

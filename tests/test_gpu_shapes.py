@@ -104,3 +104,22 @@ def test_fma_contraction_forward_and_backward(m, n, k, dtype, tol):
     torch.cuda.synchronize()
     for got, want in ((y, x @ w.T), (dx, dy @ w), (dw, dy.T @ x)):
         assert P.rel_err(got.float().cpu().numpy(), want) < tol
+
+
+@pytest.mark.parametrize("m,n,k", [(129, 64, 64), (256, 256, 64), (300, 200, 72), (19200, 768, 128), (18944, 2304, 64), (12001, 2048, 192), (12800, 2056, 64)])
+def test_linear_on_cta_pairs(m, n, k):
+    """The CTA-pair kernel at remainders of its 256-row tiles and with a last wave cut into parts of 64 to 256 columns: forward with
+    bias, GELU and residual, and the input gradient (B read across k).  One bf16 rounding of the output."""
+    import torch
+    from paper_2405_10951_b200 import binding as Bd
+    gen = torch.Generator(device="cuda").manual_seed(m + n + k)
+    mk = lambda *s: torch.randn(*s, generator=gen, device="cuda").bfloat16()
+    x, w, dy, res, bias = mk(m, k), mk(n, k) / k ** 0.5, mk(m, n), mk(m, n), torch.randn(n, generator=gen, device="cuda")
+    rel = lambda a, b: float((a.double() - b).norm() / b.norm())
+    z = x.double() @ w.double().T + bias.double()
+    assert rel(Bd.bsr_linear_forward(x, w, bias, use_tensor_cores=2), z) < 4e-3
+    want = torch.nn.functional.gelu(z) + res.double()
+    assert rel(Bd.bsr_linear_forward(x, w, bias, res, act_gelu=True, use_tensor_cores=2), want) < 4e-3
+    if m % 8 == 0:
+        dx, dw = Bd.bsr_linear_backward(x, w, dy, use_tensor_cores=2)
+        assert rel(dx, dy.double() @ w.double()) < 4e-3 and rel(dw, dy.double().T @ x.double()) < 1e-4
