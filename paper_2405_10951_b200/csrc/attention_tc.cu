@@ -115,6 +115,8 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
       mbar_init(s_full(b), 1); mbar_init(o_full(b), 1); mbar_init(p_full(b), GW); mbar_init(t_empty(b), GW); mbar_init(token(b), 1);
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    prefetch_map(&map_q);
+    prefetch_map(&map_kv);
   }
   if (warp == LOADER) {
     tmem_alloc(smem_u32(&tmem_slot), 512);
@@ -376,6 +378,7 @@ attn_fwd_tc_long_kernel(const __grid_constant__ CUtensorMap map_qkv, bf16* __res
     mbar_init(tma_bar, 1);
     mbar_init(mma_bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    prefetch_map(&map_qkv);
   }
   if (warp == 0) {
     tmem_alloc(smem_u32(&tmem_slot), 2 * KB);           // S in the first KB columns, O behind it: several CTAs share an SM
@@ -597,6 +600,8 @@ attn_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_qkv, const __grid_con
     mbar_init(mma_bar, 1);
     mbar_init(mma2_bar, 3);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    prefetch_map(&map_qkv);
+    prefetch_map(&map_do);
   }
   if (warp == 0) {
     tmem_alloc(smem_u32(&tmem_slot), 256);
@@ -812,6 +817,8 @@ attn_bwd_tc256_kernel(const __grid_constant__ CUtensorMap map_qkv, const __grid_
     mbar_init(mma_bar, 1);
     mbar_init(mma2_bar, 3);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    prefetch_map(&map_qkv);
+    prefetch_map(&map_do);
   }
   if (warp == 0) {
     tmem_alloc(smem_u32(&tmem_slot), 512);
@@ -1089,6 +1096,8 @@ attn_bwd_long_kernel(const __grid_constant__ CUtensorMap map_qkv, const __grid_c
     abort_flag = 0;
     mbar_init(full_bar(0), 1); mbar_init(full_bar(1), 1); mbar_init(s_bar, 1); mbar_init(p_bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    prefetch_map(&map_qkv);
+    prefetch_map(&map_do);
   }
   if (warp == 0) {
     tmem_alloc(smem_u32(&tmem_slot), 256);

@@ -19,6 +19,8 @@
 // copies it issued time to land, frees its tensor memory and returns.
 #include <cuda.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 #include "kernels.h"
 #include "tc_ptx.cuh"
@@ -28,14 +30,14 @@ namespace bsr {
 
 namespace tc {
 
-constexpr int BM = 128, BN_MAX = 256, BK = 64;       // tile width BN is 256, or 192 where that wastes less of the last wave
-constexpr int STAGES = 4;
+constexpr int BM = 128, BN_MAX = 256, BK = 64;       // tile width BN is 256, 192, 128 or 64: see choose_tile
 constexpr int UMMA_K = 16;
 constexpr int A_BYTES = BM * BK * 2;
-constexpr int STAGE_BYTES_MAX = A_BYTES + BN_MAX * BK * 2;
+constexpr int RING_BYTES = 4 * (A_BYTES + BN_MAX * BK * 2);        // 192 KB: 4 slabs of operands at BN = 256, 8 at 64
+constexpr int stages_for(int bn) { return RING_BYTES / (A_BYTES + bn * BK * 2) < 8 ? RING_BYTES / (A_BYTES + bn * BK * 2) : 8; }
 constexpr int EPI_WARPS = 8;                     // two warps per TMEM lane quarter, each takes half of the columns
 constexpr int STAGING_BYTES = 32 * 128;          // per epilogue warp: 32 rows x 128 bytes, 16-byte units XOR-swizzled
-constexpr int SMEM_BYTES = STAGES * STAGE_BYTES_MAX + EPI_WARPS * STAGING_BYTES + 1024 /*alignment slack*/ + 128 /*barriers*/;
+constexpr int SMEM_BYTES = RING_BYTES + EPI_WARPS * STAGING_BYTES + 1024 /*alignment slack*/ + 256 /*barriers*/;
 constexpr int THREADS = 64 + EPI_WARPS * 32;
 constexpr uint32_t TMEM_COLS = 512;
 
@@ -83,7 +85,7 @@ template <bool A_MN, bool B_MN, typename TOut, int BN, bool FP8 = false>
 __global__ void __launch_bounds__(THREADS, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, TOut* __restrict__ C,
                int M, int N, int K, Epi ep, int tiles_m, int tiles_n, int splits, int kb_per_split, GemmGroup grp, int* status) {
-  constexpr int B_BYTES = BN * BK * 2, STAGE_BYTES = A_BYTES + B_BYTES;
+  constexpr int B_BYTES = BN * BK * 2, STAGE_BYTES = A_BYTES + B_BYTES, STAGES = stages_for(BN);
   constexpr int HALF_CHUNKS = BN / 64;               // 32-column chunks per epilogue warp
   extern __shared__ unsigned char smem_dyn[];
   uint32_t base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
@@ -106,6 +108,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     for (int s = 0; s < STAGES; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
     for (int b = 0; b < 2; ++b) { mbar_init(tfull_bar(b), 1); mbar_init(tempty_bar(b), EPI_WARPS); }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    prefetch_map(&map_a);
+    prefetch_map(&map_b);
   }
   if (warp == 1) {
     tmem_alloc(smem_u32(&tmem_base_slot), TMEM_COLS);
@@ -366,6 +370,35 @@ bool make_map_u8(CUtensorMap* map, const void* ptr, uint64_t inner, uint64_t out
             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Tile width and number of splits along k (over partial sums in the workspace, reduced by a second kernel).
+// * What fits the SMs in one wave takes the narrowest tiles that still do: its time is latency -- filling the ring, one
+//   epilogue -- and a narrow tile has a short epilogue and room for more slabs in flight (200 x 1152 x 384: 12 CTAs of 192
+//   columns 5.7 us, 36 of 64 columns 4.6 us).
+// * More waves: 192 columns instead of 256 where that fills the last wave better.
+// * Splits (ws_floats > 0) and weight gradients: by estimated time in ns.  A slab costs its bytes at 126 per ns (64 a
+//   clock), a tile 2.5 us to fill and drain; the second kernel costs 3 us and its traffic.
+struct Cut { int bn, splits; };
+static Cut choose_tile(int m, int n, int k, bool a_mn, size_t ws_floats, int sms) {
+  const int tm = ceil_div(m, BM), kb = ceil_div(k, BK);
+  auto tiles = [&](int bn) { return (long)tm * ceil_div(n, bn); };
+  if (a_mn || (ws_floats > 0 && kb >= 8 && tiles(256) * 2 <= sms)) {
+    Cut best = {BN_MAX, 1};
+    double t_best = 1e30;
+    for (int bn = BN_MAX; bn >= 128; bn -= 64)
+      for (int s = 1; s <= 16; ++s) {
+        if (s > 1 && (s * 4 > kb || (size_t)s * m * n > ws_floats)) break;
+        const double slab = (A_BYTES + bn * BK * 2) / 126.0, sum = s > 1 ? 3000.0 + (s + 1.0) * m * n * 4.0 / 7000.0 : 0.0;
+        const double t = ceil_div(tiles(bn) * s, sms) * (ceil_div(kb, s) * slab + 2500.0) + sum;
+        if (t < t_best) { t_best = t; best = {bn, s}; }
+      }
+    return best;
+  }
+  if (tiles(192) <= sms)
+    for (int bn = 64; bn <= 192; bn += 64)
+      if (tiles(bn) <= sms) return {bn, 1};
+  return {ceil_div(tiles(192), sms) * 192 < ceil_div(tiles(256), sms) * 256 ? 192 : BN_MAX, 1};
+}
+
 template <bool A_MN, bool B_MN, typename TOut, int BN = BN_MAX, bool FP8 = false>
 static int launch(const Ctx& c, const CUtensorMap& ma, const CUtensorMap& mb, void* C, int m, int n, int k, const Epi& ep,
                   int tiles_m, int tiles_n, int splits, int kb_per_split, const GemmGroup& grp) {
@@ -410,31 +443,16 @@ int gemm_tc_strided(const Ctx& c, const void* A, long a_rs, long a_cs, const voi
   CUtensorMap ma, mb;
   bool ok = a_mn ? make_map(&ma, A, (uint64_t)m, (uint64_t)k, (uint64_t)lda, BK) : make_map(&ma, A, (uint64_t)k, (uint64_t)m, (uint64_t)lda, BM);
   int sms = c.sm_count > 0 ? c.sm_count : 148;
-  // Tile width: 192 columns instead of 256 where the narrower tiles fill the SMs' last wave better (a persistent CTA
-  // per SM walks ceil(tiles / SMs) tiles; the time goes with that count times the tile width).  Not for operand A
-  // read along m (weight gradients: those are split along k instead).
-  int bn = BN_MAX;
-  if (!a_mn) {
-    long w256 = (long)ceil_div(ceil_div(m, BM) * ceil_div(n, 256), sms) * 256, w192 = (long)ceil_div(ceil_div(m, BM) * ceil_div(n, 192), sms) * 192;
-    if (w192 < w256) bn = 192;
-  }
-  ok = ok && (b_mn ? make_map(&mb, B, (uint64_t)n, (uint64_t)k, (uint64_t)ldb, BK) : make_map(&mb, B, (uint64_t)k, (uint64_t)n, (uint64_t)ldb, bn));
-  if (!ok) return -2;
-  int tiles_m = ceil_div(m, BM), tiles_n = ceil_div(n, bn);
-  int total_kb = ceil_div(k, BK);
-  int splits = 1;
-  bool plain = e.bias == nullptr && e.residual == nullptr && e.act == 0;
+  const bool plain = e.bias == nullptr && e.residual == nullptr && e.act == 0;
   // split along k: weight gradients (plain float outputs) and the few-row products of the classification-only tail,
   // whose epilogue then runs in the reduction
-  if (split_ws != nullptr && tiles_m * tiles_n * 2 <= sms && total_kb >= 8 && ((out_is_float && plain) || (m <= 256 && (n % 4) == 0))) {
-    splits = sms / (tiles_m * tiles_n);
-    if (splits > total_kb / 4) splits = total_kb / 4;
-    if (splits > 16) splits = 16;
-    while (splits > 1 && (size_t)splits * m * n > split_ws_floats) --splits;
-    if (splits < 1) splits = 1;
-  }
-  int kb_per_split = ceil_div(total_kb, splits);
-  splits = ceil_div(total_kb, kb_per_split);
+  const bool may_split = split_ws != nullptr && ((out_is_float && plain) || (m <= 256 && (n % 4) == 0));
+  const Cut cut = choose_tile(m, n, k, a_mn, may_split ? split_ws_floats : 0, sms);
+  const int bn = cut.bn;
+  ok = ok && (b_mn ? make_map(&mb, B, (uint64_t)n, (uint64_t)k, (uint64_t)ldb, BK) : make_map(&mb, B, (uint64_t)k, (uint64_t)n, (uint64_t)ldb, bn));
+  if (!ok) return -2;
+  const int tiles_m = ceil_div(m, BM), tiles_n = ceil_div(n, bn), total_kb = ceil_div(k, BK);
+  const int kb_per_split = ceil_div(total_kb, cut.splits), splits = ceil_div(total_kb, kb_per_split);
   Epi ep_full;
   ep_full.bias = e.bias; ep_full.residual = e.residual; ep_full.aux_out = e.aux_out; ep_full.aux_in = e.aux_in; ep_full.act = e.act;
   // split products write plain float partials; their epilogue runs in the reduction
@@ -448,20 +466,16 @@ int gemm_tc_strided(const Ctx& c, const void* A, long a_rs, long a_cs, const voi
   if (c.prof != nullptr && c.prof->on) c.prof->begin(c.stream, 2.0 * m * n * (double)k);
   int rc;
   GemmGroup gg;
-  if (bn == 192) {
-    if (out_is_float) rc = b_mn ? launch<false, true, float, 192>(c, ma, mb, dst, m, n, k, ep, tiles_m, tiles_n, splits, kb_per_split, gg)
-                                : launch<false, false, float, 192>(c, ma, mb, dst, m, n, k, ep, tiles_m, tiles_n, splits, kb_per_split, gg);
-    else rc = b_mn ? launch<false, true, bf16, 192>(c, ma, mb, dst, m, n, k, ep, tiles_m, tiles_n, splits, kb_per_split, gg)
-                   : launch<false, false, bf16, 192>(c, ma, mb, dst, m, n, k, ep, tiles_m, tiles_n, splits, kb_per_split, gg);
-  } else if (out_is_float) {
-    if (a_mn) rc = launch<true, true, float>(c, ma, mb, dst, m, n, k, ep, tiles_m, tiles_n, splits, kb_per_split, gg);
-    else if (b_mn) rc = launch<false, true, float>(c, ma, mb, dst, m, n, k, ep, tiles_m, tiles_n, splits, kb_per_split, gg);
-    else rc = launch<false, false, float>(c, ma, mb, dst, m, n, k, ep, tiles_m, tiles_n, splits, kb_per_split, gg);
-  } else {
-    if (a_mn) rc = launch<true, true, bf16>(c, ma, mb, dst, m, n, k, ep, tiles_m, tiles_n, splits, kb_per_split, gg);
-    else if (b_mn) rc = launch<false, true, bf16>(c, ma, mb, dst, m, n, k, ep, tiles_m, tiles_n, splits, kb_per_split, gg);
-    else rc = launch<false, false, bf16>(c, ma, mb, dst, m, n, k, ep, tiles_m, tiles_n, splits, kb_per_split, gg);
-  }
+  auto run = [&](auto width) {
+    constexpr int W = decltype(width)::value;
+    auto go = [&](auto kern) { return kern(c, ma, mb, dst, m, n, k, ep, tiles_m, tiles_n, splits, kb_per_split, gg); };
+    if constexpr (W >= 128)
+      if (a_mn) return out_is_float ? go(launch<true, true, float, W>) : go(launch<true, true, bf16, W>);
+    if (out_is_float) return b_mn ? go(launch<false, true, float, W>) : go(launch<false, false, float, W>);
+    return b_mn ? go(launch<false, true, bf16, W>) : go(launch<false, false, bf16, W>);
+  };
+  rc = bn == 256 ? run(std::integral_constant<int, 256>()) : bn == 192 ? run(std::integral_constant<int, 192>())
+     : bn == 128 ? run(std::integral_constant<int, 128>()) : run(std::integral_constant<int, 64>());
   if (rc != 0) return rc;
   if (splits > 1) {
     size_t total = (size_t)m * n;
@@ -536,9 +550,7 @@ int gemm_tc_e4m3(const Ctx& c, const void* Aq, const float* a_scale, const void*
   if ((k % 16) != 0 || (n % 8) != 0 || ((uintptr_t)Aq & 15) || ((uintptr_t)Bq & 15) || ((uintptr_t)C & 15)) return -1;
   if (a_scale == nullptr || b_scale == nullptr || e.residual != nullptr || e.act == 2) return -1;
   int sms = c.sm_count > 0 ? c.sm_count : 148;
-  int bn = BN_MAX;
-  long w256 = (long)ceil_div(ceil_div(m, BM) * ceil_div(n, 256), sms) * 256, w192 = (long)ceil_div(ceil_div(m, BM) * ceil_div(n, 192), sms) * 192;
-  if (w192 < w256) bn = 192;
+  const int bn = ceil_div((long)ceil_div(m, BM) * ceil_div(n, 192), sms) * 192 < ceil_div((long)ceil_div(m, BM) * ceil_div(n, 256), sms) * 256 ? 192 : BN_MAX;
   CUtensorMap ma, mb;
   if (!make_map_u8(&ma, Aq, (uint64_t)k, (uint64_t)m, (uint64_t)k, BM) || !make_map_u8(&mb, Bq, (uint64_t)k, (uint64_t)n, (uint64_t)k, bn)) return -2;
   Epi ep;

@@ -123,3 +123,21 @@ def test_linear_on_cta_pairs(m, n, k):
     if m % 8 == 0:
         dx, dw = Bd.bsr_linear_backward(x, w, dy, use_tensor_cores=2)
         assert rel(dx, dy.double() @ w.double()) < 4e-3 and rel(dw, dy.double().T @ x.double()) < 1e-4
+
+
+@pytest.mark.parametrize("m,n,k", [(1, 64, 64), (130, 1152, 384), (200, 72, 200), (1576, 1152, 384), (1576, 384, 1544), (6304, 384, 384), (4096, 1536, 64), (2500, 3072, 128)])
+def test_linear_over_tile_widths(m, n, k):
+    """Sizes that take tiles of 64, 128, 192 and 256 columns, and weight gradients with one to sixteen shares of the reduction: the
+    residual path and the input and weight gradients.  One bf16 rounding of the output, fp32 sums for the weight gradient."""
+    import torch
+    from paper_2405_10951_b200 import binding as Bd
+    gen = torch.Generator(device="cuda").manual_seed(m + n + k)
+    mk = lambda *s: torch.randn(*s, generator=gen, device="cuda").bfloat16()
+    x, w, dy, res, bias = mk(m, k), mk(n, k) / k ** 0.5, mk(m, n), mk(m, n), torch.randn(n, generator=gen, device="cuda")
+    rel = lambda a, b: float((a.double() - b).norm() / b.norm())
+    want = x.double() @ w.double().T + bias.double()
+    assert rel(Bd.bsr_linear_forward(x, w, bias, res, use_tensor_cores=True), want + res.double()) < 4e-3
+    if m % 8 == 0:
+        ws = torch.empty(160 * 128 * 256, device="cuda")
+        dx, dw = Bd.bsr_linear_backward(x, w, dy, use_tensor_cores=True, workspace=ws)
+        assert rel(dx, dy.double() @ w.double()) < 4e-3 and rel(dw, dy.double().T @ x.double()) < 1e-4
