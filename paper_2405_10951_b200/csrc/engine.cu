@@ -172,7 +172,7 @@ struct bsr_handle {
   size_t off_escore = 0, off_delta = 0, off_ln_partials = 0, off_cs_partials = 0;
   size_t off_kept_all = 0;
   size_t off_stage = 0;
-  size_t off_split = 0, split_floats = 0;
+  size_t off_split = 0, off_split_w = 0, split_floats = 0;
   std::vector<size_t> moe_rec_eidx, moe_rec_ew;
   std::vector<size_t> score_rec;       // per drop location's block: head-mean scores [max_batch, M] of the last step
   size_t off_m_dog = 0, off_m_dzg = 0, off_m_dxg = 0, off_m_dw = 0, off_m_dsel = 0;
@@ -205,6 +205,7 @@ struct bsr_handle {
   bool slot_used[2] = {false, false};
   int host_slot = 0;
   SideLane side;                        // second lane for the reductions only the optimiser reads
+  SideLane wlane;                       // lane of the weight gradients (see block_backward)
   int use_side = 1;
   long launches_at_enable = 0;
 
@@ -486,6 +487,7 @@ size_t plan(bsr_handle* h) {
   h->off_stage = b.take(biggest * 4);
   h->split_floats = (d.dtype == BSR_DTYPE_BF16) ? (size_t)160 * 128 * 256 : 0;   // one 128x256 fp32 tile per SM
   h->off_split = b.take(h->split_floats * 4);
+  h->off_split_w = b.take(h->split_floats * 4);       // the weight gradients' own: they run on a lane of their own
   // multi-step loop state and staging; two staging slots for steps fed from host memory
   h->off_loop = b.take(256);
   h->off_lab_stage = b.take((size_t)Bm * 4);
@@ -663,6 +665,9 @@ struct GradStream {      // gradient of the residual stream: float rows, plus th
   void* c;
 };
 
+// The lane of the weight gradients (null: they stay on the stream of the step, as when launches are timed one by one).
+SideLane* lane_of(const bsr_handle* h, const Ctx& c) { return c.side != nullptr && h->wlane.stream != nullptr ? const_cast<SideLane*>(&h->wlane) : nullptr; }
+
 int block_backward(bsr_handle* h, const Ctx& c, int l, int B, GradStream dxo, GradStream dxi, bool need_dxi, const int* task_ids) {
   const bsr_dims& d = h->cfg.dims;
   const Schedule& s = h->sched;
@@ -677,8 +682,6 @@ int block_backward(bsr_handle* h, const Ctx& c, int l, int B, GradStream dxo, Gr
   size_t es = dtype_size(d.dtype);
   int Mdense = Ma;
   if (tail) { Ma = B; Mf = B; }          // FFN and projection gradients live on the classification rows only
-  Ctx cf = c;
-  cf.dtype = 0;
   float* csp = h->at<float>(h->off_cs_partials);
   float* lnp = h->at<float>(h->off_ln_partials);
   void* dz = h->base + h->off_dz;
@@ -689,6 +692,21 @@ int block_backward(bsr_handle* h, const Ctx& c, int l, int B, GradStream dxo, Gr
   void* dqkv = h->base + h->off_dqkv;
   auto op = [&](const GradStream& g) -> const void* { return bf ? g.c : (const void*)g.f; };   // GEMM operand view
   GemmEpilogue none;
+  // Weight and bias gradients are read by the optimiser only: they run on a lane of their own beside the chain of input
+  // gradients, which is all that the blocks below wait for (a batch that leaves SMs idle then uses them: DeiT-S, one
+  // image, 823 -> 740 us; batch 64 1624 -> 1531 us).  In that lane they follow one another, so one split workspace and one set of
+  // column-sum partials serve all; the chain waits for the lane only before it rewrites what the lane may still read:
+  // 0: the FFN's buffers (dz, GELU output, the block's output gradient), 1: dx', 2: dQKV.
+  Ctx cl = c;
+  cl.side = lane_of(h, c);
+  auto lane_begin = [&]() {
+    Ctx w = c;
+    w.stream = side_begin(cl);
+    if (cl.side != nullptr) { w.side = nullptr; w.split_ws = h->split_floats ? h->at<float>(h->off_split_w) : nullptr; }
+    return w;
+  };
+  auto lane_f32 = [](Ctx w) { w.dtype = 0; return w; };
+  side_join(cl, 0);
   if (is_moe(h, l)) {
     int E = d.moe_experts, K = d.moe_top_k;
     MoeBufs mb = moe_bufs(h, bb);
@@ -704,14 +722,14 @@ int block_backward(bsr_handle* h, const Ctx& c, int l, int B, GradStream dxo, Gr
     int r1 = gemm_tc_grouped_rows(c, dog, h->wb(l, "moe.fc2.weight"), 1, dzg, 0, cap, F, D, E, mb.tile_expert, eg);
     int r2 = 0, r4 = 0;
     if (pg) {
-      r2 = gemm_tc_grouped_wgrad(c, dog, mb.hg, h->gb(l, "moe.fc2.weight"), cap, D, F, E, mb.seg_start);
-      moe_seg_colsum(c, mb, dog, D, E, h->gb(l, "moe.fc2.bias"));
+      Ctx w = lane_begin();
+      r2 = gemm_tc_grouped_wgrad(w, dog, mb.hg, h->gb(l, "moe.fc2.weight"), cap, D, F, E, mb.seg_start);
+      moe_seg_colsum(w, mb, dog, D, E, h->gb(l, "moe.fc2.bias"));
+      r4 = gemm_tc_grouped_wgrad(w, dzg, mb.xg, h->gb(l, "moe.fc1.weight"), cap, F, D, E, mb.seg_start);
+      moe_seg_colsum(w, mb, dzg, F, E, h->gb(l, "moe.fc1.bias"));
+      side_end(cl, 0);
     }
     int r3 = gemm_tc_grouped_rows(c, dzg, h->wb(l, "moe.fc1.weight"), 1, dxg, 0, cap, D, F, E, mb.tile_expert, none);
-    if (pg) {
-      r4 = gemm_tc_grouped_wgrad(c, dzg, mb.xg, h->gb(l, "moe.fc1.weight"), cap, F, D, E, mb.seg_start);
-      moe_seg_colsum(c, mb, dzg, F, E, h->gb(l, "moe.fc1.bias"));
-    }
     if (r1 || r2 || r3 || r4) return set_err(h->err, BSR_ERR_CUDA, "grouped GEMM set-up failed (%d, %d, %d, %d)", r1, r2, r3, r4);
     moe_gate_bwd(c, mb, dxg, dwsel, h->wb(l, "moe.gate.weight"), task_ids, tail ? 1 : Tf, d.num_tasks, Mf, D, E, K, dy,
                  h->at<float>(h->off_m_dsel), pg ? h->gb(l, "moe.gate.weight") : nullptr);
@@ -723,17 +741,18 @@ int block_backward(bsr_handle* h, const Ctx& c, int l, int B, GradStream dxo, Gr
   if (pg) eg.aux_out = h->base + bb.hh;       // GELU(z) again, into scratch, for the weight gradient below
   gemm(c, op(dxo), D, 1, h->wb(l, "mlp.fc2.weight"), 1, F, dz, 0, Mf, F, D, eg);
   if (pg) {
-    gemm(c, op(dxo), 1, D, h->base + bb.hh, 1, F, h->gb(l, "mlp.fc2.weight"), 1, D, F, Mf, none);
+    Ctx w = lane_begin();
+    gemm(w, op(dxo), 1, D, h->base + bb.hh, 1, F, h->gb(l, "mlp.fc2.weight"), 1, D, F, Mf, none);
     // db2 = column sums of dxo: they came out of the following block's LayerNorm backward, which wrote dxo
-    if (l == d.depth - 1) colsum(cf, dxo.f, Mf, D, csp, h->gb(l, "mlp.fc2.bias"));
+    if (l == d.depth - 1) colsum(lane_f32(w), dxo.f, Mf, D, csp, h->gb(l, "mlp.fc2.bias"));
+    gemm(w, dz, 1, F, h->base + bb.y2, 1, D, h->gb(l, "mlp.fc1.weight"), 1, F, D, Mf, none);
+    colsum(w, dz, Mf, F, csp, h->gb(l, "mlp.fc1.bias"));
+    side_end(cl, 0);
   }
   // FFN first layer
   gemm(c, dz, F, 1, h->wb(l, "mlp.fc1.weight"), 1, D, dy, 0, Mf, D, F, none);
-  if (pg) {
-    gemm(c, dz, 1, F, h->base + bb.y2, 1, D, h->gb(l, "mlp.fc1.weight"), 1, F, D, Mf, none);
-    colsum(c, dz, Mf, F, csp, h->gb(l, "mlp.fc1.bias"));
   }
-  }
+  side_join(cl, 1);
   layernorm_bwd(c, dy, 0, h->at<float>(bb.xp), D, h->at<float>(bb.mean2), h->at<float>(bb.rstd2),
                 (const float*)h->wb(l, "norm2.weight"), dxo.f, dxg.f, D, shrinks ? nullptr : dxg.c, lnp,
                 pg ? h->gb(l, "norm2.weight") : nullptr, pg ? h->gb(l, "norm2.bias") : nullptr, Mf, D,
@@ -748,21 +767,26 @@ int block_backward(bsr_handle* h, const Ctx& c, int l, int B, GradStream dxo, Gr
   bool tail_cls_attn = false;
   const float* ln1_res = dxp.f;
   if (!tail) {
-    gemm(c, op(dxp), D, 1, h->wb(l, "attn.proj.weight"), 1, D, d_o, 0, Ma, D, D, none);
     if (pg) {
-      gemm(c, op(dxp), 1, D, h->base + bb.o, 1, D, h->gb(l, "attn.proj.weight"), 1, D, D, Ma, none);
-      if (shrinks) colsum(cf, dxp.f, Ma, D, csp, h->gb(l, "attn.proj.bias"));
+      Ctx w = lane_begin();
+      gemm(w, op(dxp), 1, D, h->base + bb.o, 1, D, h->gb(l, "attn.proj.weight"), 1, D, D, Ma, none);
+      if (shrinks) colsum(lane_f32(w), dxp.f, Ma, D, csp, h->gb(l, "attn.proj.bias"));
+      side_end(cl, 1);
     }
+    gemm(c, op(dxp), D, 1, h->wb(l, "attn.proj.weight"), 1, D, d_o, 0, Ma, D, D, none);
   } else {
     // B rows: dO_cls = dx'_cls Wo, dWo = dx'_cls^T o_cls; then both gradients go back into zeroed dense tensors
     void* do_cls = h->base + h->off_dy;                      // free at this point
-    gemm(c, op(dxp), D, 1, h->wb(l, "attn.proj.weight"), 1, D, do_cls, 0, B, D, D, none);
     if (pg) {
-      gemm(c, op(dxp), 1, D, h->base + bb.o_cls, 1, D, h->gb(l, "attn.proj.weight"), 1, D, D, B, none);
-      if (shrinks) colsum(cf, dxp.f, B, D, csp, h->gb(l, "attn.proj.bias"));
+      Ctx w = lane_begin();
+      gemm(w, op(dxp), 1, D, h->base + bb.o_cls, 1, D, h->gb(l, "attn.proj.weight"), 1, D, D, B, none);
+      if (shrinks) colsum(lane_f32(w), dxp.f, B, D, csp, h->gb(l, "attn.proj.bias"));
+      side_end(cl, 1);
     }
+    gemm(c, op(dxp), D, 1, h->wb(l, "attn.proj.weight"), 1, D, do_cls, 0, B, D, D, none);
     // with the classification-row attention, dqkv comes straight from do_cls; otherwise dO is scattered into a zeroed
     // dense tensor for the general kernel
+    side_join(cl, 2);
     tail_cls_attn = attention_cls_bwd(c, h->base + bb.qkv, do_cls, dqkv, B, Ta, H, hd) == 0;
     if (!tail_cls_attn) {
       cudaMemsetAsync(d_o, 0, (size_t)Mdense * D * es, c.stream);
@@ -778,16 +802,19 @@ int block_backward(bsr_handle* h, const Ctx& c, int l, int B, GradStream dxo, Gr
   // of block l-1's second FFN layer (dense FFN, trainable)
   float* prev_fc2_bias = (need_dxi && l > 0 && ((h->cfg.trainable_mask >> (l - 1)) & 1u) && !is_moe(h, l - 1)) ? h->gb(l - 1, "mlp.fc2.bias") : nullptr;
   if (!tail_cls_attn) {
+    side_join(cl, 2);
     int rc = attention_bwd(c, h->base + bb.qkv, h->base + bb.o, d_o, h->at<float>(bb.lse), h->at<float>(h->off_delta),
                            cls_extra, dqkv, B, Ta, H, hd);
     if (rc != 0) return set_err(h->err, BSR_ERR_UNSUPPORTED, "attention backward: %d tokens do not fit this kernel", Ta);
   }
   // QKV projection
-  gemm(c, dqkv, 3 * D, 1, h->wb(l, "attn.qkv.weight"), 1, D, dy, 0, Ma, D, 3 * D, none);
   if (pg) {
-    gemm(c, dqkv, 1, 3 * D, h->base + bb.y1, 1, D, h->gb(l, "attn.qkv.weight"), 1, 3 * D, D, Ma, none);
-    colsum(c, dqkv, Ma, 3 * D, csp, h->gb(l, "attn.qkv.bias"));
+    Ctx w = lane_begin();
+    gemm(w, dqkv, 1, 3 * D, h->base + bb.y1, 1, D, h->gb(l, "attn.qkv.weight"), 1, 3 * D, D, Ma, none);
+    colsum(w, dqkv, Ma, 3 * D, csp, h->gb(l, "attn.qkv.bias"));
+    side_end(cl, 2);
   }
+  gemm(c, dqkv, 3 * D, 1, h->wb(l, "attn.qkv.weight"), 1, D, dy, 0, Ma, D, 3 * D, none);
   layernorm_bwd(c, dy, 0, h->at<float>(bb.x_in), D, h->at<float>(bb.mean1), h->at<float>(bb.rstd1),
                 (const float*)h->wb(l, "norm1.weight"), ln1_res, need_dxi ? dxi.f : nullptr, D, need_dxi ? dxi.c : nullptr, lnp,
                 pg ? h->gb(l, "norm1.weight") : nullptr, pg ? h->gb(l, "norm1.bias") : nullptr, Ma, D, prev_fc2_bias);
@@ -960,6 +987,10 @@ int32_t bsr_create(const bsr_config* cfg, void* workspace, size_t bytes, bsr_han
               cudaEventCreateWithFlags(&h->side.fork, cudaEventDisableTiming) == cudaSuccess;
   for (int i = 0; i < 3 && lane; ++i) lane = cudaEventCreateWithFlags(&h->side.done[i], cudaEventDisableTiming) == cudaSuccess;
   if (!lane) { cudaGetLastError(); h->side.stream = nullptr; }
+  lane = cudaStreamCreateWithFlags(&h->wlane.stream, cudaStreamNonBlocking) == cudaSuccess &&
+         cudaEventCreateWithFlags(&h->wlane.fork, cudaEventDisableTiming) == cudaSuccess;
+  for (int i = 0; i < 3 && lane; ++i) lane = cudaEventCreateWithFlags(&h->wlane.done[i], cudaEventDisableTiming) == cudaSuccess;
+  if (!lane) { cudaGetLastError(); h->wlane.stream = nullptr; }
   *out = h;
   return BSR_OK;
 }
@@ -975,6 +1006,10 @@ int32_t bsr_destroy(bsr_handle* h) {
       if (h->ev_done[i]) cudaEventDestroy(h->ev_done[i]);
     }
     if (h->copy_stream) cudaStreamDestroy(h->copy_stream);
+    if (h->wlane.fork) cudaEventDestroy(h->wlane.fork);
+    for (int i = 0; i < 3; ++i)
+      if (h->wlane.done[i]) cudaEventDestroy(h->wlane.done[i]);
+    if (h->wlane.stream) cudaStreamDestroy(h->wlane.stream);
     if (h->side.fork) cudaEventDestroy(h->side.fork);
     for (int i = 0; i < 3; ++i)
       if (h->side.done[i]) cudaEventDestroy(h->side.done[i]);
@@ -1149,6 +1184,9 @@ static int enqueue_train_step(bsr_handle* h, const void* images, const int32_t* 
                   (const float*)h->w("norm.weight"), nullptr, nullptr, 0, nullptr, lnp, h->gradp("norm.weight"), h->gradp("norm.bias"), B, D);
   }
   side_join_all(c);                      // every gradient is complete on the main stream from here on
+  Ctx cl = c;
+  cl.side = lane_of(h, c);
+  side_join_all(cl);
   if (with_update) enqueue_optimizer(h, c);
   return BSR_OK;
 }
