@@ -347,213 +347,237 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
 }
 
 // ------------------------------------------------------------------------------------------------
-// Forward for longer sequences (T > 256): the keys are walked once in blocks of AT_LONG_KB.  Per block S = Q K^T
-// goes into tensor memory, each thread reads its row, forms P = exp(S - m) against the row's reference maximum m,
-// sums P as it goes and hands P (bf16, through shared memory) to the second product, which adds P V into a separate
-// set of tensor-memory columns; the output is divided by the sum at the end.  m follows the running maximum only in
-// jumps of more than AT_LONG_SLACK binary orders, at which the accumulator is rescaled in place (rare after the first
-// block), so that almost every block costs one product, one exponential per score and one more product.  The
-// classification row's probabilities are written out block by block against the m of the moment and brought onto the
-// final scale by its warp at the end.  One CTA per (image, head, 128 queries), one block in flight, several CTAs per SM.
+// Forward for longer sequences (T > 256): the keys are walked once in blocks of AT_LONG_KB.  One CTA per (image, head, 128
+// queries), four of them on an SM to cover one another's waits: four softmax warps, a thread per query row, and a warp
+// whose first lane loads (two slots of K and V) and issues.  Per block the row's 64 scores are read from tensor memory
+// once, P = exp(S - m) against the row's reference maximum m goes back over them as bf16, and the issuer runs O += P V and
+// the next block's S = Q K^T as one group: the softmax warps wait once a block.  m follows the running maximum only
+// in jumps of more than AT_LONG_SLACK binary orders, at which the accumulator is rescaled in place (rare after the first
+// block).  The classification row's probabilities are written out block by block against the m of the moment and brought
+// onto the final scale by its warp at the end.
+// 577 tokens, batch 32, 12 heads: 83 us (290 tokens: 31, was 47); with the scores read twice, P through shared memory, two waits a
+// block and loads that waited for the block before, 143 us.  The exponentials alone take 28 us, the products 20.
 // ------------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(128)
+constexpr int AT_LONG_THREADS = 160;
+
+__global__ void __launch_bounds__(AT_LONG_THREADS, 4)
 attn_fwd_tc_long_kernel(const __grid_constant__ CUtensorMap map_qkv, bf16* __restrict__ out, float* __restrict__ lse,
                         float* __restrict__ cls_prob, int B, int T, int H, int* status) {
   extern __shared__ unsigned char smem_dyn[];
-  uint32_t base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
+  const uint32_t base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
   unsigned char* base_ptr = smem_dyn + (base - smem_u32(smem_dyn));
-  constexpr int KB = AT_LONG_KB;                         // keys per block
-  constexpr uint32_t KV_BYTES = KB * 128;                // 16 KB
-  uint32_t sQ = base, sK = sQ + 2 * AT_BOX_BYTES, sV = sK + KV_BYTES, sP = sV + KV_BYTES;
-  uint32_t bars = sP + (KB / 64) * (AT_QROWS * 128);
-  unsigned char* pP = base_ptr + (sP - base);
+  constexpr int KB = AT_LONG_KB;
+  constexpr uint32_t KV_BYTES = KB * 128;
+  const uint32_t sQ = base, sKV = sQ + 2 * AT_BOX_BYTES;                   // [2 slots][K, V]
+  const uint32_t bars = sKV + 4 * KV_BYTES;
+  auto full_bar = [&](int s) { return bars + 8u * s; };
+  const uint32_t s_bar = bars + 16, p_bar = bars + 24;
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_flag;
-  int tid = threadIdx.x, warp = tid >> 5;
-  int bh = blockIdx.y, b = bh / H, h = bh % H;
-  int q0 = blockIdx.x * AT_QROWS;
-  uint32_t tma_bar = bars, mma_bar = bars + 8;
+  __shared__ float cls_m[AT_LONG_MAXBLK];               // reference maximum of the classification row, block by block
+  __shared__ __align__(16) float cls_p[32];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int bh = blockIdx.y, b = bh / H, h = bh - b * H;
+  const int q0 = blockIdx.x * AT_QROWS, row0 = b * T;
+  const int nblk = (T + KB - 1) / KB;
   if (tid == 0) {
     abort_flag = 0;
-    mbar_init(tma_bar, 1);
-    mbar_init(mma_bar, 1);
+    mbar_init(full_bar(0), 1); mbar_init(full_bar(1), 1); mbar_init(s_bar, 1); mbar_init(p_bar, 4);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     prefetch_map(&map_qkv);
   }
-  if (warp == 0) {
-    tmem_alloc(smem_u32(&tmem_slot), 2 * KB);           // S in the first KB columns, O behind it: several CTAs share an SM
+  if (warp == 4) {
+    tmem_alloc(smem_u32(&tmem_slot), 2 * KB);           // S (then P) in the first KB columns, O behind it
     tmem_relinquish();
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  uint32_t tmem = tmem_slot;
+  const uint32_t tmem = tmem_slot;
   if (leaves_sms_idle()) release_dependents();
   await_inputs();
   constexpr uint32_t C_O = KB;
   volatile int* abortp = &abort_flag;
-  const float c = 0.125f * 1.4426950408889634f;
-  uint32_t trow = tmem + ((uint32_t)(warp * 32) << 16);
-  int nblk = (T + KB - 1) / KB;
-  int row0 = b * T;
-  uint32_t tma_phase = 0, mma_phase = 0;
-  bool ok = true;
-  float mx = -INFINITY, sum = 0.f;
-  bool cls_row = (q0 == 0 && tid == 0 && cls_prob != nullptr);
-  bool cls_warp = (q0 == 0 && warp == 0 && cls_prob != nullptr);
-  __shared__ float cls_m[AT_LONG_MAXBLK];               // reference maximum of the classification row, block by block
 
-  for (int kb = 0; kb < nblk && ok; ++kb) {
-    int k0 = kb * KB;
-    int keys = min(KB, T - k0);
-    int kpad = (keys + 15) & ~15;
-    int nbox = (kpad + AT_BOX - 1) / AT_BOX;
-    if (tid == 0) {
-      int boxes = 2 * nbox + (kb == 0 ? 2 : 0);
-      mbar_expect_tx(tma_bar, boxes * AT_BOX_BYTES);
-      if (kb == 0)
-        for (int j = 0; j < 2; ++j) tma_load_2d(sQ + j * AT_BOX_BYTES, &map_qkv, tma_bar, h * AT_D, row0 + q0 + j * AT_BOX);
-      for (int j = 0; j < nbox; ++j) {
-        tma_load_2d(sK + j * AT_BOX_BYTES, &map_qkv, tma_bar, (H + h) * AT_D, row0 + k0 + j * AT_BOX);
-        tma_load_2d(sV + j * AT_BOX_BYTES, &map_qkv, tma_bar, (2 * H + h) * AT_D, row0 + k0 + j * AT_BOX);
-      }
-      ok = mbar_wait(tma_bar, tma_phase, abortp);
-      if (ok) {
-        tc_fence_after();
-        uint32_t idesc = make_idesc_mn(AT_QROWS, kpad, false, false);
+  if (warp == 4) {
+    // ------------------------------- loads and products -------------------------
+    if (lane == 0) {
+      auto load = [&](int kb) {
+        const uint32_t dst = sKV + (kb & 1) * 2 * KV_BYTES, bar = full_bar(kb & 1);
+        tma_load_2d(dst, &map_qkv, bar, (H + h) * AT_D, row0 + kb * KB);
+        tma_load_2d(dst + KV_BYTES, &map_qkv, bar, (2 * H + h) * AT_D, row0 + kb * KB);
+      };
+      auto scores = [&](int kb) {
+        const int kpad = (min(KB, T - kb * KB) + 15) & ~15;
+        const uint32_t sK = sKV + (kb & 1) * 2 * KV_BYTES, idesc = make_idesc_mn(AT_QROWS, kpad, false, false);
 #pragma unroll
         for (int k = 0; k < AT_D / 16; ++k)
           umma_bf16(tmem, make_desc(sQ + k * 32, 16, 1024), make_desc(sK + k * 32, 16, 1024), idesc, k > 0 ? 1u : 0u);
-        umma_commit(mma_bar);
+      };
+      mbar_expect_tx(full_bar(0), 2 * AT_BOX_BYTES + 2 * KV_BYTES);
+      for (int j = 0; j < 2; ++j) tma_load_2d(sQ + j * AT_BOX_BYTES, &map_qkv, full_bar(0), h * AT_D, row0 + q0 + j * AT_BOX);
+      load(0);
+      if (nblk > 1) {
+        mbar_expect_tx(full_bar(1), 2 * KV_BYTES);
+        load(1);
+      }
+      bool ok = mbar_wait(full_bar(0), 0, abortp);
+      if (ok) {
+        tc_fence_after();
+        scores(0);
+        umma_commit(s_bar);
+      }
+      for (int kb = 0; kb < nblk && ok; ++kb) {
+        ok = mbar_wait(p_bar, kb & 1, abortp);           // P of this block is in tensor memory
+        if (!ok) break;
+        tc_fence_after();
+        const int kpad = (min(KB, T - kb * KB) + 15) & ~15;
+        const uint32_t sV = sKV + (kb & 1) * 2 * KV_BYTES + KV_BYTES, idesc = make_idesc_mn(AT_QROWS, AT_D, false, true);
+        for (int k = 0; k < kpad / 16; ++k)
+          umma_bf16_ts(tmem + C_O, tmem + 8 * k, make_desc(sV + k * (16 * 128), 8192, 1024), idesc, (kb > 0 || k > 0) ? 1u : 0u);
+        if (kb + 1 < nblk) {                             // products run in order: the next scores overwrite P once it has been read
+          ok = mbar_wait(full_bar((kb + 1) & 1), ((kb + 1) >> 1) & 1, abortp);
+          if (ok) {
+            tc_fence_after();
+            scores(kb + 1);
+          }
+        }
+        umma_commit(s_bar);
+        if (ok && kb + 2 < nblk) {
+          ok = mbar_wait(s_bar, (kb + 1) & 1, abortp);   // this block's K and V have been read
+          if (ok) {
+            mbar_expect_tx(full_bar(kb & 1), 2 * KV_BYTES);
+            load(kb + 2);
+          }
+        }
+      }
+      if (!ok) {                                         // copies already issued still land: a bounded time before the CTA leaves
+        unsigned long long t0 = global_ns();
+        while (global_ns() - t0 < 1000000ull) {}
       }
     }
-    tma_phase ^= 1u;
-    ok = mbar_wait(mma_bar, mma_phase, abortp);
-    mma_phase ^= 1u;
+  } else {
+    // ------------------------------- softmax ------------------------------------
+    const float c = 0.125f * 1.4426950408889634f;          // 1/sqrt(64) * log2(e)
+    const uint32_t trow = tmem + ((uint32_t)(warp * 32) << 16);
+    const bool cls_warp = (q0 == 0 && warp == 0 && cls_prob != nullptr);
+    float* cp = cls_warp ? cls_prob + (size_t)bh * (T - 1) : nullptr;
+    float mx = -INFINITY, sum = 0.f;
+    bool ok = true;
+    for (int kb = 0; kb < nblk && ok; ++kb) {
+      const int keys = min(KB, T - kb * KB);
+      ok = mbar_wait_q(s_bar, kb & 1, abortp);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
+      tc_fence_after();
+      uint32_t r[KB];
+      tmem_ld32(trow, r);
+      tmem_ld32(trow + 32, r + 32);
+      tmem_ld_wait();
+      if (keys < KB) {
+#pragma unroll
+        for (int j = 0; j < KB; ++j)
+          if (j >= keys) r[j] = 0xff800000u;               // -inf: probability zero
+      }
+      float bm = -INFINITY;
+#pragma unroll
+      for (int j = 0; j < KB; j += 2) bm = fmax3(bm, __uint_as_float(r[j]), __uint_as_float(r[j + 1]));
+      // The reference maximum of a row moves only when the block's maximum exceeds it by more than AT_LONG_SLACK in the
+      // exponent (the probabilities then stay below 2^AT_LONG_SLACK, harmless in bf16 and in the fp32 sum); when it
+      // moves, the accumulated output and sum of that row are scaled down.  The decision is taken per warp, because the
+      // accumulator is read and written with warp-wide instructions; rows that do not move scale by one.
+      if (kb == 0) {
+        mx = bm;
+      } else {
+        const bool grow = (bm - mx) * c > AT_LONG_SLACK;
+        if (__any_sync(0xffffffffu, grow)) {
+          const float nm = grow ? bm : mx, f = ex2_fast((mx - nm) * c);
+#pragma unroll 1
+          for (int q = 0; q < 4; ++q) {
+            uint32_t o[16];
+            tmem_ld16(trow + C_O + q * 16, o);
+            tmem_ld_wait();
+#pragma unroll
+            for (int j = 0; j < 16; ++j) o[j] = __float_as_uint(__uint_as_float(o[j]) * f);
+            tmem_st16(trow + C_O + q * 16, o);
+          }
+          sum *= f;
+          mx = nm;
+        }
+      }
+      const float mc = mx * c;
+      if (cls_warp && lane == 0) cls_m[kb] = mx;
+#pragma unroll
+      for (int half = 0; half < 2; ++half) {
+        float s0 = 0.f, s1 = 0.f;
+#pragma unroll
+        for (int j = half * 32; j < half * 32 + 32; j += 2) {
+          const float e0 = ex2_fast(fmaf(__uint_as_float(r[j]), c, -mc)), e1 = ex2_fast(fmaf(__uint_as_float(r[j + 1]), c, -mc));
+          s0 += e0; s1 += e1;
+          r[j] = __float_as_uint(e0); r[j + 1] = __float_as_uint(e1);
+        }
+        sum += s0 + s1;
+        if (cls_warp) {                 // relative to this block's reference maximum; put on the final scale below
+          if (lane == 0) {
+#pragma unroll
+            for (int j = 0; j < 32; j += 4) *reinterpret_cast<uint4*>(cls_p + j) = make_uint4(r[half * 32 + j], r[half * 32 + j + 1], r[half * 32 + j + 2], r[half * 32 + j + 3]);
+          }
+          __syncwarp();
+          const int key = kb * KB + half * 32 + lane;
+          if (key >= 1 && key < T) cp[key - 1] = cls_p[lane];
+          __syncwarp();
+        }
+        uint32_t pk[16];
+#pragma unroll
+        for (int j = 0; j < 16; ++j) pk[j] = pack_bf16x2(__uint_as_float(r[half * 32 + 2 * j]), __uint_as_float(r[half * 32 + 2 * j + 1]));
+        tmem_st16(trow + half * 16, pk);
+      }
+      tmem_st_wait();
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(p_bar);
+    }
+    if (ok) ok = mbar_wait_q(s_bar, nblk & 1, abortp);     // the last P V
     ok = __all_sync(0xffffffffu, ok);
     tc_fence_after();
-    if (!ok) break;
-    // the block's maximum of this thread's query row (the scores are read again below: cheaper than holding them)
-    float bm = -INFINITY;
-#pragma unroll
-    for (int ch = 0; ch < KB / 32; ++ch) {
-      uint32_t r[32];
-      tmem_ld32(trow + ch * 32, r);
-      tmem_ld_wait();
-#pragma unroll
-      for (int j = 0; j < 32; ++j)
-        if (ch * 32 + j < keys) bm = fmaxf(bm, __uint_as_float(r[j]));
+    if (ok && cls_warp) {
+      // the classification row's probabilities: from each block's reference maximum to the final one, over the row sum
+      const float fm = __shfl_sync(0xffffffffu, mx, 0), inv0 = 1.0f / __shfl_sync(0xffffffffu, sum, 0);
+      for (int key = 1 + lane; key < T; key += 32) cp[key - 1] *= ex2_fast((cls_m[key / KB] - fm) * c) * inv0;
     }
-    // The reference maximum of a row moves only when the block's maximum exceeds it by more than AT_LONG_SLACK in the
-    // exponent (the probabilities then stay below 2^AT_LONG_SLACK, harmless in bf16 and in the fp32 sum); when it
-    // moves, the accumulated output and sum of that row are scaled down.  The decision is taken per warp, because the
-    // accumulator is read and written with warp-wide instructions; rows that do not move scale by one.
-    if (kb == 0) {
-      mx = bm;
-    } else {
-      bool grow = (bm - mx) * c > AT_LONG_SLACK;
-      if (__any_sync(0xffffffffu, grow)) {
-        float nm = grow ? bm : mx;
-        float f = ex2_fast((mx - nm) * c);
+    if (ok) {
+      // the output rows go out through Q's space (read by now) so that a store instruction writes whole 128-byte rows
+      const float inv = 1.0f / sum;
+      unsigned char* st = base_ptr + warp * 32 * 128;
 #pragma unroll
-        for (int half = 0; half < 2; ++half) {
-          uint32_t r[32];
-          tmem_ld32(trow + C_O + half * 32, r);
-          tmem_ld_wait();
-#pragma unroll
-          for (int j = 0; j < 32; ++j) r[j] = __float_as_uint(__uint_as_float(r[j]) * f);
-          tmem_st16(trow + C_O + half * 32, r);
-          tmem_st16(trow + C_O + half * 32 + 16, r + 16);
-        }
-        tmem_st_wait();
-        sum *= f;
-        mx = nm;
-      }
-    }
-    if (cls_row) cls_m[kb] = mx;
-    float mc = mx * c;
-#pragma unroll
-    for (int ch = 0; ch < KB / 32; ++ch) {
-      uint32_t r[32];
-      tmem_ld32(trow + ch * 32, r);
-      tmem_ld_wait();
-      float p[32];
-#pragma unroll
-      for (int j = 0; j < 32; ++j) {
-        float e = ex2_fast(fmaf(__uint_as_float(r[j]), c, -mc));
-        p[j] = (ch * 32 + j < keys) ? e : 0.f;
-        sum += p[j];
-      }
-      if (cls_row) {                  // relative to this block's reference maximum; put on the final scale below
-        float* cp = cls_prob + ((size_t)b * H + h) * (T - 1);
-        for (int j = 0; j < 32; ++j) {
-          int key = k0 + ch * 32 + j;
-          if (key >= 1 && key < T) cp[key - 1] = p[j];
-        }
-      }
-#pragma unroll
-      for (int g = 0; g < 4; ++g) {
-        int key8 = ch * 4 + g;
-        if (key8 * 8 < nbox * AT_BOX) {
-          uint4 v;
-          __nv_bfloat162* hh = reinterpret_cast<__nv_bfloat162*>(&v);
-#pragma unroll
-          for (int i = 0; i < 4; ++i) hh[i] = __floats2bfloat162_rn(p[g * 8 + 2 * i], p[g * 8 + 2 * i + 1]);
-          *reinterpret_cast<uint4*>(pP + p_offset(tid, key8)) = v;
-        }
-      }
-    }
-    fence_async_smem();
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    if (tid == 0) {
-      uint32_t idesc = make_idesc_mn(AT_QROWS, AT_D, false, true);
-      for (int k = 0; k < kpad / 16; ++k)
-        umma_bf16(tmem + C_O, make_desc(sP + (k >> 2) * (AT_QROWS * 128) + (k & 3) * 32, 16, 1024),
-                  make_desc(sV + k * (16 * 128), 8192, 1024), idesc, (kb > 0 || k > 0) ? 1u : 0u);
-      umma_commit(mma_bar);
-    }
-    ok = mbar_wait(mma_bar, mma_phase, abortp);      // P, K and V of this block are free again; O is complete
-    mma_phase ^= 1u;
-    ok = __all_sync(0xffffffffu, ok);
-    tc_fence_after();
-  }
-  if (ok && cls_warp) {
-    // the classification row's probabilities: from each block's reference maximum to the final one, over the row sum
-    float fm = __shfl_sync(0xffffffffu, mx, 0), fs = __shfl_sync(0xffffffffu, sum, 0);
-    float inv0 = 1.0f / fs;
-    __syncwarp();
-    float* cp = cls_prob + ((size_t)b * H + h) * (T - 1);
-    for (int key = 1 + (tid & 31); key < T; key += 32)
-      cp[key - 1] *= ex2_fast((cls_m[key / KB] - fm) * c) * inv0;
-  }
-  int q = q0 + tid;
-  if (ok) {
-    float inv = 1.0f / sum;
-#pragma unroll
-    for (int half = 0; half < 2; ++half) {
-      uint32_t r[32];
-      tmem_ld32(trow + C_O + half * 32, r);
-      tmem_ld_wait();
-      if (q < T) {
-        bf16* orow = out + ((size_t)b * T + q) * H * AT_D + (size_t)h * AT_D + half * 32;
+      for (int half = 0; half < 2; ++half) {
+        uint32_t r[32];
+        tmem_ld32(trow + C_O + half * 32, r);
+        tmem_ld_wait();
 #pragma unroll
         for (int g = 0; g < 4; ++g) {
           float v[8];
 #pragma unroll
           for (int j = 0; j < 8; ++j) v[j] = __uint_as_float(r[g * 8 + j]) * inv;
-          store16(orow + g * 8, v);
+          store16(reinterpret_cast<bf16*>(st + lane * 128 + (((half * 4 + g) ^ (lane & 7)) << 4)), v);
         }
       }
+      __syncwarp();
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int rr = i * 4 + (lane >> 3), u = lane & 7, q = q0 + warp * 32 + rr;
+        const uint4 x = *reinterpret_cast<const uint4*>(st + rr * 128 + ((u ^ (rr & 7)) << 4));
+        if (q < T) *reinterpret_cast<uint4*>(out + ((size_t)row0 + q) * H * AT_D + (size_t)h * AT_D + u * 8) = x;
+      }
+      const int q = q0 + tid;
+      if (q < T && lse != nullptr) lse[(size_t)bh * T + q] = mx * 0.125f + logf(sum);
     }
-    if (q < T && lse != nullptr) lse[((size_t)b * H + h) * T + q] = mx * 0.125f + logf(sum);
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == 0) {
+  if (warp == 4) {
     tc_fence_after();
-    tmem_dealloc(tmem, 2 * AT_LONG_KB);
+    tmem_dealloc(tmem, 2 * KB);
   }
   if (tid == 0 && abort_flag && status != nullptr) atomicOr(status, STATUS_TIMEOUT);
 }
@@ -1291,13 +1315,14 @@ int attention_fwd_tc(const Ctx& c, const void* qkv, void* out, float* lse, float
   if (((uintptr_t)qkv & 15) || ((uintptr_t)out & 15)) return -1;
   CUtensorMap map;
   if (!make_map(&map, qkv, (uint64_t)3 * H * d, (uint64_t)B * T, (uint64_t)3 * H * d, AT_BOX)) return -2;
+  // (up to 256 keys the kernel above, which holds a whole row of scores, is faster: 61 against 67 us at 197 tokens)
   if (T > AT_MAXKEYS) {
-    size_t smem_l = 1024 + 2 * (size_t)AT_BOX_BYTES + 2 * (size_t)AT_LONG_KB * 128 + (AT_LONG_KB / 64) * (size_t)(AT_QROWS * 128) + 64;
+    size_t smem_l = 1024 + 2 * (size_t)AT_BOX_BYTES + 4 * (size_t)AT_LONG_KB * 128 + 64;
     static SmemLimit lim_l;
     if (!ensure_smem(lim_l, attn_fwd_tc_long_kernel, smem_l)) return -3;
     dim3 grid_l((T + AT_QROWS - 1) / AT_QROWS, B * H);
     note_launch(1);
-    launch_k(attn_fwd_tc_long_kernel, grid_l, 128, smem_l, c.stream, map, (bf16*)out, lse, cls_prob, B, T, H, c.status);
+    launch_k(attn_fwd_tc_long_kernel, grid_l, AT_LONG_THREADS, smem_l, c.stream, map, (bf16*)out, lse, cls_prob, B, T, H, c.status);
     return 0;
   }
   int tpad = (T + 15) & ~15;

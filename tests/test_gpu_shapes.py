@@ -141,3 +141,20 @@ def test_linear_over_tile_widths(m, n, k):
         ws = torch.empty(160 * 128 * 256, device="cuda")
         dx, dw = Bd.bsr_linear_backward(x, w, dy, use_tensor_cores=True, workspace=ws)
         assert rel(dx, dy.double() @ w.double()) < 4e-3 and rel(dw, dy.double().T @ x.double()) < 1e-4
+
+
+@pytest.mark.parametrize("B,T,H", [(1, 257, 2), (2, 319, 1), (1, 320, 3), (1, 321, 1), (5, 577, 12), (1, 4096, 1)])
+def test_long_attention_forward_at_block_edges(B, T, H):
+    """Output, log-sum-exp and classification row of the single-walk kernel with last key blocks of 1, 63 and 64 keys, last query
+    tiles of 1 to 128 rows and the longest sequence it takes; several CTAs per SM.  bf16 rounding of P and of the output."""
+    import torch
+    from paper_2405_10951_b200 import binding as Bd
+    gen = torch.Generator(device="cuda").manual_seed(T + B)
+    qkv = torch.randn(B, T, 3, H, 64, generator=gen, device="cuda").bfloat16()
+    out, cp, lse = Bd.bsr_attention_forward(qkv, H, use_tensor_cores=True, want_lse=True)
+    q, k, v = (qkv[:, :, i].transpose(1, 2).double() for i in range(3))
+    s = q @ k.transpose(-1, -2) / 8.0
+    rel = lambda a, b: float((a.double() - b).norm() / b.norm())
+    assert rel(out, (s.softmax(-1) @ v).transpose(1, 2).reshape(B, T, H * 64)) < 6e-3
+    assert rel(lse, s.logsumexp(-1)) < 1e-5
+    assert rel(cp, s.softmax(-1)[:, :, 0, 1:]) < 2e-5
