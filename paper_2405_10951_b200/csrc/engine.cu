@@ -159,6 +159,7 @@ struct bsr_handle {
   size_t off_master = 0, off_grad = 0, off_m = 0, off_v = 0;
   size_t off_chunks = 0;
   int n_chunks = 0;
+  std::vector<int> chunk_at;            // first chunk of block l's attention half (2 l), of its FFN half (2 l + 1), of what follows the blocks (2 depth)
   std::vector<BlockBufs> bufs_train;  // per block (valid for l >= t0)
   BlockBufs bufs_frozen[2];           // ping-pong by block parity
   size_t off_x_last = 0;
@@ -206,6 +207,7 @@ struct bsr_handle {
   int host_slot = 0;
   SideLane side;                        // second lane for the reductions only the optimiser reads
   SideLane wlane;                       // lane of the weight gradients (see block_backward)
+  SideLane ulane;                       // lane of the updates that start before the backward pass has ended (see update_half)
   int use_side = 1;
   long launches_at_enable = 0;
 
@@ -309,8 +311,12 @@ size_t plan(bsr_handle* h) {
   h->weights_bytes = b.off - w0;
   // AdamW chunk table
   int nch = 0;
-  for (auto& t : h->tensors)
+  h->chunk_at.clear();
+  for (auto& t : h->tensors) {
+    if (t.name.find("norm1.weight") != std::string::npos || t.name.find("norm2.weight") != std::string::npos || t.name == "norm.weight")
+      h->chunk_at.push_back(nch);
     if (t.trainable) nch += (int)((t.numel + ADAM_CHUNK - 1) / ADAM_CHUNK);
+  }
   h->n_chunks = nch;
   h->off_chunks = b.take((size_t)nch * sizeof(AdamChunk));
   // 8-bit copies of the gradient-free prefix's LayerNorm-fed weights
@@ -668,7 +674,46 @@ struct GradStream {      // gradient of the residual stream: float rows, plus th
 // The lane of the weight gradients (null: they stay on the stream of the step, as when launches are timed one by one).
 SideLane* lane_of(const bsr_handle* h, const Ctx& c) { return c.side != nullptr && h->wlane.stream != nullptr ? const_cast<SideLane*>(&h->wlane) : nullptr; }
 
-int block_backward(bsr_handle* h, const Ctx& c, int l, int B, GradStream dxo, GradStream dxi, bool need_dxi, const int* task_ids) {
+// The update of the trainable parameters from the flat gradient buffer; learning rate and bias corrections are read
+// from device memory (the three scalars at status + 128).  Chunks first to last - 1; beside: next to other kernels.
+void enqueue_optimizer(bsr_handle* h, const Ctx& c, int first, int last, bool beside) {
+  const AdamChunk* chunks = h->at<AdamChunk>(h->off_chunks) + first;
+  if (h->cfg.optimizer == BSR_OPT_SGD)
+    sgd_momentum(c, chunks, last - first, beside, h->at<float>(h->off_master), h->at<float>(h->off_grad), h->at<float>(h->off_m),
+                 h->base + h->off_weights, h->at<float>(h->off_status + 128), h->cfg.momentum, h->cfg.weight_decay);
+  else
+    adamw(c, chunks, last - first, beside, h->at<float>(h->off_master), h->at<float>(h->off_grad), h->at<float>(h->off_m),
+          h->at<float>(h->off_v), h->base + h->off_weights, h->at<float>(h->off_status + 128), h->cfg.beta1, h->cfg.beta2, h->cfg.eps,
+          h->cfg.weight_decay);
+}
+
+// Half a block (0: attention, 1: FFN) is updated as soon as its gradients are complete and its weights have been read for
+// the last time, on a lane beside the backward pass of what is below.  The lane waits for everything enqueued so far on the
+// chain, on the reductions' lane and on the weight gradients'.
+void update_half(bsr_handle* h, const Ctx& c, const Ctx& cl, int l, int half) {
+  const cudaStream_t before[] = {c.stream, c.side->stream, cl.side->stream};
+  for (cudaStream_t s : before) {
+    cudaEventRecord(h->ulane.fork, s);
+    cudaStreamWaitEvent(h->ulane.stream, h->ulane.fork, 0);
+  }
+  Ctx u = c;
+  u.stream = h->ulane.stream;
+  enqueue_optimizer(h, u, h->chunk_at[2 * l + half], h->chunk_at[2 * l + half + 1], l > h->t0 || half == 1);
+}
+
+// Up to 16384 token rows the backward pass leaves DRAM idle and the update hides in it (a step of DeiT-S with one image 722
+// -> 708 us, with 64 images 1524 -> 1508; ViT-B with 32 images 2292 -> 2274, ViT-B/384 with 7 images 2150 -> 2117); over more
+// rows its contractions lose what the update gains (ViT-B, 128 images: 5826 -> 5860 us).  float storage has nothing to
+// gain (tiny model, four steps: 2991 -> 2997 us), nor has an expert layer, whose many weights take longer to update than its
+// backward pass has time for (64 images: 2264 -> 2278 us).  The sizes are ones that every kernel of the backward pass takes,
+// so that a step which ends in an error updates nothing.
+bool early_update(const bsr_handle* h, const Ctx& c, int B) {
+  const bsr_dims& d = h->cfg.dims;
+  return c.dtype == 1 && c.use_tc && d.dim == 64 * d.heads && (long)B * d.heads <= 65535 && h->ulane.stream != nullptr &&
+         d.moe_block_mask == 0 && h->t0 < d.depth && (long)B * h->sched.ta[0] <= 16384;
+}
+
+int block_backward(bsr_handle* h, const Ctx& c, int l, int B, GradStream dxo, GradStream dxi, bool need_dxi, const int* task_ids, bool update) {
   const bsr_dims& d = h->cfg.dims;
   const Schedule& s = h->sched;
   const BlockBufs& bb = h->bufs_train[l];
@@ -757,6 +802,7 @@ int block_backward(bsr_handle* h, const Ctx& c, int l, int B, GradStream dxo, Gr
                 (const float*)h->wb(l, "norm2.weight"), dxo.f, dxg.f, D, shrinks ? nullptr : dxg.c, lnp,
                 pg ? h->gb(l, "norm2.weight") : nullptr, pg ? h->gb(l, "norm2.bias") : nullptr, Mf, D,
                 (pg && !shrinks) ? h->gb(l, "attn.proj.bias") : nullptr);   // dx' = dxg here: its column sums are the projection's bias gradient
+  if (pg && update) update_half(h, c, cl, l, 1);
   const float* cls_extra = nullptr;
   if (shrinks) {
     gather_fuse_bwd(c, dxg.f, h->base + bb.xp_full, B, Ta - 1, D, k, h->at<int>(bb.kept), h->at<int>(bb.dropped),
@@ -818,6 +864,7 @@ int block_backward(bsr_handle* h, const Ctx& c, int l, int B, GradStream dxo, Gr
   layernorm_bwd(c, dy, 0, h->at<float>(bb.x_in), D, h->at<float>(bb.mean1), h->at<float>(bb.rstd1),
                 (const float*)h->wb(l, "norm1.weight"), ln1_res, need_dxi ? dxi.f : nullptr, D, need_dxi ? dxi.c : nullptr, lnp,
                 pg ? h->gb(l, "norm1.weight") : nullptr, pg ? h->gb(l, "norm1.bias") : nullptr, Ma, D, prev_fc2_bias);
+  if (pg && update) update_half(h, c, cl, l, 0);
   return BSR_OK;
 }
 
@@ -983,14 +1030,12 @@ int32_t bsr_create(const bsr_config* cfg, void* workspace, size_t bytes, bsr_han
     return set_err(g_error, BSR_ERR_CUDA, "workspace initialisation failed: %s", cudaGetErrorString(e));
   }
   // host objects of the side lane (no device memory); without them the reductions simply stay on the main stream
-  bool lane = cudaStreamCreateWithFlags(&h->side.stream, cudaStreamNonBlocking) == cudaSuccess &&
-              cudaEventCreateWithFlags(&h->side.fork, cudaEventDisableTiming) == cudaSuccess;
-  for (int i = 0; i < 3 && lane; ++i) lane = cudaEventCreateWithFlags(&h->side.done[i], cudaEventDisableTiming) == cudaSuccess;
-  if (!lane) { cudaGetLastError(); h->side.stream = nullptr; }
-  lane = cudaStreamCreateWithFlags(&h->wlane.stream, cudaStreamNonBlocking) == cudaSuccess &&
-         cudaEventCreateWithFlags(&h->wlane.fork, cudaEventDisableTiming) == cudaSuccess;
-  for (int i = 0; i < 3 && lane; ++i) lane = cudaEventCreateWithFlags(&h->wlane.done[i], cudaEventDisableTiming) == cudaSuccess;
-  if (!lane) { cudaGetLastError(); h->wlane.stream = nullptr; }
+  for (SideLane* lane : {&h->side, &h->wlane, &h->ulane}) {
+    bool ok = cudaStreamCreateWithFlags(&lane->stream, cudaStreamNonBlocking) == cudaSuccess &&
+              cudaEventCreateWithFlags(&lane->fork, cudaEventDisableTiming) == cudaSuccess;
+    for (int i = 0; i < 3 && ok; ++i) ok = cudaEventCreateWithFlags(&lane->done[i], cudaEventDisableTiming) == cudaSuccess;
+    if (!ok) { cudaGetLastError(); lane->stream = nullptr; }
+  }
   *out = h;
   return BSR_OK;
 }
@@ -1006,14 +1051,12 @@ int32_t bsr_destroy(bsr_handle* h) {
       if (h->ev_done[i]) cudaEventDestroy(h->ev_done[i]);
     }
     if (h->copy_stream) cudaStreamDestroy(h->copy_stream);
-    if (h->wlane.fork) cudaEventDestroy(h->wlane.fork);
-    for (int i = 0; i < 3; ++i)
-      if (h->wlane.done[i]) cudaEventDestroy(h->wlane.done[i]);
-    if (h->wlane.stream) cudaStreamDestroy(h->wlane.stream);
-    if (h->side.fork) cudaEventDestroy(h->side.fork);
-    for (int i = 0; i < 3; ++i)
-      if (h->side.done[i]) cudaEventDestroy(h->side.done[i]);
-    if (h->side.stream) cudaStreamDestroy(h->side.stream);
+    for (SideLane* lane : {&h->side, &h->wlane, &h->ulane}) {
+      if (lane->fork) cudaEventDestroy(lane->fork);
+      for (int i = 0; i < 3; ++i)
+        if (lane->done[i]) cudaEventDestroy(lane->done[i]);
+      if (lane->stream) cudaStreamDestroy(lane->stream);
+    }
   }
   delete h;
   return BSR_OK;
@@ -1139,7 +1182,6 @@ int32_t bsr_set_step(bsr_handle* h, int64_t steps_done) {
 
 // Enqueues every kernel of one step on `stream` (forward, loss, backward, AdamW reading its scalars from device memory).
 // loss_out may be null (the multi-step loop writes the loss itself); img_offset as in forward_all.
-static void enqueue_optimizer(bsr_handle* h, const Ctx& c);
 static int enqueue_train_step(bsr_handle* h, const void* images, const int32_t* labels, const int32_t* task_ids, int32_t batch,
                               void* stream, float* loss_out, int32_t* kept_out, const long long* img_offset = nullptr,
                               bool with_update = true) {
@@ -1166,6 +1208,7 @@ static int enqueue_train_step(bsr_handle* h, const void* images, const int32_t* 
   head_bwd(c, hd, xn, h->at<float>(h->off_dlogits), task_ids, h->at<float>(h->off_dxn), B);
   float* lnp = h->at<float>(h->off_ln_partials);
   bool bf = d.dtype == BSR_DTYPE_BF16;
+  const bool early = with_update && lane_of(h, c) != nullptr && early_update(h, c, B);
   if (h->t0 < d.depth) {
     GradStream dxo = {h->at<float>(h->off_dxa), bf ? (void*)(h->base + h->off_dxa_c) : nullptr};
     GradStream dxi = {h->at<float>(h->off_dxb), bf ? (void*)(h->base + h->off_dxb_c) : nullptr};
@@ -1175,7 +1218,7 @@ static int enqueue_train_step(bsr_handle* h, const void* images, const int32_t* 
     layernorm_bwd(c, h->at<float>(h->off_dxn), 1, h->at<float>(x_last), (long)Tl * D, h->at<float>(h->off_meanf), h->at<float>(h->off_rstdf),
                   (const float*)h->w("norm.weight"), nullptr, dxo.f, (long)Tl * D, dxo.c, lnp, h->gradp("norm.weight"), h->gradp("norm.bias"), B, D);
     for (int l = d.depth - 1; l >= h->t0; --l) {
-      rc = block_backward(h, c, l, B, dxo, dxi, l > h->t0, task_ids);
+      rc = block_backward(h, c, l, B, dxo, dxi, l > h->t0, task_ids, early);
       if (rc != BSR_OK) return rc;
       GradStream t = dxo; dxo = dxi; dxi = t;
     }
@@ -1187,20 +1230,14 @@ static int enqueue_train_step(bsr_handle* h, const void* images, const int32_t* 
   Ctx cl = c;
   cl.side = lane_of(h, c);
   side_join_all(cl);
-  if (with_update) enqueue_optimizer(h, c);
+  if (early) {                           // the blocks are updated or about to be; the final LayerNorm and the heads remain
+    enqueue_optimizer(h, c, h->chunk_at[2 * d.depth], h->n_chunks, false);
+    cudaEventRecord(h->ulane.fork, h->ulane.stream);
+    cudaStreamWaitEvent(c.stream, h->ulane.fork, 0);
+  } else if (with_update) {
+    enqueue_optimizer(h, c, 0, h->n_chunks, false);
+  }
   return BSR_OK;
-}
-
-// The update of the trainable parameters from the flat gradient buffer; learning rate and bias corrections are read
-// from device memory (the three scalars at status + 128).
-static void enqueue_optimizer(bsr_handle* h, const Ctx& c) {
-  if (h->cfg.optimizer == BSR_OPT_SGD)
-    sgd_momentum(c, h->at<AdamChunk>(h->off_chunks), h->n_chunks, h->at<float>(h->off_master), h->at<float>(h->off_grad),
-                 h->at<float>(h->off_m), h->base + h->off_weights, h->at<float>(h->off_status + 128), h->cfg.momentum, h->cfg.weight_decay);
-  else
-    adamw(c, h->at<AdamChunk>(h->off_chunks), h->n_chunks, h->at<float>(h->off_master), h->at<float>(h->off_grad), h->at<float>(h->off_m),
-          h->at<float>(h->off_v), h->base + h->off_weights, h->at<float>(h->off_status + 128), h->cfg.beta1, h->cfg.beta2, h->cfg.eps,
-          h->cfg.weight_decay);
 }
 
 }  // extern "C"
@@ -1330,7 +1367,7 @@ int32_t bsr_optimizer_step(bsr_handle* h, void* stream) {
   double bc2 = 1.0 - std::pow((double)h->cfg.beta2, (double)step_next);
   set_scalars(st, h->at<float>(h->off_status + 128), h->lr, (float)bc1, (float)bc2);
   Ctx c = make_ctx(h, stream);
-  enqueue_optimizer(h, c);
+  enqueue_optimizer(h, c, 0, h->n_chunks, false);
   int rc = check_cuda(h, "bsr_optimizer_step");
   if (rc == BSR_OK) h->step = step_next;
   return rc;

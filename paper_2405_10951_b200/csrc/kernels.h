@@ -214,11 +214,12 @@ void cross_entropy(const Ctx& c, const HeadDesc& h, const float* logits, const i
 void head_bwd(const Ctx& c, const HeadDesc& h, const float* xn, const float* dlogits, const int* task_ids, float* dxn, int B);
 
 struct AdamChunk { uint32_t offset; uint32_t count; int64_t shadow; uint32_t decay; uint32_t pad; };
-// scalars (device): learning rate, 1 - beta1^t, 1 - beta2^t of the step being taken.
-void adamw(const Ctx& c, const AdamChunk* chunks, int nchunks, float* master, const float* grad, float* m, float* v,
+// scalars (device): learning rate, 1 - beta1^t, 1 - beta2^t of the step being taken.  beside: the update runs next to
+// other work and takes few blocks.
+void adamw(const Ctx& c, const AdamChunk* chunks, int nchunks, bool beside, float* master, const float* grad, float* m, float* v,
            void* shadow_base, const float* scalars, float b1, float b2, float eps, float wd);
 // SGD with momentum (buf starts at zero): buf <- mu buf + (g + wd p on decayed tensors), p <- p - lr buf; lr from scalars[0].
-void sgd_momentum(const Ctx& c, const AdamChunk* chunks, int nchunks, float* master, const float* grad, float* buf,
+void sgd_momentum(const Ctx& c, const AdamChunk* chunks, int nchunks, bool beside, float* master, const float* grad, float* buf,
                   void* shadow_base, const float* scalars, float mu, float wd);
 void set_scalars(cudaStream_t s, float* dst, float a, float b, float c3);
 

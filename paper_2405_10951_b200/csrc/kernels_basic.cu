@@ -707,58 +707,117 @@ void head_bwd(const Ctx& c, const HeadDesc& h, const float* xn, const float* dlo
 //   m <- b1 m + (1-b1) g;  v <- b2 v + (1-b2) g^2;  p <- p - lr * (m/bc1) / (sqrt(v/bc2) + eps) - lr * wd * p
 // One block per chunk; a chunk never straddles two tensors.
 // ------------------------------------------------------------------------------------------------
-template <typename T>
-__global__ void adamw_kernel(const AdamChunk* __restrict__ chunks, float* __restrict__ master,
-                             const float* __restrict__ grad, float* __restrict__ m, float* __restrict__ v,
-                             T* __restrict__ shadow_base, const float* __restrict__ scalars, float b1, float b2, float eps,
-                             float wd) {
-  dependent_sync();
-  // step-dependent scalars live in device memory so that a captured graph of the step stays valid: lr, 1-b1^t, 1-b2^t
-  float lr = scalars[0], bc1 = scalars[1], bc2 = scalars[2];
-  AdamChunk ch = chunks[blockIdx.x];
-  float decay = ch.decay ? lr * wd : 0.f;
-  for (uint32_t i = threadIdx.x; i < ch.count; i += blockDim.x) {
-    size_t idx = (size_t)ch.offset + i;
-    float g = grad[idx];
-    float p = master[idx];
-    float mm = b1 * m[idx] + (1.f - b1) * g;
-    float vv = b2 * v[idx] + (1.f - b2) * g * g;
-    m[idx] = mm;
-    v[idx] = vv;
-    float np = p - lr * (mm / bc1) / (sqrtf(vv / bc2) + eps) - decay * p;
-    master[idx] = np;
-    if (ch.shadow >= 0) shadow_base[ch.shadow + i] = from_f<T>(np);
+// Bound by DRAM: 26 bytes an element with a float copy only, 30 with a bf16 one.  16-byte accesses, the loads of two groups
+// before the first store, and evict-first hints: the optimiser's state is not read again before the next update, and the
+// weights and activations of a small batch stay in L2 (DeiT-S, one image: 732 -> 722 us a step).  Blocks walk the chunk
+// table, so that a launch of UPDATE_BESIDE blocks an SM moves data without taking the slots of the kernels it runs beside
+// (one block an SM leaves the update behind: ViT-B, 128 images 5826 -> 5926 us against 5860 with three);
+// alone the update gets UPDATE_ALONE blocks an SM.
+constexpr int UPDATE_BESIDE = 3, UPDATE_ALONE = 6;
+
+// A rule reads N values an element: parameter, gradient, and the optimiser's state, which it replaces.
+struct AdamRule {
+  static constexpr int N = 4;
+  float *p, *s0, *s1;
+  const float* g;
+  float lr, bc1, bc2, b1, b2, eps, wd;
+  __device__ __forceinline__ void operator()(float* x, bool decays) const {
+    x[2] = b1 * x[2] + (1.f - b1) * x[1];
+    x[3] = b2 * x[3] + (1.f - b2) * x[1] * x[1];
+    x[0] = x[0] - lr * (x[2] / bc1) / (sqrtf(x[3] / bc2) + eps) - (decays ? lr * wd : 0.f) * x[0];
+  }
+};
+
+// SGD with momentum: buf <- mu buf + (g + wd p), p <- p - lr buf.
+struct SgdRule {
+  static constexpr int N = 3;
+  float *p, *s0, *s1;
+  const float* g;
+  float lr, mu, wd;
+  __device__ __forceinline__ void operator()(float* x, bool decays) const {
+    x[2] = mu * x[2] + (x[1] + (decays ? wd : 0.f) * x[0]);
+    x[0] = x[0] - lr * x[2];
+  }
+};
+
+template <typename T, typename Rule>
+__device__ __forceinline__ void update_chunks(const AdamChunk* __restrict__ chunks, int nchunks, const Rule& rule, T* __restrict__ shadow_base) {
+  constexpr int U = 2;
+  float* const arr[4] = {rule.p, const_cast<float*>(rule.g), rule.s0, rule.s1};
+  for (int c = blockIdx.x; c < nchunks; c += gridDim.x) {
+    const AdamChunk ch = chunks[c];
+    const uint32_t full = ch.count & ~3u, pitch = blockDim.x * 4;
+    for (uint32_t i0 = threadIdx.x * 4; i0 < full; i0 += U * pitch) {
+      float4 x[U][Rule::N];
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (i0 + u * pitch < full)
+#pragma unroll
+          for (int a = 0; a < Rule::N; ++a) x[u][a] = __ldcs(reinterpret_cast<const float4*>(arr[a] + ch.offset + i0 + u * pitch));
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const uint32_t i = i0 + u * pitch;
+        if (i >= full) continue;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          float e[4];
+#pragma unroll
+          for (int a = 0; a < Rule::N; ++a) e[a] = reinterpret_cast<const float*>(&x[u][a])[j];
+          rule(e, ch.decay != 0);
+#pragma unroll
+          for (int a = 0; a < Rule::N; ++a) reinterpret_cast<float*>(&x[u][a])[j] = e[a];
+        }
+#pragma unroll
+        for (int a = 0; a < Rule::N; ++a)
+          if (a != 1) __stcs(reinterpret_cast<float4*>(arr[a] + ch.offset + i), x[u][a]);
+        if (ch.shadow >= 0) store4(shadow_base + ch.shadow + i, reinterpret_cast<const float*>(&x[u][0]));
+      }
+    }
+    for (uint32_t i = full + threadIdx.x; i < ch.count; i += blockDim.x) {
+      float e[4];
+#pragma unroll
+      for (int a = 0; a < Rule::N; ++a) e[a] = arr[a][(size_t)ch.offset + i];
+      rule(e, ch.decay != 0);
+#pragma unroll
+      for (int a = 0; a < Rule::N; ++a)
+        if (a != 1) arr[a][(size_t)ch.offset + i] = e[a];
+      if (ch.shadow >= 0) shadow_base[ch.shadow + i] = from_f<T>(e[0]);
+    }
   }
 }
 
-// SGD with momentum on the same chunk table: buf <- mu buf + (g + wd p), p <- p - lr buf.
+// Step-dependent scalars live in device memory so that a captured graph of the step stays valid: lr, 1-b1^t, 1-b2^t.
 template <typename T>
-__global__ void sgd_kernel(const AdamChunk* __restrict__ chunks, float* __restrict__ master, const float* __restrict__ grad,
-                           float* __restrict__ buf, T* __restrict__ shadow_base, const float* __restrict__ scalars, float mu,
-                           float wd) {
+__global__ void __launch_bounds__(256)
+adamw_kernel(const AdamChunk* chunks, int nchunks, AdamRule rule, T* shadow_base, const float* scalars) {
   dependent_sync();
-  float lr = scalars[0];
-  AdamChunk ch = chunks[blockIdx.x];
-  float decay = ch.decay ? wd : 0.f;
-  for (uint32_t i = threadIdx.x; i < ch.count; i += blockDim.x) {
-    size_t idx = (size_t)ch.offset + i;
-    float p = master[idx];
-    float b = mu * buf[idx] + (grad[idx] + decay * p);
-    buf[idx] = b;
-    float np = p - lr * b;
-    master[idx] = np;
-    if (ch.shadow >= 0) shadow_base[ch.shadow + i] = from_f<T>(np);
-  }
+  rule.lr = scalars[0];
+  rule.bc1 = scalars[1];
+  rule.bc2 = scalars[2];
+  update_chunks(chunks, nchunks, rule, shadow_base);
 }
 
-void sgd_momentum(const Ctx& c, const AdamChunk* chunks, int nchunks, float* master, const float* grad, float* buf,
+template <typename T>
+__global__ void __launch_bounds__(256)
+sgd_kernel(const AdamChunk* chunks, int nchunks, SgdRule rule, T* shadow_base, const float* scalars) {
+  dependent_sync();
+  rule.lr = scalars[0];
+  update_chunks(chunks, nchunks, rule, shadow_base);
+}
+
+static int update_blocks(const Ctx& c, int nchunks, bool beside) {
+  const int cap = (c.sm_count > 0 ? c.sm_count : B200_SMS) * (beside ? UPDATE_BESIDE : UPDATE_ALONE);
+  return nchunks < cap ? nchunks : cap;
+}
+
+void sgd_momentum(const Ctx& c, const AdamChunk* chunks, int nchunks, bool beside, float* master, const float* grad, float* buf,
                   void* shadow_base, const float* scalars, float mu, float wd) {
   if (nchunks <= 0) return;
   note_launch(1);
-  if (c.dtype == 0)
-    launch_k(sgd_kernel<float>, nchunks, 256, 0, c.stream, chunks, master, grad, buf, (float*)shadow_base, scalars, mu, wd);
-  else
-    launch_k(sgd_kernel<bf16>, nchunks, 256, 0, c.stream, chunks, master, grad, buf, (bf16*)shadow_base, scalars, mu, wd);
+  const int blocks = update_blocks(c, nchunks, beside);
+  const SgdRule rule = {master, buf, nullptr, grad, 0.f, mu, wd};
+  if (c.dtype == 0) launch_k(sgd_kernel<float>, blocks, 256, 0, c.stream, chunks, nchunks, rule, (float*)shadow_base, scalars);
+  else launch_k(sgd_kernel<bf16>, blocks, 256, 0, c.stream, chunks, nchunks, rule, (bf16*)shadow_base, scalars);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -871,14 +930,14 @@ void set_scalars(cudaStream_t s, float* dst, float a, float b, float c3) {
   launch_k(set_scalars_kernel, 1, 1, 0, s, dst, a, b, c3);
 }
 
-void adamw(const Ctx& c, const AdamChunk* chunks, int nchunks, float* master, const float* grad, float* m, float* v,
+void adamw(const Ctx& c, const AdamChunk* chunks, int nchunks, bool beside, float* master, const float* grad, float* m, float* v,
            void* shadow_base, const float* scalars, float b1, float b2, float eps, float wd) {
   if (nchunks <= 0) return;
   note_launch(1);
-  if (c.dtype == 0)
-    launch_k(adamw_kernel<float>, nchunks, 256, 0, c.stream, chunks, master, grad, m, v, (float*)shadow_base, scalars, b1, b2, eps, wd);
-  else
-    launch_k(adamw_kernel<bf16>, nchunks, 256, 0, c.stream, chunks, master, grad, m, v, (bf16*)shadow_base, scalars, b1, b2, eps, wd);
+  const int blocks = update_blocks(c, nchunks, beside);
+  const AdamRule rule = {master, m, v, grad, 0.f, 1.f, 1.f, b1, b2, eps, wd};
+  if (c.dtype == 0) launch_k(adamw_kernel<float>, blocks, 256, 0, c.stream, chunks, nchunks, rule, (float*)shadow_base, scalars);
+  else launch_k(adamw_kernel<bf16>, blocks, 256, 0, c.stream, chunks, nchunks, rule, (bf16*)shadow_base, scalars);
 }
 
 // ------------------------------------------------------------------------------------------------

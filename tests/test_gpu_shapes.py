@@ -158,3 +158,29 @@ def test_long_attention_forward_at_block_edges(B, T, H):
     assert rel(out, (s.softmax(-1) @ v).transpose(1, 2).reshape(B, T, H * 64)) < 6e-3
     assert rel(lse, s.logsumexp(-1)) < 1e-5
     assert rel(cp, s.softmax(-1)[:, :, 0, 1:]) < 2e-5
+
+
+@pytest.mark.parametrize("optimizer", ["adamw", "sgd"])
+@pytest.mark.parametrize("trainable", [(0, 5), (2, 4), (5,)])
+def test_updates_beside_the_backward_pass(trainable, optimizer):
+    """Blocks updated while the backward pass goes on (frozen blocks between them, a head of 7 classes whose bias is no
+    multiple of four) equal one update after it bit for bit: every parameter, over a direct and two replayed steps."""
+    import torch
+    from paper_2405_10951_b200 import binding as Bd
+    cfg = MINI.with_(trainable=trainable, optimizer=optimizer, num_classes=(7,))
+    images, labels, task_ids, params = synth.make_workload(cfg, peaked=False)
+    whole, split = Bd.Engine(cfg), Bd.Engine(cfg)
+    with torch.cuda.stream(torch.cuda.Stream()):
+        for e in (whole, split):
+            e.set_params(params)
+        img, lab = whole.images_to_device(images), torch.as_tensor(labels).cuda()
+        for _ in range(3):
+            whole.train_step(img, lab)
+            split.forward_backward(img, lab)
+            split.optimizer_step()
+        whole.sync_status()
+        split.sync_status()
+        for n, shape in synth.param_shapes(cfg).items():
+            assert torch.equal(whole.get_tensor(n, shape), split.get_tensor(n, shape)), n
+    whole.close()
+    split.close()
