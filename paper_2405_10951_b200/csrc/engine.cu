@@ -630,11 +630,12 @@ int block_forward(bsr_handle* h, const Ctx& c, int l, int B, const BlockBufs& bb
     MoeBufs mb = moe_bufs(h, bb);
     int cap = moe_rows_cap(Mf, E, K);
     // Gate logits of every task at once as one product y Wg^T ([Mf, D] x [D, tasks E]) on the tensor cores; they land in
-    // the expert-output buffer, which is not written before the routing has consumed them.  (Small or odd gate shapes:
-    // the routing kernel forms the logits itself.)
+    // the expert-output buffer, which is not written before the routing has consumed them.  (Odd gate shapes: the
+    // routing kernel forms the logits itself, which took 31 us for the 64 rows behind the last block's attention with 32
+    // gates, against 12 us for the product and the routing from its logits.)
     int NG = d.num_tasks * E;
     const float* logits = nullptr;
-    if (c.use_tc && d.dtype == BSR_DTYPE_BF16 && Mf >= 256 && NG % 8 == 0 && (size_t)Mf * NG <= (size_t)cap * D) {
+    if (c.use_tc && d.dtype == BSR_DTYPE_BF16 && NG % 8 == 0 && (size_t)Mf * NG <= (size_t)cap * D) {
       GemmEpilogue none;
       gemm(c, h->base + bb.y2, D, 1, h->wb(l, "moe.gate.weight"), D, 1, mb.og, 1, Mf, NG, D, none);
       logits = mb.og;
@@ -776,8 +777,11 @@ int block_backward(bsr_handle* h, const Ctx& c, int l, int B, GradStream dxo, Gr
     }
     int r3 = gemm_tc_grouped_rows(c, dzg, h->wb(l, "moe.fc1.weight"), 1, dxg, 0, cap, D, F, E, mb.tile_expert, none);
     if (r1 || r2 || r3 || r4) return set_err(h->err, BSR_ERR_CUDA, "grouped GEMM set-up failed (%d, %d, %d, %d)", r1, r2, r3, r4);
-    moe_gate_bwd(c, mb, dxg, dwsel, h->wb(l, "moe.gate.weight"), task_ids, tail ? 1 : Tf, d.num_tasks, Mf, D, E, K, dy,
-                 h->at<float>(h->off_m_dsel), pg ? h->gb(l, "moe.gate.weight") : nullptr);
+    moe_gate_bwd(c, mb, dxg, dwsel, h->wb(l, "moe.gate.weight"), task_ids, tail ? 1 : Tf, Mf, D, E, K, dy, h->at<float>(h->off_m_dsel));
+    if (pg) {
+      moe_gate_wgrad(lane_begin(), mb, h->at<float>(h->off_m_dsel), task_ids, tail ? 1 : Tf, d.num_tasks, D, E, h->gb(l, "moe.gate.weight"));
+      side_end(cl, 0);
+    }
   } else {
   // FFN second layer: dz = (dxo W2) * GELU'(z); dW2 = dxo^T h; db2 = column sums of dxo
   GemmEpilogue eg;

@@ -279,7 +279,9 @@ void moe_combine(const Ctx& c, const MoeBufs& b, const float* res, float* out, i
 void moe_combine_bwd(const Ctx& c, const MoeBufs& b, const float* dout, void* dog, float* dw, int M, int D, int E, int K);
 void moe_seg_colsum(const Ctx& c, const MoeBufs& b, const void* x, int cols, int E, float* out);
 void moe_gate_bwd(const Ctx& c, const MoeBufs& b, const void* dxg, const float* dw, const void* wg, const int* task_ids,
-                  int tokens_per_image, int tasks, int M, int D, int E, int K, void* dy, float* dsel_row, float* dwg);
+                  int tokens_per_image, int M, int D, int E, int K, void* dy, float* dsel_row);
+void moe_gate_wgrad(const Ctx& c, const MoeBufs& b, const float* dsel_row, const int* task_ids, int tokens_per_image, int tasks, int D,
+                    int E, float* dwg);
 
 // ---- guard words between workspace slices ------------------------------------------------------
 // table[i]: byte offset from base of guard i (words 32-bit values each).  guards_write fills them with `word`;

@@ -6,6 +6,8 @@
 // seg_start[e] .. seg_start[e] + count[e], padded with empty rows to a multiple of 128 so that a GEMM tile never
 // mixes experts.  Within an expert rows keep token order, and every reduction runs in row order: results do not
 // depend on scheduling.
+#include <cooperative_groups.h>
+
 #include "common.cuh"
 #include "kernels.h"
 
@@ -21,8 +23,7 @@ constexpr int MOE_ROUTE_TOKENS = 16;
 static_assert(MOE_BLOCK_TOKENS % MOE_ROUTE_TOKENS == 0, "a routing block must not straddle two counting groups");
 template <typename T>
 __global__ void __launch_bounds__(MOE_ROUTE_WARPS * 32)
-moe_route_kernel(const T* __restrict__ y, const T* __restrict__ wg, const float* __restrict__ logits, int logit_stride,
-                 const int* __restrict__ task_ids, int tokens_per_image, int M, int D, int E, int K, int gate_elems_in_smem,
+moe_route_kernel(const T* __restrict__ y, const T* __restrict__ wg, const int* __restrict__ task_ids, int tokens_per_image, int M, int D, int E, int K, int gate_elems_in_smem,
                  int* __restrict__ eidx, float* __restrict__ ew, int* __restrict__ blk_counts) {
   dependent_sync();
   // A block takes MOE_ROUTE_TOKENS consecutive tokens (a divisor of MOE_BLOCK_TOKENS, so all of them fall into one
@@ -32,14 +33,12 @@ moe_route_kernel(const T* __restrict__ y, const T* __restrict__ wg, const float*
   // in a fixed (butterfly) order; lane e keeps logit e.  The top k then come from k warp-wide maxima (among equal
   // logits the lowest expert id, found with a ballot).  Few registers, so many tokens are in flight per SM: the work
   // per token is a chain of dependent loads.  The per-group expert counts (zeroed before the launch) are integer sums.
-  // When `logits` is given (row stride logit_stride, the E logits of task t at column t E), the products were formed
-  // by a GEMM over all tasks' gates beforehand and lane e just reads its logit.
   extern __shared__ __align__(16) unsigned char route_smem[];
   __shared__ int counts[MOE_MAX_E];
   constexpr int N = Pack<T>::N;
   if (threadIdx.x < MOE_MAX_E) counts[threadIdx.x] = 0;
   const T* gates = wg;
-  if (logits == nullptr && gate_elems_in_smem > 0) {
+  if (gate_elems_in_smem > 0) {
     T* sg = reinterpret_cast<T*>(route_smem);
     for (int i = threadIdx.x * N; i < gate_elems_in_smem; i += blockDim.x * N)
       *reinterpret_cast<uint4*>(sg + i) = *reinterpret_cast<const uint4*>(wg + i);
@@ -56,9 +55,6 @@ moe_route_kernel(const T* __restrict__ y, const T* __restrict__ wg, const float*
     const T* yr = y + (size_t)tok * D;
     const T* gt = gates + (size_t)task * E * D;
     float logit = -INFINITY;                      // lane e: logit of expert e
-    if (logits != nullptr) {
-      if (lane < E) logit = logits[(size_t)tok * logit_stride + task * E + lane];
-    } else
 #pragma unroll 4
     for (int e = 0; e < E; ++e) {
       float acc = 0.f;
@@ -108,12 +104,75 @@ moe_route_kernel(const T* __restrict__ y, const T* __restrict__ wg, const float*
     atomicAdd(&blk_counts[(size_t)(blockIdx.x * MOE_ROUTE_TOKENS / MOE_BLOCK_TOKENS) * E + threadIdx.x], counts[threadIdx.x]);
 }
 
+// ---- the same from logits that a GEMM over all tasks' gates formed beforehand (row stride logit_stride, the E logits of
+// task t at column t E) -------------------------------------------------------------------------------------------------
+// A thread per token and a block per counting group: a token's logits are one or two cache lines, its top k need no other
+// lane, and the group's counts leave with plain stores, so that nothing has to be zeroed before.  Bound by latency
+// (6464 tokens, 16 experts: a warp per token, 16 tokens a block and a zeroing launch before took 11.7 us, this 5.7 us).
+__global__ void __launch_bounds__(MOE_BLOCK_TOKENS)
+moe_route_logits_kernel(const float* __restrict__ logits, int logit_stride, const int* __restrict__ task_ids, int tokens_per_image,
+                        int M, int E, int K, int* __restrict__ eidx, float* __restrict__ ew, int* __restrict__ blk_counts) {
+  __shared__ int counts[MOE_MAX_E];
+  if (threadIdx.x < MOE_MAX_E) counts[threadIdx.x] = 0;
+  dependent_sync();
+  __syncthreads();
+  const int tok = blockIdx.x * MOE_BLOCK_TOKENS + threadIdx.x;
+  if (tok < M) {
+    const int task = task_ids ? task_ids[tok / tokens_per_image] : 0;
+    const float* row = logits + (size_t)tok * logit_stride + task * E;
+    float lg[MOE_MAX_E];
+#pragma unroll
+    for (int e = 0; e < MOE_MAX_E; ++e) lg[e] = e < E ? row[e] : -INFINITY;
+    float sel[MOE_MAX_K];
+    int sid[MOE_MAX_K];
+    uint32_t open = E >= 32 ? 0xffffffffu : (1u << E) - 1u;
+#pragma unroll
+    for (int i = 0; i < MOE_MAX_K; ++i) {
+      if (i < K) {
+        float best = -INFINITY;
+#pragma unroll
+        for (int e = 0; e < MOE_MAX_E; ++e)
+          if ((open >> e) & 1u) best = fmaxf(best, lg[e]);
+        int bi = __ffs(open) - 1;                   // nothing compares equal (a NaN among the logits): lowest open id
+        float bv = 0.f;
+        bool found = false;
+#pragma unroll
+        for (int e = 0; e < MOE_MAX_E; ++e)         // the lowest id wins among equals
+          if (((open >> e) & 1u) && !found && lg[e] == best) { bi = e; found = true; }
+#pragma unroll
+        for (int e = 0; e < MOE_MAX_E; ++e) bv = e == bi ? lg[e] : bv;
+        sel[i] = bv;
+        sid[i] = bi;
+        open &= ~(1u << bi);
+      }
+    }
+    float den = 0.f;
+#pragma unroll
+    for (int i = 0; i < MOE_MAX_K; ++i)
+      if (i < K) den += expf(sel[i] - sel[0]);
+#pragma unroll
+    for (int i = 0; i < MOE_MAX_K; ++i) {
+      if (i < K) {
+        eidx[(size_t)tok * K + i] = sid[i];
+        ew[(size_t)tok * K + i] = expf(sel[i] - sel[0]) / den;
+        atomicAdd(&counts[sid[i]], 1);              // integer counts: order-independent
+      }
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < E) blk_counts[(size_t)blockIdx.x * E + threadIdx.x] = counts[threadIdx.x];
+}
+
 // ---- segment table and row assignment in one kernel ---------------------------------------------------------------
 // A block per group of MOE_BLOCK_TOKENS tokens.  Every block sums the per-group expert counts itself (a few KB): the
 // totals give the start of every expert's segment (padded to 128 rows), the counts of the groups before its own give
 // its place inside each segment.  Then the position of every (token, slot) inside its expert's segment, in token order.
-// Block 0 also publishes the segment starts and the expert of every 128-row tile for the grouped GEMMs.
-__global__ void __launch_bounds__(256)
+// Block 0 also publishes the segment starts and the expert of every 128-row tile for the grouped GEMMs; the empty rows of
+// an expert are marked by the block of the same number.
+// The group's entries are staged in shared memory beside the counts' loads: one trip to memory instead of one per 32
+// entries (with a warp per expert 12.6 -> 7.5 us for 6464 tokens and 16 experts, and the launch that emptied row_token before is gone).
+constexpr int MOE_ASSIGN_WARPS = 16;             // at least 128 threads: they mark an expert's empty rows at once
+__global__ void __launch_bounds__(MOE_ASSIGN_WARPS * 32)
 moe_assign_kernel(const int* __restrict__ eidx, const float* __restrict__ ew, const int* __restrict__ blk_counts, int nblk,
                   int tiles_cap, int M, int E, int K, int* __restrict__ seg_start, int* __restrict__ tile_expert,
                   int* __restrict__ pos, int* __restrict__ row_token, float* __restrict__ row_w) {
@@ -121,9 +180,14 @@ moe_assign_kernel(const int* __restrict__ eidx, const float* __restrict__ ew, co
   __shared__ int total[MOE_MAX_E];
   __shared__ int before[MOE_MAX_E];
   __shared__ int start[MOE_MAX_E + 1];
+  __shared__ int entry[MOE_BLOCK_TOKENS * MOE_MAX_K];
   int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int e = warp; e < E; e += 8) {
+  const int t0 = blockIdx.x * MOE_BLOCK_TOKENS;
+  const int n_entries = min(MOE_BLOCK_TOKENS, M - t0) * K;
+  for (int i = threadIdx.x; i < n_entries; i += blockDim.x) entry[i] = eidx[(size_t)t0 * K + i];
+  for (int e = warp; e < E; e += MOE_ASSIGN_WARPS) {
     int all = 0, pre = 0;
+#pragma unroll 4
     for (int g = lane; g < nblk; g += 32) {
       int cnt = blk_counts[(size_t)g * E + e];
       all += cnt;
@@ -134,13 +198,16 @@ moe_assign_kernel(const int* __restrict__ eidx, const float* __restrict__ ew, co
     if (lane == 0) { total[e] = all; before[e] = pre; }
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    int s = 0;
-    for (int i = 0; i < E; ++i) {
-      start[i] = s;
-      s += (total[i] + 127) & ~127;
+  if (warp == 0) {
+    const int rows = lane < E ? (total[lane] + 127) & ~127 : 0;
+    int s = rows;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      int below = __shfl_up_sync(0xffffffffu, s, o);
+      if (lane >= o) s += below;
     }
-    start[E] = s;
+    if (lane < E) start[lane + 1] = s;
+    if (lane == 0) start[0] = 0;
   }
   __syncthreads();
   if (blockIdx.x == 0) {
@@ -152,15 +219,17 @@ moe_assign_kernel(const int* __restrict__ eidx, const float* __restrict__ ew, co
       tile_expert[t] = ex;
     }
   }
-  int t0 = blockIdx.x * MOE_BLOCK_TOKENS;
-  int n_entries = min(MOE_BLOCK_TOKENS, M - t0) * K;
+  for (int e = blockIdx.x; e < E; e += gridDim.x) {
+    const int r = start[e] + total[e] + threadIdx.x;   // fewer than 128 rows
+    if (r < start[e + 1]) row_token[r] = -1;
+  }
   uint32_t lt = (1u << lane) - 1u;
-  for (int e = warp; e < E; e += 8) {
+  for (int e = warp; e < E; e += MOE_ASSIGN_WARPS) {
     int base = start[e] + before[e];
     int run = 0;
     for (int i0 = 0; i0 < n_entries; i0 += 32) {
       int i = i0 + lane;
-      bool hit = i < n_entries && eidx[(size_t)t0 * K + i] == e;
+      bool hit = i < n_entries && entry[i] == e;
       uint32_t m = __ballot_sync(0xffffffffu, hit);
       if (hit) {
         int r = base + run + __popc(m & lt);
@@ -237,39 +306,77 @@ __global__ void moe_combine_bwd_kernel(const float* __restrict__ dout, const flo
   if (lane == 0) dw[warp] = dot;
 }
 
-// ---- per-expert column sums (bias gradients): out[e][col] = sum over the expert's rows of x[r][col] -----------------
-template <typename T>
+// ---- sums over an expert's rows ----------------------------------------------------------------------------------------
+//   bias gradients:  out[e][col] = sum over expert e's rows of x[r][col]
+//   gate gradients (GATE):  out[task][e][col] = sum over expert e's rows of that task of dsel[r] * x[r][col]
+// Bound by the latency of the rows' loads: an expert's rows are split over the CTAs of a cluster (SEG_SPLIT) and over the
+// warps of each, a lane has the loads of SEG_U rows in flight, and the partial sums meet in shared memory, added in a fixed
+// order.  6464 tokens, 16 experts, top 2: one CTA an expert and one row in flight took 23 us (384 columns) for the bias and
+// 40 us for the gate gradient, this 11 and 12 us.
+constexpr int SEG_SPLIT = 8, SEG_U = 4;
+
+template <typename T, bool GATE>
 __global__ void __launch_bounds__(256)
-moe_seg_colsum_kernel(const T* __restrict__ x, const int* __restrict__ seg_start, int cols, float* __restrict__ out) {
+moe_seg_sum_kernel(const T* __restrict__ x, const float* __restrict__ dsel_row, const int* __restrict__ row_token,
+                   const int* __restrict__ seg_start, const int* __restrict__ task_ids, int tokens_per_image, int cols, int E,
+                   float* __restrict__ out) {
+  namespace cg = cooperative_groups;
   dependent_sync();
-  constexpr int N = Pack<T>::N;
-  __shared__ float sm[8][32 * N];
-  int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  int e = blockIdx.y;
-  int col0 = (blockIdx.x * 32 + tx) * N;
+  constexpr int N = Pack<T>::N, W = 32 * N;
+  __shared__ float sm[8][W];
+  __shared__ float part[W];
+  cg::cluster_group cluster = cg::this_cluster();
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int e = blockIdx.y, task = blockIdx.z / SEG_SPLIT, rank = blockIdx.z % SEG_SPLIT;
+  const int col0 = (blockIdx.x * 32 + tx) * N;
+  const int end = seg_start[e + 1];
   float acc[N];
 #pragma unroll
   for (int j = 0; j < N; ++j) acc[j] = 0.f;
   if (col0 < cols) {
-    for (int r = seg_start[e] + ty; r < seg_start[e + 1]; r += 8) {
-      float v[N];
-      load16(x + (size_t)r * cols + col0, v);
+    for (int r0 = seg_start[e] + rank * 8 + ty; r0 < end; r0 += SEG_U * SEG_SPLIT * 8) {
+      float w[SEG_U], v[SEG_U][N];
+      bool use[SEG_U];
 #pragma unroll
-      for (int j = 0; j < N; ++j) acc[j] += v[j];
+      for (int u = 0; u < SEG_U; ++u) {
+        const int r = r0 + u * SEG_SPLIT * 8;
+        use[u] = r < end;
+        w[u] = 1.f;
+        if constexpr (GATE) {
+          const int tok = use[u] ? row_token[r] : -1;
+          w[u] = use[u] ? dsel_row[r] : 0.f;
+          use[u] = tok >= 0 && (task_ids ? task_ids[tok / tokens_per_image] : 0) == task;
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < SEG_U; ++u)
+        if (use[u]) load16(x + (size_t)(r0 + u * SEG_SPLIT * 8) * cols + col0, v[u]);
+#pragma unroll
+      for (int u = 0; u < SEG_U; ++u)
+        if (use[u])
+#pragma unroll
+          for (int j = 0; j < N; ++j) acc[j] = GATE ? fmaf(w[u], v[u][j], acc[j]) : acc[j] + v[u][j];
     }
   }
 #pragma unroll
   for (int j = 0; j < N; ++j) sm[ty][tx * N + j] = acc[j];
   __syncthreads();
-  for (int c = threadIdx.x; c < 32 * N; c += blockDim.x) {
-    int col = blockIdx.x * 32 * N + c;
-    if (col < cols) {
-      float s = 0.f;
+  for (int c = threadIdx.x; c < W; c += blockDim.x) {
+    float s = 0.f;
 #pragma unroll
-      for (int w = 0; w < 8; ++w) s += sm[w][c];
-      out[(size_t)e * cols + col] = s;
-    }
+    for (int w = 0; w < 8; ++w) s += sm[w][c];
+    part[c] = s;
   }
+  cluster.sync();
+  constexpr int SHARE = W / SEG_SPLIT;                 // columns that each CTA of the cluster adds up
+  if (threadIdx.x < SHARE) {
+    const int c = rank * SHARE + threadIdx.x, col = blockIdx.x * W + c;
+    float s = 0.f;
+#pragma unroll
+    for (int q = 0; q < SEG_SPLIT; ++q) s += *cluster.map_shared_rank(&part[c], q);
+    if (col < cols) out[((size_t)task * E + e) * cols + col] = s;
+  }
+  cluster.sync();                                      // no CTA leaves while another may still read its partial sums
 }
 
 // ---- gate backward, token side: d(selected logits) and the gradient of the layer input -----------------------------
@@ -310,48 +417,6 @@ __global__ void moe_gate_bwd_kernel(const T* __restrict__ dxg, const float* __re
   }
 }
 
-// ---- gate backward, weight side: dWg[task][e] = sum over expert e's rows of that task of dsel[r] * xg[r] --------------
-template <typename T>
-__global__ void __launch_bounds__(256)
-moe_gate_wgrad_kernel(const T* __restrict__ xg, const float* __restrict__ dsel_row, const int* __restrict__ row_token,
-                      const int* __restrict__ seg_start, const int* __restrict__ task_ids, int tokens_per_image, int D, int E,
-                      float* __restrict__ dwg) {
-  dependent_sync();
-  constexpr int N = Pack<T>::N;
-  __shared__ float sm[8][32 * N];
-  int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  int e = blockIdx.y, task = blockIdx.z;
-  int col0 = (blockIdx.x * 32 + tx) * N;
-  float acc[N];
-#pragma unroll
-  for (int j = 0; j < N; ++j) acc[j] = 0.f;
-  if (col0 < D) {
-    for (int r = seg_start[e] + ty; r < seg_start[e + 1]; r += 8) {
-      int tok = row_token[r];
-      if (tok < 0) continue;
-      int tk = task_ids ? task_ids[tok / tokens_per_image] : 0;
-      if (tk != task) continue;
-      float c = dsel_row[r];
-      float v[N];
-      load16(xg + (size_t)r * D + col0, v);
-#pragma unroll
-      for (int j = 0; j < N; ++j) acc[j] = fmaf(c, v[j], acc[j]);
-    }
-  }
-#pragma unroll
-  for (int j = 0; j < N; ++j) sm[ty][tx * N + j] = acc[j];
-  __syncthreads();
-  for (int c = threadIdx.x; c < 32 * N; c += blockDim.x) {
-    int col = blockIdx.x * 32 * N + c;
-    if (col < D) {
-      float s = 0.f;
-#pragma unroll
-      for (int w = 0; w < 8; ++w) s += sm[w][c];
-      dwg[((size_t)task * E + e) * D + col] = s;
-    }
-  }
-}
-
 // =================================================================================================
 // launchers
 // =================================================================================================
@@ -363,24 +428,27 @@ void moe_route(const Ctx& c, const MoeBufs& b, const void* y, const void* wg, co
   int nblk = moe_blocks(M);
   int rows_cap = moe_rows_cap(M, E, K);
   note_launch(3);
-  size_t es = c.dtype == 0 ? 4 : 2;
-  size_t gate_elems = (size_t)(num_tasks < 1 ? 1 : num_tasks) * E * D;
-  size_t smem = gate_elems * es;
-  if (smem > 16 * 1024 || logits != nullptr) { smem = 0; gate_elems = 0; }       // not worth staging for 16 tokens: the gates are read through L1 instead
-  static SmemLimit lim[2];
-  int rblk = ceil_div(M, MOE_ROUTE_TOKENS);
-  cudaMemsetAsync(b.blk_counts, 0, (size_t)nblk * E * sizeof(int), c.stream);
-  if (c.dtype == 0) {
-    ensure_smem(lim[0], moe_route_kernel<float>, smem);
-    launch_k(moe_route_kernel<float>, rblk, MOE_ROUTE_WARPS * 32, smem, c.stream, (const float*)y, (const float*)wg, logits, logit_stride, task_ids, tokens_per_image, M, D, E, K,
-                                                                        (int)gate_elems, b.eidx, b.ew, b.blk_counts);
+  if (logits != nullptr) {
+    launch_k(moe_route_logits_kernel, nblk, MOE_BLOCK_TOKENS, 0, c.stream, logits, logit_stride, task_ids, tokens_per_image, M, E, K, b.eidx, b.ew, b.blk_counts);
   } else {
-    ensure_smem(lim[1], moe_route_kernel<bf16>, smem);
-    launch_k(moe_route_kernel<bf16>, rblk, MOE_ROUTE_WARPS * 32, smem, c.stream, (const bf16*)y, (const bf16*)wg, logits, logit_stride, task_ids, tokens_per_image, M, D, E, K,
-                                                                       (int)gate_elems, b.eidx, b.ew, b.blk_counts);
+    size_t es = c.dtype == 0 ? 4 : 2;
+    size_t gate_elems = (size_t)(num_tasks < 1 ? 1 : num_tasks) * E * D;
+    size_t smem = gate_elems * es;
+    if (smem > 16 * 1024) { smem = 0; gate_elems = 0; }       // not worth staging for 16 tokens: the gates are read through L1 instead
+    static SmemLimit lim[2];
+    int rblk = ceil_div(M, MOE_ROUTE_TOKENS);
+    cudaMemsetAsync(b.blk_counts, 0, (size_t)nblk * E * sizeof(int), c.stream);
+    if (c.dtype == 0) {
+      ensure_smem(lim[0], moe_route_kernel<float>, smem);
+      launch_k(moe_route_kernel<float>, rblk, MOE_ROUTE_WARPS * 32, smem, c.stream, (const float*)y, (const float*)wg, task_ids, tokens_per_image, M, D, E, K,
+               (int)gate_elems, b.eidx, b.ew, b.blk_counts);
+    } else {
+      ensure_smem(lim[1], moe_route_kernel<bf16>, smem);
+      launch_k(moe_route_kernel<bf16>, rblk, MOE_ROUTE_WARPS * 32, smem, c.stream, (const bf16*)y, (const bf16*)wg, task_ids, tokens_per_image, M, D, E, K,
+               (int)gate_elems, b.eidx, b.ew, b.blk_counts);
+    }
   }
-  cudaMemsetAsync(b.row_token, 0xFF, (size_t)rows_cap * sizeof(int), c.stream);
-  launch_k(moe_assign_kernel, nblk, 256, 0, c.stream, b.eidx, b.ew, b.blk_counts, nblk, rows_cap / 128, M, E, K, b.seg_start, b.tile_expert,
+  launch_k(moe_assign_kernel, nblk, MOE_ASSIGN_WARPS * 32, 0, c.stream, b.eidx, b.ew, b.blk_counts, nblk, rows_cap / 128, M, E, K, b.seg_start, b.tile_expert,
                                                 b.pos, b.row_token, b.row_w);
   int blocks = ceil_div((long)rows_cap * 32, 256);
   if (c.dtype == 0) launch_k(moe_gather_kernel<float>, blocks, 256, 0, c.stream, (const float*)y, b.row_token, b.seg_start, E, D, (float*)b.xg, rows_cap, M, c.status);
@@ -403,23 +471,33 @@ void moe_combine_bwd(const Ctx& c, const MoeBufs& b, const float* dout, void* do
     launch_k(moe_combine_bwd_kernel<bf16>, blocks, 256, 0, c.stream, dout, b.og, b.row_token, b.row_w, b.seg_start, E, D, (bf16*)dog, dw, rows_cap);
 }
 
-void moe_seg_colsum(const Ctx& c, const MoeBufs& b, const void* x, int cols, int E, float* out) {
+template <typename T, bool GATE>
+static void seg_sum(const Ctx& c, const void* x, const float* dsel_row, const MoeBufs& b, const int* task_ids, int tokens_per_image,
+                    int cols, int E, int tasks, float* out) {
   note_launch(1);
-  if (c.dtype == 0) launch_k(moe_seg_colsum_kernel<float>, dim3(ceil_div(cols, 128), E), 256, 0, c.stream, (const float*)x, b.seg_start, cols, out);
-  else launch_k(moe_seg_colsum_kernel<bf16>, dim3(ceil_div(cols, 256), E), 256, 0, c.stream, (const bf16*)x, b.seg_start, cols, out);
+  launch_cluster(moe_seg_sum_kernel<T, GATE>, dim3(ceil_div(cols, 32 * Pack<T>::N), E, tasks * SEG_SPLIT), 256, 0, c.stream, dim3(1, 1, SEG_SPLIT),
+                 (const T*)x, dsel_row, b.row_token, b.seg_start, task_ids, tokens_per_image, cols, E, out);
+}
+
+void moe_seg_colsum(const Ctx& c, const MoeBufs& b, const void* x, int cols, int E, float* out) {
+  if (c.dtype == 0) seg_sum<float, false>(c, x, nullptr, b, nullptr, 1, cols, E, 1, out);
+  else seg_sum<bf16, false>(c, x, nullptr, b, nullptr, 1, cols, E, 1, out);
+}
+
+void moe_gate_wgrad(const Ctx& c, const MoeBufs& b, const float* dsel_row, const int* task_ids, int tokens_per_image, int tasks, int D,
+                    int E, float* dwg) {
+  if (c.dtype == 0) seg_sum<float, true>(c, b.xg, dsel_row, b, task_ids, tokens_per_image, D, E, tasks, dwg);
+  else seg_sum<bf16, true>(c, b.xg, dsel_row, b, task_ids, tokens_per_image, D, E, tasks, dwg);
 }
 
 void moe_gate_bwd(const Ctx& c, const MoeBufs& b, const void* dxg, const float* dw, const void* wg, const int* task_ids,
-                  int tokens_per_image, int tasks, int M, int D, int E, int K, void* dy, float* dsel_row, float* dwg) {
-  note_launch(2);
+                  int tokens_per_image, int M, int D, int E, int K, void* dy, float* dsel_row) {
+  note_launch(1);
   int blocks = ceil_div((long)M * 32, 256);
-  if (c.dtype == 0) {
+  if (c.dtype == 0)
     launch_k(moe_gate_bwd_kernel<float>, blocks, 256, 0, c.stream, (const float*)dxg, dw, b.pos, b.eidx, b.ew, (const float*)wg, task_ids, tokens_per_image, M, D, E, K, (float*)dy, dsel_row);
-    if (dwg != nullptr) launch_k(moe_gate_wgrad_kernel<float>, dim3(ceil_div(D, 128), E, tasks), 256, 0, c.stream, (const float*)b.xg, dsel_row, b.row_token, b.seg_start, task_ids, tokens_per_image, D, E, dwg);
-  } else {
+  else
     launch_k(moe_gate_bwd_kernel<bf16>, blocks, 256, 0, c.stream, (const bf16*)dxg, dw, b.pos, b.eidx, b.ew, (const bf16*)wg, task_ids, tokens_per_image, M, D, E, K, (bf16*)dy, dsel_row);
-    if (dwg != nullptr) launch_k(moe_gate_wgrad_kernel<bf16>, dim3(ceil_div(D, 256), E, tasks), 256, 0, c.stream, (const bf16*)b.xg, dsel_row, b.row_token, b.seg_start, task_ids, tokens_per_image, D, E, dwg);
-  }
 }
 
 }  // namespace bsr

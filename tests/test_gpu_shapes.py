@@ -184,3 +184,14 @@ def test_updates_beside_the_backward_pass(trainable, optimizer):
             assert torch.equal(whole.get_tensor(n, shape), split.get_tensor(n, shape)), n
     whole.close()
     split.close()
+
+
+@pytest.mark.parametrize("experts,top_k,batch,classes", [(32, 4, 7, (10,)), (32, 1, 5, (10, 6)), (8, 3, 9, (10,)), (1, 1, 8, (5,) * 4)])
+def test_expert_routing_and_row_sums_at_their_limits(experts, top_k, batch, classes):
+    """One expert and the most, one slot and the most, token counts no multiple of a counting group, experts with fewer
+    rows than a cluster has row lanes and one with all of them; tolerance of every bf16 step."""
+    cfg = Config("mini_moe_shapes", 64, 8, 128, 2, 4, 256, classes, batch, (1, 2, 3), (1,), 7, 10, dtype="bf16", seed=4,
+                 moe_experts=experts, moe_top_k=top_k, moe_blocks=(0, 2))
+    images, labels, task_ids, params = synth.make_workload(cfg, peaked=False)
+    gpu = P.run_gpu_step(cfg, images, labels, task_ids, params)
+    P.compare_step(cfg, images, labels, task_ids, params, gpu, P.BF16_TOL, P.BF16_EXACT_MARGIN, P.BF16_SCORE_TOL)
