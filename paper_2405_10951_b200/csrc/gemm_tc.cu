@@ -280,49 +280,6 @@ __global__ void splitk_reduce_kernel(const float* __restrict__ partial, float* _
   *reinterpret_cast<float4*>(out + i) = acc;
 }
 
-// The same reduction followed by the epilogue the GEMM kernel would have applied (bias, GELU with optional copy of the
-// pre-activation, GELU derivative of a stored pre-activation, residual), for products whose few tiles are split along k.
-template <typename TOut>
-__global__ void splitk_reduce_epi_kernel(const float* __restrict__ partial, TOut* __restrict__ out, int m, int n, int splits, Epi ep) {
-  dependent_sync();
-  size_t total = (size_t)m * n;
-  size_t i = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) * 4;
-  if (i >= total) return;
-  float4 a4 = *reinterpret_cast<const float4*>(partial + i);
-  for (int s = 1; s < splits; ++s) {
-    float4 v = *reinterpret_cast<const float4*>(partial + (size_t)s * total + i);
-    a4.x += v.x; a4.y += v.y; a4.z += v.z; a4.w += v.w;
-  }
-  float v[4] = {a4.x, a4.y, a4.z, a4.w};
-  int col = (int)(i % (size_t)n);                    // n is a multiple of 4: the four values share a row
-  if (ep.bias != nullptr) {
-    float4 bb = *reinterpret_cast<const float4*>(ep.bias + col);
-    v[0] += bb.x; v[1] += bb.y; v[2] += bb.z; v[3] += bb.w;
-  }
-  if (ep.act == 1) {
-    if (ep.aux_out != nullptr) store4(reinterpret_cast<TOut*>(ep.aux_out) + i, v);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) v[j] = gelu_f(v[j]);
-  } else if (ep.act == 2) {
-    float z[4];
-    load4(reinterpret_cast<const bf16*>(ep.aux_in) + i, z);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) v[j] *= gelu_grad_f(z[j]);
-    if (ep.aux_out != nullptr) {            // GELU(z), recomputed for the weight gradient that follows
-#pragma unroll
-      for (int j = 0; j < 4; ++j) z[j] = gelu_f(z[j]);
-      store4(reinterpret_cast<bf16*>(ep.aux_out) + i, z);
-    }
-  }
-  if (ep.residual != nullptr) {
-    float r[4];
-    load4(reinterpret_cast<const TOut*>(ep.residual) + i, r);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) v[j] += r[j];
-  }
-  store4(out + i, v);
-}
-
 static EncodeFn lookup_encode_fn() {
   void* p = nullptr;
   cudaDriverEntryPointQueryResult q;
@@ -375,13 +332,13 @@ bool make_map_u8(CUtensorMap* map, const void* ptr, uint64_t inner, uint64_t out
 //   epilogue -- and a narrow tile has a short epilogue and room for more slabs in flight (200 x 1152 x 384: 12 CTAs of 192
 //   columns 5.7 us, 36 of 64 columns 4.6 us).
 // * More waves: 192 columns instead of 256 where that fills the last wave better.
-// * Splits (ws_floats > 0) and weight gradients: by estimated time in ns.  A slab costs its bytes at 126 per ns (64 a
+// * Weight gradients, split where there is a workspace (ws_floats > 0): by estimated time in ns.  A slab costs its bytes at 126 per ns (64 a
 //   clock), a tile 2.5 us to fill and drain; the second kernel costs 3 us and its traffic.
 struct Cut { int bn, splits; };
 static Cut choose_tile(int m, int n, int k, bool a_mn, size_t ws_floats, int sms) {
   const int tm = ceil_div(m, BM), kb = ceil_div(k, BK);
   auto tiles = [&](int bn) { return (long)tm * ceil_div(n, bn); };
-  if (a_mn || (ws_floats > 0 && kb >= 8 && tiles(256) * 2 <= sms)) {
+  if (a_mn) {
     Cut best = {BN_MAX, 1};
     double t_best = 1e30;
     for (int bn = BN_MAX; bn >= 128; bn -= 64)
@@ -440,27 +397,23 @@ int gemm_tc_strided(const Ctx& c, const void* A, long a_rs, long a_cs, const voi
   if (a_mn && (m % 8) != 0) return -1;
   if (a_mn && !b_mn) return -1;                 // combination not instantiated
   if (out_is_float && e.act != 0) return -1;    // activations belong to bf16 outputs
+  if (!a_mn) {
+    const int rc = gemm_tc_small(c, A, lda, B, ldb, b_mn, C, out_is_float, m, n, k, e);
+    if (rc != -1) return rc;
+  }
   CUtensorMap ma, mb;
   bool ok = a_mn ? make_map(&ma, A, (uint64_t)m, (uint64_t)k, (uint64_t)lda, BK) : make_map(&ma, A, (uint64_t)k, (uint64_t)m, (uint64_t)lda, BM);
   int sms = c.sm_count > 0 ? c.sm_count : 148;
   const bool plain = e.bias == nullptr && e.residual == nullptr && e.act == 0;
-  // split along k: weight gradients (plain float outputs) and the few-row products of the classification-only tail,
-  // whose epilogue then runs in the reduction
-  const bool may_split = split_ws != nullptr && ((out_is_float && plain) || (m <= 256 && (n % 4) == 0));
+  const bool may_split = split_ws != nullptr && out_is_float && plain;      // weight gradients
   const Cut cut = choose_tile(m, n, k, a_mn, may_split ? split_ws_floats : 0, sms);
   const int bn = cut.bn;
   ok = ok && (b_mn ? make_map(&mb, B, (uint64_t)n, (uint64_t)k, (uint64_t)ldb, BK) : make_map(&mb, B, (uint64_t)k, (uint64_t)n, (uint64_t)ldb, bn));
   if (!ok) return -2;
   const int tiles_m = ceil_div(m, BM), tiles_n = ceil_div(n, bn), total_kb = ceil_div(k, BK);
   const int kb_per_split = ceil_div(total_kb, cut.splits), splits = ceil_div(total_kb, kb_per_split);
-  Epi ep_full;
-  ep_full.bias = e.bias; ep_full.residual = e.residual; ep_full.aux_out = e.aux_out; ep_full.aux_in = e.aux_in; ep_full.act = e.act;
-  // split products write plain float partials; their epilogue runs in the reduction
-  const bool deferred = splits > 1 && !(out_is_float && plain);
-  Epi ep = ep_full;
-  if (splits > 1) { ep.bias = nullptr; ep.residual = nullptr; ep.aux_out = nullptr; ep.aux_in = nullptr; ep.act = 0; }
-  const int final_is_float = out_is_float;
-  if (splits > 1) out_is_float = 1;
+  Epi ep;
+  ep.bias = e.bias; ep.residual = e.residual; ep.aux_out = e.aux_out; ep.aux_in = e.aux_in; ep.act = e.act;
   void* dst = (splits > 1) ? (void*)split_ws : C;
   if (splits > 1) side_join(c, 2);         // the previous split sum has read the workspace
   if (c.prof != nullptr && c.prof->on) c.prof->begin(c.stream, 2.0 * m * n * (double)k);
@@ -478,16 +431,8 @@ int gemm_tc_strided(const Ctx& c, const void* A, long a_rs, long a_cs, const voi
      : bn == 128 ? run(std::integral_constant<int, 128>()) : run(std::integral_constant<int, 64>());
   if (rc != 0) return rc;
   if (splits > 1) {
-    size_t total = (size_t)m * n;
-    if (!deferred) {                       // a weight gradient: only the optimiser reads the sum
-      splitk_reduce(side_begin(c), split_ws, (float*)C, total, splits);
-      side_end(c, 2);
-    } else {
-      note_launch(1);
-      int blocks = ceil_div((long)(total / 4), 256);
-      if (final_is_float) launch_k(splitk_reduce_epi_kernel<float>, blocks, 256, 0, c.stream, split_ws, (float*)C, m, n, splits, ep_full);
-      else launch_k(splitk_reduce_epi_kernel<bf16>, blocks, 256, 0, c.stream, split_ws, (bf16*)C, m, n, splits, ep_full);
-    }
+    splitk_reduce(side_begin(c), split_ws, (float*)C, (size_t)m * n, splits);      // only the optimiser reads the sum
+    side_end(c, 2);
   }
   if (c.prof != nullptr && c.prof->on) c.prof->end(c.stream);
   return 0;

@@ -163,6 +163,9 @@ int gemm_tc_grouped_wgrad(const Ctx& c, const void* dY, const void* X, float* dW
 // The same on CTA pairs (tcgen05 cta_group::2, 256 x 256 tiles): A contiguous along k, no split.
 int gemm_tc2_strided(const Ctx& c, const void* A, long a_rs, long a_cs, const void* B, long b_rs, long b_cs, void* C,
                      int out_is_float, int m, int n, int k, const GemmEpilogue& e);
+// Products of few tiles (A along k; B along k, or along n when b_mn): k split over clusters.  -1: not a product for it.
+int gemm_tc_small(const Ctx& c, const void* A, long lda, const void* B, long ldb, int b_mn, void* C, int out_is_float, int m, int n, int k,
+                  const GemmEpilogue& e);
 void splitk_reduce(cudaStream_t s, const float* partial, float* out, size_t n, int splits);
 // Diagnostic: one CTA whose bounded wait expires after limit_ns and which then tears down as the GEMM kernels do.
 void wait_expiry_selftest(const Ctx& c, unsigned long long limit_ns);

@@ -195,3 +195,22 @@ def test_expert_routing_and_row_sums_at_their_limits(experts, top_k, batch, clas
     images, labels, task_ids, params = synth.make_workload(cfg, peaked=False)
     gpu = P.run_gpu_step(cfg, images, labels, task_ids, params)
     P.compare_step(cfg, images, labels, task_ids, params, gpu, P.BF16_TOL, P.BF16_EXACT_MARGIN, P.BF16_SCORE_TOL)
+
+
+@pytest.mark.parametrize("m,n,k", [(1, 768, 768), (7, 1152, 1152), (127, 776, 776), (129, 1160, 3080), (200, 768, 1600), (600, 1152, 3072), (1000, 1160, 1216)])
+def test_linear_split_over_clusters(m, n, k):
+    """Few-tile products whose reduction is split over 2, 4 and 8 CTAs: rows and columns past the last tile, shares of rows that do
+    not divide a tile, reductions that are no multiple of a slab; forward with bias, GELU and residual, and the input gradient."""
+    import torch
+    from paper_2405_10951_b200 import binding as Bd
+    gen = torch.Generator(device="cuda").manual_seed(m + n + k)
+    mk = lambda *s: torch.randn(*s, generator=gen, device="cuda").bfloat16()
+    x, w, dy, res, bias = mk(m, k), mk(n, k) / k ** 0.5, mk(m, n), mk(m, n), torch.randn(n, generator=gen, device="cuda")
+    rel = lambda a, b: float((a.double() - b).norm() / b.norm())
+    z = x.double() @ w.double().T + bias.double()
+    assert rel(Bd.bsr_linear_forward(x, w, bias, use_tensor_cores=True), z) < 4e-3
+    want = torch.nn.functional.gelu(z) + res.double()
+    assert rel(Bd.bsr_linear_forward(x, w, bias, res, act_gelu=True, use_tensor_cores=True), want) < 4e-3
+    if m % 8 == 0:
+        dx, _ = Bd.bsr_linear_backward(x, w, dy, use_tensor_cores=True)
+        assert rel(dx, dy.double() @ w.double()) < 4e-3
