@@ -108,7 +108,8 @@ moe_route_kernel(const T* __restrict__ y, const T* __restrict__ wg, const int* _
 // task t at column t E) -------------------------------------------------------------------------------------------------
 // A thread per token and a block per counting group: a token's logits are one or two cache lines, its top k need no other
 // lane, and the group's counts leave with plain stores, so that nothing has to be zeroed before.  Bound by latency
-// (6464 tokens, 16 experts: a warp per token, 16 tokens a block and a zeroing launch before took 11.7 us, this 5.7 us).
+// (16 experts, mean over the six layers of ViT-S with 64 images, 12608 tokens and fewer: a warp per token, 16 tokens a block
+// and a zeroing launch before took 11.7 us, this 5.7 us).
 __global__ void __launch_bounds__(MOE_BLOCK_TOKENS)
 moe_route_logits_kernel(const float* __restrict__ logits, int logit_stride, const int* __restrict__ task_ids, int tokens_per_image,
                         int M, int E, int K, int* __restrict__ eidx, float* __restrict__ ew, int* __restrict__ blk_counts) {
@@ -170,7 +171,7 @@ moe_route_logits_kernel(const float* __restrict__ logits, int logit_stride, cons
 // Block 0 also publishes the segment starts and the expert of every 128-row tile for the grouped GEMMs; the empty rows of
 // an expert are marked by the block of the same number.
 // The group's entries are staged in shared memory beside the counts' loads: one trip to memory instead of one per 32
-// entries (with a warp per expert 12.6 -> 7.5 us for 6464 tokens and 16 experts, and the launch that emptied row_token before is gone).
+// entries (with a warp per expert 12.6 -> 7.5 us in the same layers, and the launch that emptied row_token before is gone).
 constexpr int MOE_ASSIGN_WARPS = 16;             // at least 128 threads: they mark an expert's empty rows at once
 __global__ void __launch_bounds__(MOE_ASSIGN_WARPS * 32)
 moe_assign_kernel(const int* __restrict__ eidx, const float* __restrict__ ew, const int* __restrict__ blk_counts, int nblk,
@@ -311,8 +312,8 @@ __global__ void moe_combine_bwd_kernel(const float* __restrict__ dout, const flo
 //   gate gradients (GATE):  out[task][e][col] = sum over expert e's rows of that task of dsel[r] * x[r][col]
 // Bound by the latency of the rows' loads: an expert's rows are split over the CTAs of a cluster (SEG_SPLIT) and over the
 // warps of each, a lane has the loads of SEG_U rows in flight, and the partial sums meet in shared memory, added in a fixed
-// order.  6464 tokens, 16 experts, top 2: one CTA an expert and one row in flight took 23 us (384 columns) for the bias and
-// 40 us for the gate gradient, this 11 and 12 us.
+// order.  16 experts, top 2, mean over the two trained layers of ViT-S with 64 images: one CTA an expert and one row in
+// flight took 23 us for a bias and 40 us for the gate gradient, this 11 and 12 us.
 constexpr int SEG_SPLIT = 8, SEG_U = 4;
 
 template <typename T, bool GATE>
