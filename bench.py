@@ -67,7 +67,7 @@ def step_bytes(cfg, batch, fp):
 # (dram__bytes_read.sum + dram__bytes_write.sum of every gemm_tc_kernel launch of the step, divided by their number),
 # from the one-pass ncu launch lists summarised in profiles/launch_list_<workload>_step.txt, taken at the batch sizes
 # bench.py runs.  Absent (null in the output) for a workload whose list has not been taken on the kernel as it stands.
-GEMM_DRAM_BYTES_PER_LAUNCH = {"vit_b": 82660169, "deit_s": 15886456, "vit_b_384": 39582905}
+GEMM_DRAM_BYTES_PER_LAUNCH = {"vit_b": 82634556, "deit_s": 15844225, "moe_vit_s": 21736962}
 
 
 def peaks():
