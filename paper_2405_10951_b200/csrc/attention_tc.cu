@@ -65,6 +65,11 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
   __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<uint32_t*>(&h);
 }
+// Two floats as a pair of bf16 plus the pair that the rounding left.
+__device__ __forceinline__ void split_bf16x2(float a, float b, uint32_t& hi, uint32_t& lo) {
+  hi = pack_bf16x2(a, b);
+  lo = pack_bf16x2(a - __uint_as_float(hi << 16), b - __uint_as_float(hi & 0xffff0000u));
+}
 // Four neighbouring lanes hold a row of four 16-byte units each; afterwards lane j of them holds unit j of the four rows.
 // Stored so, an instruction writes 64 bytes of 8 rows instead of 16 bytes of 32 rows (197 tokens, batch 128, 12 heads: 59.1
 // -> 55.6 us).
@@ -1125,10 +1130,14 @@ attn_bwd_tc256_kernel(const __grid_constant__ CUtensorMap map_qkv, const __grid_
 //   KV = true : rows are keys.  S^T = K Q_i^T and dP^T = V dO_i^T, with lse and delta of the block's queries from shared
 //               memory; dV += P^T dO_i and dK += dS^T Q_i.
 // Either way the row operand of the second products is what the threads have just computed, so it goes back into tensor
-// memory (bf16, over the score columns its writer has consumed) and is read from there: nothing is transposed and
-// nothing passes through shared memory.  What bounds it is the chain product -> read -> exponential -> write -> product of
+// memory (over the score columns its writer has consumed) and is read from there: nothing is transposed and nothing passes
+// through shared memory.  P and dS stay 32-bit values in effect: each goes back as two bf16 numbers, the value rounded and
+// what the rounding left (2^-17 of the value is lost), in the columns that held the score, and both are multiplied: the
+// error of dQ, dK and dV against 64 bits is that of their rounding to bf16, 1.66e-3, as with fp32 P and dS (rounded to bf16
+// once they gave 2.35e-3).  What bounds it is the chain product -> read -> exponential -> write -> product of
 // one block; 256 tensor-memory columns and 66 KB of shared memory let two CTAs share an SM and overlap their chains.
-// 577 tokens, 12 heads: 450 us at batch 32, 128 us at batch 7, where the FP32-FMA kernels it replaces took 2.4 ms.
+// 577 tokens, 12 heads: 495 us at batch 32 and 141 at batch 7, 290 tokens at batch 32 161 us (429, 121 and 141 us with P and dS
+// rounded to bf16 once).
 // No step leaves a loop early: after a wait that expired the remaining steps only keep the barriers in step.
 // ------------------------------------------------------------------------------------------------
 constexpr int BL_COLS = 64;
@@ -1277,17 +1286,17 @@ attn_bwd_long_kernel(const __grid_constant__ CUtensorMap map_qkv, const __grid_c
 #pragma unroll
             for (int j = 0; j < 16; ++j) dsum = fmaf(p[j], dp[j], dsum);
           } else {
-            uint32_t pk[8];
+            uint32_t pk[16];
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
               const float d0 = KV ? stats[s & 1][1][cc + 2 * j] : dl, d1 = KV ? stats[s & 1][1][cc + 2 * j + 1] : dl;
-              pk[j] = pack_bf16x2(p[2 * j] * (dp[2 * j] - d0) * 0.125f, p[2 * j + 1] * (dp[2 * j + 1] - d1) * 0.125f);
+              split_bf16x2(p[2 * j] * (dp[2 * j] - d0) * 0.125f, p[2 * j + 1] * (dp[2 * j + 1] - d1) * 0.125f, pk[j], pk[8 + j]);
             }
-            tmem_st8(trow + C_DP + half * 32 + g * 8, pk);
+            tmem_st16(trow + C_DP + cc, pk);
             if (KV) {
 #pragma unroll
-              for (int j = 0; j < 8; ++j) pk[j] = pack_bf16x2(p[2 * j], p[2 * j + 1]);
-              tmem_st8(trow + C_S + half * 32 + g * 8, pk);
+              for (int j = 0; j < 8; ++j) split_bf16x2(p[2 * j], p[2 * j + 1], pk[j], pk[8 + j]);
+              tmem_st16(trow + C_S + cc, pk);
             }
           }
         }
@@ -1305,11 +1314,11 @@ attn_bwd_long_kernel(const __grid_constant__ CUtensorMap map_qkv, const __grid_c
     if (products && tid == 0 && ok && !abort_flag) {
       const uint32_t idesc = make_idesc_mn(AT_QROWS, AT_D, false, true);
       const bool first = KV ? s == 0 : s == nt;
-      for (int k = 0; k < cpad / 16; ++k)
-        umma_bf16_ts(tmem + C_A1, tmem + C_DP + (k >> 1) * 32 + (k & 1) * 8, make_desc(sC1 + k * 2048, 8192, 1024), idesc, (first && k == 0) ? 0u : 1u);
+      for (int i = 0; i < cpad / 8; ++i)                  // 16 columns of the block: their upper halves, then their lower ones
+        umma_bf16_ts(tmem + C_A1, tmem + C_DP + i * 8, make_desc(sC1 + (i >> 1) * 2048, 8192, 1024), idesc, (first && i == 0) ? 0u : 1u);
       if (KV)
-        for (int k = 0; k < cpad / 16; ++k)
-          umma_bf16_ts(tmem + C_A2, tmem + C_S + (k >> 1) * 32 + (k & 1) * 8, make_desc(sC2 + k * 2048, 8192, 1024), idesc, (first && k == 0) ? 0u : 1u);
+        for (int i = 0; i < cpad / 8; ++i)
+          umma_bf16_ts(tmem + C_A2, tmem + C_S + i * 8, make_desc(sC2 + (i >> 1) * 2048, 8192, 1024), idesc, (first && i == 0) ? 0u : 1u);
       umma_commit(p_bar);
     }
   }
@@ -1390,7 +1399,7 @@ int attention_bwd_tc(const Ctx& c, const void* qkv, const void* dout, const floa
   if (!make_map(&mq, qkv, (uint64_t)3 * H * d, (uint64_t)B * T, (uint64_t)3 * H * d, AT_BOX)) return -2;
   if (!make_map(&mg, dout, (uint64_t)H * d, (uint64_t)B * T, (uint64_t)H * d, AT_BOX)) return -2;
   // Up to 256 tokens the kernels below, which form every score once or twice instead of three times, are faster: 228 against
-  // 318 us at 197 tokens, 51 against 118 us at 100 (batch 128, 12 heads).
+  // 318 us at 197 tokens, 51 against 118 us at 100 (batch 128, 12 heads; the longer kernels then still with P and dS rounded once).
   if (T > 2 * AT_QROWS) {
     size_t smem_l = 1024 + 4 * 2 * (size_t)AT_BOX_BYTES + 64;
     static SmemLimit lim_q, lim_kv;

@@ -214,3 +214,39 @@ def test_linear_split_over_clusters(m, n, k):
     if m % 8 == 0:
         dx, _ = Bd.bsr_linear_backward(x, w, dy, use_tensor_cores=True)
         assert rel(dx, dy.double() @ w.double()) < 4e-3
+
+
+@pytest.mark.parametrize("scale,with_score_grad", [(0.3, True), (1.0, False), (2.0, True)])
+@pytest.mark.parametrize("B,T,H", [(2, 290, 3), (2, 577, 6)])
+def test_long_attention_backward_is_as_exact_as_fp32_probabilities(B, T, H, scale, with_score_grad):
+    """dQ, dK and dV beyond 256 tokens against 64 bits, beside the FP32-FMA kernels on the same inputs.  P and dS enter the products
+    with 16 bits of mantissa (2^-17 lost), which adds (2^-17 / 1.66e-3)^2 / 2 = 1e-5 of itself to the error that the rounding of
+    the outputs leaves; 1 % covers scores and sums in another order.  P and dS rounded to bf16 once give 1.4 times that error."""
+    import ctypes as C
+
+    import torch
+    from paper_2405_10951_b200 import binding as Bd
+    gen = torch.Generator(device="cuda").manual_seed(T + B)
+    qkv = (torch.randn(B, T, 3, H, 64, generator=gen, device="cuda") * scale).bfloat16()
+    do = torch.randn(B, T, H * 64, generator=gen, device="cuda").bfloat16()
+    sg = 3.0 * torch.randn(B, T - 1, generator=gen, device="cuda") if with_score_grad else None
+    q, k, v = (qkv[:, :, i].transpose(1, 2).double() for i in range(3))
+    s = q @ k.transpose(-1, -2) / 8.0
+    lse = s.logsumexp(-1)
+    prob, dov = (s - lse.unsqueeze(-1)).exp(), do.double().view(B, T, H, 64).transpose(1, 2)
+    dp = dov @ v.transpose(-1, -2)
+    if sg is not None:
+        dp[:, :, 0, 1:] += sg.double().unsqueeze(1) / H
+    ds = prob * (dp - (prob * dp).sum(-1, keepdim=True)) / 8.0
+    want = (ds @ k, ds.transpose(-1, -2) @ q, prob.transpose(-1, -2) @ dov)
+    lse32, delta, p = lse.float().contiguous(), torch.empty(B * H * T, device="cuda"), lambda t: None if t is None else C.c_void_p(t.data_ptr())
+    err = []
+    for mode in (0, 1):
+        out = torch.empty_like(qkv)
+        assert Bd.lib().bsr_attention_backward(p(qkv), p(do), p(lse32), p(sg), Bd.DTYPE_BF16, B, T, H, 64, p(out), p(delta), mode,
+                                               C.c_void_p(torch.cuda.current_stream().cuda_stream)) == Bd.BSR_OK
+        torch.cuda.synchronize()
+        got = out.permute(2, 0, 3, 1, 4).double()
+        err.append([float((got[i] - w).norm() / w.norm()) for i, w in enumerate(want)])
+    for name, fma, tensor in zip(("dq", "dk", "dv"), *err):
+        assert tensor <= 1.01 * fma, (name, fma, tensor)
