@@ -221,7 +221,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         tc_fence_after();
         return w;
       };
-      ok = epilogue_tile<TOut, FP8>(ready, ep, wk.bias_off, C + wk.c_off, M, N, mt * BM + quarter * 32, nt * BN + chalf * HALF_CHUNKS * 32, HALF_CHUNKS,
+      ok = epilogue_tile<TOut, FP8, (BN <= 128)>(ready, ep, wk.bias_off, C + wk.c_off, M, N, mt * BM + quarter * 32, nt * BN + chalf * HALF_CHUNKS * 32, HALF_CHUNKS,
                                     tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * BN + chalf * HALF_CHUNKS * 32),
                                     wk.kb0 >= wk.kb1, st, lane);
       if (!ok) break;
@@ -414,6 +414,7 @@ int gemm_tc_strided(const Ctx& c, const void* A, long a_rs, long a_cs, const voi
   const int kb_per_split = ceil_div(total_kb, cut.splits), splits = ceil_div(total_kb, kb_per_split);
   Epi ep;
   ep.bias = e.bias; ep.residual = e.residual; ep.aux_out = e.aux_out; ep.aux_in = e.aux_in; ep.act = e.act;
+  ep.exact = exact_gelu(m, k);             // (tiles of 64 or 128 columns up to 9472 of them)
   void* dst = (splits > 1) ? (void*)split_ws : C;
   if (splits > 1) side_join(c, 2);         // the previous split sum has read the workspace
   if (c.prof != nullptr && c.prof->on) c.prof->begin(c.stream, 2.0 * m * n * (double)k);

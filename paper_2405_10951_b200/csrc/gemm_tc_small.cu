@@ -177,11 +177,21 @@ gemm_tc_small_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
     v[0] += bias.x; v[1] += bias.y; v[2] += bias.z; v[3] += bias.w;
     if (ep.act == 1) {
       if (ep.aux_out != nullptr) store4(reinterpret_cast<TOut*>(ep.aux_out) + at(r0 + local), v);
-      gelu_fast2(v[0], v[1]);
-      gelu_fast2(v[2], v[3]);
+      if (ep.exact) {
+        gelu_exact2(v[0], v[1]);
+        gelu_exact2(v[2], v[3]);
+      } else {
+        gelu_fast2(v[0], v[1]);
+        gelu_fast2(v[2], v[3]);
+      }
     } else if (ep.act == 2) {
-      gelu_grad_mul2h(v[0], v[1], z[p][0], z[p][1], z[p][0], z[p][1]);
-      gelu_grad_mul2h(v[2], v[3], z[p][2], z[p][3], z[p][2], z[p][3]);
+      if (ep.exact) {
+        gelu_grad_exact2(v[0], v[1], z[p][0], z[p][1]);
+        gelu_grad_exact2(v[2], v[3], z[p][2], z[p][3]);
+      } else {
+        gelu_grad_mul2h(v[0], v[1], z[p][0], z[p][1], z[p][0], z[p][1]);
+        gelu_grad_mul2h(v[2], v[3], z[p][2], z[p][3], z[p][2], z[p][3]);
+      }
       if (ep.aux_out != nullptr) store4(reinterpret_cast<bf16*>(ep.aux_out) + at(r0 + local), z[p]);
     }
     if (ep.residual != nullptr) { v[0] += res[p][0]; v[1] += res[p][1]; v[2] += res[p][2]; v[3] += res[p][3]; }
@@ -233,6 +243,7 @@ int gemm_tc_small(const Ctx& c, const void* A, long lda, const void* B, long ldb
   if (!(b_mn ? make_map(&mb, B, (uint64_t)n, (uint64_t)k, (uint64_t)ldb, BK) : make_map(&mb, B, (uint64_t)k, (uint64_t)n, (uint64_t)ldb, BN))) return -2;
   Epi ep;
   ep.bias = e.bias; ep.residual = e.residual; ep.aux_out = e.aux_out; ep.aux_in = e.aux_in; ep.act = e.act;
+  ep.exact = exact_gelu(m, k);
   const bool timed = c.prof != nullptr && c.prof->on;
   if (timed) c.prof->begin(c.stream, 2.0 * m * n * (double)k);
   const int rc = out_is_float ? (b_mn ? launch<true, float>(c, ma, mb, C, m, n, k, ep, splits) : launch<false, float>(c, ma, mb, C, m, n, k, ep, splits))

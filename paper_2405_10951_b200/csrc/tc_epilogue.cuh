@@ -15,6 +15,7 @@ struct Epi {
   void* aux_out = nullptr;
   const void* aux_in = nullptr;
   int act = 0;
+  bool exact = false;              // activation to fp32 precision: see exact_gelu
   // operands quantised with one scale per row of A and per row of B (8-bit floating point): the accumulator of
   // (row, col) is multiplied by row_scale[row] * col_scale[col] before the bias
   const float* row_scale = nullptr;
@@ -96,6 +97,54 @@ __device__ __forceinline__ void gelu_grad_mul2h(float& g0, float& g1, float z0, 
   h0 = z0 * p0; h1 = z1 * p1;
   g0 *= fmaf(d0, e0, p0);
   g1 *= fmaf(d1, e1, p1);
+}
+
+// The polynomial above is off by up to 4e-6 of Phi, which near z = -4 is a tenth of GELU itself and twenty times its rounding to
+// bf16.  The classification rows of the last block and other products of few rows and a long reduction take GELU and its
+// derivative to 7e-6 of their values: Phi(-t) = exp(-t^2 / 2) R(t), R a polynomial of degree 11 in 2 t / 5.75 - 1 fitted to
+// erfc(t / sqrt 2) exp(t^2 / 2) / 2 in double precision on 0 <= t <= 5.75 (relative error 6e-6; beyond, Phi(-t) < 5e-9 and too large
+// by less than t / 5.75).  At many rows its exponential would be felt (25216 x 3072 x 768: GELU already adds 11 us to 75); with
+// few a launch waits for its operands (128 x 3072 x 768: 6.5 -> 6.9 us; erff and expf 7.4).
+inline bool exact_gelu(int m, int k) { return m <= 256 && k > 448; }
+// z <- Phi(z) of two values; e = exp(-z^2 / 2).
+__device__ __forceinline__ void phi_exact2(float& z0, float& z1, float& e0, float& e1) {
+  float u0, u1, p0, p1;
+  uint64_t z = pack2(z0, z1);
+  unpack2(mul2(z, z), u0, u1);
+  const float kh = -0.5f * 1.4426950408889634f;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e0) : "f"(u0 * kh));
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e1) : "f"(u1 * kh));
+  const uint64_t x = fma2(pack2(fminf(fabsf(z0), 5.75f), fminf(fabsf(z1), 5.75f)), dup2(2.0f / 5.75f), dup2(-1.0f));
+  uint64_t r = dup2(-0.003139214925281772f);
+  r = fma2(r, x, dup2(0.006516454073486045f));
+  r = fma2(r, x, dup2(-0.0026901766723877356f));
+  r = fma2(r, x, dup2(0.0023635298203356254f));
+  r = fma2(r, x, dup2(-0.01276389393510076f));
+  r = fma2(r, x, dup2(0.022197755375759323f));
+  r = fma2(r, x, dup2(-0.02989035800599237f));
+  r = fma2(r, x, dup2(0.04333526234265012f));
+  r = fma2(r, x, dup2(-0.06198110430277863f));
+  r = fma2(r, x, dup2(0.08334893928193564f));
+  r = fma2(r, x, dup2(-0.10580940246565074f));
+  r = fma2(r, x, dup2(0.12596105591795748f));
+  unpack2(mul2(r, pack2(e0, e1)), p0, p1);
+  z0 = z0 < 0.0f ? p0 : 1.0f - p0;
+  z1 = z1 < 0.0f ? p1 : 1.0f - p1;
+}
+__device__ __forceinline__ void gelu_exact2(float& z0, float& z1) {
+  float p0 = z0, p1 = z1, e0, e1;
+  phi_exact2(p0, p1, e0, e1);
+  z0 *= p0;
+  z1 *= p1;
+}
+// g <- g * GELU'(z), z <- GELU(z), two values.
+__device__ __forceinline__ void gelu_grad_exact2(float& g0, float& g1, float& z0, float& z1) {
+  float p0 = z0, p1 = z1, e0, e1;
+  phi_exact2(p0, p1, e0, e1);
+  g0 *= fmaf(z0 * 0.39894228040143268f, e0, p0);
+  g1 *= fmaf(z1 * 0.39894228040143268f, e1, p1);
+  z0 *= p0;
+  z1 *= p1;
 }
 
 // 16-byte global load of data that is read once (residual stream, stored pre-activations).
@@ -187,7 +236,8 @@ template <> __device__ __forceinline__ uint4 ChunkIO<bf16>::pack(const float* f)
 // v[j]: accumulator of (row0 + lane, col0 + j).  All lanes of the warp take part (row0, col0 are warp-uniform).
 // z: the chunk of the stored pre-activation for act == 2, already in this lane's row order (overwritten).
 // sbias, scol: the chunk's 32 bias values and column scales in shared memory (null: none), rs: this lane's row scale.
-template <typename TOut>
+// EXACT: the kernel is one that ep.exact may ask for the exact activation.
+template <typename TOut, bool EXACT>
 __device__ __forceinline__ void epilogue_chunk(const uint32_t* r, const Epi& ep, const float* sbias, const float* scol, float rs, TOut* Cs, int M,
                                                int N, int row0, int col0, unsigned char* st, int lane, float* z) {
   if (row0 < M && col0 < N) {
@@ -210,10 +260,19 @@ __device__ __forceinline__ void epilogue_chunk(const uint32_t* r, const Epi& ep,
     }
     if (ep.act == 1) {
       if (ep.aux_out != nullptr) ChunkIO<TOut>::store((TOut*)ep.aux_out, N, row0, col0, M, N, st, lane, v);
+      if (EXACT && ep.exact) {
 #pragma unroll
-      for (int j = 0; j < 32; j += 2) gelu_fast2(v[j], v[j + 1]);
+        for (int j = 0; j < 32; j += 2) gelu_exact2(v[j], v[j + 1]);
+      } else {
+#pragma unroll
+        for (int j = 0; j < 32; j += 2) gelu_fast2(v[j], v[j + 1]);
+      }
     } else if (ep.act == 2) {
-      if (ep.aux_out != nullptr) {          // GELU(z) recomputed for the weight gradient of the second FFN layer
+      if (EXACT && ep.exact) {
+#pragma unroll
+        for (int j = 0; j < 32; j += 2) gelu_grad_exact2(v[j], v[j + 1], z[j], z[j + 1]);
+        if (ep.aux_out != nullptr) ChunkIO<bf16>::store((bf16*)ep.aux_out, N, row0, col0, M, N, st, lane, z);
+      } else if (ep.aux_out != nullptr) {   // GELU(z) recomputed for the weight gradient of the second FFN layer
 #pragma unroll
         for (int j = 0; j < 32; j += 2) gelu_grad_mul2h(v[j], v[j + 1], z[j], z[j + 1], z[j], z[j + 1]);
         ChunkIO<bf16>::store((bf16*)ep.aux_out, N, row0, col0, M, N, st, lane, z);
@@ -298,7 +357,7 @@ __device__ __forceinline__ void chunk_land_bf16(const uint4* x, unsigned char* s
 // are added, they came from L2 -- the operand ring leaves hardly any L1 -- and took 900 of the 1700 clocks of a chunk) and
 // the first chunk of the residual or of the stored pre-activation, whose next chunk is always on its way.
 // empty: no products were accumulated (an expert without tokens): the result is zero.  st: this warp's staging buffer, 4 KB.
-template <typename TOut, bool FP8, typename Ready>
+template <typename TOut, bool FP8, bool EXACT, typename Ready>
 __device__ __forceinline__ bool epilogue_tile(Ready ready, const Epi& ep, int bias_off, TOut* Cs, int M, int N, int row0, int cb, int nc, uint32_t taddr,
                                               bool empty, unsigned char* st, int lane) {
   const float* bias = ep.bias == nullptr ? nullptr : ep.bias + bias_off;
@@ -354,7 +413,7 @@ __device__ __forceinline__ bool epilogue_tile(Ready ready, const Epi& ep, int bi
       uint32_t r[32];
       tmem_ld32(taddr + cc * 32, r);
       tmem_ld_wait();
-      epilogue_chunk<TOut>(r, ep, bias != nullptr ? sbias + cc * 32 : nullptr, FP8 ? sbias + 128 + cc * 32 : nullptr, rs, Cs, M, N, row0, cb + cc * 32, st,
+      epilogue_chunk<TOut, EXACT>(r, ep, bias != nullptr ? sbias + cc * 32 : nullptr, FP8 ? sbias + 128 + cc * 32 : nullptr, rs, Cs, M, N, row0, cb + cc * 32, st,
                            lane, z);
     }
   }

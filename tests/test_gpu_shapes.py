@@ -250,3 +250,20 @@ def test_long_attention_backward_is_as_exact_as_fp32_probabilities(B, T, H, scal
         err.append([float((got[i] - w).norm() / w.norm()) for i, w in enumerate(want)])
     for name, fma, tensor in zip(("dq", "dk", "dv"), *err):
         assert tensor <= 1.01 * fma, (name, fma, tensor)
+
+
+@pytest.mark.parametrize("m,n,k", [(1, 3072, 768), (7, 1536, 768), (128, 3072, 768), (200, 5000, 520), (256, 384, 1536)])
+@pytest.mark.parametrize("bias", [0.0, -3.0, -3.8])
+def test_gelu_of_few_row_products_is_exact(m, n, k, bias):
+    """GELU where products of few rows and a long reduction apply it, down to the tail where a polynomial for Phi fails: nothing but
+    the rounding of the outputs, at most 2^-9 of each (and fp32 sums, a hundredth of that)."""
+    import torch
+    from paper_2405_10951_b200 import binding as Bd
+    gen = torch.Generator(device="cuda").manual_seed(m + n)
+    x = torch.randn(m, k, generator=gen, device="cuda").bfloat16()
+    w = (0.02 * torch.randn(n, k, generator=gen, device="cuda")).bfloat16()
+    b = torch.full((n,), bias, device="cuda")
+    z = x.double() @ w.double().T + b.double()
+    want = 0.5 * z * torch.special.erfc(-z / 2 ** 0.5)
+    got = Bd.bsr_linear_forward(x, w, b, act_gelu=True, use_tensor_cores=True).double()
+    assert float((got - want).norm() / want.norm()) < 1.01 * 2 ** -9
