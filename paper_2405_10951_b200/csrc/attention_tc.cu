@@ -1393,7 +1393,8 @@ namespace bsr {
 int attention_bwd_tc(const Ctx& c, const void* qkv, const void* dout, const float* lse, const float* cls_extra, float* delta,
                      void* dqkv, int B, int T, int H, int d) {
   using namespace tc;
-  if (c.dtype != 1 || d != AT_D || T < 1 || (T > 2 * AT_QROWS && delta == nullptr) || (long)B * H > 65535) return -1;
+  if (c.dtype != 1 || d != AT_D || T < 1) return -1;
+  if (T > 2 * AT_QROWS && (delta == nullptr || (long)B * H > 65535)) return -1;      // there (image, head) is the grid's second dimension
   if (((uintptr_t)qkv & 15) || ((uintptr_t)dout & 15) || ((uintptr_t)dqkv & 15)) return -1;
   CUtensorMap mq, mg;
   if (!make_map(&mq, qkv, (uint64_t)3 * H * d, (uint64_t)B * T, (uint64_t)3 * H * d, AT_BOX)) return -2;

@@ -267,3 +267,26 @@ def test_gelu_of_few_row_products_is_exact(m, n, k, bias):
     want = 0.5 * z * torch.special.erfc(-z / 2 ** 0.5)
     got = Bd.bsr_linear_forward(x, w, b, act_gelu=True, use_tensor_cores=True).double()
     assert float((got - want).norm() / want.norm()) < 1.01 * 2 ** -9
+
+
+def test_attention_backward_of_more_pairs_than_a_grid_dimension():
+    """Up to 256 tokens the tensor-core kernels take any number of (image, head) pairs: 65544 of them, bit for bit as in small batches."""
+    import ctypes as C
+
+    import torch
+    from paper_2405_10951_b200 import binding as Bd
+    B, T, H = 5462, 5, 12
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    qkv = torch.randn(B, T, 3, H, 64, generator=gen, device="cuda").bfloat16()
+    do = torch.randn(B, T, H * 64, generator=gen, device="cuda").bfloat16()
+    _, _, lse = Bd.bsr_attention_forward(qkv, H, use_tensor_cores=True, want_lse=True)
+    p = lambda t: C.c_void_p(t.data_ptr())
+
+    def backward(a, b):
+        out = torch.empty_like(qkv[a:b])
+        rc = Bd.lib().bsr_attention_backward(p(qkv[a:b]), p(do[a:b]), p(lse[a:b]), None, Bd.DTYPE_BF16, b - a, T, H, 64, p(out), None, 1,
+                                             C.c_void_p(torch.cuda.current_stream().cuda_stream))
+        assert rc == Bd.BSR_OK
+        return out
+    whole = backward(0, B)
+    assert torch.equal(whole[:7], backward(0, 7)) and torch.equal(whole[-7:], backward(B - 7, B))
