@@ -256,10 +256,12 @@ int32_t bsr_set_gemm_mode(bsr_handle* h, int32_t mode);
 /* bsr_train_step replays a captured CUDA graph of its ~200 launches (unless the caller is capturing `stream`): the first
  * call with a given set of pointers and batch enqueues its kernels one by one, the second captures them, later calls
  * with the same arguments replay the graph.  The key of a captured graph is (images, labels, task ids, loss and
- * kept-index pointers, batch, kernel mode); the handle keeps the eight most recently used graphs, so an input pipeline
- * should rotate through at most eight sets of buffers (bsr_profile.graph_captures counts captures: it stops growing once
- * a pipeline fits).  bsr_eval_forward does the same with a graph per batch size, whatever the pointers.  on = 0 turns this
- * off (every call enqueues its kernels one by one); the results are identical.  No counterpart in the paper. */
+ * kept-index pointers, batch, kernel mode); the handle keeps eight graphs, so an input pipeline should rotate through
+ * at most eight sets of buffers.  With more, the calls that find no graph enqueue their kernels one by one; a graph gives
+ * way to a new key only after 256 calls without it (bsr_profile.graph_captures counts captures: it stops growing).
+ * bsr_eval_forward does the same with a graph per batch size, whatever the pointers: eight batch sizes, besides the
+ * graphs of the steps.  on = 0 turns this off (every call enqueues its kernels one by one); the results are
+ * identical.  No counterpart in the paper. */
 int32_t bsr_set_graph_mode(bsr_handle* h, int32_t on);
 
 /* Measurement support (no counterpart in the paper).  bsr_profile_enable resets the counters; with
@@ -273,7 +275,7 @@ typedef struct {
   uint64_t gemm_launches;
   double gemm_flops;
   double gemm_ms;
-  uint64_t graph_captures;          /* training-step graphs captured by this handle since it was created */
+  uint64_t graph_captures;          /* graphs (steps and inference) captured by this handle since it was created */
 } bsr_profile;
 int32_t bsr_profile_enable(bsr_handle* h, int32_t time_gemms);
 int32_t bsr_profile_read(bsr_handle* h, void* stream, bsr_profile* out_host);

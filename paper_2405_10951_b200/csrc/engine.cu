@@ -180,18 +180,24 @@ struct bsr_handle {
   GemmProfile prof;
   // Captured graphs.  The key is everything a captured launch has baked in: the caller's pointers, the batch, the kernel
   // mode and which path it is (a training step, a step of the multi-step loop, forward and backward alone; inference bakes
-  // in no caller's pointer: those go through EvalIo).  Up to GRAPH_CACHE graphs of either kind are kept; the least
-  // recently used one is dropped.  A key is captured when it comes round the second time (`seen`): a first pass, or an input
-  // pipeline that never returns to a buffer, does not pay for a graph it will not replay (a first DeiT-S step at batch 64
-  // took 2.93 ms with the capture in it).
+  // in no caller's pointer: those go through EvalIo).  A key is captured when it comes round the second time (`seen`): a first
+  // pass, or an input pipeline that never returns to a buffer, does not pay for a graph it will not replay (a first DeiT-S step
+  // at batch 64 took 2.93 ms with the capture in it).  Up to GRAPH_CACHE graphs of either kind are kept.  A caller that goes round
+  // more keys than that replays the graphs there are and enqueues the rest: a graph gives way, to a key that has come round
+  // twice, only after GRAPH_IDLE calls without it, so that captures stay rare whatever the order of the keys (DeiT-S, 16
+  // images, nine sets of buffers in turn: 907 us a step; 2461 with the least recently used graph evicted on every miss, which
+  // captured on every call).
   struct StepGraph { const void* images; const void* labels; const void* tasks; void* loss; void* kept; int batch; int mode; int loop;
                      cudaGraphExec_t exec; long launches; uint64_t last_use; };
-  static constexpr size_t GRAPH_CACHE = 8;
-  std::vector<StepGraph> graphs, eval_graphs;
-  std::vector<StepGraph> seen;
+  static constexpr size_t GRAPH_CACHE = 8, GRAPH_SEEN = 4 * GRAPH_CACHE;
+  static constexpr uint64_t GRAPH_IDLE = 32 * GRAPH_CACHE;
+  struct GraphSet {
+    std::vector<StepGraph> graphs, seen;
+    uint64_t calls = 0;
+  };
+  GraphSet step_graphs, eval_graphs;
   cudaStream_t capture_stream = nullptr;   // graphs are captured here, whatever stream they are replayed on
-  uint64_t graph_clock = 0;
-  uint64_t graph_captures = 0;        // how many times a step was captured (a pipeline that cycles through more buffers than the cache holds re-captures every step)
+  uint64_t graph_captures = 0;        // how many graphs were captured, of either kind
   int use_graph = 1;
   // multi-step loop and host-buffer step
   // E4M3 copies of the QKV and first-FFN weights of the dense blocks before t0 (frozen_fp8), with a scale per row
@@ -1047,8 +1053,8 @@ int32_t bsr_create(const bsr_config* cfg, void* workspace, size_t bytes, bsr_han
 int32_t bsr_destroy(bsr_handle* h) {
   if (h != nullptr) {
     for (cudaEvent_t ev : h->prof.events) cudaEventDestroy(ev);
-    for (auto& g : h->graphs) cudaGraphExecDestroy(g.exec);
-    for (auto& g : h->eval_graphs) cudaGraphExecDestroy(g.exec);
+    for (auto* set : {&h->step_graphs, &h->eval_graphs})
+      for (auto& g : set->graphs) cudaGraphExecDestroy(g.exec);
     if (h->capture_stream) cudaStreamDestroy(h->capture_stream);
     for (int i = 0; i < 2; ++i) {
       if (h->ev_copied[i]) cudaEventDestroy(h->ev_copied[i]);
@@ -1248,11 +1254,11 @@ static int enqueue_train_step(bsr_handle* h, const void* images, const int32_t* 
 
 // Runs `enqueue(stream)` (which puts one step's kernels on a stream) either directly or, when the caller's stream is not
 // itself being captured and no per-launch events are asked for, as a CUDA graph that is captured the second time its key
-// comes round and replayed from then on.  at_once: the caller knows that the key will come round again.
+// comes round and replayed from then on, as far as the set has room.  at_once: the caller replays the graph itself a few times.
 template <typename Enqueue>
-static int run_graphed(bsr_handle* h, cudaStream_t st, std::vector<bsr_handle::StepGraph>& cache, const bsr_handle::StepGraph& key, bool at_once,
-                       uint64_t* captures, Enqueue enqueue) {
+static int run_graphed(bsr_handle* h, cudaStream_t st, bsr_handle::GraphSet& set, const bsr_handle::StepGraph& key, bool at_once, Enqueue enqueue) {
   int rc;
+  auto& cache = set.graphs;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   const bool legacy = st == nullptr || st == cudaStreamLegacy;
   bool can_graph = h->use_graph && !h->prof.on && (legacy || (cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone));
@@ -1270,20 +1276,27 @@ static int run_graphed(bsr_handle* h, cudaStream_t st, std::vector<bsr_handle::S
     return BSR_OK;
   };
   if (!can_graph) return direct();
-  for (auto& g : cache)
-    if (same(g)) {
-      g_kernel_launches += g.launches;
-      g.last_use = ++h->graph_clock;
-      return replay(g);
+  ++set.calls;
+  size_t lru = 0;
+  for (size_t i = 0; i < cache.size(); ++i) {
+    if (same(cache[i])) {
+      g_kernel_launches += cache[i].launches;
+      cache[i].last_use = set.calls;
+      return replay(cache[i]);
     }
+    if (cache[i].last_use < cache[lru].last_use) lru = i;
+  }
+  const bool full = cache.size() >= bsr_handle::GRAPH_CACHE;
   if (!at_once) {
-    bool known = false;
-    for (auto& g : h->seen) known = known || same(g);
-    if (!known) {
-      if (h->seen.size() >= 4 * bsr_handle::GRAPH_CACHE) h->seen.erase(h->seen.begin());
-      h->seen.push_back(key);
+    size_t at = 0;
+    while (at < set.seen.size() && !same(set.seen[at])) ++at;
+    if (at == set.seen.size()) {
+      if (at >= bsr_handle::GRAPH_SEEN) set.seen.erase(set.seen.begin());
+      set.seen.push_back(key);
       return direct();
     }
+    if (full && set.calls - cache[lru].last_use <= bsr_handle::GRAPH_IDLE) return direct();
+    set.seen.erase(set.seen.begin() + at);
   }
   if (h->capture_stream == nullptr && cudaStreamCreateWithFlags(&h->capture_stream, cudaStreamNonBlocking) != cudaSuccess) {
     h->capture_stream = nullptr;
@@ -1299,17 +1312,14 @@ static int run_graphed(bsr_handle* h, cudaStream_t st, std::vector<bsr_handle::S
     return rc;
   }
   bsr_handle::StepGraph sg = key;
-  sg.exec = nullptr; sg.launches = g_kernel_launches - before; sg.last_use = ++h->graph_clock;
+  sg.exec = nullptr; sg.launches = g_kernel_launches - before; sg.last_use = set.calls;
   if (ce != cudaSuccess || graph == nullptr || cudaGraphInstantiate(&sg.exec, graph, 0) != cudaSuccess) {
     if (graph) cudaGraphDestroy(graph);
     return direct();                                     // nothing ran during the capture
   }
   cudaGraphDestroy(graph);
-  if (captures != nullptr) ++*captures;
-  if (cache.size() >= bsr_handle::GRAPH_CACHE) {         // drop the least recently used graph
-    size_t lru = 0;
-    for (size_t i = 1; i < cache.size(); ++i)
-      if (cache[i].last_use < cache[lru].last_use) lru = i;
+  ++h->graph_captures;
+  if (full) {
     cudaGraphExecDestroy(cache[lru].exec);
     cache.erase(cache.begin() + lru);
   }
@@ -1337,7 +1347,7 @@ int32_t bsr_train_step(bsr_handle* h, const void* images, const int32_t* labels,
   double bc2 = 1.0 - std::pow((double)h->cfg.beta2, (double)step_next);
   set_scalars(st, h->at<float>(h->off_status + 128), h->lr, (float)bc1, (float)bc2);
   auto key = graph_key(h, images, labels, task_ids, loss_out, kept_out, batch, 0);
-  rc = run_graphed(h, st, h->graphs, key, false, &h->graph_captures,
+  rc = run_graphed(h, st, h->step_graphs, key, false,
                    [&](cudaStream_t s) { return enqueue_train_step(h, images, labels, task_ids, batch, s, loss_out, kept_out); });
   if (rc == BSR_OK) h->step = step_next;
   return rc;
@@ -1350,7 +1360,7 @@ int32_t bsr_forward_backward(bsr_handle* h, const void* images, const int32_t* l
   if (labels == nullptr || loss_out == nullptr) return set_err(h->err, BSR_ERR_INVALID_ARG, "labels_dev and loss_dev_out must not be null");
   if (h->cfg.dims.num_tasks > 1 && task_ids == nullptr) return set_err(h->err, BSR_ERR_INVALID_ARG, "task_ids_dev is required with several tasks");
   auto key = graph_key(h, images, labels, task_ids, loss_out, kept_out, batch, 2);
-  return run_graphed(h, (cudaStream_t)stream, h->graphs, key, false, &h->graph_captures, [&](cudaStream_t s) {
+  return run_graphed(h, (cudaStream_t)stream, h->step_graphs, key, false, [&](cudaStream_t s) {
     return enqueue_train_step(h, images, labels, task_ids, batch, s, loss_out, kept_out, nullptr, false);
   });
 }
@@ -1396,7 +1406,7 @@ int32_t bsr_train_steps(bsr_handle* h, const void* images, const int32_t* labels
   float* scalars = h->at<float>(h->off_status + 128);
   auto key = graph_key(h, images, labels, task_ids, loss_out, kept_out, batch, 1);
   for (int i = 0; i < n_steps; ++i) {
-    rc = run_graphed(h, st, h->graphs, key, n_steps > 2, &h->graph_captures, [&](cudaStream_t s) {
+    rc = run_graphed(h, st, h->step_graphs, key, n_steps > 2, [&](cudaStream_t s) {
       loop_begin(s, ls, scalars, labels, task_ids, lab_stage, task_stage, batch);
       int r = enqueue_train_step(h, images, lab_stage, task_stage, batch, s, nullptr, kept_out, &ls->image_offset);
       loop_end(s, ls, h->at<float>(h->off_loss), loss_out);
@@ -1486,7 +1496,7 @@ int32_t bsr_eval_forward(bsr_handle* h, const void* images, const int32_t* task_
   };
   cudaGetLastError();
   eval_begin(st, io, value, task_ids, tasks, batch);
-  if (relative) return run_graphed(h, st, h->eval_graphs, key, false, nullptr, enqueue);
+  if (relative) return run_graphed(h, st, h->eval_graphs, key, false, enqueue);
   rc = enqueue(st);
   return rc != BSR_OK ? rc : check_cuda(h, "bsr_eval_forward");
 }

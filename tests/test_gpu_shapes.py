@@ -290,3 +290,31 @@ def test_attention_backward_of_more_pairs_than_a_grid_dimension():
         return out
     whole = backward(0, B)
     assert torch.equal(whole[:7], backward(0, 7)) and torch.equal(whole[-7:], backward(B - 7, B))
+
+
+def test_more_keys_than_graphs_capture_no_more_than_the_cache_holds():
+    """Ten sets of step buffers and ten batch sizes of inference in turn: eight graphs of each kind, the rest enqueued, results as
+    without graphs.  A batch size that stays alone long enough then takes the place of an idle one."""
+    import torch
+    from paper_2405_10951_b200 import binding as Bd
+    cfg = MINI.with_(optimizer="sgd", lr=0.0, weight_decay=0.0)
+    images, labels, _, params = synth.make_workload(cfg, peaked=True)
+    eng = Bd.Engine(cfg, max_batch=12)
+    eng.set_params(params)
+    with torch.cuda.stream(torch.cuda.Stream()):
+        img, lab = eng.images_to_device(images), torch.as_tensor(labels).cuda()
+        loss, bufs = torch.zeros(1, device="cuda"), [torch.roll(img, i, 0).clone() for i in range(10)]
+        evals = [torch.randn(b, *img.shape[1:], device="cuda").to(img.dtype) for b in range(1, 11)]
+        runs = []
+        for graphs in (False, True):
+            eng.set_graph_mode(graphs)
+            for _ in range(4):
+                got = [eng.train_step(b, lab, out=(loss, None))[0].clone() for b in bufs] + [eng.eval_forward(x, want_kept=False)[0] for x in evals]
+            runs.append(got)
+        assert all(torch.equal(a, b) for a, b in zip(*runs))
+        assert eng.profile_read()["graph_captures"] == 16
+        for _ in range(300):
+            eng.eval_forward(evals[9], want_kept=False)
+        eng.sync_status()
+        assert eng.profile_read()["graph_captures"] == 17
+    eng.close()
