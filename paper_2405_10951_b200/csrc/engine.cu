@@ -706,6 +706,20 @@ void update_half(bsr_handle* h, const Ctx& c, const Ctx& cl, int l, int half) {
   Ctx u = c;
   u.stream = h->ulane.stream;
   enqueue_optimizer(h, u, h->chunk_at[2 * l + half], h->chunk_at[2 * l + half + 1], l > h->t0 || half == 1);
+  h->ulane.pending[0] = true;
+}
+
+// The stream of the step waits for whatever its lanes still have in flight.
+void join_lanes(bsr_handle* h, const Ctx& c) {
+  side_join_all(c);
+  Ctx cl = c;
+  cl.side = lane_of(h, c);
+  side_join_all(cl);
+  if (h->ulane.pending[0]) {
+    cudaEventRecord(h->ulane.fork, h->ulane.stream);
+    cudaStreamWaitEvent(c.stream, h->ulane.fork, 0);
+    h->ulane.pending[0] = false;
+  }
 }
 
 // Up to 16384 token rows the backward pass leaves DRAM idle and the update hides in it (a step of DeiT-S with one image 722
@@ -1192,12 +1206,10 @@ int32_t bsr_set_step(bsr_handle* h, int64_t steps_done) {
 
 // Enqueues every kernel of one step on `stream` (forward, loss, backward, AdamW reading its scalars from device memory).
 // loss_out may be null (the multi-step loop writes the loss itself); img_offset as in forward_all.
-static int enqueue_train_step(bsr_handle* h, const void* images, const int32_t* labels, const int32_t* task_ids, int32_t batch,
-                              void* stream, float* loss_out, int32_t* kept_out, const long long* img_offset = nullptr,
-                              bool with_update = true) {
+static int enqueue_step_kernels(bsr_handle* h, const Ctx& c, const void* images, const int32_t* labels, const int32_t* task_ids, int32_t batch,
+                                float* loss_out, int32_t* kept_out, const long long* img_offset, bool with_update) {
   int rc;
   const bsr_dims& d = h->cfg.dims;
-  Ctx c = make_ctx(h, stream);
   int D = d.dim, B = batch;
   size_t es = dtype_size(d.dtype);
   size_t x_last = 0;
@@ -1242,12 +1254,21 @@ static int enqueue_train_step(bsr_handle* h, const void* images, const int32_t* 
   side_join_all(cl);
   if (early) {                           // the blocks are updated or about to be; the final LayerNorm and the heads remain
     enqueue_optimizer(h, c, h->chunk_at[2 * d.depth], h->n_chunks, false);
-    cudaEventRecord(h->ulane.fork, h->ulane.stream);
-    cudaStreamWaitEvent(c.stream, h->ulane.fork, 0);
   } else if (with_update) {
     enqueue_optimizer(h, c, 0, h->n_chunks, false);
   }
   return BSR_OK;
+}
+
+// On every way out, a refusal half-way included, the lanes end in `stream`: what they run is then covered by a wait for that
+// stream, and none of their events is left recorded in a capture that has been abandoned.
+static int enqueue_train_step(bsr_handle* h, const void* images, const int32_t* labels, const int32_t* task_ids, int32_t batch,
+                              void* stream, float* loss_out, int32_t* kept_out, const long long* img_offset = nullptr,
+                              bool with_update = true) {
+  Ctx c = make_ctx(h, stream);
+  int rc = enqueue_step_kernels(h, c, images, labels, task_ids, batch, loss_out, kept_out, img_offset, with_update);
+  join_lanes(h, c);
+  return rc;
 }
 
 }  // extern "C"

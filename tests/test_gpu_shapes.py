@@ -318,3 +318,31 @@ def test_more_keys_than_graphs_capture_no_more_than_the_cache_holds():
         eng.sync_status()
         assert eng.profile_read()["graph_captures"] == 17
     eng.close()
+
+
+def test_a_step_refused_half_way_leaves_nothing_in_flight():
+    """730 tokens fit the attention backward on the tensor cores but not the one on FMAs, which refuses while reductions and weight
+    gradients of the block above are on their lanes, here inside a capture.  The next step equals that of a new handle."""
+    import torch
+    from paper_2405_10951_b200 import binding as Bd
+    cfg = Config("mini_730", 432, 16, 128, 2, 3, 256, (10,), 1, (0, 1, 2), (), 1, 1, dtype="bf16", seed=2)
+    images, labels, _, params = synth.make_workload(cfg, peaked=False)
+    shapes = synth.param_shapes(cfg)
+    got = []
+    with torch.cuda.stream(torch.cuda.Stream()):
+        for refused in (True, False):
+            eng = Bd.Engine(cfg)
+            eng.set_params(params)
+            img, lab = eng.images_to_device(images), torch.as_tensor(labels).cuda()
+            if refused:
+                eng.set_gemm_mode(0)
+                for _ in range(2):
+                    with pytest.raises(Bd.BsrError) as e:
+                        eng.train_steps(img.expand(3, *img.shape).contiguous(), lab.expand(3, -1).contiguous(), total_steps=3)
+                    assert e.value.status == -2          # BSR_ERR_UNSUPPORTED
+                eng.set_gemm_mode(1)
+            loss = eng.train_step(img, lab)[0]
+            eng.sync_status()
+            got.append([loss.clone()] + [eng.get_tensor("grad/" + n, shapes[n]) for n in shapes if n.startswith(("blocks", "head"))])
+            eng.close()
+    assert all(torch.equal(a, b) for a, b in zip(*got))
