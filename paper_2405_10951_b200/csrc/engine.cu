@@ -173,7 +173,7 @@ struct bsr_handle {
   size_t off_escore = 0, off_delta = 0, off_ln_partials = 0, off_cs_partials = 0;
   size_t off_kept_all = 0;
   size_t off_stage = 0;
-  size_t off_split = 0, off_split_w = 0, split_floats = 0;
+  size_t off_split = 0, split_floats = 0;
   std::vector<size_t> moe_rec_eidx, moe_rec_ew;
   std::vector<size_t> score_rec;       // per drop location's block: head-mean scores [max_batch, M] of the last step
   size_t off_m_dog = 0, off_m_dzg = 0, off_m_dxg = 0, off_m_dw = 0, off_m_dsel = 0;
@@ -499,7 +499,6 @@ size_t plan(bsr_handle* h) {
   h->off_stage = b.take(biggest * 4);
   h->split_floats = (d.dtype == BSR_DTYPE_BF16) ? (size_t)160 * 128 * 256 : 0;   // one 128x256 fp32 tile per SM
   h->off_split = b.take(h->split_floats * 4);
-  h->off_split_w = b.take(h->split_floats * 4);       // the weight gradients' own: they run on a lane of their own
   // multi-step loop state and staging; two staging slots for steps fed from host memory
   h->off_loop = b.take(256);
   h->off_lab_stage = b.take((size_t)Bm * 4);
@@ -768,7 +767,7 @@ int block_backward(bsr_handle* h, const Ctx& c, int l, int B, GradStream dxo, Gr
   auto lane_begin = [&]() {
     Ctx w = c;
     w.stream = side_begin(cl);
-    if (cl.side != nullptr) { w.side = nullptr; w.split_ws = h->split_floats ? h->at<float>(h->off_split_w) : nullptr; }
+    if (cl.side != nullptr) w.side = nullptr;
     return w;
   };
   auto lane_f32 = [](Ctx w) { w.dtype = 0; return w; };

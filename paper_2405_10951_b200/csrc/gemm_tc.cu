@@ -405,7 +405,7 @@ int gemm_tc_strided(const Ctx& c, const void* A, long a_rs, long a_cs, const voi
   bool ok = a_mn ? make_map(&ma, A, (uint64_t)m, (uint64_t)k, (uint64_t)lda, BK) : make_map(&ma, A, (uint64_t)k, (uint64_t)m, (uint64_t)lda, BM);
   int sms = c.sm_count > 0 ? c.sm_count : 148;
   const bool plain = e.bias == nullptr && e.residual == nullptr && e.act == 0;
-  const bool may_split = split_ws != nullptr && out_is_float && plain;      // weight gradients
+  const bool may_split = a_mn && split_ws != nullptr && out_is_float && plain;      // weight gradients, the workspace's only users
   const Cut cut = choose_tile(m, n, k, a_mn, may_split ? split_ws_floats : 0, sms);
   const int bn = cut.bn;
   ok = ok && (b_mn ? make_map(&mb, B, (uint64_t)n, (uint64_t)k, (uint64_t)ldb, BK) : make_map(&mb, B, (uint64_t)k, (uint64_t)n, (uint64_t)ldb, bn));

@@ -75,3 +75,11 @@ def test_workspace_size_and_validation():
     c.max_batch = 0
     with pytest.raises(Bd.BsrError):
         Bd.bsr_workspace_bytes(c)
+
+
+def test_workspace_holds_one_split_workspace():
+    """A bf16 handle needs one 128 x 256 float tile per SM (160 of them) for partial sums of weight gradients; without tensors to
+    speak of, its workspace is that and less than as much again."""
+    cfg = synth.Config("mini", 32, 16, 64, 1, 2, 64, (2,), 1, (1,), (), 1, 1, dtype="bf16")
+    split = 160 * 128 * 256 * 4
+    assert split < Bd.bsr_workspace_bytes(Bd.make_config(cfg)) < 2 * split
