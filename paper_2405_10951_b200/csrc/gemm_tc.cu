@@ -81,7 +81,7 @@ __device__ __forceinline__ Work decode_work(int w, int tiles_m, int tiles_n, int
 
 // FP8: both operands are E4M3 bytes, K-major; a k-slab is still 128 bytes of every row, i.e. 128 elements instead of
 // 64, and the MMA consumes 32 elements per instruction, so the staging and the descriptors are those of the bf16 kernel.
-template <bool A_MN, bool B_MN, typename TOut, int BN, bool FP8 = false>
+template <bool A_MN, bool B_MN, typename TOut, int BN, bool FP8 = false, bool EXACT = false>
 __global__ void __launch_bounds__(THREADS, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, TOut* __restrict__ C,
                int M, int N, int K, Epi ep, int tiles_m, int tiles_n, int splits, int kb_per_split, GemmGroup grp, int* status) {
@@ -221,7 +221,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         tc_fence_after();
         return w;
       };
-      ok = epilogue_tile<TOut, FP8, (BN <= 128)>(ready, ep, wk.bias_off, C + wk.c_off, M, N, mt * BM + quarter * 32, nt * BN + chalf * HALF_CHUNKS * 32, HALF_CHUNKS,
+      ok = epilogue_tile<TOut, FP8, EXACT>(ready, ep, wk.bias_off, C + wk.c_off, M, N, mt * BM + quarter * 32, nt * BN + chalf * HALF_CHUNKS * 32, HALF_CHUNKS,
                                     tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * BN + chalf * HALF_CHUNKS * 32),
                                     wk.kb0 >= wk.kb1, st, lane);
       if (!ok) break;
@@ -356,10 +356,10 @@ static Cut choose_tile(int m, int n, int k, bool a_mn, size_t ws_floats, int sms
   return {ceil_div(tiles(192), sms) * 192 < ceil_div(tiles(256), sms) * 256 ? 192 : BN_MAX, 1};
 }
 
-template <bool A_MN, bool B_MN, typename TOut, int BN = BN_MAX, bool FP8 = false>
+template <bool A_MN, bool B_MN, typename TOut, int BN = BN_MAX, bool FP8 = false, bool EXACT = false>
 static int launch(const Ctx& c, const CUtensorMap& ma, const CUtensorMap& mb, void* C, int m, int n, int k, const Epi& ep,
                   int tiles_m, int tiles_n, int splits, int kb_per_split, const GemmGroup& grp) {
-  auto kern = gemm_tc_kernel<A_MN, B_MN, TOut, BN, FP8>;
+  auto kern = gemm_tc_kernel<A_MN, B_MN, TOut, BN, FP8, EXACT>;
   static SmemLimit lim;
   if (!ensure_smem(lim, kern, SMEM_BYTES)) return -3;
   int work = tiles_m * tiles_n * splits;
@@ -414,7 +414,7 @@ int gemm_tc_strided(const Ctx& c, const void* A, long a_rs, long a_cs, const voi
   const int kb_per_split = ceil_div(total_kb, cut.splits), splits = ceil_div(total_kb, kb_per_split);
   Epi ep;
   ep.bias = e.bias; ep.residual = e.residual; ep.aux_out = e.aux_out; ep.aux_in = e.aux_in; ep.act = e.act;
-  ep.exact = exact_gelu(m, k);             // (tiles of 64 or 128 columns up to 9472 of them)
+  const bool exact = !a_mn && e.act != 0 && exact_gelu(m, k);       // (tiles of 64 or 128 columns up to 9472 of them)
   void* dst = (splits > 1) ? (void*)split_ws : C;
   if (splits > 1) side_join(c, 2);         // the previous split sum has read the workspace
   if (c.prof != nullptr && c.prof->on) c.prof->begin(c.stream, 2.0 * m * n * (double)k);
@@ -423,6 +423,8 @@ int gemm_tc_strided(const Ctx& c, const void* A, long a_rs, long a_cs, const voi
   auto run = [&](auto width) {
     constexpr int W = decltype(width)::value;
     auto go = [&](auto kern) { return kern(c, ma, mb, dst, m, n, k, ep, tiles_m, tiles_n, splits, kb_per_split, gg); };
+    if constexpr (W <= 128)
+      if (exact) return b_mn ? go(launch<false, true, bf16, W, false, true>) : go(launch<false, false, bf16, W, false, true>);
     if constexpr (W >= 128)
       if (a_mn) return out_is_float ? go(launch<true, true, float, W>) : go(launch<true, true, bf16, W>);
     if (out_is_float) return b_mn ? go(launch<false, true, float, W>) : go(launch<false, false, float, W>);

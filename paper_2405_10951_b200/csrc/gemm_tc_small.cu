@@ -45,7 +45,7 @@ __device__ __forceinline__ void send16(uint32_t dst, const uint32_t* v) {
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
-template <bool B_MN, typename TOut>
+template <bool B_MN, typename TOut, bool EXACT>
 __global__ void __launch_bounds__(THREADS, 2)
 gemm_tc_small_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, TOut* __restrict__ C,
                      int M, int N, int K, Epi ep, int stages, int* status) {
@@ -177,7 +177,7 @@ gemm_tc_small_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
     v[0] += bias.x; v[1] += bias.y; v[2] += bias.z; v[3] += bias.w;
     if (ep.act == 1) {
       if (ep.aux_out != nullptr) store4(reinterpret_cast<TOut*>(ep.aux_out) + at(r0 + local), v);
-      if (ep.exact) {
+      if (EXACT) {
         gelu_exact2(v[0], v[1]);
         gelu_exact2(v[2], v[3]);
       } else {
@@ -185,7 +185,7 @@ gemm_tc_small_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
         gelu_fast2(v[2], v[3]);
       }
     } else if (ep.act == 2) {
-      if (ep.exact) {
+      if (EXACT) {
         gelu_grad_exact2(v[0], v[1], z[p][0], z[p][1]);
         gelu_grad_exact2(v[2], v[3], z[p][2], z[p][3]);
       } else {
@@ -204,9 +204,9 @@ gemm_tc_small_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
   }
 }
 
-template <bool B_MN, typename TOut>
+template <bool B_MN, typename TOut, bool EXACT = false>
 static int launch(const Ctx& c, const CUtensorMap& ma, const CUtensorMap& mb, void* C, int m, int n, int k, const Epi& ep, int splits) {
-  auto kern = gemm_tc_small_kernel<B_MN, TOut>;
+  auto kern = gemm_tc_small_kernel<B_MN, TOut, EXACT>;
   const int slabs = ceil_div(ceil_div(k, BK), splits), stages = slabs < MAX_STAGES ? slabs : MAX_STAGES;
   auto bytes = [](int st) { return (size_t)st * STAGE_BYTES + RECV_BYTES + 1024; };
   static SmemLimit lim;
@@ -243,11 +243,14 @@ int gemm_tc_small(const Ctx& c, const void* A, long lda, const void* B, long ldb
   if (!(b_mn ? make_map(&mb, B, (uint64_t)n, (uint64_t)k, (uint64_t)ldb, BK) : make_map(&mb, B, (uint64_t)k, (uint64_t)n, (uint64_t)ldb, BN))) return -2;
   Epi ep;
   ep.bias = e.bias; ep.residual = e.residual; ep.aux_out = e.aux_out; ep.aux_in = e.aux_in; ep.act = e.act;
-  ep.exact = exact_gelu(m, k);
   const bool timed = c.prof != nullptr && c.prof->on;
   if (timed) c.prof->begin(c.stream, 2.0 * m * n * (double)k);
-  const int rc = out_is_float ? (b_mn ? launch<true, float>(c, ma, mb, C, m, n, k, ep, splits) : launch<false, float>(c, ma, mb, C, m, n, k, ep, splits))
-                              : (b_mn ? launch<true, bf16>(c, ma, mb, C, m, n, k, ep, splits) : launch<false, bf16>(c, ma, mb, C, m, n, k, ep, splits));
+  const bool exact = e.act != 0 && exact_gelu(m, k);
+  auto go = [&](auto kern) { return kern(c, ma, mb, C, m, n, k, ep, splits); };
+  int rc;
+  if (out_is_float) rc = b_mn ? go(launch<true, float>) : go(launch<false, float>);
+  else if (exact) rc = b_mn ? go(launch<true, bf16, true>) : go(launch<false, bf16, true>);
+  else rc = b_mn ? go(launch<true, bf16>) : go(launch<false, bf16>);
   if (timed) c.prof->end(c.stream);
   return rc;
 }

@@ -15,7 +15,6 @@ struct Epi {
   void* aux_out = nullptr;
   const void* aux_in = nullptr;
   int act = 0;
-  bool exact = false;              // activation to fp32 precision: see exact_gelu
   // operands quantised with one scale per row of A and per row of B (8-bit floating point): the accumulator of
   // (row, col) is multiplied by row_scale[row] * col_scale[col] before the bias
   const float* row_scale = nullptr;
@@ -236,7 +235,7 @@ template <> __device__ __forceinline__ uint4 ChunkIO<bf16>::pack(const float* f)
 // v[j]: accumulator of (row0 + lane, col0 + j).  All lanes of the warp take part (row0, col0 are warp-uniform).
 // z: the chunk of the stored pre-activation for act == 2, already in this lane's row order (overwritten).
 // sbias, scol: the chunk's 32 bias values and column scales in shared memory (null: none), rs: this lane's row scale.
-// EXACT: the kernel is one that ep.exact may ask for the exact activation.
+// EXACT: activations as exact_gelu has them.
 template <typename TOut, bool EXACT>
 __device__ __forceinline__ void epilogue_chunk(const uint32_t* r, const Epi& ep, const float* sbias, const float* scol, float rs, TOut* Cs, int M,
                                                int N, int row0, int col0, unsigned char* st, int lane, float* z) {
@@ -260,7 +259,7 @@ __device__ __forceinline__ void epilogue_chunk(const uint32_t* r, const Epi& ep,
     }
     if (ep.act == 1) {
       if (ep.aux_out != nullptr) ChunkIO<TOut>::store((TOut*)ep.aux_out, N, row0, col0, M, N, st, lane, v);
-      if (EXACT && ep.exact) {
+      if (EXACT) {
 #pragma unroll
         for (int j = 0; j < 32; j += 2) gelu_exact2(v[j], v[j + 1]);
       } else {
@@ -268,7 +267,7 @@ __device__ __forceinline__ void epilogue_chunk(const uint32_t* r, const Epi& ep,
         for (int j = 0; j < 32; j += 2) gelu_fast2(v[j], v[j + 1]);
       }
     } else if (ep.act == 2) {
-      if (EXACT && ep.exact) {
+      if (EXACT) {
 #pragma unroll
         for (int j = 0; j < 32; j += 2) gelu_grad_exact2(v[j], v[j + 1], z[j], z[j + 1]);
         if (ep.aux_out != nullptr) ChunkIO<bf16>::store((bf16*)ep.aux_out, N, row0, col0, M, N, st, lane, z);
