@@ -206,10 +206,17 @@ void gemm(const Ctx& c, const void* A, long a_rs, long a_cs, const void* B, long
   // there), and slabs past the end arrive as zeros.  Weight gradients reduce over batch x tokens rows, which an odd batch
   // leaves odd: at batch 45 of ViT-B they took 515 us a launch on FP32 FMAs, 18 us on the tensor cores.
   if (c.dtype == 1 && c.use_tc && (n % 8) == 0) {
-    // CTA pairs where a wide output over many rows keeps all of them busy (QKV and first FFN layer of ViT-B from batch 61):
-    // 25216 x 2304 x 768 73.1 -> 71.4 us, and less power, which is what limits a long run (ViT-B step at batch 128 5.81 -> 5.72 ms,
-    // inference 3.93 -> 3.86 ms).  Narrower outputs lose (25216 x 768 x 3072: 92 -> 107 us; B read across k: 159 -> 166 us).
-    const bool pairs = c.use_tc >= 2 ? m > 128 : (m >= 12000 && n >= 2048 && a_cs == 1 && b_cs == 1);
+    // CTA pairs where a wide output over many rows keeps all of them busy (QKV and first FFN layer of ViT-B from batch 61).  us with
+    // one CTA a tile / with pairs, launch after launch, at 12608, 16351 and 25216 rows:
+    //   2304 columns, k = 768     52.6 / 49.7   56.4 / 55.2   82.7 / 82.2     (9000 and 11000 rows: 39.1 / 39.6, 44.8 / 45.0)
+    //   3072 columns, k = 768     65.3 / 58.6   81.9 / 71.0   112  / 110      (with GELU 72.9 / 74.6, 97.6 / 97.8, 114 / 125)
+    //   2048 columns, k = 768     43.4 / 43.3   50.0 / 49.7   79.3 / 77.0     (1536 columns 33.0 / 32.3, 37.8 / 37.0, 52.3 / 53.9)
+    //   2304 columns, k = 640     42.6 / 42.0   48.4 / 50.2   71.2 / 75.3     (k = 512: 36.7 / 40.3, 42.2 / 48.4, 58.3 / 68.2)
+    // A pair stages half of B on each SM, which also takes less power, and power is what limits a run of steps: there GELU's products
+    // are as fast either way (with them on single CTAs a ViT-B step at batch 128 5.79 against 5.77 ms, inference 3.96 and 3.96).
+    // Below k = 640 the set-up of a pair's tile shows more than that.  Float outputs and B read across k lose on pairs
+    // (25216 x 768 x 3072: 92 -> 107 us; 159 -> 166 us).
+    const bool pairs = c.use_tc >= 2 ? m > 128 : (m >= 12000 && n >= 2048 && k >= 640 && a_cs == 1 && b_cs == 1);
     if (pairs && gemm_tc2_strided(c, A, a_rs, a_cs, B, b_rs, b_cs, C, out_is_float, m, n, k, e) == 0) return;
     if (gemm_tc_strided(c, A, a_rs, a_cs, B, b_rs, b_cs, C, out_is_float, m, n, k, e, c.split_ws, c.split_ws_floats) == 0) return;
   }
