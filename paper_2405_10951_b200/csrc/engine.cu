@@ -721,16 +721,20 @@ void join_lanes(bsr_handle* h, const Ctx& c) {
   }
 }
 
-// Up to 16384 token rows the backward pass leaves DRAM idle and the update hides in it (a step of DeiT-S with one image 722
-// -> 708 us, with 64 images 1524 -> 1508; ViT-B with 32 images 2292 -> 2274, ViT-B/384 with 7 images 2150 -> 2117); over more
-// rows its contractions lose what the update gains (ViT-B, 128 images: 5826 -> 5860 us).  float storage has nothing to
-// gain (tiny model, four steps: 2991 -> 2997 us), nor has an expert layer, whose many weights take longer to update than its
-// backward pass has time for (64 images: 2264 -> 2278 us).  The sizes are ones that every kernel of the backward pass takes,
-// so that a step which ends in an error updates nothing.
+// As long as the residual stream (rows x width) has no more than 8 Mi values the backward pass leaves DRAM idle and the update hides
+// in it.  us a step, update at the end -> early, by values:
+//   0.1 M  DeiT-S, one image      722 -> 708       7.1 M  ViT-B/384, 16 images   2131 -> 2098
+//   3.1 M  ViT-B/384, 7 images   2150 -> 2117      9.7 M  DeiT-S, 128 images     2394 -> 2390 (blocks 4, 8, 12: 3570 -> 3567)
+//   4.8 M  DeiT-S, 64 images     1504 -> 1492      9.7 M  ViT-B, 64 images       3279 -> 3303
+//   4.8 M  ViT-B, 32 images      2292 -> 2274     12.6 M  ViT-B, 83 images       3987 -> 3995 (blocks 4, 8, 12: 5671 -> 5702)
+//   6.8 M  ViT-B, 45 images      2485 -> 2491     19.4 M  ViT-B, 128 images      5826 -> 5860
+// float storage has nothing to gain (tiny model, four steps: 2991 -> 2997 us), nor has an expert layer, whose many weights take
+// longer to update than its backward pass has time for (64 images: 2264 -> 2278 us).  The sizes are ones that every kernel of
+// the backward pass takes, so that a step which ends in an error updates nothing.
 bool early_update(const bsr_handle* h, const Ctx& c, int B) {
   const bsr_dims& d = h->cfg.dims;
   return c.dtype == 1 && c.use_tc && d.dim == 64 * d.heads && (long)B * d.heads <= 65535 && h->ulane.stream != nullptr &&
-         d.moe_block_mask == 0 && h->t0 < d.depth && (long)B * h->sched.ta[0] <= 16384;
+         d.moe_block_mask == 0 && h->t0 < d.depth && (long)B * h->sched.ta[0] * d.dim <= (8l << 20);
 }
 
 int block_backward(bsr_handle* h, const Ctx& c, int l, int B, GradStream dxo, GradStream dxi, bool need_dxi, const int* task_ids, bool update) {
