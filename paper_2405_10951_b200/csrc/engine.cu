@@ -731,11 +731,12 @@ void join_lanes(bsr_handle* h, const Ctx& c) {
 // float storage has nothing to gain (tiny model, four steps: 2991 -> 2997 us), nor has an expert layer, whose many weights take
 // longer to update than its backward pass has time for (64 images: 2264 -> 2278 us).  The sizes are ones that every kernel of
 // the backward pass takes, so that a step which ends in an error updates nothing.
-bool early_update(const bsr_handle* h, const Ctx& c, int B) {
+bool update_can_be_early(const bsr_handle* h, int B) {
   const bsr_dims& d = h->cfg.dims;
-  return c.dtype == 1 && c.use_tc && d.dim == 64 * d.heads && (long)B * d.heads <= 65535 && h->ulane.stream != nullptr &&
-         d.moe_block_mask == 0 && h->t0 < d.depth && (long)B * h->sched.ta[0] * d.dim <= (8l << 20);
+  return d.dtype == BSR_DTYPE_BF16 && d.dim == 64 * d.heads && (long)B * d.heads <= 65535 && d.moe_block_mask == 0 && h->t0 < d.depth &&
+         (long)B * h->sched.ta[0] * d.dim <= (8l << 20);
 }
+bool early_update(const bsr_handle* h, const Ctx& c, int B) { return c.use_tc && h->ulane.stream != nullptr && update_can_be_early(h, B); }
 
 int block_backward(bsr_handle* h, const Ctx& c, int l, int B, GradStream dxo, GradStream dxi, bool need_dxi, const int* task_ids, bool update) {
   const bsr_dims& d = h->cfg.dims;
@@ -1013,16 +1014,16 @@ int32_t bsr_create(const bsr_config* cfg, void* workspace, size_t bytes, bsr_han
   h->base = (char*)workspace;
   h->bytes = bytes;
   h->lr = cfg->lr;
-  int dev = 0;
-  cudaDeviceProp prop;
-  if (cudaGetDevice(&dev) != cudaSuccess || cudaGetDeviceProperties(&prop, dev) != cudaSuccess) {
+  int dev = 0, major = 0, minor = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&h->sm_count, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, dev) != cudaSuccess) {
     delete h;
     return set_err(g_error, BSR_ERR_CUDA, "no usable CUDA device: %s", cudaGetErrorString(cudaGetLastError()));
   }
-  h->sm_count = prop.multiProcessorCount;
-  if (prop.major != 10) {
+  if (major != 10) {
     delete h;
-    return set_err(g_error, BSR_ERR_UNSUPPORTED, "this library is built for sm_100a only (device is sm_%d%d)", prop.major, prop.minor);
+    return set_err(g_error, BSR_ERR_UNSUPPORTED, "this library is built for sm_100a only (device is sm_%d%d)", major, minor);
   }
   // optimiser state and status start at zero; the chunk table is uploaded once
   cudaMemsetAsync(h->base + h->off_status, 0, 256, 0);
@@ -1056,13 +1057,17 @@ int32_t bsr_create(const bsr_config* cfg, void* workspace, size_t bytes, bsr_han
     delete h;
     return set_err(g_error, BSR_ERR_CUDA, "workspace initialisation failed: %s", cudaGetErrorString(e));
   }
-  // host objects of the side lane (no device memory); without them the reductions simply stay on the main stream
-  for (SideLane* lane : {&h->side, &h->wlane, &h->ulane}) {
+  // host objects of the lanes (no device memory); without them the work simply stays on the main stream.  The updates' lane is
+  // made where a batch of one could use it, and takes one event.
+  auto make_lane = [](SideLane* lane, int buffers) {
     bool ok = cudaStreamCreateWithFlags(&lane->stream, cudaStreamNonBlocking) == cudaSuccess &&
               cudaEventCreateWithFlags(&lane->fork, cudaEventDisableTiming) == cudaSuccess;
-    for (int i = 0; i < 3 && ok; ++i) ok = cudaEventCreateWithFlags(&lane->done[i], cudaEventDisableTiming) == cudaSuccess;
+    for (int i = 0; i < buffers && ok; ++i) ok = cudaEventCreateWithFlags(&lane->done[i], cudaEventDisableTiming) == cudaSuccess;
     if (!ok) { cudaGetLastError(); lane->stream = nullptr; }
-  }
+  };
+  make_lane(&h->side, 3);
+  if (h->t0 < cfg->dims.depth) make_lane(&h->wlane, 3);
+  if (update_can_be_early(h, 1)) make_lane(&h->ulane, 0);
   *out = h;
   return BSR_OK;
 }
