@@ -250,7 +250,8 @@ int32_t bsr_selftest_wait_expiry(bsr_handle* h, uint64_t limit_ns, void* stream)
 
 /* Which kernels run the dense contractions and attention of a bf16 handle (no counterpart in the paper):
  * 0 = the FP32-FMA kernels of the fp32 configuration (slow; a cross-check), 1 = tcgen05 kernels, one CTA per tile or
- * CTA pairs (cta_group::2) by size (the default), 2 = as 1 but GEMMs with more than 128 rows run on CTA pairs. */
+ * CTA pairs (cta_group::2) by size (the default), 2 = as 1, but of the products that CTA pairs take (forward, bf16
+ * output) all with more than 128 rows run on them. */
 int32_t bsr_set_gemm_mode(bsr_handle* h, int32_t mode);
 
 /* bsr_train_step replays a captured CUDA graph of its ~200 launches (unless the caller is capturing `stream`): the first

@@ -214,10 +214,10 @@ void gemm(const Ctx& c, const void* A, long a_rs, long a_cs, const void* B, long
     //   2304 columns, k = 640     42.6 / 42.0   48.4 / 50.2   71.2 / 75.3     (k = 512: 36.7 / 40.3, 42.2 / 48.4, 58.3 / 68.2)
     // A pair stages half of B on each SM, which also takes less power, and power is what limits a run of steps: there GELU's products
     // are as fast either way (with them on single CTAs a ViT-B step at batch 128 5.79 against 5.77 ms, inference 3.96 and 3.96).
-    // Below k = 640 the set-up of a pair's tile shows more than that.  Float outputs and B read across k lose on pairs
-    // (25216 x 768 x 3072: 92 -> 107 us; 159 -> 166 us).
-    const bool pairs = c.use_tc >= 2 ? m > 128 : (m >= 12000 && n >= 2048 && k >= 640 && a_cs == 1 && b_cs == 1);
-    if (pairs && gemm_tc2_strided(c, A, a_rs, a_cs, B, b_rs, b_cs, C, out_is_float, m, n, k, e) == 0) return;
+    // Below k = 640 the set-up of a pair's tile shows more than that.  Float outputs and B read across k
+    // lost on pairs (25216 x 768 x 3072: 92 -> 107 us; 159 -> 166 us) and are not built for them.
+    const bool pairs = a_cs == 1 && b_cs == 1 && !out_is_float && (c.use_tc >= 2 ? m > 128 : (m >= 12000 && n >= 2048 && k >= 640));
+    if (pairs && gemm_tc2(c, A, a_rs, B, b_rs, C, m, n, k, e) == 0) return;
     if (gemm_tc_strided(c, A, a_rs, a_cs, B, b_rs, b_cs, C, out_is_float, m, n, k, e, c.split_ws, c.split_ws_floats) == 0) return;
   }
   note_launch(1);

@@ -8,13 +8,13 @@
 // dX = dY W, and both operands of the weight-gradient product dW = dY^T X, Eq. 2 and Eq. 4 of the
 // paper).  No operand is transposed in memory; the shared-memory descriptors say how to read it.
 //
-// Kernel shape: persistent, one CTA per SM, 128 x 256 output tiles, k in slabs of 64.  Tiles are walked with the
-// column index fastest, so that the CTAs running at one time share rows of A and find them in L2.
+// Kernel shape: persistent, one CTA per SM, output tiles of 128 rows and 64 to 256 columns (choose_tile), k in slabs of 64.
+// Tiles are walked with the column index fastest, so that the CTAs running at one time share rows of A and find them in L2.
 //   warp 0      : TMA producer (one lane)
 //   warp 1      : tensor-memory allocation, MMA issue (one lane)
 //   warps 2..9  : epilogue, two warps per TMEM lane quarter; chunks of 32 x 32 outputs go through a staging
-//                 buffer so that global loads and stores are row-contiguous; two accumulator buffers of 256
-//                 columns let the epilogue of one tile overlap the main loop of the next.
+//                 buffer so that global loads and stores are row-contiguous; two accumulator buffers, a
+//                 tile wide each, let the epilogue of one tile overlap the main loop of the next.
 // Every wait is bounded: on expiry the CTA raises STATUS_TIMEOUT in the status word, gives the
 // copies it issued time to land, frees its tensor memory and returns.
 #include <cuda.h>
@@ -302,17 +302,6 @@ bool make_map(CUtensorMap* map, const void* ptr, uint64_t inner, uint64_t outer,
   cuuint32_t box[2] = {64, box_outer};
   cuuint32_t estr[2] = {1, 1};
   return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(ptr), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-            CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-bool make_map_chunks(CUtensorMap* map, const void* ptr, uint64_t extent, uint64_t outer, uint64_t ld, uint32_t box_chunks) {
-  EncodeFn fn = encode_fn();
-  if (fn == nullptr) return false;
-  cuuint64_t dims[3] = {64, outer, extent / 64};
-  cuuint64_t strides[2] = {ld * 2, 128};
-  cuuint32_t box[3] = {64, 64, box_chunks};
-  cuuint32_t estr[3] = {1, 1, 1};
-  return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 

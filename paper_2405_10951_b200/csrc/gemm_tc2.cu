@@ -1,6 +1,6 @@
 // bf16 GEMM on CTA pairs: tcgen05.mma cta_group::2 with a 256 x 256 accumulator tile spread over the tensor
-// memory of two SMs.  Same contract as the single-CTA kernel for an operand A read along k, but each SM stages only its
-// own 128 rows of A and its own half of the columns of B per k-slab: 32 KB instead of 48 KB for the same number of
+// memory of two SMs.  Same contract as the single-CTA kernel for operands read along k and a bf16 output, but each SM stages
+// only its own 128 rows of A and its own half of the columns of B per k-slab: 32 KB instead of 48 KB for the same number of
 // multiply-accumulates.  That is what bounds the single-CTA kernel's main loop: four slabs of 48 KB in flight cover less
 // than the 2000-odd clocks a slab takes to arrive; six slabs of 32 KB fit here.
 //
@@ -83,14 +83,13 @@ __device__ __forceinline__ void mbar_arrive_leader(uint32_t bar) {
 
 // The tiles of one pair.  Whole tiles go round in as many full waves as there are; the tiles of a last wave that would leave
 // pairs idle are cut along n into as many parts as there are pairs for them (25216 rows are 98.5 tiles of 256: at 768 columns
-// 297 tiles on 74 pairs, the last wave a single tile).  Parts are multiples of UNIT columns: 64, or 128 where B is read
-// across k (64-column chunks for each CTA).  Stepping to the next whole tile takes no division.
+// 297 tiles on 74 pairs, the last wave a single tile).  Parts are multiples of UNIT columns.  Stepping to the next whole tile
+// takes no division.
 struct Tile {
   int mt, n0, width;
 };
-template <int UNIT>
+constexpr int UNIT = 64, UNITS = BN / UNIT;
 struct Walk {
-  static constexpr int UNITS = BN / UNIT;
   int i, row, nt, step, full, items, parts, workers;
   __device__ __forceinline__ static int part_units(int parts) { return (UNITS + parts - 1) / parts; }
   __device__ __forceinline__ Walk(int tiles_m, int tiles_n, int worker, int workers_) {
@@ -127,10 +126,9 @@ struct Walk {
   }
 };
 
-template <bool B_MN, typename TOut>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
 gemm_tc2_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, const __grid_constant__ CUtensorMap map_part,
-                int wide, TOut* __restrict__ C, int M, int N, int K, Epi ep, int tiles_m, int tiles_n, int* status) {
+                bf16* __restrict__ C, int M, int N, int K, Epi ep, int tiles_m, int tiles_n, int* status) {
   extern __shared__ unsigned char smem_dyn[];
   uint32_t base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
   uint32_t staging0 = base + STAGES * STAGE_BYTES;
@@ -164,7 +162,7 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
   uint32_t tmem_base = tmem_base_slot;
   await_inputs();                           // (fills the SMs: see release_dependents)
   volatile int* abortp = &abort_flag;
-  Walk<B_MN ? 128 : 64> walk(tiles_m, tiles_n, blockIdx.x >> 1, gridDim.x >> 1);
+  Walk walk(tiles_m, tiles_n, blockIdx.x >> 1, gridDim.x >> 1);
   Tile t;
 
   if (warp == 0) {
@@ -177,7 +175,6 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
       while (ok && walk.next(N, tiles_n, t)) {
         const int m0 = t.mt * (2 * BM) + (int)rank * BM;        // this CTA's rows of A
         const int cols = t.width >> 1, n0 = t.n0 + (int)rank * cols;   // this CTA's share of B
-        const bool whole = t.width == BN && wide;
         const uint32_t bytes = 2u * (uint32_t)(A_BYTES + cols * (BK * 2));
         for (int kb = 0; kb < total_kb; ++kb) {
           if (!mbar_wait(empty_bar(stage), phase ^ 1u, abortp)) { ok = false; break; }
@@ -185,14 +182,10 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
           if (leader) mbar_expect_tx(full_bar(stage), bytes);
           const uint32_t sa = base + stage * STAGE_BYTES, sb = sa + A_BYTES;
           tma_load_2d_pair(sa, &map_a, fb, kb * BK, m0);
-          if (whole) {
-            if (!B_MN) tma_load_2d_pair(sb, &map_b, fb, kb * BK, n0);
-            else tma_load_3d_pair(sb, &map_b, fb, 0, kb * BK, n0 >> 6);
+          if (t.width == BN) {
+            tma_load_2d_pair(sb, &map_b, fb, kb * BK, n0);
           } else {
-            for (int j = 0; j < cols; j += B_MN ? 64 : 32) {
-              if (!B_MN) tma_load_2d_pair(sb + j * 128, &map_part, fb, kb * BK, n0 + j);
-              else tma_load_2d_pair(sb + j * (BK * 2), &map_part, fb, n0 + j, kb * BK);
-            }
+            for (int j = 0; j < cols; j += UNIT / 2) tma_load_2d_pair(sb + j * 128, &map_part, fb, kb * BK, n0 + j);
           }
           ++armed;
           if (++stage == STAGES) { stage = 0; phase ^= 1u; }
@@ -206,10 +199,10 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
   } else if (warp == 1) {
     // ------------------------------- MMA issuer (leader CTA only) ---------------------------
     if (lane == 0 && leader) {
-      constexpr uint32_t idesc0 = make_idesc_mn(2 * BM, 0, false, B_MN);
-      constexpr uint32_t A_KSTEP = (UMMA_K * 2) >> 4, B_KSTEP = (B_MN ? UMMA_K * 128 : UMMA_K * 2) >> 4;
+      constexpr uint32_t idesc0 = make_idesc_mn(2 * BM, 0, false, false);
+      constexpr uint32_t KSTEP = (UMMA_K * 2) >> 4;
       const uint64_t desc_a0 = make_desc(base, 16, 1024);
-      const uint64_t desc_b0 = B_MN ? make_desc(base + A_BYTES, BK * 128, 1024) : make_desc(base + A_BYTES, 16, 1024);
+      const uint64_t desc_b0 = make_desc(base + A_BYTES, 16, 1024);
       int stage = 0;
       uint32_t phase = 0;
       int local = 0;
@@ -226,7 +219,7 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
           const uint64_t off = (uint64_t)((stage * STAGE_BYTES) >> 4);
 #pragma unroll
           for (int k = 0; k < BK / UMMA_K; ++k)
-            umma_bf16_pair(d_tmem, desc_a0 + off + (uint64_t)(k * A_KSTEP), desc_b0 + off + (uint64_t)(k * B_KSTEP), idesc, (kb > 0 || k > 0) ? 1u : 0u);
+            umma_bf16_pair(d_tmem, desc_a0 + off + (uint64_t)(k * KSTEP), desc_b0 + off + (uint64_t)(k * KSTEP), idesc, (kb > 0 || k > 0) ? 1u : 0u);
           umma_commit_pair(empty_bar(stage));
           if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
@@ -246,7 +239,7 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
         tc_fence_after();
         return w;
       };
-      if (!epilogue_tile<TOut, false, false>(ready, ep, 0, C, M, N, t.mt * (2 * BM) + (int)rank * BM + quarter * 32, t.n0 + chalf * nc * 32, nc,
+      if (!epilogue_tile<bf16, false, false>(ready, ep, 0, C, M, N, t.mt * (2 * BM) + (int)rank * BM + quarter * 32, t.n0 + chalf * nc * 32, nc,
                                       tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * BN + chalf * nc * 32), false, st, lane))
         break;
       tc_fence_before();
@@ -265,52 +258,29 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
   if (threadIdx.x == 0 && abort_flag && status != nullptr) atomicOr(status, STATUS_TIMEOUT);
 }
 
-template <bool B_MN, typename TOut>
-static int launch(const Ctx& c, const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorMap& mp, int wide, void* C, int m, int n, int k,
-                  const Epi& ep, int tiles_m, int tiles_n) {
-  auto kern = gemm_tc2_kernel<B_MN, TOut>;
-  static SmemLimit lim;
-  if (!ensure_smem(lim, kern, SMEM_BYTES)) return -3;
-  const long work = (long)tiles_m * tiles_n * (BN / (B_MN ? 128 : 64));
-  const int pairs = (c.sm_count > 0 ? c.sm_count : B200_SMS) / 2;
-  note_launch(1);
-  launch_k(kern, 2 * (int)(work < pairs ? work : pairs), THREADS, SMEM_BYTES, c.stream, ma, mb, mp, wide, (TOut*)C, m, n, k, ep, tiles_m, tiles_n, c.status);
-  return 0;
-}
-
 }  // namespace tc2
 
-// Same contract as gemm_tc_strided without splits, on CTA pairs; A contiguous along k.  Returns non-zero when the problem is
+// C[m, n] (bf16) = epilogue(A B^T) for operands contiguous along k, rows lda and ldb apart.  Returns non-zero when the problem is
 // not taken.
-int gemm_tc2_strided(const Ctx& c, const void* A, long a_rs, long a_cs, const void* B, long b_rs, long b_cs, void* C,
-                     int out_is_float, int m, int n, int k, const GemmEpilogue& e) {
+int gemm_tc2(const Ctx& c, const void* A, long lda, const void* B, long ldb, void* C, int m, int n, int k, const GemmEpilogue& e) {
   using namespace tc2;
-  const bool b_mn = b_cs != 1;
-  if (a_cs != 1 || (b_mn && b_rs != 1)) return -1;
-  const long lda = a_rs, ldb = b_mn ? b_cs : b_rs;
   if ((lda % 8) != 0 || (ldb % 8) != 0 || ((uintptr_t)A & 15) || ((uintptr_t)B & 15) || ((uintptr_t)C & 15)) return -1;
   if ((n % 8) != 0) return -1;
-  if (out_is_float && e.act != 0) return -1;
   CUtensorMap ma, mb, mp;
-  bool ok = tc::make_map(&ma, A, (uint64_t)k, (uint64_t)m, (uint64_t)lda, BM);
-  const int wide = !b_mn || n % 64 == 0;       // whole tiles of B in one copy
-  if (!b_mn) {
-    ok = ok && tc::make_map(&mb, B, (uint64_t)k, (uint64_t)n, (uint64_t)ldb, BN / 2) && tc::make_map(&mp, B, (uint64_t)k, (uint64_t)n, (uint64_t)ldb, 32);
-  } else {
-    ok = ok && tc::make_map(&mp, B, (uint64_t)n, (uint64_t)k, (uint64_t)ldb, BK);
-    if (ok && wide) ok = tc::make_map_chunks(&mb, B, (uint64_t)n, (uint64_t)k, (uint64_t)ldb, BN / 128);
-    else mb = mp;
-  }
-  if (!ok) return -2;
-  const int tiles_m = ceil_div(m, 2 * BM), tiles_n = ceil_div(n, BN);
+  if (!tc::make_map(&ma, A, (uint64_t)k, (uint64_t)m, (uint64_t)lda, BM) || !tc::make_map(&mb, B, (uint64_t)k, (uint64_t)n, (uint64_t)ldb, BN / 2) ||
+      !tc::make_map(&mp, B, (uint64_t)k, (uint64_t)n, (uint64_t)ldb, UNIT / 2))
+    return -2;
+  static SmemLimit lim;
+  if (!ensure_smem(lim, gemm_tc2_kernel, SMEM_BYTES)) return -3;
+  const int tiles_m = ceil_div(m, 2 * BM), tiles_n = ceil_div(n, BN), pairs = (c.sm_count > 0 ? c.sm_count : B200_SMS) / 2;
+  const long work = (long)tiles_m * tiles_n * UNITS;
   tc::Epi ep;
   ep.bias = e.bias; ep.residual = e.residual; ep.aux_out = e.aux_out; ep.aux_in = e.aux_in; ep.act = e.act;
   if (c.prof != nullptr && c.prof->on) c.prof->begin(c.stream, 2.0 * m * n * (double)k);
-  int rc;
-  if (out_is_float) rc = b_mn ? launch<true, float>(c, ma, mb, mp, wide, C, m, n, k, ep, tiles_m, tiles_n) : launch<false, float>(c, ma, mb, mp, wide, C, m, n, k, ep, tiles_m, tiles_n);
-  else rc = b_mn ? launch<true, bf16>(c, ma, mb, mp, wide, C, m, n, k, ep, tiles_m, tiles_n) : launch<false, bf16>(c, ma, mb, mp, wide, C, m, n, k, ep, tiles_m, tiles_n);
+  note_launch(1);
+  launch_k(gemm_tc2_kernel, 2 * (int)(work < pairs ? work : pairs), THREADS, SMEM_BYTES, c.stream, ma, mb, mp, (bf16*)C, m, n, k, ep, tiles_m, tiles_n, c.status);
   if (c.prof != nullptr && c.prof->on) c.prof->end(c.stream);
-  return rc;
+  return 0;
 }
 
 }  // namespace bsr

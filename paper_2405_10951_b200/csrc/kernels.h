@@ -160,9 +160,8 @@ int gemm_tc_grouped_rows(const Ctx& c, const void* A, const void* Bst, int b_mn,
 // dW[e][m, n] = sum over rows r of expert e's segment of dY[r, m] * X[r, n]  (float out).
 int gemm_tc_grouped_wgrad(const Ctx& c, const void* dY, const void* X, float* dW, int rows_cap, int m, int n, int experts,
                           const int* seg_start);
-// The same on CTA pairs (tcgen05 cta_group::2, 256 x 256 tiles): A contiguous along k, no split.
-int gemm_tc2_strided(const Ctx& c, const void* A, long a_rs, long a_cs, const void* B, long b_rs, long b_cs, void* C,
-                     int out_is_float, int m, int n, int k, const GemmEpilogue& e);
+// The same on CTA pairs (tcgen05 cta_group::2, 256 x 256 tiles): both operands along k, bf16 output, no split.
+int gemm_tc2(const Ctx& c, const void* A, long lda, const void* B, long ldb, void* C, int m, int n, int k, const GemmEpilogue& e);
 // Products of few tiles (A along k; B along k, or along n when b_mn): k split over clusters.  -1: not a product for it.
 int gemm_tc_small(const Ctx& c, const void* A, long lda, const void* B, long ldb, int b_mn, void* C, int out_is_float, int m, int n, int k,
                   const GemmEpilogue& e);

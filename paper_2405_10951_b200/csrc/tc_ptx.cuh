@@ -60,12 +60,6 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
       "l"(map), "r"(bar), "r"(c0), "r"(c1)
       : "memory");
 }
-__device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1, int c2) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];" ::"r"(dst),
-      "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2)
-      : "memory");
-}
 
 __device__ __forceinline__ void tmem_alloc(uint32_t smem_dst, uint32_t cols) {
   asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_dst), "r"(cols) : "memory");
@@ -183,9 +177,6 @@ EncodeFn encode_fn();
 // 2-D bf16 tensor map with 128-byte swizzle: `inner` contiguous elements per row, `outer` rows `ld` elements apart,
 // box {64, box_outer}.
 bool make_map(CUtensorMap* map, const void* ptr, uint64_t inner, uint64_t outer, uint64_t ld, uint32_t box_outer);
-// MN-major operand as 64-element chunks: dims {64, outer, extent / 64}, box {64, 64, box_chunks}: one copy fills box_chunks chunks
-// of [64 k-rows][128 bytes].  `extent` (contiguous) must be a multiple of 64.
-bool make_map_chunks(CUtensorMap* map, const void* ptr, uint64_t extent, uint64_t outer, uint64_t ld, uint32_t box_chunks);
 // The same for 8-bit elements: rows of `inner` bytes `ld` bytes apart, box {128 bytes, box_outer rows}.
 bool make_map_u8(CUtensorMap* map, const void* ptr, uint64_t inner, uint64_t outer, uint64_t ld, uint32_t box_outer);
 

@@ -109,7 +109,7 @@ def test_fma_contraction_forward_and_backward(m, n, k, dtype, tol):
 @pytest.mark.parametrize("m,n,k", [(129, 64, 64), (256, 256, 64), (300, 200, 72), (19200, 768, 128), (18944, 2304, 64), (12001, 2048, 192), (12800, 2056, 64)])
 def test_linear_on_cta_pairs(m, n, k):
     """The CTA-pair kernel at remainders of its 256-row tiles and with a last wave cut into parts of 64 to 256 columns: forward with
-    bias, GELU and residual, and the input gradient (B read across k).  One bf16 rounding of the output."""
+    bias, GELU and residual; the gradients, which CTA pairs do not take, as with single CTAs.  One bf16 rounding of the output."""
     import torch
     from paper_2405_10951_b200 import binding as Bd
     gen = torch.Generator(device="cuda").manual_seed(m + n + k)
