@@ -316,14 +316,14 @@ __global__ void moe_combine_bwd_kernel(const float* __restrict__ dout, const flo
 // flight took 23 us for a bias and 40 us for the gate gradient, this 11 and 12 us.
 constexpr int SEG_SPLIT = 8, SEG_U = 4;
 
-template <typename T, bool GATE>
+template <bool GATE>
 __global__ void __launch_bounds__(256)
-moe_seg_sum_kernel(const T* __restrict__ x, const float* __restrict__ dsel_row, const int* __restrict__ row_token,
+moe_seg_sum_kernel(const bf16* __restrict__ x, const float* __restrict__ dsel_row, const int* __restrict__ row_token,
                    const int* __restrict__ seg_start, const int* __restrict__ task_ids, int tokens_per_image, int cols, int E,
                    float* __restrict__ out) {
   namespace cg = cooperative_groups;
   dependent_sync();
-  constexpr int N = Pack<T>::N, W = 32 * N;
+  constexpr int N = Pack<bf16>::N, W = 32 * N;
   __shared__ float sm[8][W];
   __shared__ float part[W];
   cg::cluster_group cluster = cg::this_cluster();
@@ -472,23 +472,22 @@ void moe_combine_bwd(const Ctx& c, const MoeBufs& b, const float* dout, void* do
     launch_k(moe_combine_bwd_kernel<bf16>, blocks, 256, 0, c.stream, dout, b.og, b.row_token, b.row_w, b.seg_start, E, D, (bf16*)dog, dw, rows_cap);
 }
 
-template <typename T, bool GATE>
+// (bf16 only, as expert layers are)
+template <bool GATE>
 static void seg_sum(const Ctx& c, const void* x, const float* dsel_row, const MoeBufs& b, const int* task_ids, int tokens_per_image,
                     int cols, int E, int tasks, float* out) {
   note_launch(1);
-  launch_cluster(moe_seg_sum_kernel<T, GATE>, dim3(ceil_div(cols, 32 * Pack<T>::N), E, tasks * SEG_SPLIT), 256, 0, c.stream, dim3(1, 1, SEG_SPLIT),
-                 (const T*)x, dsel_row, b.row_token, b.seg_start, task_ids, tokens_per_image, cols, E, out);
+  launch_cluster(moe_seg_sum_kernel<GATE>, dim3(ceil_div(cols, 32 * Pack<bf16>::N), E, tasks * SEG_SPLIT), 256, 0, c.stream, dim3(1, 1, SEG_SPLIT),
+                 (const bf16*)x, dsel_row, b.row_token, b.seg_start, task_ids, tokens_per_image, cols, E, out);
 }
 
 void moe_seg_colsum(const Ctx& c, const MoeBufs& b, const void* x, int cols, int E, float* out) {
-  if (c.dtype == 0) seg_sum<float, false>(c, x, nullptr, b, nullptr, 1, cols, E, 1, out);
-  else seg_sum<bf16, false>(c, x, nullptr, b, nullptr, 1, cols, E, 1, out);
+  seg_sum<false>(c, x, nullptr, b, nullptr, 1, cols, E, 1, out);
 }
 
 void moe_gate_wgrad(const Ctx& c, const MoeBufs& b, const float* dsel_row, const int* task_ids, int tokens_per_image, int tasks, int D,
                     int E, float* dwg) {
-  if (c.dtype == 0) seg_sum<float, true>(c, b.xg, dsel_row, b, task_ids, tokens_per_image, D, E, tasks, dwg);
-  else seg_sum<bf16, true>(c, b.xg, dsel_row, b, task_ids, tokens_per_image, D, E, tasks, dwg);
+  seg_sum<true>(c, b.xg, dsel_row, b, task_ids, tokens_per_image, D, E, tasks, dwg);
 }
 
 void moe_gate_bwd(const Ctx& c, const MoeBufs& b, const void* dxg, const float* dw, const void* wg, const int* task_ids,
