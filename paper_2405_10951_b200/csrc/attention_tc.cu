@@ -26,8 +26,6 @@ constexpr int AT_LONG_KB = 64;                   // keys per block of the kernel
 
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
-// Byte offset of element (row, key) in a probability tile stored as 64-key chunks of [128 rows x 128 bytes],
-// 16-byte units XOR-swizzled with the row (the layout TMA produces for a 128-byte-swizzled operand tile).
 __device__ __forceinline__ float fmax3(float a, float b, float c) {
   float d;
   asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
@@ -37,10 +35,6 @@ __device__ __forceinline__ float ex2_fast(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
-}
-__device__ __forceinline__ uint32_t p_offset(int row, int key8) {   // key8: index of a group of 8 keys
-  int chunk = key8 >> 3, unit = key8 & 7;
-  return (uint32_t)(chunk * (AT_QROWS * 128) + row * 128 + ((unit ^ (row & 7)) << 4));
 }
 
 // ------------------------------------------------------------------------------------------------
