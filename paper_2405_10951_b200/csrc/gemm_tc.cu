@@ -40,6 +40,17 @@ constexpr int STAGING_BYTES = 32 * 128;          // per epilogue warp: 32 rows x
 constexpr int SMEM_BYTES = RING_BYTES + EPI_WARPS * STAGING_BYTES + 1024 /*alignment slack*/ + 256 /*barriers*/;
 constexpr int THREADS = 64 + EPI_WARPS * 32;
 constexpr uint32_t TMEM_COLS = 512;
+// Weight gradients (A read along m, float output) reduce over every row of the batch.  The tensor core's accumulator loses up to a
+// bit of its last place with each addition, always towards zero, so that its error grows with their number: 4.8e-6 over 8864
+// rows and 1.4e-5 over 25216, where fp32 FMAs have 1.0e-6 over 8864.  So it only ever holds a few slabs of k: the epilogue warps
+// add them up in registers while the next ones are formed in the other accumulator.
+//   error against 64 bits, sums of    all   8 slabs  4       2       1          us of dX and dW, all   8      4      2      1
+//   1576 x 768 x 768               1.6e-6   4.7e-7   2.3e-7  1.4e-7  1.1e-7                      17.7  18.0   18.6   20.0   22.2
+//   8864 x 2304 x 768              4.8e-6   4.7e-7   2.4e-7  1.6e-7  1.7e-7                      56.4  57.2   57.8   61.2   69.2
+//   25216 x 2304 x 768             1.4e-5   4.8e-7   2.7e-7  2.2e-7  2.6e-7                       141   143    144    153    169
+// Four, then; where few slabs are all there is, FMAs do better than that (200 rows 9.3e-8, four slabs 1.8e-7, one 7.6e-8), and a
+// launch is short anyway: one.
+constexpr int sum_slabs(int k) { return k <= 1024 ? 1 : 4; }
 
 // Instruction descriptor: D = f32, A = B = bf16, M = 128, N = bn, operand majors as given.
 __host__ __device__ constexpr uint32_t make_idesc(bool a_mn, bool b_mn, int bn) {
@@ -84,9 +95,11 @@ __device__ __forceinline__ Work decode_work(int w, int tiles_m, int tiles_n, int
 template <bool A_MN, bool B_MN, typename TOut, int BN, bool FP8 = false, bool EXACT = false>
 __global__ void __launch_bounds__(THREADS, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, TOut* __restrict__ C,
-               int M, int N, int K, Epi ep, int tiles_m, int tiles_n, int splits, int kb_per_split, GemmGroup grp, int* status) {
+               int M, int N, int K, Epi ep, int tiles_m, int tiles_n, int splits, int kb_per_split, int slabs, GemmGroup grp, int* status) {
   constexpr int B_BYTES = BN * BK * 2, STAGE_BYTES = A_BYTES + B_BYTES, STAGES = stages_for(BN);
   constexpr int HALF_CHUNKS = BN / 64;               // 32-column chunks per epilogue warp
+  constexpr bool SUMS = A_MN;                        // a weight gradient: sums of `slabs` slabs, see sum_slabs
+  static_assert(!SUMS || sizeof(TOut) == 4, "weight gradients are float");
   extern __shared__ unsigned char smem_dyn[];
   uint32_t base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
   uint32_t staging0 = base + STAGES * STAGE_BYTES;
@@ -175,31 +188,34 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       for (int w = blockIdx.x; w < work_items && ok; w += gridDim.x) {
         Work wk = decode_work(w, tiles_m, tiles_n, total_kb, kb_per_split, grp, (size_t)M * N);
         if (!wk.active) continue;
-        int kb0 = wk.kb0, kb1 = wk.kb1;
-        int buf = local & 1;
-        if (!mbar_wait(tempty_bar(buf), ((local >> 1) & 1) ^ 1u, abortp)) { ok = false; break; }
-        tc_fence_after();
-        uint32_t d_tmem = tmem_base + buf * BN;
-        for (int kb = kb0; kb < kb1; ++kb) {
-          if (!mbar_wait(full_bar(stage), phase, abortp)) { ok = false; break; }
+        int kb = wk.kb0;
+        do {
+          int buf = local & 1;
+          if (!mbar_wait(tempty_bar(buf), ((local >> 1) & 1) ^ 1u, abortp)) { ok = false; break; }
           tc_fence_after();
-          // descriptors of this stage: only the 16-byte-unit address field (low bits) moves with the stage and the k step
-          uint64_t da = desc_a0 + (uint64_t)((stage * STAGE_BYTES) >> 4), db = desc_b0 + (uint64_t)((stage * STAGE_BYTES) >> 4);
-          if (FP8) {
+          uint32_t d_tmem = tmem_base + buf * BN;
+          const int first = kb, last = SUMS ? min(wk.kb1, kb + slabs) : wk.kb1;
+          for (; kb < last; ++kb) {
+            if (!mbar_wait(full_bar(stage), phase, abortp)) { ok = false; break; }
+            tc_fence_after();
+            // descriptors of this stage: only the 16-byte-unit address field (low bits) moves with the stage and the k step
+            uint64_t da = desc_a0 + (uint64_t)((stage * STAGE_BYTES) >> 4), db = desc_b0 + (uint64_t)((stage * STAGE_BYTES) >> 4);
+            if (FP8) {
 #pragma unroll
-            for (int k = 0; k < BK / UMMA_K; ++k)       // four steps of 32 bytes along k, as for bf16
-              umma_e4m3(d_tmem, da + (uint64_t)(k * A_KSTEP), db + (uint64_t)(k * B_KSTEP), idesc, (kb > kb0 || k > 0) ? 1u : 0u);
-          } else {
-            umma_bf16(d_tmem, da, db, idesc, kb > kb0 ? 1u : 0u);
+              for (int k = 0; k < BK / UMMA_K; ++k)       // four steps of 32 bytes along k, as for bf16
+                umma_e4m3(d_tmem, da + (uint64_t)(k * A_KSTEP), db + (uint64_t)(k * B_KSTEP), idesc, (kb > first || k > 0) ? 1u : 0u);
+            } else {
+              umma_bf16(d_tmem, da, db, idesc, kb > first ? 1u : 0u);
 #pragma unroll
-            for (int k = 1; k < BK / UMMA_K; ++k)
-              umma_bf16_acc(d_tmem, da + (uint64_t)(k * A_KSTEP), db + (uint64_t)(k * B_KSTEP), idesc);
+              for (int k = 1; k < BK / UMMA_K; ++k)
+                umma_bf16_acc(d_tmem, da + (uint64_t)(k * A_KSTEP), db + (uint64_t)(k * B_KSTEP), idesc);
+            }
+            umma_commit(empty_bar(stage));
+            if (++stage == STAGES) { stage = 0; phase ^= 1u; }
           }
-          umma_commit(empty_bar(stage));
-          if (++stage == STAGES) { stage = 0; phase ^= 1u; }
-        }
-        if (ok) umma_commit(tfull_bar(buf));
-        ++local;
+          if (ok) umma_commit(tfull_bar(buf));
+          ++local;
+        } while (ok && kb < wk.kb1);
       }
     }
   } else {
@@ -214,21 +230,50 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       Work wk = decode_work(w, tiles_m, tiles_n, total_kb, kb_per_split, grp, (size_t)M * N);
       if (!wk.active) continue;
       int nt = wk.nt, mt = wk.mt;
-      int buf = local & 1;
+      const uint32_t trow = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(chalf * HALF_CHUNKS * 32);
+      const int row0 = mt * BM + quarter * 32, cb = nt * BN + chalf * HALF_CHUNKS * 32;
       auto ready = [&]() {
-        bool w = mbar_wait(tfull_bar(buf), (local >> 1) & 1, abortp);
+        bool w = mbar_wait(tfull_bar(local & 1), (local >> 1) & 1, abortp);
         w = __all_sync(0xffffffffu, w);
         tc_fence_after();
         return w;
       };
-      ok = epilogue_tile<TOut, FP8, EXACT>(ready, ep, wk.bias_off, C + wk.c_off, M, N, mt * BM + quarter * 32, nt * BN + chalf * HALF_CHUNKS * 32, HALF_CHUNKS,
-                                    tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * BN + chalf * HALF_CHUNKS * 32),
-                                    wk.kb0 >= wk.kb1, st, lane);
-      if (!ok) break;
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(tempty_bar(buf));
-      ++local;
+      auto release = [&]() {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(tempty_bar(local & 1));
+        ++local;
+      };
+      if constexpr (SUMS) {
+        uint32_t sum[HALF_CHUNKS * 32];
+#pragma unroll
+        for (int j = 0; j < HALF_CHUNKS * 32; ++j) sum[j] = 0u;
+        int kb = wk.kb0;
+        do {
+          ok = ready();
+          if (!ok) break;
+          if (kb < wk.kb1) {                             // (an expert without tokens has no slab: its gradient is zero)
+#pragma unroll
+            for (int c0 = 0; c0 < HALF_CHUNKS * 32; c0 += 16) {
+              uint32_t r[16];
+              tmem_ld16(trow + (uint32_t)((local & 1) * BN + c0), r);
+              tmem_ld_wait();
+#pragma unroll
+              for (int j = 0; j < 16; ++j) sum[c0 + j] = __float_as_uint(__uint_as_float(sum[c0 + j]) + __uint_as_float(r[j]));
+            }
+          }
+          release();
+          kb += slabs;
+        } while (kb < wk.kb1);
+        if (!ok) break;
+#pragma unroll
+        for (int cc = 0; cc < HALF_CHUNKS; ++cc)
+          epilogue_chunk_f32(sum + cc * 32, make_float4(0.f, 0.f, 0.f, 0.f), (float*)C + wk.c_off, M, N, row0, cb + cc * 32, st, lane, nullptr, false);
+      } else {
+        ok = epilogue_tile<TOut, FP8, EXACT>(ready, ep, wk.bias_off, C + wk.c_off, M, N, row0, cb, HALF_CHUNKS, trow + (uint32_t)((local & 1) * BN), st, lane);
+        if (!ok) break;
+        release();
+      }
     }
   }
   tc_fence_before();
@@ -355,7 +400,7 @@ static int launch(const Ctx& c, const CUtensorMap& ma, const CUtensorMap& mb, vo
   int sms = c.sm_count > 0 ? c.sm_count : 148;
   int grid = work < sms ? work : sms;
   note_launch(1);
-  launch_k(kern, grid, THREADS, SMEM_BYTES, c.stream, ma, mb, (TOut*)C, m, n, k, ep, tiles_m, tiles_n, splits, kb_per_split, grp, c.status);
+  launch_k(kern, grid, THREADS, SMEM_BYTES, c.stream, ma, mb, (TOut*)C, m, n, k, ep, tiles_m, tiles_n, splits, kb_per_split, sum_slabs(k), grp, c.status);
   return 0;
 }
 
@@ -384,7 +429,8 @@ int gemm_tc_strided(const Ctx& c, const void* A, long a_rs, long a_cs, const voi
   if ((lda % 8) != 0 || (ldb % 8) != 0 || ((uintptr_t)A & 15) || ((uintptr_t)B & 15) || ((uintptr_t)C & 15)) return -1;
   if ((n % 8) != 0) return -1;
   if (a_mn && (m % 8) != 0) return -1;
-  if (a_mn && !b_mn) return -1;                 // combination not instantiated
+  const bool plain = e.bias == nullptr && e.residual == nullptr && e.act == 0;
+  if (a_mn && !(b_mn && out_is_float && plain)) return -1;       // a weight gradient, or not instantiated
   if (out_is_float && e.act != 0) return -1;    // activations belong to bf16 outputs
   if (!a_mn) {
     const int rc = gemm_tc_small(c, A, lda, B, ldb, b_mn, C, out_is_float, m, n, k, e);
@@ -393,9 +439,7 @@ int gemm_tc_strided(const Ctx& c, const void* A, long a_rs, long a_cs, const voi
   CUtensorMap ma, mb;
   bool ok = a_mn ? make_map(&ma, A, (uint64_t)m, (uint64_t)k, (uint64_t)lda, BK) : make_map(&ma, A, (uint64_t)k, (uint64_t)m, (uint64_t)lda, BM);
   int sms = c.sm_count > 0 ? c.sm_count : 148;
-  const bool plain = e.bias == nullptr && e.residual == nullptr && e.act == 0;
-  const bool may_split = a_mn && split_ws != nullptr && out_is_float && plain;      // weight gradients, the workspace's only users
-  const Cut cut = choose_tile(m, n, k, a_mn, may_split ? split_ws_floats : 0, sms);
+  const Cut cut = choose_tile(m, n, k, a_mn, a_mn && split_ws != nullptr ? split_ws_floats : 0, sms);      // weight gradients may be split
   const int bn = cut.bn;
   ok = ok && (b_mn ? make_map(&mb, B, (uint64_t)n, (uint64_t)k, (uint64_t)ldb, BK) : make_map(&mb, B, (uint64_t)k, (uint64_t)n, (uint64_t)ldb, bn));
   if (!ok) return -2;
@@ -415,7 +459,7 @@ int gemm_tc_strided(const Ctx& c, const void* A, long a_rs, long a_cs, const voi
     if constexpr (W <= 128)
       if (exact) return b_mn ? go(launch<false, true, bf16, W, false, true>) : go(launch<false, false, bf16, W, false, true>);
     if constexpr (W >= 128)
-      if (a_mn) return out_is_float ? go(launch<true, true, float, W>) : go(launch<true, true, bf16, W>);
+      if (a_mn) return go(launch<true, true, float, W>);
     if (out_is_float) return b_mn ? go(launch<false, true, float, W>) : go(launch<false, false, float, W>);
     return b_mn ? go(launch<false, true, bf16, W>) : go(launch<false, false, bf16, W>);
   };

@@ -240,7 +240,7 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
         return w;
       };
       if (!epilogue_tile<bf16, false, false>(ready, ep, 0, C, M, N, t.mt * (2 * BM) + (int)rank * BM + quarter * 32, t.n0 + chalf * nc * 32, nc,
-                                      tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * BN + chalf * nc * 32), false, st, lane))
+                                      tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * BN + chalf * nc * 32), st, lane))
         break;
       tc_fence_before();
       __syncwarp();

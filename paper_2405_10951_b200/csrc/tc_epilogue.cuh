@@ -355,10 +355,10 @@ __device__ __forceinline__ void chunk_land_bf16(const uint4* x, unsigned char* s
 // waits for the accumulators; what does not depend on them is fetched before: bias and column scales (read where they
 // are added, they came from L2 -- the operand ring leaves hardly any L1 -- and took 900 of the 1700 clocks of a chunk) and
 // the first chunk of the residual or of the stored pre-activation, whose next chunk is always on its way.
-// empty: no products were accumulated (an expert without tokens): the result is zero.  st: this warp's staging buffer, 4 KB.
+// st: this warp's staging buffer, 4 KB.
 template <typename TOut, bool FP8, bool EXACT, typename Ready>
 __device__ __forceinline__ bool epilogue_tile(Ready ready, const Epi& ep, int bias_off, TOut* Cs, int M, int N, int row0, int cb, int nc, uint32_t taddr,
-                                              bool empty, unsigned char* st, int lane) {
+                                              unsigned char* st, int lane) {
   const float* bias = ep.bias == nullptr ? nullptr : ep.bias + bias_off;
   uint4 xn[8];
   if constexpr (sizeof(TOut) == 4) {           // float outputs (never with an activation) are transposed once
@@ -383,10 +383,6 @@ __device__ __forceinline__ bool epilogue_tile(Ready ready, const Epi& ep, int bi
       uint32_t r[32];
       tmem_ld32(taddr + cc * 32, r);
       tmem_ld_wait();
-      if (empty) {
-#pragma unroll
-        for (int j = 0; j < 32; ++j) r[j] = 0u;
-      }
       epilogue_chunk_f32(r, bb, (float*)Cs, M, N, row0, cb + cc * 32, st, lane, xc, has_res);
     }
   } else {
