@@ -63,11 +63,10 @@ def step_bytes(cfg, batch, fp):
     return float(images + fp["weight_bytes"] + 2 * fp["saved_activation_bytes"] + 30 * fp["trainable_params"])
 
 
-# DRAM traffic of the dominant kernel (tcgen05 GEMM), bytes per launch averaged over the GEMM launches of one step
-# (dram__bytes_read.sum + dram__bytes_write.sum of every gemm_tc_kernel launch of the step, divided by their number),
-# from the one-pass ncu launch lists summarised in profiles/launch_list_<workload>_step.txt, taken at the batch sizes
-# bench.py runs.  Absent (null in the output) for a workload whose list has not been taken on the kernel as it stands.
-GEMM_DRAM_BYTES_PER_LAUNCH = {"vit_b": 82634556, "deit_s": 15844225, "moe_vit_s": 21736962}
+# DRAM traffic of the tcgen05 GEMM kernels, bytes per launch averaged over the GEMM launches of one step, by workload.  Empty (null
+# in the output): counters are not collected over whole steps of full-size workloads; profiles/ has the DRAM bytes of single
+# launches of each kernel, and the launch lists of steps there hold durations alone.
+GEMM_DRAM_BYTES_PER_LAUNCH = {}
 
 
 def peaks():
@@ -383,7 +382,7 @@ def main():
                             else "bsr_train_step_host (host buffers in, loss to host memory)")},
             "gpu_launches": int(launches),
             # the dominant kernel: all tcgen05 GEMM launches of a step, each bracketed by CUDA events on the launching stream
-            "roofline": {"bound": "tensor", "kernel": "gemm_tc_kernel (tcgen05 bf16 GEMM, all launches of a step)",
+            "roofline": {"bound": "tensor", "kernel": "tcgen05 GEMM kernels (gemm_tc_kernel, gemm_tc2_kernel, gemm_tc_small_kernel): all launches of a step",
                          "achieved": gemm_tflops, "peak": pk["tflops_burst"], "unit": "TFLOP/s",
                          "frac": gemm_tflops / pk["tflops_burst"], "traffic": traffic,
                          "peak_source": pk["source"] + " burst (cuBLAS bf16 GEMM timed alone); sustained " + f"{pk['tflops']:.0f}",

@@ -16,6 +16,9 @@
  *     the caller keeps ownership of that block and of every input and output buffer;
  *   - bsr_train_step / bsr_eval_forward only enqueue work on `stream` and do not synchronise;
  *     results are in device memory once the stream reaches that point;
+ *   - results are reproducible: the same calls on the same data give the same bits.  In fp32 the logits of an image do not
+ *     depend on the other images of its batch either; in bf16 the number of rows decides how a product is cut, and so the
+ *     order of its fp32 sums, and the logits of an image in different batches agree to what their rounding makes of that;
  *   - tensors are dense row-major; linear weights are [out_features, in_features].
  *
  * Parameter names (bsr_set_param / bsr_get_tensor), L = dim, F = mlp_hidden:
