@@ -125,7 +125,7 @@ static inline void note_launch(int n = 1) { g_kernel_launches += n; }
 // touches global memory only after await_inputs(), and every CTA of every kernel calls it, so completion of a kernel
 // still implies completion of all before it.  A kernel that allocates tensor memory releases only after its allocation:
 // otherwise the next kernel's CTA could take the columns first and wait for this one for good.
-// It saves launch latency and prologue: a DeiT-S step of one image (199 launches) 1072 -> 945 us, of 64 images 1737 -> 1692 us.
+// It saves launch latency and prologue: a DeiT-S step of one image (199 launches) 746 -> 659 us, of 64 images 1572 -> 1492 us.
 // Kernels that fill the SMs with one large CTA each (GEMM, attention) do not release: the next kernel's CTAs would pile up on
 // the SMs whose CTA leaves first instead of spreading over all of them (ViT-B at batch 128: 5336 us without, 5341 us so,
 // 5534 us with a release at their start).  On at most half of the SMs they do: the next kernel finds the others idle.

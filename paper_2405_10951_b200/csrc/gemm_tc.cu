@@ -42,15 +42,19 @@ constexpr int THREADS = 64 + EPI_WARPS * 32;
 constexpr uint32_t TMEM_COLS = 512;
 // Weight gradients (A read along m, float output) reduce over every row of the batch.  The tensor core's accumulator loses up to a
 // bit of its last place with each addition, always towards zero, so that its error grows with their number: 4.8e-6 over 8864
-// rows and 1.4e-5 over 25216, where fp32 FMAs have 1.0e-6 over 8864.  So it only ever holds a few slabs of k: the epilogue warps
-// add them up in registers while the next ones are formed in the other accumulator.
+// rows and 1.4e-5 over 25216.  So it only ever holds a few slabs of k: the epilogue warps add them up in registers while the
+// next ones are formed in the other accumulator.  Longer sums take less time:
 //   error against 64 bits, sums of    all   8 slabs  4       2       1          us of dX and dW, all   8      4      2      1
 //   1576 x 768 x 768               1.6e-6   4.7e-7   2.3e-7  1.4e-7  1.1e-7                      17.7  18.0   18.6   20.0   22.2
 //   8864 x 2304 x 768              4.8e-6   4.7e-7   2.4e-7  1.6e-7  1.7e-7                      56.4  57.2   57.8   61.2   69.2
 //   25216 x 2304 x 768             1.4e-5   4.8e-7   2.7e-7  2.2e-7  2.6e-7                       141   143    144    153    169
-// Four, then; where few slabs are all there is, FMAs do better than that (200 rows 9.3e-8, four slabs 1.8e-7, one 7.6e-8), and a
-// launch is short anyway: one.
-constexpr int sum_slabs(int k) { return k <= 1024 ? 1 : 4; }
+// and the lines lie where the error stays below that of one fp32 FMA after the other, which these sums had before:
+//   rows    200      320      328      1024     1032     4096     4104     8864     25216
+//   FMAs    9.3e-8   1.2e-7   1.2e-7   2.5e-7   2.5e-7   6.1e-7   6.1e-7   1.0e-6   2.0e-6
+//   here    7.6e-8   8.0e-8   1.2e-7   1.3e-7   2.3e-7   2.4e-7   4.5e-7   4.1e-7   4.7e-7
+// (64 rows are one slab: 6.6e-8 against 5.2e-8.)  An expert's rows, never summed by FMAs, stay one sum (64 images, 16 experts:
+// 2154 us a step, 2172 with sums of four slabs).
+constexpr int sum_slabs(int k) { return k <= 320 ? 1 : k <= 1024 ? 2 : k <= 4096 ? 4 : 8; }
 
 // Instruction descriptor: D = f32, A = B = bf16, M = 128, N = bn, operand majors as given.
 __host__ __device__ constexpr uint32_t make_idesc(bool a_mn, bool b_mn, int bn) {
@@ -400,7 +404,7 @@ static int launch(const Ctx& c, const CUtensorMap& ma, const CUtensorMap& mb, vo
   int sms = c.sm_count > 0 ? c.sm_count : 148;
   int grid = work < sms ? work : sms;
   note_launch(1);
-  launch_k(kern, grid, THREADS, SMEM_BYTES, c.stream, ma, mb, (TOut*)C, m, n, k, ep, tiles_m, tiles_n, splits, kb_per_split, sum_slabs(k), grp, c.status);
+  launch_k(kern, grid, THREADS, SMEM_BYTES, c.stream, ma, mb, (TOut*)C, m, n, k, ep, tiles_m, tiles_n, splits, kb_per_split, grp.mode == 2 ? 1 << 20 : sum_slabs(k), grp, c.status);
   return 0;
 }
 
