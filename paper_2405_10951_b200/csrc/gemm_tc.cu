@@ -365,11 +365,17 @@ bool make_map_u8(CUtensorMap* map, const void* ptr, uint64_t inner, uint64_t out
             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// 192 columns instead of 256 where that fills the last wave better.
+static int wave_width(int m, int n, int sms) {
+  const long tm = ceil_div(m, BM);
+  return ceil_div(tm * ceil_div(n, 192), sms) * 192 < ceil_div(tm * ceil_div(n, BN_MAX), sms) * BN_MAX ? 192 : BN_MAX;
+}
+
 // Tile width and number of splits along k (over partial sums in the workspace, reduced by a second kernel).
 // * What fits the SMs in one wave takes the narrowest tiles that still do: its time is latency -- filling the ring, one
 //   epilogue -- and a narrow tile has a short epilogue and room for more slabs in flight (200 x 1152 x 384: 12 CTAs of 192
 //   columns 5.7 us, 36 of 64 columns 4.6 us).
-// * More waves: 192 columns instead of 256 where that fills the last wave better.
+// * More waves: wave_width.
 // * Weight gradients, split where there is a workspace (ws_floats > 0): by estimated time in ns.  A slab costs its bytes at 126 per ns (64 a
 //   clock), a tile 2.5 us to fill and drain; the second kernel costs 3 us and its traffic.
 struct Cut { int bn, splits; };
@@ -391,7 +397,7 @@ static Cut choose_tile(int m, int n, int k, bool a_mn, size_t ws_floats, int sms
   if (tiles(192) <= sms)
     for (int bn = 64; bn <= 192; bn += 64)
       if (tiles(bn) <= sms) return {bn, 1};
-  return {ceil_div(tiles(192), sms) * 192 < ceil_div(tiles(256), sms) * 256 ? 192 : BN_MAX, 1};
+  return {wave_width(m, n, sms), 1};
 }
 
 template <bool A_MN, bool B_MN, typename TOut, int BN = BN_MAX, bool FP8 = false, bool EXACT = false>
@@ -535,7 +541,7 @@ int gemm_tc_e4m3(const Ctx& c, const void* Aq, const float* a_scale, const void*
   if ((k % 16) != 0 || (n % 8) != 0 || ((uintptr_t)Aq & 15) || ((uintptr_t)Bq & 15) || ((uintptr_t)C & 15)) return -1;
   if (a_scale == nullptr || b_scale == nullptr || e.residual != nullptr || e.act == 2) return -1;
   int sms = c.sm_count > 0 ? c.sm_count : 148;
-  const int bn = ceil_div((long)ceil_div(m, BM) * ceil_div(n, 192), sms) * 192 < ceil_div((long)ceil_div(m, BM) * ceil_div(n, 256), sms) * 256 ? 192 : BN_MAX;
+  const int bn = wave_width(m, n, sms);    // (the gradient-free prefix: many rows)
   CUtensorMap ma, mb;
   if (!make_map_u8(&ma, Aq, (uint64_t)k, (uint64_t)m, (uint64_t)k, BM) || !make_map_u8(&mb, Bq, (uint64_t)k, (uint64_t)n, (uint64_t)k, bn)) return -2;
   Epi ep;
