@@ -39,7 +39,7 @@ struct Tensor {
 struct BlockBufs {          // byte offsets into the workspace; filled for frozen (scratch) and trainable (arena) blocks
   size_t x_in, y1, qkv, o, xp_full, xp, y2, z, hh, x_out;
   size_t mean1, rstd1, lse, mean2, rstd2, p, s, kept, dropped;
-  size_t o_cls, xin_cls;    // classification rows of o and of the block input (last block only)
+  size_t o_cls;             // classification rows of o (last block only)
   // MoE blocks: routing tables and expert-ordered buffers
   size_t m_eidx, m_ew, m_pos, m_row_token, m_row_w, m_seg, m_tile, m_cnt, m_off, m_xg, m_zg, m_hg, m_og;
 };
@@ -167,7 +167,7 @@ struct bsr_handle {
   size_t block_saved_bytes[BSR_MAX_DEPTH] = {};
   // scratch
   size_t off_patches = 0, off_emb = 0;
-  size_t off_xn = 0, off_meanf = 0, off_rstdf = 0, off_logits = 0, off_per_image = 0, off_dlogits = 0, off_dxn = 0;
+  size_t off_xn = 0, off_xhat = 0, off_logits = 0, off_per_image = 0, off_dlogits = 0, off_dxn = 0;
   size_t off_dxa = 0, off_dxb = 0, off_dz = 0, off_dy = 0, off_dxg = 0, off_dxp = 0, off_do = 0, off_dqkv = 0;
   size_t off_dxa_c = 0, off_dxb_c = 0, off_dxg_c = 0, off_dxp_c = 0;
   size_t off_escore = 0, off_delta = 0, off_ln_partials = 0, off_cs_partials = 0;
@@ -403,7 +403,6 @@ size_t plan(bsr_handle* h) {
     bb.hh = 0;
     bb.x_out = b.take(Mf * D * 4);
     bb.o_cls = b.take((size_t)Bm * D * es);
-    bb.xin_cls = b.take((size_t)Bm * D * 4);
     if (moe) take_moe(bb, l, s.tf[l]);
     next_in = bb.x_out;
     h->block_saved_bytes[l] = b.off - block0;
@@ -436,7 +435,6 @@ size_t plan(bsr_handle* h) {
     bb.kept = b.take((size_t)Bm * (T0 - 1) * 4);
     bb.dropped = b.take((size_t)Bm * (T0 - 1) * 4);
     bb.o_cls = b.take((size_t)Bm * D * es);
-    bb.xin_cls = b.take((size_t)Bm * D * 4);
     if (d.moe_block_mask != 0) take_moe(bb, 0, T0);          // frozen MoE blocks share one set sized for the longest sequence
     size_t in1 = h->bufs_frozen[1].x_in, out1 = h->bufs_frozen[1].x_out;
     h->bufs_frozen[1] = bb;
@@ -454,8 +452,7 @@ size_t plan(bsr_handle* h) {
     h->off_yq_s = b.take(M0 * 4);
   }
   h->off_xn = b.take((size_t)Bm * D * 4);
-  h->off_meanf = b.take((size_t)Bm * 4);
-  h->off_rstdf = b.take((size_t)Bm * 4);
+  h->off_xhat = b.take((size_t)Bm * D * 4);
   h->off_logits = b.take((size_t)Bm * cmax * 4);
   h->off_per_image = b.take((size_t)Bm * 4);
   h->off_dlogits = b.take((size_t)Bm * cmax * 4);
@@ -575,8 +572,8 @@ int block_forward(bsr_handle* h, const Ctx& c, int l, int B, const BlockBufs& bb
                      h->base + bb.qkv, Ma, 3 * D, D, e1) != 0)
       return set_err(h->err, BSR_ERR_CUDA, "8-bit GEMM set-up failed");
   } else {
-    layernorm_fwd(c, h->at<float>(bb.x_in), D, (const float*)h->wb(l, "norm1.weight"), (const float*)h->wb(l, "norm1.bias"),
-                  h->base + bb.y1, 0, save ? h->at<float>(bb.mean1) : nullptr, save ? h->at<float>(bb.rstd1) : nullptr, Ma, D, d.ln_eps);
+    layernorm_fwd(c, h->at<float>(bb.x_in), (const float*)h->wb(l, "norm1.weight"), (const float*)h->wb(l, "norm1.bias"),
+                  h->base + bb.y1, save ? h->at<float>(bb.mean1) : nullptr, save ? h->at<float>(bb.rstd1) : nullptr, Ma, D, d.ln_eps);
     gemm(c, h->base + bb.y1, D, 1, h->wb(l, "attn.qkv.weight"), D, 1, h->base + bb.qkv, 0, Ma, 3 * D, D, e1);
   }
   size_t es = dtype_size(d.dtype);
@@ -589,18 +586,16 @@ int block_forward(bsr_handle* h, const Ctx& c, int l, int B, const BlockBufs& bb
     if (rc != 0) return set_err(h->err, BSR_ERR_UNSUPPORTED, "attention: %d tokens of head dimension %d do not fit this kernel", Ta, hd);
   }
   const void* proj_in = h->base + bb.o;
-  const void* proj_res = h->base + bb.x_in;
   if (tail) {                  // from here on: B rows
     if (!cls_attn) copy_rows(c.stream, h->base + bb.o, (long)Ta * D * es, h->base + bb.o_cls, (long)D * es, B, (int)(D * es));
-    copy_rows(c.stream, h->base + bb.x_in, (long)Ta * D * 4, h->base + bb.xin_cls, (long)D * 4, B, D * 4);
     proj_in = h->base + bb.o_cls;
-    proj_res = h->base + bb.xin_cls;
     Ma = B;
     Mf = B;
   }
   GemmEpilogue e2;
   e2.bias = (const float*)h->wb(l, "attn.proj.bias");
-  e2.residual = proj_res;
+  e2.residual = h->base + bb.x_in;
+  if (tail) e2.residual_ld = (long)Ta * D;       // its classification rows
   void* xp_dst = h->base + (shrinks ? bb.xp_full : bb.xp);
   gemm(c, proj_in, D, 1, h->wb(l, "attn.proj.weight"), D, 1, xp_dst, 1, Ma, D, D, e2);
   if (is_drop) {
@@ -627,8 +622,8 @@ int block_forward(bsr_handle* h, const Ctx& c, int l, int B, const BlockBufs& bb
     gemm(c, h->base + bb.hh, F, 1, h->wb(l, "mlp.fc2.weight"), F, 1, h->base + bb.x_out, 1, Mf, D, F, q4);
     return BSR_OK;
   }
-  layernorm_fwd(c, h->at<float>(bb.xp), D, (const float*)h->wb(l, "norm2.weight"), (const float*)h->wb(l, "norm2.bias"),
-                h->base + bb.y2, 0, save ? h->at<float>(bb.mean2) : nullptr, save ? h->at<float>(bb.rstd2) : nullptr, Mf, D, d.ln_eps);
+  layernorm_fwd(c, h->at<float>(bb.xp), (const float*)h->wb(l, "norm2.weight"), (const float*)h->wb(l, "norm2.bias"),
+                h->base + bb.y2, save ? h->at<float>(bb.mean2) : nullptr, save ? h->at<float>(bb.rstd2) : nullptr, Mf, D, d.ln_eps);
   if (is_moe(h, l)) {
     // MoE layer in place of the FFN (Section 5.2): route, run the chosen experts as grouped GEMMs, combine
     int E = d.moe_experts, K = d.moe_top_k;
@@ -826,8 +821,8 @@ int block_backward(bsr_handle* h, const Ctx& c, int l, int B, GradStream dxo, Gr
   gemm(c, dz, F, 1, h->wb(l, "mlp.fc1.weight"), 1, D, dy, 0, Mf, D, F, none);
   }
   side_join(cl, 1);
-  layernorm_bwd(c, dy, 0, h->at<float>(bb.xp), D, h->at<float>(bb.mean2), h->at<float>(bb.rstd2),
-                (const float*)h->wb(l, "norm2.weight"), dxo.f, dxg.f, D, shrinks ? nullptr : dxg.c, lnp,
+  layernorm_bwd(c, dy, h->at<float>(bb.xp), h->at<float>(bb.mean2), h->at<float>(bb.rstd2),
+                (const float*)h->wb(l, "norm2.weight"), dxo.f, 1, dxg.f, shrinks ? nullptr : dxg.c, lnp,
                 pg ? h->gb(l, "norm2.weight") : nullptr, pg ? h->gb(l, "norm2.bias") : nullptr, Mf, D,
                 (pg && !shrinks) ? h->gb(l, "attn.proj.bias") : nullptr);   // dx' = dxg here: its column sums are the projection's bias gradient
   if (pg && update) update_half(h, c, cl, l, 1);
@@ -839,7 +834,6 @@ int block_backward(bsr_handle* h, const Ctx& c, int l, int B, GradStream dxo, Gr
   }
   // attention output projection
   bool tail_cls_attn = false;
-  const float* ln1_res = dxp.f;
   if (!tail) {
     if (pg) {
       Ctx w = lane_begin();
@@ -849,7 +843,7 @@ int block_backward(bsr_handle* h, const Ctx& c, int l, int B, GradStream dxo, Gr
     }
     gemm(c, op(dxp), D, 1, h->wb(l, "attn.proj.weight"), 1, D, d_o, 0, Ma, D, D, none);
   } else {
-    // B rows: dO_cls = dx'_cls Wo, dWo = dx'_cls^T o_cls; then both gradients go back into zeroed dense tensors
+    // B rows: dO_cls = dx'_cls Wo, dWo = dx'_cls^T o_cls; the other rows have no gradient
     void* do_cls = h->base + h->off_dy;                      // free at this point
     if (pg) {
       Ctx w = lane_begin();
@@ -866,10 +860,6 @@ int block_backward(bsr_handle* h, const Ctx& c, int l, int B, GradStream dxo, Gr
       cudaMemsetAsync(d_o, 0, (size_t)Mdense * D * es, c.stream);
       copy_rows(c.stream, do_cls, (long)D * es, d_o, (long)Ta * D * es, B, (int)(D * es));
     }
-    float* dense_res = h->at<float>(h->off_dxp);
-    cudaMemsetAsync(dense_res, 0, (size_t)Mdense * D * 4, c.stream);
-    copy_rows(c.stream, dxp.f, (long)D * 4, dense_res, (long)Ta * D * 4, B, D * 4);
-    ln1_res = dense_res;
     Ma = Mdense;
   }
   // the gradient this block hands to block l-1 is that block's output gradient: its column sums are the bias gradient
@@ -889,8 +879,8 @@ int block_backward(bsr_handle* h, const Ctx& c, int l, int B, GradStream dxo, Gr
     side_end(cl, 2);
   }
   gemm(c, dqkv, 3 * D, 1, h->wb(l, "attn.qkv.weight"), 1, D, dy, 0, Ma, D, 3 * D, none);
-  layernorm_bwd(c, dy, 0, h->at<float>(bb.x_in), D, h->at<float>(bb.mean1), h->at<float>(bb.rstd1),
-                (const float*)h->wb(l, "norm1.weight"), ln1_res, need_dxi ? dxi.f : nullptr, D, need_dxi ? dxi.c : nullptr, lnp,
+  layernorm_bwd(c, dy, h->at<float>(bb.x_in), h->at<float>(bb.mean1), h->at<float>(bb.rstd1),
+                (const float*)h->wb(l, "norm1.weight"), dxp.f, tail ? Ta : 1, need_dxi ? dxi.f : nullptr, need_dxi ? dxi.c : nullptr, lnp,
                 pg ? h->gb(l, "norm1.weight") : nullptr, pg ? h->gb(l, "norm1.bias") : nullptr, Ma, D, prev_fc2_bias);
   if (pg && update) update_half(h, c, cl, l, 0);
   return BSR_OK;
@@ -912,6 +902,20 @@ HeadDesc head_desc(bsr_handle* h) {
     hd.db[t] = h->gradp(n + ".bias");
   }
   return hd;
+}
+
+HeadRow head_row(const bsr_handle* h, size_t x_last) {
+  const bsr_dims& d = h->cfg.dims;
+  HeadRow r;
+  r.x = h->at<float>(x_last);
+  r.x_stride = (long)(cls_tail(h, d.depth - 1) ? 1 : h->sched.tf[d.depth - 1]) * d.dim;   // rows per image in the last block's output
+  r.gamma = (const float*)h->w("norm.weight"); r.beta = (const float*)h->w("norm.bias");
+  r.eps = d.ln_eps;
+  r.logits = h->at<float>(h->off_logits); r.dlogits = h->at<float>(h->off_dlogits);
+  r.xn = h->at<float>(h->off_xn); r.xhat = h->at<float>(h->off_xhat);
+  r.per_image = h->at<float>(h->off_per_image); r.dxn = h->at<float>(h->off_dxn);
+  r.dx = nullptr;
+  return r;
 }
 
 // Forward through all blocks.  train: blocks >= t0 write the activation arena.  Returns the offset of the last output.
@@ -1025,12 +1029,9 @@ int32_t bsr_create(const bsr_config* cfg, void* workspace, size_t bytes, bsr_han
     delete h;
     return set_err(g_error, BSR_ERR_UNSUPPORTED, "this library is built for sm_100a only (device is sm_%d%d)", major, minor);
   }
-  // optimiser state and status start at zero; the chunk table is uploaded once
-  cudaMemsetAsync(h->base + h->off_status, 0, 256, 0);
-  cudaMemsetAsync(h->base + h->off_m, 0, h->n_flat * 4, 0);
-  cudaMemsetAsync(h->base + h->off_v, 0, h->n_flat * 4, 0);
-  cudaMemsetAsync(h->base + h->off_grad, 0, h->n_flat * 4, 0);
-  cudaMemsetAsync(h->base + h->off_master, 0, h->n_flat * 4, 0);
+  // Optimiser state and status start at zero, and so does all else: memory that an earlier handle had may still hold its guard
+  // words.  The chunk table is uploaded once.
+  cudaMemsetAsync(h->base, 0, need, 0);
   std::vector<AdamChunk> chunks;
   for (auto& t : h->tensors) {
     if (!t.trainable) continue;
@@ -1066,7 +1067,7 @@ int32_t bsr_create(const bsr_config* cfg, void* workspace, size_t bytes, bsr_han
     if (!ok) { cudaGetLastError(); lane->stream = nullptr; }
   };
   make_lane(&h->side, 3);
-  if (h->t0 < cfg->dims.depth) make_lane(&h->wlane, 3);
+  if (h->t0 < cfg->dims.depth) make_lane(&h->wlane, 4);
   if (update_can_be_early(h, 1)) make_lane(&h->ulane, 0);
   *out = h;
   return BSR_OK;
@@ -1085,8 +1086,8 @@ int32_t bsr_destroy(bsr_handle* h) {
     if (h->copy_stream) cudaStreamDestroy(h->copy_stream);
     for (SideLane* lane : {&h->side, &h->wlane, &h->ulane}) {
       if (lane->fork) cudaEventDestroy(lane->fork);
-      for (int i = 0; i < 3; ++i)
-        if (lane->done[i]) cudaEventDestroy(lane->done[i]);
+      for (cudaEvent_t ev : lane->done)
+        if (ev) cudaEventDestroy(ev);
       if (lane->stream) cudaStreamDestroy(lane->stream);
     }
   }
@@ -1223,42 +1224,38 @@ static int enqueue_step_kernels(bsr_handle* h, const Ctx& c, const void* images,
   size_t x_last = 0;
   rc = forward_all(h, c, images, B, true, &x_last, task_ids, img_offset);
   if (rc != BSR_OK) return rc;
-  int Tl = cls_tail(h, d.depth - 1) ? 1 : h->sched.tf[d.depth - 1];   // rows per image in the last block's output
-  HeadDesc hd = head_desc(h);
-  float* xn = h->at<float>(h->off_xn);
-  layernorm_fwd(c, h->at<float>(x_last), (long)Tl * D, (const float*)h->w("norm.weight"), (const float*)h->w("norm.bias"), xn, 1,
-                h->at<float>(h->off_meanf), h->at<float>(h->off_rstdf), B, D, d.ln_eps);
-  head_fwd(c, hd, xn, task_ids, h->at<float>(h->off_logits), B);
-  cross_entropy(c, hd, h->at<float>(h->off_logits), labels, task_ids, h->at<float>(h->off_per_image), h->at<float>(h->off_dlogits),
-                h->at<float>(h->off_loss), B);
-  if (loss_out != nullptr) cudaMemcpyAsync(loss_out, h->at<float>(h->off_loss), 4, cudaMemcpyDeviceToDevice, c.stream);
   if (kept_out != nullptr && kept_total(h, B) > 0)
     cudaMemcpyAsync(kept_out, h->base + h->off_kept_all, kept_total(h, B) * 4, cudaMemcpyDeviceToDevice, c.stream);
-  // backward: head, final LayerNorm, trainable blocks in reverse, nothing before the earliest one
-  head_bwd(c, hd, xn, h->at<float>(h->off_dlogits), task_ids, h->at<float>(h->off_dxn), B);
-  float* lnp = h->at<float>(h->off_ln_partials);
-  bool bf = d.dtype == BSR_DTYPE_BF16;
+  // head, loss and final LayerNorm forward and backward in one launch; what they sum over the images beside the blocks' backward pass
+  HeadDesc hd = head_desc(h);
+  HeadRow row = head_row(h, x_last);
+  const bool blocks = h->t0 < d.depth, bf = d.dtype == BSR_DTYPE_BF16;
+  GradStream dxo = {blocks ? h->at<float>(h->off_dxa) : nullptr, blocks && bf ? (void*)(h->base + h->off_dxa_c) : nullptr};
+  if (blocks && row.x_stride != D) {                     // only the classification rows of the last block's output receive a gradient
+    cudaMemsetAsync(dxo.f, 0, (size_t)B * row.x_stride * 4, c.stream);
+    if (bf) cudaMemsetAsync(dxo.c, 0, (size_t)B * row.x_stride * es, c.stream);
+  }
+  row.dx = dxo.f;
+  head_chain(c, hd, row, nullptr, labels, task_ids, dxo.c, B);
+  Ctx cl = c;
+  cl.side = lane_of(h, c);
+  {
+    Ctx w = c;
+    w.stream = side_begin(cl);
+    head_grads(w, hd, row, task_ids, h->gradp("norm.weight"), h->gradp("norm.bias"), h->at<float>(h->off_loss), loss_out, B);
+    side_end(cl, 3);
+  }
+  // backward through the trainable blocks in reverse, nothing before the earliest one
   const bool early = with_update && lane_of(h, c) != nullptr && early_update(h, c, B);
-  if (h->t0 < d.depth) {
-    GradStream dxo = {h->at<float>(h->off_dxa), bf ? (void*)(h->base + h->off_dxa_c) : nullptr};
+  if (blocks) {
     GradStream dxi = {h->at<float>(h->off_dxb), bf ? (void*)(h->base + h->off_dxb_c) : nullptr};
-    // only the classification rows of the last block's output receive a gradient
-    cudaMemsetAsync(dxo.f, 0, (size_t)B * Tl * D * 4, c.stream);
-    if (bf) cudaMemsetAsync(dxo.c, 0, (size_t)B * Tl * D * es, c.stream);
-    layernorm_bwd(c, h->at<float>(h->off_dxn), 1, h->at<float>(x_last), (long)Tl * D, h->at<float>(h->off_meanf), h->at<float>(h->off_rstdf),
-                  (const float*)h->w("norm.weight"), nullptr, dxo.f, (long)Tl * D, dxo.c, lnp, h->gradp("norm.weight"), h->gradp("norm.bias"), B, D);
     for (int l = d.depth - 1; l >= h->t0; --l) {
       rc = block_backward(h, c, l, B, dxo, dxi, l > h->t0, task_ids, early);
       if (rc != BSR_OK) return rc;
       GradStream t = dxo; dxo = dxi; dxi = t;
     }
-  } else {
-    layernorm_bwd(c, h->at<float>(h->off_dxn), 1, h->at<float>(x_last), (long)Tl * D, h->at<float>(h->off_meanf), h->at<float>(h->off_rstdf),
-                  (const float*)h->w("norm.weight"), nullptr, nullptr, 0, nullptr, lnp, h->gradp("norm.weight"), h->gradp("norm.bias"), B, D);
   }
   side_join_all(c);                      // every gradient is complete on the main stream from here on
-  Ctx cl = c;
-  cl.side = lane_of(h, c);
   side_join_all(cl);
   if (early) {                           // the blocks are updated or about to be; the final LayerNorm and the heads remain
     enqueue_optimizer(h, c, h->chunk_at[2 * d.depth], h->n_chunks, false);
@@ -1514,13 +1511,8 @@ int32_t bsr_eval_forward(bsr_handle* h, const void* images, const int32_t* task_
     size_t x_last = 0;
     int r = relative ? forward_all(h, c, h->base, batch, false, &x_last, tasks, &io->image_offset) : forward_all(h, c, images, batch, false, &x_last, tasks);
     if (r != BSR_OK) return r;
-    int Tl = cls_tail(h, d.depth - 1) ? 1 : h->sched.tf[d.depth - 1];   // rows per image in the last block's output
-    HeadDesc hd = head_desc(h);
-    float* xn = h->at<float>(h->off_xn);
-    layernorm_fwd(c, h->at<float>(x_last), (long)Tl * d.dim, (const float*)h->w("norm.weight"), (const float*)h->w("norm.bias"), xn, 1,
-                  nullptr, nullptr, batch, d.dim, d.ln_eps);
-    head_fwd(c, hd, xn, tasks, h->at<float>(h->off_logits), batch);
-    eval_end(c.stream, io, h->at<float>(h->off_logits), (size_t)batch * hd.cmax, h->at<int>(h->off_kept_all), kept_total(h, batch));
+    head_chain(c, head_desc(h), head_row(h, x_last), io, nullptr, tasks, nullptr, batch);
+    eval_end(c.stream, io, h->at<int>(h->off_kept_all), kept_total(h, batch));
     return BSR_OK;
   };
   cudaGetLastError();

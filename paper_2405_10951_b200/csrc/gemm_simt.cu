@@ -66,6 +66,7 @@ struct SimtEpi {
   TC* aux_out;
   const T* aux_in;
   int M, N, act;
+  long res_ld;
   // four consecutive columns of one row
   __device__ __forceinline__ void operator()(int gm, int gn, const float* acc) const {
     if (gm >= M) return;
@@ -83,7 +84,7 @@ struct SimtEpi {
         v *= gelu_grad_f(z);
         if (aux_out != nullptr) reinterpret_cast<T*>(aux_out)[o] = from_f<T>(gelu_f(z));     // GELU(z), storage type
       }
-      if (residual != nullptr) v += to_f(residual[o]);
+      if (residual != nullptr) v += to_f(residual[(size_t)gm * res_ld + gn + j]);
       C[o] = from_f<TC>(v);
     }
   }
@@ -193,7 +194,7 @@ static void launch_simt(const Ctx& c, const void* A, long a_rs, long a_cs, const
   splits = ceil_div(k, per) < 1 ? 1 : ceil_div(k, per);
   const long lda = ak ? a_rs : a_cs, ldb = bk ? b_rs : b_cs;
   const size_t quad = 4 * sizeof(T);
-  SimtEpi<T, TC> epi = {(TC*)C, e.bias, (const TC*)e.residual, (TC*)e.aux_out, (const T*)e.aux_in, m, n, e.act};
+  SimtEpi<T, TC> epi = {(TC*)C, e.bias, (const TC*)e.residual, (TC*)e.aux_out, (const T*)e.aux_in, m, n, e.act, e.residual_ld ? e.residual_ld : n};
   launch_cluster(gemm_simt_kernel<T, TC>, dim3(tiles_n, ceil_div(m, SG_BM), splits), SG_THREADS, 0, c.stream, dim3(1, 1, splits), (const T*)A, lda, (int)ak,
                  (int)(lda % 4 == 0 && (uintptr_t)A % quad == 0), (const T*)B, ldb, (int)bk, (int)(ldb % 4 == 0 && (uintptr_t)B % quad == 0), k, per, epi);
 }

@@ -456,7 +456,7 @@ int gemm_tc_strided(const Ctx& c, const void* A, long a_rs, long a_cs, const voi
   const int tiles_m = ceil_div(m, BM), tiles_n = ceil_div(n, bn), total_kb = ceil_div(k, BK);
   const int kb_per_split = ceil_div(total_kb, cut.splits), splits = ceil_div(total_kb, kb_per_split);
   Epi ep;
-  ep.bias = e.bias; ep.residual = e.residual; ep.aux_out = e.aux_out; ep.aux_in = e.aux_in; ep.act = e.act;
+  ep.bias = e.bias; ep.residual = e.residual; ep.res_ld = (int)(e.residual_ld ? e.residual_ld : n); ep.aux_out = e.aux_out; ep.aux_in = e.aux_in; ep.act = e.act;
   const bool exact = !a_mn && e.act != 0 && exact_gelu(m, k);       // (tiles of 64 or 128 columns up to 9472 of them)
   void* dst = (splits > 1) ? (void*)split_ws : C;
   if (splits > 1) side_join(c, 2);         // the previous split sum has read the workspace
@@ -502,7 +502,7 @@ int gemm_tc_grouped_rows(const Ctx& c, const void* A, const void* Bst, int b_mn,
   g.b_stride = b_mn ? k : n;
   g.bias_stride = n;
   Epi ep;
-  ep.bias = e.bias; ep.residual = e.residual; ep.aux_out = e.aux_out; ep.aux_in = e.aux_in; ep.act = e.act;
+  ep.bias = e.bias; ep.residual = e.residual; ep.res_ld = (int)(e.residual_ld ? e.residual_ld : n); ep.aux_out = e.aux_out; ep.aux_in = e.aux_in; ep.act = e.act;
   int tiles_m = rows_cap / BM, tiles_n = ceil_div(n, BN_MAX);
   if (c.prof != nullptr && c.prof->on) c.prof->begin(c.stream, 2.0 * rows_cap * n * (double)k);
   int rc;

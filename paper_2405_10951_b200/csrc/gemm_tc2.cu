@@ -275,7 +275,7 @@ int gemm_tc2(const Ctx& c, const void* A, long lda, const void* B, long ldb, voi
   const int tiles_m = ceil_div(m, 2 * BM), tiles_n = ceil_div(n, BN), pairs = (c.sm_count > 0 ? c.sm_count : B200_SMS) / 2;
   const long work = (long)tiles_m * tiles_n * UNITS;
   tc::Epi ep;
-  ep.bias = e.bias; ep.residual = e.residual; ep.aux_out = e.aux_out; ep.aux_in = e.aux_in; ep.act = e.act;
+  ep.bias = e.bias; ep.residual = e.residual; ep.res_ld = (int)(e.residual_ld ? e.residual_ld : n); ep.aux_out = e.aux_out; ep.aux_in = e.aux_in; ep.act = e.act;
   if (c.prof != nullptr && c.prof->on) c.prof->begin(c.stream, 2.0 * m * n * (double)k);
   note_launch(1);
   launch_k(gemm_tc2_kernel, 2 * (int)(work < pairs ? work : pairs), THREADS, SMEM_BYTES, c.stream, ma, mb, mp, (bf16*)C, m, n, k, ep, tiles_m, tiles_n, c.status);

@@ -131,7 +131,7 @@ gemm_tc_small_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_con
   if (ep.bias != nullptr && col < N) bias = __ldg(reinterpret_cast<const float4*>(ep.bias + col));
 #pragma unroll
   for (int p = 0; p < PASSES; ++p) {
-    if (ep.residual != nullptr && mine(p)) load4(reinterpret_cast<const TOut*>(ep.residual) + at(r0 + p * 16 + sub), res[p]);
+    if (ep.residual != nullptr && mine(p)) load4(reinterpret_cast<const TOut*>(ep.residual) + (size_t)(mt * BM + r0 + p * 16 + sub) * ep.res_ld + col, res[p]);
     if (ep.act == 2 && mine(p)) load4(reinterpret_cast<const bf16*>(ep.aux_in) + at(r0 + p * 16 + sub), z[p]);
   }
 
@@ -242,7 +242,7 @@ int gemm_tc_small(const Ctx& c, const void* A, long lda, const void* B, long ldb
   if (!make_map(&ma, A, (uint64_t)k, (uint64_t)m, (uint64_t)lda, BM)) return -2;
   if (!(b_mn ? make_map(&mb, B, (uint64_t)n, (uint64_t)k, (uint64_t)ldb, BK) : make_map(&mb, B, (uint64_t)k, (uint64_t)n, (uint64_t)ldb, BN))) return -2;
   Epi ep;
-  ep.bias = e.bias; ep.residual = e.residual; ep.aux_out = e.aux_out; ep.aux_in = e.aux_in; ep.act = e.act;
+  ep.bias = e.bias; ep.residual = e.residual; ep.res_ld = (int)(e.residual_ld ? e.residual_ld : n); ep.aux_out = e.aux_out; ep.aux_in = e.aux_in; ep.act = e.act;
   const bool timed = c.prof != nullptr && c.prof->on;
   if (timed) c.prof->begin(c.stream, 2.0 * m * n * (double)k);
   const bool exact = e.act != 0 && exact_gelu(m, k);

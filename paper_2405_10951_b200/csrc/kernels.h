@@ -43,8 +43,8 @@ struct GemmProfile {
 struct SideLane {
   cudaStream_t stream = nullptr;
   cudaEvent_t fork = nullptr;
-  cudaEvent_t done[3] = {nullptr, nullptr, nullptr};   // 0: LayerNorm partials, 1: column-sum partials, 2: split-k workspace
-  bool pending[3] = {false, false, false};
+  cudaEvent_t done[4] = {};   // 0: LayerNorm partials, 1: column-sum partials, 2: split-k workspace, 3: what the step writes once
+  bool pending[4] = {};
 };
 
 struct Ctx {
@@ -67,7 +67,7 @@ inline void side_join(const Ctx& c, int which) {
   }
 }
 inline void side_join_all(const Ctx& c) {
-  for (int w = 0; w < 3; ++w) side_join(c, w);
+  for (int w = 0; w < 4; ++w) side_join(c, w);
 }
 // Stream for a reduction of buffer `which`: the side lane, made to wait for everything enqueued on the main stream so far
 // (the main stream itself when there is no side lane).  side_end marks the reduction as in flight.
@@ -91,18 +91,17 @@ void patchify(const Ctx& c, const void* images, void* patches, int B, int C, int
 void assemble_tokens(const Ctx& c, const void* emb, const float* cls, const float* pos, float* x, int B, int N, int D);
 
 // ---- LayerNorm (the residual stream is float in every configuration) ----------------------------
-// y[r] = LN(x[r]) * g + b for `rows` rows of length D; row r of x starts at x + r * x_stride elements.
-// y takes the storage dtype unless y_is_float.  mean/rstd (optional) receive the row statistics.
-void layernorm_fwd(const Ctx& c, const float* x, long x_stride, const float* g, const float* b, void* y, int y_is_float,
-                   float* mean, float* rstd, int rows, int D, float eps);
-// dx[r] = dres[r] + LN'(dy[r]) (float; rows dx_stride apart); dx_copy (optional, bf16 configurations) receives
+// y[r] = LN(x[r]) * g + b for `rows` rows of length D; y takes the storage dtype.  mean/rstd (optional) receive the row statistics.
+void layernorm_fwd(const Ctx& c, const float* x, const float* g, const float* b, void* y, float* mean, float* rstd, int rows, int D, float eps);
+// dx[r] = dres[r] + LN'(dy[r]) (float); dx_copy (optional, bf16 configurations) receives
 // the same rows in the storage dtype.  Partial sums of dgamma/dbeta go to `partials` ([2][groups][D]) and are
 // reduced in a fixed order; with dx_colsum the column sums of dx (a bias gradient of the layer that produced the
-// normalised input's predecessor) come out of the same pass ([3][groups][D] partials).  dx may be null (only parameter gradients wanted); dres may be null.
-// dy is in the storage dtype, or float [rows, D] when dy_is_float (head path).
-void layernorm_bwd(const Ctx& c, const void* dy, int dy_is_float, const float* x, long x_stride, const float* mean,
-                   const float* rstd, const float* g, const float* dres, float* dx, long dx_stride, void* dx_copy,
-                   float* partials, float* dgamma, float* dbeta, int rows, int D, float* dx_colsum = nullptr);
+// normalised input's predecessor) come out of the same pass ([3][groups][D] partials).  dx may be null (only parameter gradients
+// wanted); dres may be null, and holds only every dres_period-th row (rows 0, dres_period, ... of dx, the others' being zero).
+// dy is in the storage dtype.
+void layernorm_bwd(const Ctx& c, const void* dy, const float* x, const float* mean, const float* rstd, const float* g, const float* dres,
+                   int dres_period, float* dx, void* dx_copy, float* partials, float* dgamma, float* dbeta, int rows, int D,
+                   float* dx_colsum = nullptr);
 int layernorm_bwd_groups(const Ctx& c, int rows);
 
 // ---- column sums (bias gradients) -------------------------------------------------------------
@@ -127,6 +126,7 @@ struct GemmGroup {
 struct GemmEpilogue {
   const float* bias = nullptr;      // [n]
   const void* residual = nullptr;   // [m, n] in the output type, added last
+  long residual_ld = 0;             // elements between its rows (0: n)
   int act = 0;                      // 0 none, 1 GELU (pre-activation optionally stored), 2 multiply by GELU'(aux_in)
   void* aux_out = nullptr;          // act 1: pre-activation [m, n], output type; act 2 (optional): GELU(aux_in) [m, n], storage type
   const void* aux_in = nullptr;     // act 2: pre-activation [m, n], storage type
@@ -210,10 +210,33 @@ struct HeadDesc {
   float* dw[4];           // gradients (float)
   float* db[4];
 };
-void head_fwd(const Ctx& c, const HeadDesc& h, const float* xn, const int* task_ids, float* logits, int B);
-void cross_entropy(const Ctx& c, const HeadDesc& h, const float* logits, const int* labels, const int* task_ids,
-                   float* per_image, float* dlogits, float* loss, int B);
-void head_bwd(const Ctx& c, const HeadDesc& h, const float* xn, const float* dlogits, const int* task_ids, float* dxn, int B);
+// Inference replayed from a graph: what differs from call to call lives in device memory, written before the replay.
+struct EvalIo {
+  long long image_offset;    // elements from the base the captured patch kernel reads from to this call's images
+  float* logits;             // where this call wants its logits ...
+  int* kept;                 // ... and the kept positions (may be null)
+};
+// One image's row through the head and back.  x: the last block's output, rows x_stride apart (dx alike).
+struct HeadRow {
+  const float* x;
+  long x_stride;
+  const float* gamma;     // final LayerNorm
+  const float* beta;
+  float eps;
+  float* logits;          // [B, cmax]
+  float* dlogits;         // [B, cmax] (in inference: scratch for very many classes)
+  // training
+  float* xn;              // [B, D] normalised rows
+  float* xhat;            // [B, D] the same without scale and shift
+  float* per_image;       // [B] loss
+  float* dxn;             // [B, D] gradient of xn
+  float* dx;              // gradient of x (null: not wanted)
+};
+// Final LayerNorm and logits (eval, optional: also to where it says); with labels also the loss, its gradient and that of x
+// (dx_copy, optional: the same rows in bf16).
+void head_chain(const Ctx& c, const HeadDesc& h, const HeadRow& io, const EvalIo* eval, const int* labels, const int* task_ids, void* dx_copy, int B);
+// The sums over images: gradients of the heads and of the final LayerNorm, and the mean loss (to loss and, optionally, loss_copy).
+void head_grads(const Ctx& c, const HeadDesc& h, const HeadRow& io, const int* task_ids, float* dgamma, float* dbeta, float* loss, float* loss_copy, int B);
 
 struct AdamChunk { uint32_t offset; uint32_t count; int64_t shadow; uint32_t decay; uint32_t pad; };
 // scalars (device): learning rate, 1 - beta1^t, 1 - beta2^t of the step being taken.  beside: the update runs next to
@@ -242,14 +265,8 @@ void loop_begin(cudaStream_t s, LoopState* st, float* scalars, const int* labels
 // End of a step: loss_out[i] = loss, counters advance.
 void loop_end(cudaStream_t s, LoopState* st, const float* loss, float* loss_out);
 
-// Inference replayed from a graph: what differs from call to call lives in device memory, written before the replay.
-struct EvalIo {
-  long long image_offset;    // elements from the base the captured patch kernel reads from to this call's images
-  float* logits;             // where this call wants its logits ...
-  int* kept;                 // ... and the kept positions (may be null)
-};
 void eval_begin(cudaStream_t s, EvalIo* io, const EvalIo& value, const int* tasks, int* task_stage, int batch);
-void eval_end(cudaStream_t s, const EvalIo* io, const float* logits, size_t n_logits, const int* kept, size_t n_kept);
+void eval_end(cudaStream_t s, const EvalIo* io, const int* kept, size_t n_kept);
 
 // dst row r = src row r (row_bytes a multiple of 16), independent pitches: gathers / scatters token rows.
 void copy_rows(cudaStream_t s, const void* src, long src_pitch_bytes, void* dst, long dst_pitch_bytes, int rows, int row_bytes);

@@ -111,14 +111,14 @@ void assemble_tokens(const Ctx& c, const void* emb, const float* cls, const floa
 // NCH = 16-byte chunks of the row each lane holds (D <= 128 * NCH); instantiated for 2, 3, 4, 6 and 8.
 
 template <typename TY, int NCH>
-__global__ void layernorm_fwd_kernel(const float* __restrict__ x, long x_stride, const float* __restrict__ g,
+__global__ void layernorm_fwd_kernel(const float* __restrict__ x, const float* __restrict__ g,
                                      const float* __restrict__ b, TY* __restrict__ y, float* __restrict__ mean,
                                      float* __restrict__ rstd, int rows, int D, float eps) {
   dependent_sync();
   int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   int lane = threadIdx.x & 31;
   if (warp >= rows) return;
-  const float* xr = x + (long)warp * x_stride;
+  const float* xr = x + (long)warp * D;
   int chunks = D / 4;
   float v[(NCH * 4)];
   float sum = 0.f;
@@ -163,21 +163,21 @@ __global__ void layernorm_fwd_kernel(const float* __restrict__ x, long x_stride,
 }
 
 template <typename TY>
-static void launch_ln_fwd(const Ctx& c, const float* x, long x_stride, const float* g, const float* b, TY* y, float* mean,
+static void launch_ln_fwd(const Ctx& c, const float* x, const float* g, const float* b, TY* y, float* mean,
                           float* rstd, int rows, int D, float eps) {
   int threads = 256;
   int blocks = ceil_div((long)rows * 32, threads);
   int nch = ceil_div(D, 128);
-#define BSR_LN_FWD(N) launch_k(layernorm_fwd_kernel<TY, N>, blocks, threads, 0, c.stream, x, x_stride, g, b, y, mean, rstd, rows, D, eps)
+#define BSR_LN_FWD(N) launch_k(layernorm_fwd_kernel<TY, N>, blocks, threads, 0, c.stream, x, g, b, y, mean, rstd, rows, D, eps)
   if (nch <= 2) BSR_LN_FWD(2); else if (nch == 3) BSR_LN_FWD(3); else if (nch == 4) BSR_LN_FWD(4); else if (nch <= 6) BSR_LN_FWD(6); else BSR_LN_FWD(8);
 #undef BSR_LN_FWD
 }
 
-void layernorm_fwd(const Ctx& c, const float* x, long x_stride, const float* g, const float* b, void* y, int y_is_float,
-                   float* mean, float* rstd, int rows, int D, float eps) {
+void layernorm_fwd(const Ctx& c, const float* x, const float* g, const float* b, void* y, float* mean, float* rstd, int rows, int D,
+                   float eps) {
   note_launch(1);
-  if (c.dtype == 0 || y_is_float) launch_ln_fwd<float>(c, x, x_stride, g, b, (float*)y, mean, rstd, rows, D, eps);
-  else launch_ln_fwd<bf16>(c, x, x_stride, g, b, (bf16*)y, mean, rstd, rows, D, eps);
+  if (c.dtype == 0) launch_ln_fwd<float>(c, x, g, b, (float*)y, mean, rstd, rows, D, eps);
+  else launch_ln_fwd<bf16>(c, x, g, b, (bf16*)y, mean, rstd, rows, D, eps);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -316,11 +316,11 @@ void layernorm_fwd_e4m3(const Ctx& c, const float* x, long x_stride, const float
 // storage dtype for the GEMMs that consume them.
 constexpr int LNB_WARPS = 8;
 
-template <typename TDY, typename TC, int NCH>
-__global__ void __launch_bounds__(256, 2) layernorm_bwd_kernel(const TDY* __restrict__ dy, const float* __restrict__ x, long x_stride,
+template <typename T, int NCH>
+__global__ void __launch_bounds__(256, 2) layernorm_bwd_kernel(const T* __restrict__ dy, const float* __restrict__ x,
                                      const float* __restrict__ mean, const float* __restrict__ rstd,
-                                     const float* __restrict__ g, const float* __restrict__ dres, float* __restrict__ dx,
-                                     long dx_stride, TC* __restrict__ dx_copy, float* __restrict__ partials, int rows, int D, int nsum) {
+                                     const float* __restrict__ g, const float* __restrict__ dres, int dres_period, float* __restrict__ dx,
+                                     T* __restrict__ dx_copy, float* __restrict__ partials, int rows, int D, int nsum) {
   dependent_sync();
   extern __shared__ float sm[];   // [LNB_WARPS][nsum][D]: dgamma, dbeta and (nsum == 3) the column sums of dx
   int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -338,8 +338,10 @@ __global__ void __launch_bounds__(256, 2) layernorm_bwd_kernel(const TDY* __rest
     }
   }
   for (int r = blockIdx.x * LNB_WARPS + warp; r < rows; r += gridDim.x * LNB_WARPS) {
-    const float* xr = x + (long)r * x_stride;
-    const TDY* dyr = dy + (long)r * D;
+    const float* xr = x + (long)r * D;
+    const T* dyr = dy + (long)r * D;
+    const int rr = r / dres_period;
+    const float* res = dx != nullptr && dres != nullptr && rr * dres_period == r ? dres + (long)rr * D : nullptr;
     float mu = mean[r], rs = rstd[r];
     float xh[(NCH * 4)], dh[(NCH * 4)], o[(NCH * 4)];
 #pragma unroll
@@ -348,7 +350,7 @@ __global__ void __launch_bounds__(256, 2) layernorm_bwd_kernel(const TDY* __rest
       if (ch < chunks) {
         load16(xr + ch * 4, xh + i * 4);
         load4(dyr + ch * 4, dh + i * 4);
-        if (dx != nullptr && dres != nullptr) load16(dres + (long)r * D + ch * 4, o + i * 4);
+        if (res != nullptr) load16(res + ch * 4, o + i * 4);
         else {
 #pragma unroll
           for (int j = 0; j < 4; ++j) o[i * 4 + j] = 0.f;
@@ -384,7 +386,7 @@ __global__ void __launch_bounds__(256, 2) layernorm_bwd_kernel(const TDY* __rest
     s1 = warp_sum(s1) / (float)D;
     s2 = warp_sum(s2) / (float)D;
     if (dx != nullptr) {
-      float* dxr = dx + (long)r * dx_stride;
+      float* dxr = dx + (long)r * D;
 #pragma unroll
       for (int i = 0; i < NCH; ++i) {
         int ch = lane + i * 32;
@@ -392,7 +394,7 @@ __global__ void __launch_bounds__(256, 2) layernorm_bwd_kernel(const TDY* __rest
 #pragma unroll
           for (int j = 0; j < 4; ++j) o[i * 4 + j] += rs * (dh[i * 4 + j] - s1 - xh[i * 4 + j] * s2);
           store16(dxr + ch * 4, o + i * 4);
-          if (dx_copy != nullptr) store4(dx_copy + (long)r * dx_stride + ch * 4, o + i * 4);
+          if (dx_copy != nullptr) store4(dx_copy + (long)r * D + ch * 4, o + i * 4);
           if (nsum == 3) {
             float4 ps = *reinterpret_cast<const float4*>(mine + 2 * D + ch * 4);
             ps.x += o[i * 4]; ps.y += o[i * 4 + 1]; ps.z += o[i * 4 + 2]; ps.w += o[i * 4 + 3];
@@ -441,36 +443,30 @@ int layernorm_bwd_groups(const Ctx& c, int rows) {
   return want < cap ? (want < 1 ? 1 : want) : cap;
 }
 
-template <typename TDY, typename TC>
-static void launch_ln_bwd(const Ctx& c, int groups, size_t smem, const void* dy, const float* x, long x_stride, const float* mean,
-                          const float* rstd, const float* g, const float* dres, float* dx, long dx_stride, void* dx_copy,
-                          float* partials, int rows, int D, int nsum) {
+template <typename T>
+static void launch_ln_bwd(const Ctx& c, int groups, size_t smem, const void* dy, const float* x, const float* mean, const float* rstd,
+                          const float* g, const float* dres, int dres_period, float* dx, void* dx_copy, float* partials, int rows, int D, int nsum) {
   int nch = ceil_div(D, 128);
 #define BSR_LN_BWD(N)                                                                                                   \
   do {                                                                                                                  \
     static SmemLimit lim;                                                                                               \
-    ensure_smem(lim, layernorm_bwd_kernel<TDY, TC, N>, smem);                                                           \
-    launch_k(layernorm_bwd_kernel<TDY, TC, N>, groups, LNB_WARPS * 32, smem, c.stream, (const TDY*)dy, x, x_stride, mean, rstd, g, dres, \
-                                                                                 dx, dx_stride, (TC*)dx_copy, partials, rows, D, nsum); \
+    ensure_smem(lim, layernorm_bwd_kernel<T, N>, smem);                                                                 \
+    launch_k(layernorm_bwd_kernel<T, N>, groups, LNB_WARPS * 32, smem, c.stream, (const T*)dy, x, mean, rstd, g, dres, dres_period, \
+                                                                           dx, (T*)dx_copy, partials, rows, D, nsum);   \
   } while (0)
   if (nch <= 2) BSR_LN_BWD(2); else if (nch == 3) BSR_LN_BWD(3); else if (nch == 4) BSR_LN_BWD(4); else if (nch <= 6) BSR_LN_BWD(6); else BSR_LN_BWD(8);
 #undef BSR_LN_BWD
 }
 
-void layernorm_bwd(const Ctx& c, const void* dy, int dy_is_float, const float* x, long x_stride, const float* mean,
-                   const float* rstd, const float* g, const float* dres, float* dx, long dx_stride, void* dx_copy,
-                   float* partials, float* dgamma, float* dbeta, int rows, int D, float* dx_colsum) {
+void layernorm_bwd(const Ctx& c, const void* dy, const float* x, const float* mean, const float* rstd, const float* g, const float* dres,
+                   int dres_period, float* dx, void* dx_copy, float* partials, float* dgamma, float* dbeta, int rows, int D, float* dx_colsum) {
   note_launch(2);
   int groups = layernorm_bwd_groups(c, rows);
   int nsum = (dx_colsum != nullptr && dx != nullptr) ? 3 : 2;
   size_t smem = (size_t)LNB_WARPS * nsum * D * sizeof(float);
   side_join(c, 0);                                                     // the previous reduction has read the partials
-  if (c.dtype == 0)
-    launch_ln_bwd<float, float>(c, groups, smem, dy, x, x_stride, mean, rstd, g, dres, dx, dx_stride, nullptr, partials, rows, D, nsum);
-  else if (dy_is_float)
-    launch_ln_bwd<float, bf16>(c, groups, smem, dy, x, x_stride, mean, rstd, g, dres, dx, dx_stride, dx_copy, partials, rows, D, nsum);
-  else
-    launch_ln_bwd<bf16, bf16>(c, groups, smem, dy, x, x_stride, mean, rstd, g, dres, dx, dx_stride, dx_copy, partials, rows, D, nsum);
+  if (c.dtype == 0) launch_ln_bwd<float>(c, groups, smem, dy, x, mean, rstd, g, dres, dres_period, dx, nullptr, partials, rows, D, nsum);
+  else launch_ln_bwd<bf16>(c, groups, smem, dy, x, mean, rstd, g, dres, dres_period, dx, dx_copy, partials, rows, D, nsum);
   if (dgamma == nullptr && nsum == 2) return;                          // a frozen block in the gradient path: only dx is wanted
   dim3 grid(ceil_div(D, 16), nsum);
   cudaStream_t rs = side_begin(c);                                     // only the optimiser reads these sums
@@ -549,157 +545,6 @@ void colsum(const Ctx& c, const void* x, int rows, int cols, float* partials, fl
   cudaStream_t rs = side_begin(c);
   launch_k(reduce_partials_kernel, dim3(ceil_div(cols, 16), 1), 256, 0, rs, partials, groups, cols, out, out, nullptr);
   side_end(c, 1);
-}
-
-// ------------------------------------------------------------------------------------------------
-// Classification head on the normalised classification token, cross-entropy, head backward.
-// ------------------------------------------------------------------------------------------------
-struct HeadDev {
-  int num_tasks, cmax, D;
-  int ncls[4];
-  const void* w[4];
-  const float* bias[4];
-  float* dw[4];
-  float* db[4];
-};
-
-template <typename T>
-__global__ void head_fwd_kernel(HeadDev h, const float* __restrict__ xn, const int* __restrict__ task_ids,
-                                float* __restrict__ logits, int B) {
-  dependent_sync();
-  int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (warp >= B * h.cmax) return;
-  int b = warp / h.cmax, cls = warp % h.cmax;
-  int t = task_ids ? task_ids[b] : 0;
-  if (cls >= h.ncls[t]) {
-    if (lane == 0) logits[warp] = -INFINITY;
-    return;
-  }
-  const T* w = (const T*)h.w[t] + (size_t)cls * h.D;
-  const float* xr = xn + (size_t)b * h.D;
-  float s = 0.f;
-  for (int d = lane; d < h.D; d += 32) s += xr[d] * to_f(w[d]);
-  s = warp_sum(s);
-  if (lane == 0) logits[warp] = s + h.bias[t][cls];
-}
-
-static HeadDev to_dev(const HeadDesc& h) {
-  HeadDev d;
-  d.num_tasks = h.num_tasks; d.cmax = h.cmax; d.D = h.D;
-  for (int i = 0; i < 4; ++i) { d.ncls[i] = h.ncls[i]; d.w[i] = h.w[i]; d.bias[i] = h.bias[i]; d.dw[i] = h.dw[i]; d.db[i] = h.db[i]; }
-  return d;
-}
-
-void head_fwd(const Ctx& c, const HeadDesc& h, const float* xn, const int* task_ids, float* logits, int B) {
-  note_launch(1);
-  int threads = 256, blocks = ceil_div((long)B * h.cmax * 32, threads);
-  if (c.dtype == 0) launch_k(head_fwd_kernel<float>, blocks, threads, 0, c.stream, to_dev(h), xn, task_ids, logits, B);
-  else launch_k(head_fwd_kernel<bf16>, blocks, threads, 0, c.stream, to_dev(h), xn, task_ids, logits, B);
-}
-
-// One warp per image: loss_b = logsumexp(logits) - logits[label]; dlogits = (softmax - onehot) / B.
-__global__ void cross_entropy_kernel(HeadDev h, const float* __restrict__ logits, const int* __restrict__ labels,
-                                     const int* __restrict__ task_ids, float* __restrict__ per_image,
-                                     float* __restrict__ dlogits, int B, int* status) {
-  dependent_sync();
-  int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (warp >= B) return;
-  int t = task_ids ? task_ids[warp] : 0;
-  // labels and task ids come from the caller: in every build a value outside its range raises STATUS_CHECK and is
-  // clamped, instead of indexing outside the logits
-  if (t < 0 || t >= h.num_tasks) {
-    if (lane == 0 && status != nullptr) atomicOr(status, STATUS_CHECK);
-    t = 0;
-  }
-  int n = h.ncls[t];
-  const float* lr = logits + (size_t)warp * h.cmax;
-  float mx = -INFINITY;
-  for (int i = lane; i < n; i += 32) mx = fmaxf(mx, lr[i]);
-  mx = warp_max(mx);
-  float se = 0.f;
-  for (int i = lane; i < n; i += 32) se += expf(lr[i] - mx);
-  se = warp_sum(se);
-  int label = labels[warp];
-  if (label < 0 || label >= n) {
-    if (lane == 0 && status != nullptr) atomicOr(status, STATUS_CHECK);
-    label = 0;
-  }
-  float inv = 1.0f / se, invB = 1.0f / (float)B;
-  for (int i = lane; i < h.cmax; i += 32) {
-    float g = 0.f;
-    if (i < n) g = (expf(lr[i] - mx) * inv - (i == label ? 1.f : 0.f)) * invB;
-    dlogits[(size_t)warp * h.cmax + i] = g;
-  }
-  if (lane == 0) per_image[warp] = logf(se) + mx - lr[label];
-}
-
-// Single warp: mean of the per-image losses, lanes stride the images, fixed order.
-__global__ void loss_reduce_kernel(const float* __restrict__ per_image, int B, float* __restrict__ loss, int* status) {
-  dependent_sync();
-  int lane = threadIdx.x;
-  float s = 0.f;
-  for (int i = lane; i < B; i += 32) s += per_image[i];
-  s = warp_sum(s);
-  if (lane == 0) {
-    float l = s / (float)B;
-    *loss = l;
-    if (status != nullptr && !isfinite(l)) atomicOr(status, STATUS_NONFINITE);
-  }
-}
-
-void cross_entropy(const Ctx& c, const HeadDesc& h, const float* logits, const int* labels, const int* task_ids,
-                   float* per_image, float* dlogits, float* loss, int B) {
-  note_launch(2);
-  int threads = 128, blocks = ceil_div((long)B * 32, threads);
-  launch_k(cross_entropy_kernel, blocks, threads, 0, c.stream, to_dev(h), logits, labels, task_ids, per_image, dlogits, B, c.status);
-  launch_k(loss_reduce_kernel, 1, 32, 0, c.stream, per_image, B, loss, c.status);
-}
-
-// dW_t[c, d] = sum_b [task(b) = t] dlogits[b, c] xn[b, d];  db_t[c] = sum_b [..] dlogits[b, c]
-__global__ void head_wgrad_kernel(HeadDev h, const float* __restrict__ xn, const float* __restrict__ dlogits,
-                                  const int* __restrict__ task_ids, int B, int t) {
-  dependent_sync();
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  int n = h.ncls[t];
-  if (i >= n * (h.D + 1)) return;
-  int cls = i / (h.D + 1), d = i % (h.D + 1);
-  // branch-free and unrolled: the loads of eight images are in flight together; the sum still runs in image order
-  float s = 0.f;
-#pragma unroll 8
-  for (int b = 0; b < B; ++b) {
-    int tb = task_ids ? task_ids[b] : 0;
-    float g = (tb == t) ? dlogits[(size_t)b * h.cmax + cls] : 0.f;
-    float x = (d < h.D) ? xn[(size_t)b * h.D + d] : 1.f;
-    s = fmaf(g, x, s);
-  }
-  if (d < h.D) h.dw[t][(size_t)cls * h.D + d] = s;
-  else h.db[t][cls] = s;
-}
-
-template <typename T>
-__global__ void head_dgrad_kernel(HeadDev h, const float* __restrict__ dlogits, const int* __restrict__ task_ids,
-                                  float* __restrict__ dxn, int B) {
-  dependent_sync();
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= B * h.D) return;
-  int b = i / h.D, d = i % h.D;
-  int t = task_ids ? task_ids[b] : 0;
-  const T* w = (const T*)h.w[t];
-  float s = 0.f;
-  for (int cidx = 0; cidx < h.ncls[t]; ++cidx) s += dlogits[(size_t)b * h.cmax + cidx] * to_f(w[(size_t)cidx * h.D + d]);
-  dxn[i] = s;
-}
-
-void head_bwd(const Ctx& c, const HeadDesc& h, const float* xn, const float* dlogits, const int* task_ids, float* dxn, int B) {
-  note_launch(h.num_tasks + 1);
-  HeadDev hd = to_dev(h);
-  for (int t = 0; t < h.num_tasks; ++t) {
-    int total = h.ncls[t] * (h.D + 1);
-    launch_k(head_wgrad_kernel, ceil_div(total, 128), 128, 0, c.stream, hd, xn, dlogits, task_ids, B, t);
-  }
-  int total = B * h.D;
-  if (c.dtype == 0) launch_k(head_dgrad_kernel<float>, ceil_div(total, 128), 128, 0, c.stream, hd, dlogits, task_ids, dxn, B);
-  else launch_k(head_dgrad_kernel<bf16>, ceil_div(total, 128), 128, 0, c.stream, hd, dlogits, task_ids, dxn, B);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -875,23 +720,22 @@ __global__ void eval_begin_kernel(EvalIo* io, EvalIo value, const int* __restric
   if (tasks != nullptr)
     for (int j = threadIdx.x; j < batch; j += blockDim.x) task_stage[j] = tasks[j];
 }
-__global__ void eval_end_kernel(const EvalIo* io, const float* __restrict__ logits, size_t n_logits, const int* __restrict__ kept, size_t n_kept) {
+__global__ void eval_end_kernel(const EvalIo* io, const int* __restrict__ kept, size_t n_kept) {
   dependent_sync();
-  EvalIo out = *io;
+  int* out = io->kept;
   size_t step = (size_t)gridDim.x * blockDim.x, i0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  for (size_t i = i0; i < n_logits; i += step) out.logits[i] = logits[i];
-  if (out.kept != nullptr)
-    for (size_t i = i0; i < n_kept; i += step) out.kept[i] = kept[i];
+  if (out != nullptr)
+    for (size_t i = i0; i < n_kept; i += step) out[i] = kept[i];
 }
 void eval_begin(cudaStream_t s, EvalIo* io, const EvalIo& value, const int* tasks, int* task_stage, int batch) {
   note_launch(1);
   launch_k(eval_begin_kernel, 1, 128, 0, s, io, value, tasks, task_stage, batch);
 }
-void eval_end(cudaStream_t s, const EvalIo* io, const float* logits, size_t n_logits, const int* kept, size_t n_kept) {
+void eval_end(cudaStream_t s, const EvalIo* io, const int* kept, size_t n_kept) {
+  if (n_kept == 0) return;
   note_launch(1);
-  size_t n = n_logits > n_kept ? n_logits : n_kept;
-  int blocks = ceil_div((long)n, 256);
-  launch_k(eval_end_kernel, blocks < 64 ? blocks : 64, 256, 0, s, io, logits, n_logits, kept, n_kept);
+  int blocks = ceil_div((long)n_kept, 256);
+  launch_k(eval_end_kernel, blocks < 64 ? blocks : 64, 256, 0, s, io, kept, n_kept);
 }
 
 // Guard words after every workspace slice: one warp per guard.

@@ -12,6 +12,7 @@ namespace tc {
 struct Epi {
   const float* bias = nullptr;
   const void* residual = nullptr;
+  int res_ld = 0;                   // elements between its rows
   void* aux_out = nullptr;
   const void* aux_in = nullptr;
   int act = 0;
@@ -282,7 +283,7 @@ __device__ __forceinline__ void epilogue_chunk(const uint32_t* r, const Epi& ep,
     }
     if (ep.residual != nullptr) {
       float rr[32];
-      ChunkIO<TOut>::load((const TOut*)ep.residual, N, row0, col0, M, N, st, lane, rr);
+      ChunkIO<TOut>::load((const TOut*)ep.residual, ep.res_ld, row0, col0, M, N, st, lane, rr);
 #pragma unroll
       for (int j = 0; j < 32; ++j) v[j] += rr[j];
     }
@@ -368,7 +369,7 @@ __device__ __forceinline__ bool epilogue_tile(Ready ready, const Epi& ep, int bi
       return bias != nullptr && col < N ? __ldg(reinterpret_cast<const float4*>(bias + col)) : make_float4(0.f, 0.f, 0.f, 0.f);
     };
     float4 bn = bias4(0);
-    if (has_res) chunk_issue((const float*)ep.residual, N, row0, cb, M, N, lane, xn);
+    if (has_res) chunk_issue((const float*)ep.residual, ep.res_ld, row0, cb, M, N, lane, xn);
     if (!ready()) return false;
 #pragma unroll 1
     for (int cc = 0; cc < nc; ++cc) {
@@ -378,7 +379,7 @@ __device__ __forceinline__ bool epilogue_tile(Ready ready, const Epi& ep, int bi
       const float4 bb = bn;
       if (cc + 1 < nc) {
         bn = bias4(cc + 1);
-        if (has_res) chunk_issue((const float*)ep.residual, N, row0, cb + (cc + 1) * 32, M, N, lane, xn);
+        if (has_res) chunk_issue((const float*)ep.residual, ep.res_ld, row0, cb + (cc + 1) * 32, M, N, lane, xn);
       }
       uint32_t r[32];
       tmem_ld32(taddr + cc * 32, r);

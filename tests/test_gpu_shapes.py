@@ -364,3 +364,14 @@ def test_weight_gradients_are_summed_to_fp32(m, n, k, mean):
     for ws in (None, torch.empty(160 * 128 * 256, device="cuda")):
         _, dw = Bd.bsr_linear_backward(x, w, dy, use_tensor_cores=True, workspace=ws)
         assert float((dw.double() - want).norm() / want.norm()) < (additions + 10) * 2 ** -24
+
+
+@pytest.mark.parametrize("drop", [(), (2,)])
+@pytest.mark.parametrize("classes,dim,batch", [((1,), 64, 2), ((16, 31, 33), 64, 7), ((32, 100), 1024, 33), ((9000,), 128, 3), ((10,), 8, 1)])
+def test_head_over_numbers_of_classes(classes, dim, batch, drop):
+    """One, two, four and eight CTAs an image, slices beyond shared memory, several tasks, narrow and wide rows; with a drop location in the
+    last block the head reads one row of many."""
+    cfg = Config("mini_head", 16, 4, dim, max(1, dim // 64), 3, 2 * dim, classes, batch, (1, 2), drop, 1, 2, dtype="fp32", seed=len(classes))
+    images, labels, task_ids, params = synth.make_workload(cfg, peaked=dim >= 64)
+    gpu = P.run_gpu_step(cfg, images, labels, task_ids, params)
+    P.compare_step(cfg, images, labels, task_ids, params, gpu, P.FP32_TOL, P.EXACT_MARGIN, P.FP32_TOL)
