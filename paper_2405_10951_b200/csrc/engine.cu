@@ -38,7 +38,7 @@ struct Tensor {
 
 struct BlockBufs {          // byte offsets into the workspace; filled for frozen (scratch) and trainable (arena) blocks
   size_t x_in, y1, qkv, o, xp_full, xp, y2, z, hh, x_out;
-  size_t mean1, rstd1, lse, mean2, rstd2, p, s, kept, dropped;
+  size_t mean1, rstd1, lse, mean2, rstd2, p, s, dropped;
   size_t o_cls;             // classification rows of o (last block only)
   // MoE blocks: routing tables and expert-ordered buffers
   size_t m_eidx, m_ew, m_pos, m_row_token, m_row_w, m_seg, m_tile, m_cnt, m_off, m_xg, m_zg, m_hg, m_og;
@@ -393,7 +393,6 @@ size_t plan(bsr_handle* h) {
     if (s.k[l] >= 0) {
       bb.p = b.take((size_t)Bm * H * (s.ta[l] - 1) * 4);
       bb.s = h->score_rec[l];
-      bb.kept = b.take((size_t)Bm * (s.ta[l] - 1) * 4);
       bb.dropped = b.take((size_t)Bm * (s.ta[l] - 1) * 4);
     }
     bb.mean2 = b.take(Mf * 4); bb.rstd2 = b.take(Mf * 4);
@@ -432,7 +431,6 @@ size_t plan(bsr_handle* h) {
     bb.hh = b.take(M0 * F * es);
     bb.p = b.take((size_t)Bm * H * (T0 - 1) * 4);
     bb.s = b.take((size_t)Bm * (T0 - 1) * 4);
-    bb.kept = b.take((size_t)Bm * (T0 - 1) * 4);
     bb.dropped = b.take((size_t)Bm * (T0 - 1) * 4);
     bb.o_cls = b.take((size_t)Bm * D * es);
     if (d.moe_block_mask != 0) take_moe(bb, 0, T0);          // frozen MoE blocks share one set sized for the longest sequence
@@ -551,7 +549,8 @@ MoeBufs moe_bufs(const bsr_handle* h, const BlockBufs& bb) {
   return m;
 }
 
-int block_forward(bsr_handle* h, const Ctx& c, int l, int B, const BlockBufs& bb, bool save, int* kept_out, const int* task_ids) {
+// kept: the library's copy of the positions this block keeps, kept_copy: the caller's.
+int block_forward(bsr_handle* h, const Ctx& c, int l, int B, const BlockBufs& bb, bool save, int* kept, KeptCopy kept_copy, const int* task_ids) {
   const bsr_dims& d = h->cfg.dims;
   const Schedule& s = h->sched;
   int D = d.dim, F = d.mlp_hidden, H = d.heads, hd = D / H;
@@ -559,8 +558,6 @@ int block_forward(bsr_handle* h, const Ctx& c, int l, int B, const BlockBufs& bb
   int Ma = B * Ta, Mf = B * Tf;
   bool is_drop = k >= 0;
   bool shrinks = is_drop && Tf != Ta;
-  Ctx cf = c;                // the residual stream is float whatever the storage dtype
-  cf.dtype = 0;
   // gradient-free prefix with 8-bit operands: the LayerNorm output leaves as E4M3 rows and meets the E4M3 weight copy
   const bool fp8 = !save && l < h->t0 && h->cfg.frozen_fp8 && h->q_qkv[l] != 0 && c.use_tc;
   GemmEpilogue e1;
@@ -598,18 +595,27 @@ int block_forward(bsr_handle* h, const Ctx& c, int l, int B, const BlockBufs& bb
   if (tail) e2.residual_ld = (long)Ta * D;       // its classification rows
   void* xp_dst = h->base + (shrinks ? bb.xp_full : bb.xp);
   gemm(c, proj_in, D, 1, h->wb(l, "attn.proj.weight"), D, 1, xp_dst, 1, Ma, D, D, e2);
+  const float *g2 = (const float*)h->wb(l, "norm2.weight"), *b2 = (const float*)h->wb(l, "norm2.bias");
+  float *mean2 = save ? h->at<float>(bb.mean2) : nullptr, *rstd2 = save ? h->at<float>(bb.rstd2) : nullptr;
+  const bool fp8_ffn = fp8 && !is_moe(h, l);
+  bool normed = false;         // the second LayerNorm's output is there already
   if (is_drop) {
     int M = Ta - 1;
-    token_select(c.stream, h->at<float>(bb.p), B, H, M, k, h->at<float>(bb.s), h->at<int>(bb.kept), h->at<int>(bb.dropped));
-    if (kept_out != nullptr)
-      cudaMemcpyAsync(kept_out, h->base + bb.kept, (size_t)B * k * sizeof(int), cudaMemcpyDeviceToDevice, c.stream);
-    if (shrinks)
-      gather_fuse(cf, h->base + bb.xp_full, B, M, D, k, h->at<int>(bb.kept), h->at<int>(bb.dropped), h->at<float>(bb.s),
-                  h->cfg.fuse_mode, h->base + bb.xp);
+    const float* p = h->at<float>(bb.p);
+    float* scores = h->at<float>(bb.s);
+    int* dropped = h->at<int>(bb.dropped);
+    if (shrinks && select_gather(c, p, h->at<float>(bb.xp_full), B, H, M, D, k, h->cfg.fuse_mode, scores, kept, dropped, kept_copy, h->at<float>(bb.xp),
+                                 g2, b2, fp8_ffn ? nullptr : h->base + bb.y2, mean2, rstd2, d.ln_eps) == 0) {
+      normed = !fp8_ffn;
+    } else {
+      token_select(c.stream, p, B, H, M, k, scores, kept, dropped, kept_copy);
+      Ctx cf = c;              // the residual stream is float whatever the storage dtype
+      cf.dtype = 0;
+      if (shrinks) gather_fuse(cf, h->base + bb.xp_full, B, M, D, k, kept, dropped, scores, h->cfg.fuse_mode, h->base + bb.xp);
+    }
   }
-  if (fp8 && !is_moe(h, l)) {
-    layernorm_fwd_e4m3(c, h->at<float>(bb.xp), D, (const float*)h->wb(l, "norm2.weight"), (const float*)h->wb(l, "norm2.bias"),
-                       h->base + h->off_yq, h->at<float>(h->off_yq_s), Mf, D, d.ln_eps);
+  if (fp8_ffn) {
+    layernorm_fwd_e4m3(c, h->at<float>(bb.xp), D, g2, b2, h->base + h->off_yq, h->at<float>(h->off_yq_s), Mf, D, d.ln_eps);
     GemmEpilogue q3;
     q3.bias = (const float*)h->wb(l, "mlp.fc1.bias");
     q3.act = 1;
@@ -622,8 +628,7 @@ int block_forward(bsr_handle* h, const Ctx& c, int l, int B, const BlockBufs& bb
     gemm(c, h->base + bb.hh, F, 1, h->wb(l, "mlp.fc2.weight"), F, 1, h->base + bb.x_out, 1, Mf, D, F, q4);
     return BSR_OK;
   }
-  layernorm_fwd(c, h->at<float>(bb.xp), (const float*)h->wb(l, "norm2.weight"), (const float*)h->wb(l, "norm2.bias"),
-                h->base + bb.y2, save ? h->at<float>(bb.mean2) : nullptr, save ? h->at<float>(bb.rstd2) : nullptr, Mf, D, d.ln_eps);
+  if (!normed) layernorm_fwd(c, h->at<float>(bb.xp), g2, b2, h->base + bb.y2, mean2, rstd2, Mf, D, d.ln_eps);
   if (is_moe(h, l)) {
     // MoE layer in place of the FFN (Section 5.2): route, run the chosen experts as grouped GEMMs, combine
     int E = d.moe_experts, K = d.moe_top_k;
@@ -663,6 +668,14 @@ int block_forward(bsr_handle* h, const Ctx& c, int l, int B, const BlockBufs& bb
   e4.residual = h->base + bb.xp;
   gemm(c, h->base + bb.hh, F, 1, h->wb(l, "mlp.fc2.weight"), F, 1, h->base + bb.x_out, 1, Mf, D, F, e4);
   return BSR_OK;
+}
+
+// Kept positions recorded before block l's.
+size_t kept_before(const bsr_handle* h, int B, int l) {
+  size_t n = 0;
+  for (int i = 0; i < l; ++i)
+    if (h->sched.k[i] >= 0) n += (size_t)B * h->sched.k[i];
+  return n;
 }
 
 // Backward of one trainable block (Eq. 2-5).  dxo: gradient at the block output [B*Tf, D]; dxi receives the
@@ -741,6 +754,7 @@ int block_backward(bsr_handle* h, const Ctx& c, int l, int B, GradStream dxo, Gr
   int Ta = s.ta[l], Tf = s.tf[l], k = s.k[l];
   int Ma = B * Ta, Mf = B * Tf;
   bool shrinks = k >= 0 && Tf != Ta;
+  const int* kept = h->at<int>(h->off_kept_all) + kept_before(h, B, l);
   bool bf = d.dtype == BSR_DTYPE_BF16;
   bool tail = cls_tail(h, l);
   bool pg = (h->cfg.trainable_mask >> l) & 1u;     // a frozen block inside the gradient path only passes gradients on (Eq. 2)
@@ -828,7 +842,7 @@ int block_backward(bsr_handle* h, const Ctx& c, int l, int B, GradStream dxo, Gr
   if (pg && update) update_half(h, c, cl, l, 1);
   const float* cls_extra = nullptr;
   if (shrinks) {
-    gather_fuse_bwd(c, dxg.f, h->base + bb.xp_full, B, Ta - 1, D, k, h->at<int>(bb.kept), h->at<int>(bb.dropped),
+    gather_fuse_bwd(c, dxg.f, h->base + bb.xp_full, B, Ta - 1, D, k, kept, h->at<int>(bb.dropped),
                     h->at<float>(bb.s), h->cfg.fuse_mode, dxp.f, dxp.c, h->at<float>(h->off_escore), h->base + bb.xp);
     if (h->cfg.fuse_mode != BSR_FUSE_NONE) cls_extra = h->at<float>(h->off_escore);
   }
@@ -919,7 +933,8 @@ HeadRow head_row(const bsr_handle* h, size_t x_last) {
 }
 
 // Forward through all blocks.  train: blocks >= t0 write the activation arena.  Returns the offset of the last output.
-int forward_all(bsr_handle* h, const Ctx& c, const void* images, int B, bool train, size_t* x_last_off, const int* task_ids,
+// kept_copy: where the caller wants the kept positions (the library's own copy apart).
+int forward_all(bsr_handle* h, const Ctx& c, const void* images, int B, bool train, size_t* x_last_off, const int* task_ids, KeptCopy kept_copy,
                 const long long* img_offset = nullptr) {
   const bsr_dims& d = h->cfg.dims;
   int D = d.dim;
@@ -932,8 +947,6 @@ int forward_all(bsr_handle* h, const Ctx& c, const void* images, int B, bool tra
   int first_train = train ? h->t0 : d.depth;
   size_t x0 = (first_train == 0) ? h->bufs_train[0].x_in : h->bufs_frozen[0].x_in;
   assemble_tokens(c, h->base + h->off_emb, (const float*)h->w("cls_token"), (const float*)h->w("pos_embed"), h->at<float>(x0), B, N, D);
-  int* kept_all = h->at<int>(h->off_kept_all);
-  size_t kept_off = 0;
   size_t cur = x0;
   for (int l = 0; l < d.depth; ++l) {
     BlockBufs bb;
@@ -947,9 +960,11 @@ int forward_all(bsr_handle* h, const Ctx& c, const void* images, int B, bool tra
     bb.x_in = cur;
     if (is_moe(h, l)) { bb.m_eidx = h->moe_rec_eidx[l]; bb.m_ew = h->moe_rec_ew[l]; }
     if (h->sched.k[l] >= 0) bb.s = h->score_rec[l];
-    int* kept_dst = nullptr;
-    if (h->sched.k[l] >= 0) { kept_dst = kept_all + kept_off; kept_off += (size_t)B * h->sched.k[l]; }
-    int rc = block_forward(h, c, l, B, bb, save, kept_dst, task_ids);
+    const size_t kept_off = kept_before(h, B, l);
+    KeptCopy kc = kept_copy;
+    if (kc.dst != nullptr) kc.dst += kept_off;
+    kc.off = kept_off;
+    int rc = block_forward(h, c, l, B, bb, save, h->at<int>(h->off_kept_all) + kept_off, kc, task_ids);
     if (rc != BSR_OK) return rc;
     cur = bb.x_out;
   }
@@ -957,12 +972,7 @@ int forward_all(bsr_handle* h, const Ctx& c, const void* images, int B, bool tra
   return BSR_OK;
 }
 
-size_t kept_total(const bsr_handle* h, int B) {
-  size_t n = 0;
-  for (int l = 0; l < h->cfg.dims.depth; ++l)
-    if (h->sched.k[l] >= 0) n += (size_t)B * h->sched.k[l];
-  return n;
-}
+size_t kept_total(const bsr_handle* h, int B) { return kept_before(h, B, h->cfg.dims.depth); }
 
 int check_batch(bsr_handle* h, const void* images, int batch) {
   if (h == nullptr) return set_err(g_error, BSR_ERR_INVALID_ARG, "handle is null");
@@ -1222,10 +1232,10 @@ static int enqueue_step_kernels(bsr_handle* h, const Ctx& c, const void* images,
   int D = d.dim, B = batch;
   size_t es = dtype_size(d.dtype);
   size_t x_last = 0;
-  rc = forward_all(h, c, images, B, true, &x_last, task_ids, img_offset);
+  KeptCopy kept_copy;
+  kept_copy.dst = kept_out;
+  rc = forward_all(h, c, images, B, true, &x_last, task_ids, kept_copy, img_offset);
   if (rc != BSR_OK) return rc;
-  if (kept_out != nullptr && kept_total(h, B) > 0)
-    cudaMemcpyAsync(kept_out, h->base + h->off_kept_all, kept_total(h, B) * 4, cudaMemcpyDeviceToDevice, c.stream);
   // head, loss and final LayerNorm forward and backward in one launch; what they sum over the images beside the blocks' backward pass
   HeadDesc hd = head_desc(h);
   HeadRow row = head_row(h, x_last);
@@ -1509,10 +1519,11 @@ int32_t bsr_eval_forward(bsr_handle* h, const void* images, const int32_t* task_
   auto enqueue = [&](cudaStream_t s) -> int {
     Ctx c = make_ctx(h, s);
     size_t x_last = 0;
-    int r = relative ? forward_all(h, c, h->base, batch, false, &x_last, tasks, &io->image_offset) : forward_all(h, c, images, batch, false, &x_last, tasks);
+    KeptCopy kept_copy;
+    kept_copy.eval = io;
+    int r = relative ? forward_all(h, c, h->base, batch, false, &x_last, tasks, kept_copy, &io->image_offset) : forward_all(h, c, images, batch, false, &x_last, tasks, kept_copy);
     if (r != BSR_OK) return r;
     head_chain(c, head_desc(h), head_row(h, x_last), io, nullptr, tasks, nullptr, batch);
-    eval_end(c.stream, io, h->at<int>(h->off_kept_all), kept_total(h, batch));
     return BSR_OK;
   };
   cudaGetLastError();

@@ -190,9 +190,25 @@ int attention_cls_fwd(const Ctx& c, const void* qkv, void* out_cls, int B, int T
 int attention_cls_bwd(const Ctx& c, const void* qkv, const void* dout_cls, void* dqkv, int B, int T, int H, int d);
 
 // ---- token selection --------------------------------------------------------------------------
-void token_select(cudaStream_t s, const float* p, int B, int H, int M, int k, float* scores, int* kept, int* dropped);
+// Inference replayed from a graph: what differs from call to call lives in device memory, written before the replay.
+struct EvalIo {
+  long long image_offset;    // elements from the base the captured patch kernel reads from to this call's images
+  float* logits;             // where this call wants its logits ...
+  int* kept;                 // ... and the kept positions (may be null)
+};
+// Where the caller wants a drop location's kept positions beside the library's own copy: `dst`, or `off` positions into what `eval` names.
+struct KeptCopy {
+  int* dst = nullptr;
+  const EvalIo* eval = nullptr;
+  size_t off = 0;
+};
+void token_select(cudaStream_t s, const float* p, int B, int H, int M, int k, float* scores, int* kept, int* dropped, KeptCopy copy = KeptCopy());
 void gather_fuse(const Ctx& c, const void* x, int B, int M, int D, int k, const int* kept, const int* dropped,
                  const float* scores, int fuse, void* out);
+// Selection, compaction and the LayerNorm of the compacted rows in one launch (float rows, k < M): out [B, 1+k+f, D]; with y
+// also its LayerNorm in the storage dtype (mean, rstd optional).  Non-zero when it does not take the problem.
+int select_gather(const Ctx& c, const float* p, const float* x, int B, int H, int M, int D, int k, int fuse, float* scores, int* kept, int* dropped,
+                  KeptCopy copy, float* out, const float* g, const float* b, void* y, float* mean, float* rstd, float eps);
 // Backward of the compaction: dx [B, 1+M, D] from dout [B, 1+k+f, D]; escore [B, M] = gradient arriving at the fusion
 // weight of each dropped token (<g_fused, x_j> for the weighted sum), 0 for kept ones.  fuse: 0 none, 1 weighted sum,
 // 2 weighted mean (needs fwd_out, the forward pass's compacted tensor [B, 1+k+1, D] float, for the fused row).
@@ -209,12 +225,6 @@ struct HeadDesc {
   const float* bias[4];
   float* dw[4];           // gradients (float)
   float* db[4];
-};
-// Inference replayed from a graph: what differs from call to call lives in device memory, written before the replay.
-struct EvalIo {
-  long long image_offset;    // elements from the base the captured patch kernel reads from to this call's images
-  float* logits;             // where this call wants its logits ...
-  int* kept;                 // ... and the kept positions (may be null)
 };
 // One image's row through the head and back.  x: the last block's output, rows x_stride apart (dx alike).
 struct HeadRow {
@@ -266,7 +276,6 @@ void loop_begin(cudaStream_t s, LoopState* st, float* scalars, const int* labels
 void loop_end(cudaStream_t s, LoopState* st, const float* loss, float* loss_out);
 
 void eval_begin(cudaStream_t s, EvalIo* io, const EvalIo& value, const int* tasks, int* task_stage, int batch);
-void eval_end(cudaStream_t s, const EvalIo* io, const int* kept, size_t n_kept);
 
 // dst row r = src row r (row_bytes a multiple of 16), independent pitches: gathers / scatters token rows.
 void copy_rows(cudaStream_t s, const void* src, long src_pitch_bytes, void* dst, long dst_pitch_bytes, int rows, int row_bytes);

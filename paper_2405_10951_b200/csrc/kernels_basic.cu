@@ -2,6 +2,7 @@
 // backward, column sums, head/loss, AdamW, conversions.  All reductions run in a fixed order.
 #include "common.cuh"
 #include "kernels.h"
+#include "layernorm.cuh"
 
 namespace bsr {
 
@@ -116,50 +117,10 @@ __global__ void layernorm_fwd_kernel(const float* __restrict__ x, const float* _
                                      float* __restrict__ rstd, int rows, int D, float eps) {
   dependent_sync();
   int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  int lane = threadIdx.x & 31;
   if (warp >= rows) return;
-  const float* xr = x + (long)warp * D;
-  int chunks = D / 4;
-  float v[(NCH * 4)];
-  float sum = 0.f;
-#pragma unroll
-  for (int i = 0; i < NCH; ++i) {
-    int ch = lane + i * 32;
-    if (ch < chunks) {
-      load16(xr + ch * 4, v + i * 4);
-#pragma unroll
-      for (int j = 0; j < 4; ++j) sum += v[i * 4 + j];
-    }
-  }
-  float mu = warp_sum(sum) / (float)D;
-  float sq = 0.f;
-#pragma unroll
-  for (int i = 0; i < NCH; ++i) {
-    int ch = lane + i * 32;
-    if (ch < chunks) {
-#pragma unroll
-      for (int j = 0; j < 4; ++j) { float t = v[i * 4 + j] - mu; sq += t * t; }
-    }
-  }
-  float rs = rsqrtf(warp_sum(sq) / (float)D + eps);
-  if (lane == 0) {
-    if (mean) mean[warp] = mu;
-    if (rstd) rstd[warp] = rs;
-  }
-  TY* yr = y + (long)warp * D;
-#pragma unroll
-  for (int i = 0; i < NCH; ++i) {
-    int ch = lane + i * 32;
-    if (ch < chunks) {
-      float4 gg = *reinterpret_cast<const float4*>(g + ch * 4), bb = *reinterpret_cast<const float4*>(b + ch * 4);
-      float o[4];
-      o[0] = (v[i * 4 + 0] - mu) * rs * gg.x + bb.x;
-      o[1] = (v[i * 4 + 1] - mu) * rs * gg.y + bb.y;
-      o[2] = (v[i * 4 + 2] - mu) * rs * gg.z + bb.z;
-      o[3] = (v[i * 4 + 3] - mu) * rs * gg.w + bb.w;
-      store4(yr + ch * 4, o);
-    }
-  }
+  float v[NCH * 4];
+  ln_load_row<NCH>(x + (long)warp * D, D, v);
+  ln_write_row<TY, NCH>(v, g, b, y + (long)warp * D, mean ? mean + warp : nullptr, rstd ? rstd + warp : nullptr, D, eps);
 }
 
 template <typename TY>
@@ -720,24 +681,10 @@ __global__ void eval_begin_kernel(EvalIo* io, EvalIo value, const int* __restric
   if (tasks != nullptr)
     for (int j = threadIdx.x; j < batch; j += blockDim.x) task_stage[j] = tasks[j];
 }
-__global__ void eval_end_kernel(const EvalIo* io, const int* __restrict__ kept, size_t n_kept) {
-  dependent_sync();
-  int* out = io->kept;
-  size_t step = (size_t)gridDim.x * blockDim.x, i0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (out != nullptr)
-    for (size_t i = i0; i < n_kept; i += step) out[i] = kept[i];
-}
 void eval_begin(cudaStream_t s, EvalIo* io, const EvalIo& value, const int* tasks, int* task_stage, int batch) {
   note_launch(1);
   launch_k(eval_begin_kernel, 1, 128, 0, s, io, value, tasks, task_stage, batch);
 }
-void eval_end(cudaStream_t s, const EvalIo* io, const int* kept, size_t n_kept) {
-  if (n_kept == 0) return;
-  note_launch(1);
-  int blocks = ceil_div((long)n_kept, 256);
-  launch_k(eval_end_kernel, blocks < 64 ? blocks : 64, 256, 0, s, io, kept, n_kept);
-}
-
 // Guard words after every workspace slice: one warp per guard.
 __global__ void guards_write_kernel(char* base, const unsigned long long* __restrict__ table, int n, int words, uint32_t word) {
   dependent_sync();

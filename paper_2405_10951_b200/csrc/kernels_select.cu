@@ -1,6 +1,11 @@
 // Token importance, per-image top-K and the compaction between MHSA and FFN (paper Section 4.1, Eq. 6).
+#include <cooperative_groups.h>
+
+#include <type_traits>
+
 #include "common.cuh"
 #include "kernels.h"
+#include "layernorm.cuh"
 
 namespace bsr {
 
@@ -10,13 +15,19 @@ __device__ __forceinline__ uint32_t ordered_key(float f) {
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
+// The caller's copy of a drop location's kept positions, [B, k] (null: none).
+__device__ __forceinline__ int* kept_copy_dst(const KeptCopy& c) {
+  if (c.dst != nullptr) return c.dst;
+  return c.eval != nullptr && c.eval->kept != nullptr ? c.eval->kept + c.off : nullptr;
+}
+
 // One warp per image.  Scores are the head mean of the classification token's attention row, summed in
 // head order and divided by H in float.  The K-th largest key is found bit by bit (largest t with
 // count(key >= t) >= K); ties at the threshold go to the lower index; both index lists come out ascending.
 constexpr int SEL_WARPS = 4;
 
 __global__ void token_select_kernel(const float* __restrict__ p, int B, int H, int M, int k,
-                                    float* __restrict__ scores, int* __restrict__ kept, int* __restrict__ dropped) {
+                                    float* __restrict__ scores, int* __restrict__ kept, int* __restrict__ dropped, KeptCopy copy) {
   dependent_sync();
   extern __shared__ uint32_t keys_all[];
   int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -24,6 +35,7 @@ __global__ void token_select_kernel(const float* __restrict__ p, int B, int H, i
   if (b >= B) return;
   uint32_t* keys = keys_all + (size_t)warp * M;
   const float* pb = p + (size_t)b * H * M;
+  int* kcopy = kept_copy_dst(copy);
   for (int j = lane; j < M; j += 32) {
     float acc = pb[j];
     for (int h = 1; h < H; ++h) acc = acc + pb[(size_t)h * M + j];
@@ -56,8 +68,11 @@ __global__ void token_select_kernel(const float* __restrict__ p, int B, int H, i
     bool keep = valid && (key > t || (is_eq && eq_rank < need_eq));
     uint32_t keep_mask = __ballot_sync(0xffffffffu, keep);
     uint32_t drop_mask = __ballot_sync(0xffffffffu, valid && !keep);
-    if (keep) kept[(size_t)b * k + n_kept + __popc(keep_mask & lt_mask)] = j;
-    else if (valid) dropped[(size_t)b * (M - k) + n_drop + __popc(drop_mask & lt_mask)] = j;
+    if (keep) {
+      size_t at = (size_t)b * k + n_kept + __popc(keep_mask & lt_mask);
+      kept[at] = j;
+      if (kcopy != nullptr) kcopy[at] = j;
+    } else if (valid) dropped[(size_t)b * (M - k) + n_drop + __popc(drop_mask & lt_mask)] = j;
     n_kept += __popc(keep_mask);
     n_drop += __popc(drop_mask);
     eq_seen += __popc(eq_mask);
@@ -70,12 +85,13 @@ __global__ void token_select_kernel(const float* __restrict__ p, int B, int H, i
 template <int IPL>
 __global__ void __launch_bounds__(SEL_WARPS * 32)
 token_select_reg_kernel(const float* __restrict__ p, int B, int H, int M, int k, float* __restrict__ scores,
-                        int* __restrict__ kept, int* __restrict__ dropped) {
+                        int* __restrict__ kept, int* __restrict__ dropped, KeptCopy copy) {
   dependent_sync();
   int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int b = blockIdx.x * SEL_WARPS + warp;
   if (b >= B) return;
   const float* pb = p + (size_t)b * H * M;
+  int* kcopy = kept_copy_dst(copy);
   uint32_t key[IPL];
   float acc[IPL];
   // head sum in head order per token; the IPL loads of one head are independent, so many are in flight
@@ -142,22 +158,25 @@ token_select_reg_kernel(const float* __restrict__ p, int B, int H, int M, int k,
     bool keep = valid && (key[i] > t || (is_eq && eq_rank < need_eq));
     uint32_t keep_mask = __ballot_sync(0xffffffffu, keep);
     uint32_t drop_mask = __ballot_sync(0xffffffffu, valid && !keep);
-    if (keep) kept[(size_t)b * k + n_kept + __popc(keep_mask & lt_mask)] = j;
-    else if (valid) dropped[(size_t)b * (M - k) + n_drop + __popc(drop_mask & lt_mask)] = j;
+    if (keep) {
+      size_t at = (size_t)b * k + n_kept + __popc(keep_mask & lt_mask);
+      kept[at] = j;
+      if (kcopy != nullptr) kcopy[at] = j;
+    } else if (valid) dropped[(size_t)b * (M - k) + n_drop + __popc(drop_mask & lt_mask)] = j;
     n_kept += __popc(keep_mask);
     n_drop += __popc(drop_mask);
     eq_seen += __popc(eq_mask);
   }
 }
 
-void token_select(cudaStream_t s, const float* p, int B, int H, int M, int k, float* scores, int* kept, int* dropped) {
+void token_select(cudaStream_t s, const float* p, int B, int H, int M, int k, float* scores, int* kept, int* dropped, KeptCopy copy) {
   note_launch(1);
   int blocks = ceil_div(B, SEL_WARPS), threads = SEL_WARPS * 32;
-  if (M <= 256) { launch_k(token_select_reg_kernel<8>, blocks, threads, 0, s, p, B, H, M, k, scores, kept, dropped); return; }
-  if (M <= 640) { launch_k(token_select_reg_kernel<20>, blocks, threads, 0, s, p, B, H, M, k, scores, kept, dropped); return; }
+  if (M <= 256) { launch_k(token_select_reg_kernel<8>, blocks, threads, 0, s, p, B, H, M, k, scores, kept, dropped, copy); return; }
+  if (M <= 640) { launch_k(token_select_reg_kernel<20>, blocks, threads, 0, s, p, B, H, M, k, scores, kept, dropped, copy); return; }
   size_t smem = (size_t)SEL_WARPS * M * sizeof(uint32_t);
   if (smem > 48 * 1024) cudaFuncSetAttribute(token_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  launch_k(token_select_kernel, blocks, threads, smem, s, p, B, H, M, k, scores, kept, dropped);
+  launch_k(token_select_kernel, blocks, threads, smem, s, p, B, H, M, k, scores, kept, dropped, copy);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -253,6 +272,216 @@ void gather_fuse(const Ctx& c, const void* x, int B, int M, int D, int k, const 
     launch_k(gather_fuse_kernel<float>, grid, GF_THREADS, 0, c.stream, (const float*)x, M, D, k, kept, dropped, scores, do_fuse, (float*)out, copy_splits, c.status);
   else
     launch_k(gather_fuse_kernel<bf16>, grid, GF_THREADS, 0, c.stream, (const bf16*)x, M, D, k, kept, dropped, scores, do_fuse, (bf16*)out, copy_splits, c.status);
+}
+
+// Selection, compaction and the LayerNorm that follows, one image per cluster of eight CTAs.  As three launches each waited for the
+// one before: the selection is one warp's work (9 us of inference with one image), and the compacted rows went out to be read again.
+// Here every CTA selects for itself -- a thread has up to four tokens' keys, the K-th largest is found two bits at a time, three
+// counts to a warp reduction and one barrier each -- and then takes every eighth row of each kind:
+//   dropped rows : threads own four columns and add up s_j x_j; rank 0 combines the eight parts, read through distributed shared
+//                  memory, in rank order (the order of gather_fuse_kernel, whatever the batch), and finishes the fused row;
+//   kept rows    : a warp a row, taken from a counter; the row is in registers, so its LayerNorm costs no second pass.
+// Scores, kept and dropped lists are those of token_select, ties at the K-th key going to the lower index.
+// us a step, three launches -> one: ViT-B, 1 / 8 / 32 images 920 -> 884 / 1210 -> 1170 / 1951 -> 1916, DeiT-S, 8 / 24 images 772 -> 756 /
+// 971 -> 956, ViT-B/384, 7 images 1691 -> 1666.  Images that fill the SMs by themselves gain nothing from it and the selection is made eight
+// times over (DeiT-S, 64 images 1493 -> 1499; ViT-B, 128 images 5836 -> 5852): beyond SGA_MAXIMAGES the three launches stay.
+constexpr int SGA_MAXIMAGES = 48;
+constexpr int SGA_THREADS = 256, SGA_RANKS = 8, SGA_MAXM = 1023;   // three counts of up to 1023 share one warp reduction
+constexpr int SGA_MAXD = 1024;
+// Kept rows are shared out over as many clusters an image as the SMs have room for; the first has the dropped ones.
+constexpr int SGA_MAXCLUSTERS = 4;
+
+template <int IPT, typename TY>
+__global__ void __launch_bounds__(SGA_THREADS)
+select_gather_kernel(const float* __restrict__ p, const float* __restrict__ x, int clusters, int H, int M, int D, int k, int fuse, float* __restrict__ scores,
+                     int* __restrict__ kept, int* __restrict__ dropped, KeptCopy copy, float* __restrict__ out, const float* __restrict__ g,
+                     const float* __restrict__ be, TY* __restrict__ y, float* __restrict__ mean, float* __restrict__ rstd, float eps) {
+  dependent_sync();
+  __shared__ float sc[SGA_MAXM + 1];
+  __shared__ int list[SGA_MAXM + 1];                      // kept positions, then dropped ones, each ascending
+  __shared__ __align__(16) float part[SGA_MAXD];
+  __shared__ int next_row;
+  constexpr int NCH = SGA_MAXD / 128;
+  cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int rank = blockIdx.x % SGA_RANKS, b = blockIdx.x / SGA_RANKS / clusters, share = blockIdx.x / SGA_RANKS - b * clusters;
+  const bool first = share == 0, lead = first && rank == 0;
+  const float* pb = p + (size_t)b * H * M;
+  constexpr int WARPS = SGA_THREADS / 32;
+  __shared__ __align__(16) uint32_t counts[2][WARPS];
+  __shared__ int n_gt[IPT * WARPS], n_eq[IPT * WARPS], at_kept[IPT * WARPS], at_drop[IPT * WARPS], eq_left[IPT * WARPS];
+  if (tid == 0) next_row = share * SGA_RANKS + rank;
+  uint32_t key[IPT];                                       // token i * SGA_THREADS + tid; absent ones 0, below every candidate
+#pragma unroll
+  for (int i = 0; i < IPT; ++i) {
+    const int j = i * SGA_THREADS + tid;
+    key[i] = 0u;
+    if (j < M) {
+      float acc = 0.f;
+      for (int h = 0; h < H; h += 12) {                    // the loads of twelve heads at once, the sum in head order
+        float v[12];
+#pragma unroll
+        for (int u = 0; u < 12; ++u)
+          if (h + u < H) v[u] = pb[(size_t)(h + u) * M + j];
+#pragma unroll
+        for (int u = 0; u < 12; ++u)
+          if (h + u < H) acc = h + u == 0 ? v[u] : acc + v[u];
+      }
+      const float s = acc / (float)H;
+      sc[j] = s;
+      key[i] = ordered_key(s);
+      if (lead) scores[(size_t)b * M + j] = s;
+    }
+  }
+  uint32_t t = 0;
+  for (int bit = 30; bit >= 0; bit -= 2) {
+    const uint32_t c1 = t | (1u << bit), c2 = t | (2u << bit), c3 = t | (3u << bit);
+    uint32_t cnt = 0;
+#pragma unroll
+    for (int i = 0; i < IPT; ++i) cnt += (key[i] >= c1 ? 1u : 0u) + (key[i] >= c2 ? 1u << 10 : 0u) + (key[i] >= c3 ? 1u << 20 : 0u);
+    cnt = __reduce_add_sync(0xffffffffu, cnt);
+    uint32_t* row = counts[(bit >> 1) & 1];
+    if (lane == 0) row[warp] = cnt;
+    __syncthreads();
+    const uint4 x = reinterpret_cast<const uint4*>(row)[0], z = reinterpret_cast<const uint4*>(row)[1];
+    cnt = ((x.x + x.y) + (x.z + x.w)) + ((z.x + z.y) + (z.z + z.w));
+    if ((cnt >> 20) >= (uint32_t)k) t = c3;
+    else if (((cnt >> 10) & 1023u) >= (uint32_t)k) t = c2;
+    else if ((cnt & 1023u) >= (uint32_t)k) t = c1;
+  }
+  // positions: groups of 32 tokens in token order (IPT * WARPS <= 32 of them, a lane of warp 0 each); of the keys equal to the K-th the
+  // first ones are kept
+  const uint32_t lt_mask = (1u << lane) - 1u;
+  uint32_t gt_mask[IPT], eq_mask[IPT];
+#pragma unroll
+  for (int i = 0; i < IPT; ++i) {
+    const bool valid = i * SGA_THREADS + tid < M;
+    gt_mask[i] = __ballot_sync(0xffffffffu, valid && key[i] > t);
+    eq_mask[i] = __ballot_sync(0xffffffffu, valid && key[i] == t);
+    if (lane == 0) { n_gt[i * WARPS + warp] = __popc(gt_mask[i]); n_eq[i * WARPS + warp] = __popc(eq_mask[i]); }
+  }
+  __syncthreads();
+  if (warp == 0) {
+    const bool have = lane < IPT * WARPS;
+    const int gt = have ? n_gt[lane] : 0, eq = have ? n_eq[lane] : 0;
+    const int need_eq = k - __reduce_add_sync(0xffffffffu, gt);
+    auto before = [&](int v) {                             // sum over the lanes below
+      int s = v;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, s, o);
+        if (lane >= o) s += u;
+      }
+      return s - v;
+    };
+    const int left = max(0, need_eq - before(eq)), kept_here = gt + min(eq, left), at = before(kept_here);
+    if (have) { eq_left[lane] = left; at_kept[lane] = at; at_drop[lane] = k + min(lane * 32, M) - at; }
+  }
+  __syncthreads();
+  int* kcopy = lead ? kept_copy_dst(copy) : nullptr;
+#pragma unroll
+  for (int i = 0; i < IPT; ++i) {
+    const int j = i * SGA_THREADS + tid, w = i * WARPS + warp;
+    const uint32_t bit = 1u << lane;
+    const int eq_before = __popc(eq_mask[i] & lt_mask);
+    const bool keep = (gt_mask[i] & bit) != 0 || ((eq_mask[i] & bit) != 0 && eq_before < eq_left[w]);
+    const uint32_t keep_mask = __ballot_sync(0xffffffffu, keep);
+    if (j >= M) continue;
+    const int n = __popc(keep_mask & lt_mask), at = keep ? at_kept[w] + n : at_drop[w] + lane - n;
+    list[at] = j;
+    if (lead) {
+      if (keep) {
+        kept[(size_t)b * k + at] = j;
+        if (kcopy != nullptr) kcopy[(size_t)b * k + at] = j;
+      } else {
+        dropped[(size_t)b * (M - k) + at - k] = j;
+      }
+    }
+  }
+  __syncthreads();
+  const int nd = M - k, t_out = 1 + k + (fuse ? 1 : 0), col = tid * 4;
+  const float* xb = x + (size_t)b * (1 + M) * D;
+  const bool has = fuse && first && col < D;
+  if (has) {
+    float acc[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int i0 = rank; i0 < nd; i0 += 8 * SGA_RANKS) {    // eight rows at once, added in order
+      float v[8][4];
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (i0 + u * SGA_RANKS < nd) load16(xb + (size_t)(1 + list[k + i0 + u * SGA_RANKS]) * D + col, v[u]);
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (i0 + u * SGA_RANKS < nd) {
+          const float w = sc[list[k + i0 + u * SGA_RANKS]];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) acc[e] += w * v[u][e];
+        }
+    }
+    store16(part + col, acc);
+  }
+  auto finish_row = [&](int r, const float* src) {         // row r of the image's output, by one warp
+    const size_t ro = (size_t)b * t_out + r;
+    float v[NCH * 4];
+    ln_load_row<NCH>(src, D, v);
+    float* dst = out + ro * D;
+#pragma unroll
+    for (int i = 0; i < NCH; ++i)
+      if (lane + i * 32 < D / 4) store16(dst + (lane + i * 32) * 4, v + i * 4);
+    if (y != nullptr) ln_write_row<TY, NCH>(v, g, be, y + ro * D, mean ? mean + ro : nullptr, rstd ? rstd + ro : nullptr, D, eps);
+  };
+  while (true) {
+    int r = 0;
+    if (lane == 0) r = atomicAdd(&next_row, clusters * SGA_RANKS);
+    r = __shfl_sync(0xffffffffu, r, 0);
+    if (r > k) break;
+    finish_row(r, r == 0 ? xb : xb + (size_t)(1 + list[r - 1]) * D);
+  }
+  if (!fuse || !first) return;
+  cluster.sync();
+  if (rank == 0 && has) {
+    float o[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int r = 0; r < SGA_RANKS; ++r) {
+      float v[4];
+      load16(cluster.map_shared_rank(part, r) + col, v);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) o[e] += v[e];
+    }
+    store16(part + col, o);                                // (a thread rewrites what it alone reads)
+  }
+  cluster.sync();                                          // no CTA leaves while rank 0 may still read its part
+  if (rank == 0 && warp == 0) {
+    if (fuse == 2) {                                       // weighted mean: by the sum of the dropped tokens' weights, in a fixed order
+      float ws = 0.f;
+      for (int i = lane; i < nd; i += 32) ws += sc[list[k + i]];
+      ws = warp_sum(ws);
+      for (int c = lane; c < D; c += 32) part[c] = part[c] / ws;
+      __syncwarp();
+    }
+    finish_row(1 + k, part);
+  }
+}
+
+int select_gather(const Ctx& c, const float* p, const float* x, int B, int H, int M, int D, int k, int fuse, float* scores, int* kept, int* dropped,
+                  KeptCopy copy, float* out, const float* g, const float* b, void* y, float* mean, float* rstd, float eps) {
+  if (B > SGA_MAXIMAGES || M > SGA_MAXM || D > SGA_MAXD || D % 4 != 0 || k >= M) return -1;
+  note_launch(1);
+  const int sms = c.sm_count > 0 ? c.sm_count : B200_SMS;
+  int clusters = sms / (B * SGA_RANKS);
+  clusters = clusters < 1 ? 1 : clusters > SGA_MAXCLUSTERS ? SGA_MAXCLUSTERS : clusters;
+  auto go = [&](auto kern, auto* yt) {
+    launch_cluster(kern, dim3(B * clusters * SGA_RANKS), SGA_THREADS, 0, c.stream, dim3(SGA_RANKS, 1, 1), p, x, clusters, H, M, D, k, fuse, scores, kept, dropped, copy, out, g, b,
+                   yt, mean, rstd, eps);
+  };
+  auto pick = [&](auto* yt) {
+    using TY = std::remove_pointer_t<decltype(yt)>;
+    if (M <= SGA_THREADS) go(select_gather_kernel<1, TY>, yt);
+    else if (M <= 3 * SGA_THREADS) go(select_gather_kernel<3, TY>, yt);
+    else go(select_gather_kernel<4, TY>, yt);
+  };
+  if (c.dtype == 0) pick((float*)y);
+  else pick((bf16*)y);
+  return 0;
 }
 
 // Backward of the compaction, one warp per input row (the index sets are constants, the fusion weights are

@@ -375,3 +375,19 @@ def test_head_over_numbers_of_classes(classes, dim, batch, drop):
     images, labels, task_ids, params = synth.make_workload(cfg, peaked=dim >= 64)
     gpu = P.run_gpu_step(cfg, images, labels, task_ids, params)
     P.compare_step(cfg, images, labels, task_ids, params, gpu, P.FP32_TOL, P.EXACT_MARGIN, P.FP32_TOL)
+
+
+@pytest.mark.parametrize("dtype,grid,keep,fuse,dim,heads,batch", [
+    ("fp32", 16, (1, 2), 1, 64, 4, 3), ("fp32", 17, (3, 10), 2, 192, 3, 1), ("fp32", 25, (7, 10), 0, 64, 4, 2), ("fp32", 26, (1, 100), 1, 128, 8, 1),
+    ("fp32", 31, (99, 100), 2, 64, 4, 1), ("fp32", 32, (1, 2), 1, 64, 4, 1), ("fp32", 3, (1, 3), 1, 1024, 16, 9),
+    ("bf16", 16, (1, 2), 2, 128, 2, 3), ("bf16", 26, (7, 10), 1, 64, 1, 2)])
+def test_selection_compaction_and_layernorm_in_one_launch(dtype, grid, keep, fuse, dim, heads, batch):
+    """Register counts of the selection (256, 640 tokens) and the longest row it takes (1023; 1024 go the general way), one kept
+    token, few dropped ones, no fused token, rows of 64 to 1024 columns; a frozen and a trainable drop location."""
+    cfg = Config("mini_select", 4 * grid, 4, dim, heads, 3, 2 * dim, (10,), batch, (1, 2), (0, 1), keep[0], keep[1], dtype=dtype, fuse_mode=fuse, seed=grid)
+    images, labels, task_ids, params = synth.make_workload(cfg, peaked=dtype == "fp32")
+    gpu = P.run_gpu_step(cfg, images, labels, task_ids, params)
+    if dtype == "fp32":
+        P.compare_step(cfg, images, labels, task_ids, params, gpu, P.FP32_TOL, P.EXACT_MARGIN, P.FP32_TOL)
+    else:
+        P.compare_step(cfg, images, labels, task_ids, params, gpu, P.BF16_TOL, P.BF16_EXACT_MARGIN, P.BF16_SCORE_TOL)
