@@ -109,6 +109,13 @@ __device__ __forceinline__ int warp_sum_int(int v) {
   return v;
 }
 
+// 16 bytes from global to shared memory, on their own; a group of copies is committed, and all but the newest N groups waited for.
+__device__ __forceinline__ void copy16_async(void* dst, const void* src, int bytes = 16) {      // bytes: what is copied, zeros follow
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void copies_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
 // Exact GELU x * Phi(x) and its derivative Phi(x) + x * phi(x).
 __device__ __forceinline__ float gelu_f(float x) { return 0.5f * x * (1.0f + erff(x * 0.70710678118654752f)); }
 __device__ __forceinline__ float gelu_grad_f(float x) {

@@ -1,7 +1,9 @@
 // FP32-FMA dense contraction with arbitrary operand strides.  It is the contraction of the fp32
-// configuration (TF32 tensor-core math cannot hold a 1e-4 relative tolerance) and the fall-back for
-// bf16 problems the tcgen05 kernel does not take (tiny or unaligned shapes).
+// configuration (TF32 tensor-core math cannot hold a 1e-4 relative tolerance; gemm_simt_small_kernel wherever rows are aligned) and the
+// fall-back for bf16 problems the tcgen05 kernel does not take (tiny or unaligned shapes).
 #include <cooperative_groups.h>
+
+#include <type_traits>
 
 #include "common.cuh"
 #include "kernels.h"
@@ -67,9 +69,41 @@ struct SimtEpi {
   const T* aux_in;
   int M, N, act;
   long res_ld;
+  bool vec;                                  // all float, rows of whole aligned groups of four
   // four consecutive columns of one row
   __device__ __forceinline__ void operator()(int gm, int gn, const float* acc) const {
     if (gm >= M) return;
+    if constexpr (sizeof(T) == 4) {
+      if (vec) {
+        if (gn >= N) return;
+        const size_t o = (size_t)gm * N + gn;
+        float v[4], x[4];
+        if (bias != nullptr) load16(bias + gn, x);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) v[j] = bias != nullptr ? acc[j] + x[j] : acc[j];
+        if (act == 1) {
+          if (aux_out != nullptr) store16(aux_out + o, v);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) v[j] = gelu_f(v[j]);
+        } else if (act == 2) {
+          load16(aux_in + o, x);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) v[j] *= gelu_grad_f(x[j]);
+          if (aux_out != nullptr) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) x[j] = gelu_f(x[j]);
+            store16(aux_out + o, x);
+          }
+        }
+        if (residual != nullptr) {
+          load16(residual + (size_t)gm * res_ld + gn, x);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) v[j] += x[j];
+        }
+        store16(C + o, v);
+        return;
+      }
+    }
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       if (gn + j >= N) continue;
@@ -169,6 +203,226 @@ gemm_simt_kernel(const T* __restrict__ A, long lda, int a_kmajor, int a_vec, con
   cluster.sync();                          // no CTA leaves while another may still read its partial tile
 }
 
+__device__ __forceinline__ uint64_t simt_pack2(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void simt_unpack2(uint64_t r, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(r)); }
+__device__ __forceinline__ uint64_t simt_fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+// The same for products of few tiles (the fp32 configuration's own: 520 x 192 x 192 is 27 tiles of 64).  Tiles of 32 x 32, a CTA of
+// 256 threads in four groups of 64: every group forms the whole tile, 4 x 4 products a
+// thread (two an instruction, fma.rn.f32x2), over a quarter of each slab of 64 along k, and the four sums are added in
+// group order through shared memory.  So eight warps share the latency of a tile that two would otherwise work on.  Slabs
+// arrive by cp.async, up to three in flight beside the one worked on: k is split over a cluster beyond 256, so these are most of them.
+// us of a launch in a row of launches, tiles of 64 / this, forward and both products of the backward:
+//   520 x 192 x 192   11.7 / 3.4   25.1 / 7.9    2080 x 576 x 192   24.1 / 17.4   62.0 / 42.4
+//   520 x 576 x 192   12.8 / 7.3   28.9 / 16.7   2080 x 768 x 192   37.9 / 23.3   77.3 / 55.9
+//   520 x 192 x 768   16.4 / 10.5  30.7 / 17.2   8192 x 768 x 768   361 / 368     860 / 632
+// and the error against 64 bits falls, forward 1.8e-7 -> 1.0e-7, input gradients 1.8e-7 -> 1.3e-7, weight gradients over 2080 rows
+// 4.1e-7 -> 2.2e-7.  A step of the fp32 configuration: batch 1 / 8 / 32 559 -> 367 / 749 -> 439 / 1162 -> 827 us.
+// Rows of a slab lie where quarter-warps read them without bank conflicts: [row][64 + 4] where the operand is
+// contiguous along k (fragments of four k), [k][32 + 4] where along its own index.
+constexpr int SS_BM = 32, SS_BN = 32, SS_BK = 64, SS_THREADS = 256, SS_GROUPS = 4, SS_STAGES = 4;
+constexpr long SS_MANY = 8192;
+constexpr int SS_KLD = SS_BK + 4, SS_MLD = SS_BM + 4;
+constexpr int SS_OPERAND = SS_BK * SS_MLD;                    // floats of a slab of one operand, either layout (32 x 68 or 64 x 36)
+static_assert(SS_OPERAND >= SS_BM * SS_KLD, "either layout fits");
+constexpr size_t SS_SMEM = (size_t)SS_STAGES * 2 * SS_OPERAND * sizeof(float);
+
+// Slab k0 .. k0 + 63 of rows r0 .. r0 + 31; what lies beyond R rows or K columns becomes zero.  Base and row pitch are multiples of 16 bytes.
+template <bool KMAJOR>
+__device__ __forceinline__ void ss_load(const float* __restrict__ P, long ld, int r0, int k0, int R, int K, float* S) {
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const int i = q * SS_THREADS + threadIdx.x;
+    int left;
+    const float* src;
+    float* dst;
+    if (KMAJOR) {
+      const int r = i >> 4, k = (i & 15) * 4;
+      left = r0 + r < R ? K - (k0 + k) : 0;
+      src = P + (long)(r0 + r) * ld + k0 + k;
+      dst = S + r * SS_KLD + k;
+    } else {
+      const int k = i >> 3, r = (i & 7) * 4;
+      left = k0 + k < K ? R - (r0 + r) : 0;
+      src = P + (long)(k0 + k) * ld + r0 + r;
+      dst = S + k * SS_MLD + r;
+    }
+    const int bytes = left >= 4 ? 16 : left > 0 ? left * 4 : 0;
+    copy16_async(dst, bytes > 0 ? src : P, bytes);
+  }
+}
+// Four rows at k .. k + 3: v[row][k].  Rows r, r + 8, r + 16, r + 24 of an operand contiguous along k, r .. r + 3 of the other kind.
+template <bool KMAJOR>
+__device__ __forceinline__ void ss_frag(const float* S, int r, int k, float (&v)[4][4]) {
+  if (KMAJOR) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) load16(S + (r + i * 8) * SS_KLD + k, v[i]);
+  } else {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      float t[4];
+      load16(S + (k + j) * SS_MLD + r, t);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) v[i][j] = t[i];
+    }
+  }
+}
+
+template <bool A_K, bool B_K>
+__global__ void __launch_bounds__(SS_THREADS)
+gemm_simt_small_kernel(const float* __restrict__ A, long lda, const float* __restrict__ B, long ldb, int K, int k_per_split, SimtEpi<float, float> epi) {
+  extern __shared__ __align__(16) float ss[];
+  if (leaves_sms_idle()) release_dependents();
+  await_inputs();
+  const int tid = threadIdx.x, grp = tid >> 6, ty = (tid & 63) >> 3, tx = tid & 7;
+  const int m0 = blockIdx.y * SS_BM, n0 = blockIdx.x * SS_BN;
+  const int splits = gridDim.z, rank = blockIdx.z;
+  const int kb = rank * k_per_split, ke = min(K, kb + k_per_split), slabs = (ke - kb + SS_BK - 1) / SS_BK;
+  auto stage = [&](int i) {
+    if (i < slabs) {
+      float* S = ss + (i % SS_STAGES) * 2 * SS_OPERAND;
+      ss_load<A_K>(A, lda, m0, kb + i * SS_BK, epi.M, ke, S);
+      ss_load<B_K>(B, ldb, n0, kb + i * SS_BK, epi.N, ke, S + SS_OPERAND);
+    }
+    copies_commit();
+  };
+#pragma unroll
+  for (int i = 0; i < SS_STAGES - 1; ++i) stage(i);
+  // Pairs of one instruction: where both operands come four k at a time, even and odd k (each a sum of its own), otherwise two columns.
+  constexpr bool KP = A_K && B_K;
+  constexpr int PAIRS = KP ? 4 : 2;
+  uint64_t acc[4][PAIRS];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < PAIRS; ++j) acc[i][j] = 0ull;
+  for (int s = 0; s < slabs; ++s) {
+    copies_wait<SS_STAGES - 2>();
+    __syncthreads();
+    stage(s + SS_STAGES - 1);                                 // into the slab that every thread left before this barrier
+    const float* As = ss + (s % SS_STAGES) * 2 * SS_OPERAND;
+    const float* Bs = As + SS_OPERAND;
+#pragma unroll
+    for (int kk = 0; kk < SS_BK / SS_GROUPS; kk += 4) {
+      const int k = grp * (SS_BK / SS_GROUPS) + kk;
+      float a[4][4], b[4][4];
+      ss_frag<A_K>(As, A_K ? ty : ty * 4, k, a);
+      ss_frag<B_K>(Bs, B_K ? tx : tx * 4, k, b);
+      if constexpr (KP) {
+#pragma unroll
+        for (int j = 0; j < 4; j += 2)
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int n = 0; n < 4; ++n) acc[i][n] = simt_fma2(simt_pack2(a[i][j], a[i][j + 1]), simt_pack2(b[n][j], b[n][j + 1]), acc[i][n]);
+      } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const uint64_t b0 = simt_pack2(b[0][j], b[1][j]), b1 = simt_pack2(b[2][j], b[3][j]);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const uint64_t av = simt_pack2(a[i][j], a[i][j]);
+            acc[i][0] = simt_fma2(av, b0, acc[i][0]);
+            acc[i][1] = simt_fma2(av, b1, acc[i][1]);
+          }
+        }
+      }
+    }
+  }
+  // the groups' tiles [4][32][32 + 4] over the operand buffers
+  copies_wait<0>();
+  __syncthreads();
+  constexpr int TLD = SS_BN + 4;
+  static_assert(SS_GROUPS * SS_BM * TLD <= SS_STAGES * 2 * SS_OPERAND, "the groups' tiles fit");
+  float* tile = ss + grp * SS_BM * TLD;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int r = A_K ? ty + i * 8 : ty * 4 + i;
+    float c[4];
+    if constexpr (KP) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        float even, odd;
+        simt_unpack2(acc[i][j], even, odd);
+        c[j] = even + odd;
+      }
+    } else {
+      simt_unpack2(acc[i][0], c[0], c[1]);
+      simt_unpack2(acc[i][1], c[2], c[3]);
+    }
+    if (B_K) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) tile[r * TLD + tx + j * 8] = c[j];
+    } else {
+      store16(tile + r * TLD + tx * 4, c);
+    }
+  }
+  __syncthreads();
+  const int r = tid >> 3, c4 = (tid & 7) * 4;                 // a thread has four columns of a row
+  float v[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+  for (int g = 0; g < SS_GROUPS; ++g) {
+    float t[4];
+    load16(ss + (g * SS_BM + r) * TLD + c4, t);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) v[j] += t[j];
+  }
+  if (splits == 1) {
+    epi(m0 + r, n0 + c4, v);
+    return;
+  }
+  // every rank finishes its share of the tile's rows, the others' sums read through distributed shared memory in rank order
+  cg::cluster_group cluster = cg::this_cluster();
+  store16(ss + r * TLD + c4, v);                              // (a thread rewrites what it alone has read)
+  cluster.sync();
+  const int share = (SS_BM + splits - 1) / splits;
+  if (r < share && rank * share + r < SS_BM) {
+    const int row = rank * share + r;
+    float4 x[SG_MAXSPLIT];
+#pragma unroll
+    for (int q = 0; q < SG_MAXSPLIT; ++q)
+      if (q < splits) x[q] = *reinterpret_cast<const float4*>(cluster.map_shared_rank(ss, q) + row * TLD + c4);
+    float o[4] = {x[0].x, x[0].y, x[0].z, x[0].w};
+#pragma unroll
+    for (int q = 1; q < SG_MAXSPLIT; ++q)
+      if (q < splits) { o[0] += x[q].x; o[1] += x[q].y; o[2] += x[q].z; o[3] += x[q].w; }
+    epi(m0 + row, n0 + c4, o);
+  }
+  cluster.sync();                                             // no CTA leaves while another may still read its tile
+}
+
+// Splits of the reduction: by its length alone for a layer's output or input gradient, so that an image's result does not
+// depend on the batch; weight gradients by what fills the SMs.  Non-zero: not a product for this kernel.
+static int launch_simt_small(const Ctx& c, const float* A, long lda, bool ak, const float* B, long ldb, bool bk, int m, int n, int k,
+                             const SimtEpi<float, float>& epi) {
+  if (lda % 4 != 0 || ldb % 4 != 0 || (uintptr_t)A % 16 != 0 || (uintptr_t)B % 16 != 0) return -1;
+  const int sms = c.sm_count > 0 ? c.sm_count : B200_SMS;
+  const long tiles = (long)ceil_div(m, SS_BM) * ceil_div(n, SS_BN);
+  if (ceil_div(m, SS_BM) > 65535) return -1;
+  int splits = ceil_div(k, 256) < SG_MAXSPLIT ? ceil_div(k, 256) : SG_MAXSPLIT;
+  if (!ak)
+    while (splits > 1 && tiles * splits > 4l * sms) --splits;
+  const int per = ceil_div(ceil_div(k, splits), SS_BK) * SS_BK;
+  splits = ceil_div(k, per) < 1 ? 1 : ceil_div(k, per);
+  // many tiles along k on both sides: nothing is idle, and tiles of 64 read shared memory less often
+  if (ak && bk && tiles * splits > SS_MANY) return -1;
+  auto go = [&](auto kern, SmemLimit& lim) {
+    if (!ensure_smem(lim, kern, SS_SMEM)) return -3;
+    launch_cluster(kern, dim3(ceil_div(n, SS_BN), ceil_div(m, SS_BM), splits), SS_THREADS, SS_SMEM, c.stream, dim3(1, 1, splits), A, lda, B, ldb, k, per, epi);
+    return 0;
+  };
+  static SmemLimit l0, l1, l2, l3;
+  return ak ? (bk ? go(gemm_simt_small_kernel<true, true>, l0) : go(gemm_simt_small_kernel<true, false>, l1))
+            : (bk ? go(gemm_simt_small_kernel<false, true>, l2) : go(gemm_simt_small_kernel<false, false>, l3));
+}
+
 template <typename T, typename TC>
 static void launch_simt(const Ctx& c, const void* A, long a_rs, long a_cs, const void* B, long b_rs, long b_cs, void* C, int m, int n, int k,
                         const GemmEpilogue& e) {
@@ -194,7 +448,11 @@ static void launch_simt(const Ctx& c, const void* A, long a_rs, long a_cs, const
   splits = ceil_div(k, per) < 1 ? 1 : ceil_div(k, per);
   const long lda = ak ? a_rs : a_cs, ldb = bk ? b_rs : b_cs;
   const size_t quad = 4 * sizeof(T);
-  SimtEpi<T, TC> epi = {(TC*)C, e.bias, (const TC*)e.residual, (TC*)e.aux_out, (const T*)e.aux_in, m, n, e.act, e.residual_ld ? e.residual_ld : n};
+  SimtEpi<T, TC> epi = {(TC*)C, e.bias, (const TC*)e.residual, (TC*)e.aux_out, (const T*)e.aux_in, m, n, e.act, e.residual_ld ? e.residual_ld : n,
+                         sizeof(T) == 4 && sizeof(TC) == 4 && n % 4 == 0 && e.residual_ld % 4 == 0 &&
+                             (((uintptr_t)C | (uintptr_t)e.bias | (uintptr_t)e.residual | (uintptr_t)e.aux_out | (uintptr_t)e.aux_in) & 15) == 0};
+  if constexpr (std::is_same<T, float>::value)
+    if (launch_simt_small(c, (const float*)A, lda, ak, (const float*)B, ldb, bk, m, n, k, epi) == 0) return;
   launch_cluster(gemm_simt_kernel<T, TC>, dim3(tiles_n, ceil_div(m, SG_BM), splits), SG_THREADS, 0, c.stream, dim3(1, 1, splits), (const T*)A, lda, (int)ak,
                  (int)(lda % 4 == 0 && (uintptr_t)A % quad == 0), (const T*)B, ldb, (int)bk, (int)(ldb % 4 == 0 && (uintptr_t)B % quad == 0), k, per, epi);
 }

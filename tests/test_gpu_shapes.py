@@ -391,3 +391,20 @@ def test_selection_compaction_and_layernorm_in_one_launch(dtype, grid, keep, fus
         P.compare_step(cfg, images, labels, task_ids, params, gpu, P.FP32_TOL, P.EXACT_MARGIN, P.FP32_TOL)
     else:
         P.compare_step(cfg, images, labels, task_ids, params, gpu, P.BF16_TOL, P.BF16_EXACT_MARGIN, P.BF16_SCORE_TOL)
+
+
+@pytest.mark.parametrize("m,n,k", [(1, 4, 4), (31, 36, 60), (32, 32, 64), (33, 68, 260), (100, 192, 516), (7, 200, 2052), (9000, 512, 512)])
+def test_fp32_products_in_small_tiles(m, n, k):
+    """Edges of the 32 x 32 tiles and 64-deep slabs, one to eight parts of k, and the number of tiles beyond which tiles of 64 take over; sums of at
+    most a few hundred fp32 additions in a row keep a relative error below 2e-6."""
+    import torch
+    from paper_2405_10951_b200 import binding as Bd
+    g = torch.Generator(device="cuda").manual_seed(m + n + k)
+    x, w, dy = (torch.randn(s, generator=g, device="cuda") for s in ((m, k), (n, k), (m, n)))
+    bias, res = torch.randn(n, generator=g, device="cuda"), torch.randn(m, n, generator=g, device="cuda")
+    rel = lambda a, b: float((a.double() - b).norm() / b.norm())
+    z = x.double() @ w.double().T + bias.double()
+    assert rel(Bd.bsr_linear_forward(x, w, bias, res), z + res.double()) < 2e-6
+    assert rel(Bd.bsr_linear_forward(x, w, bias, act_gelu=True), torch.nn.functional.gelu(z)) < 2e-6
+    dx, dw = Bd.bsr_linear_backward(x, w, dy)
+    assert rel(dx, dy.double() @ w.double()) < 2e-6 and rel(dw, dy.double().T @ x.double()) < 2e-6
