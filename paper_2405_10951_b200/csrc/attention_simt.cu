@@ -2,6 +2,10 @@
 // query (or key) row with the head's K/V (or Q/dO) resident in shared memory.  Used by the fp32
 // configuration, and by bf16 problems until the tensor-core attention takes them.
 //
+// What bounds it is the latency of a short chain: K and V arrive by cp.async (a load and a store a row and warp, one after the other,
+// were half of the time), and a warp forms the scores of up to four groups of 32 keys side by side.  A step of the fp32
+// configuration: batch 1 / 8 / 32 367 -> 315 / 439 -> 383 / 827 -> 748 us.
+//
 // Layout: qkv [B, T, 3, H, d], out/dout [B, T, H*d], lse/delta [B, H, T], cls_prob [B, H, T-1].
 // The forward kernel also emits the classification token's attention row (Eq. 6: the token
 // importance scores), and the backward kernels accept a gradient arriving at that row.
@@ -13,13 +17,25 @@ namespace bsr {
 constexpr int AT_WARPS = 8;
 constexpr int AT_MAXD = 64;
 
+// Four bytes from global to shared memory, on their own (the rows' pitch there allows no wider copies).
+__device__ __forceinline__ void copy4_async(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copies_done() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 template <typename T> struct Row;
 template <> struct Row<float> {
   __device__ static int stride(int d) { return d + 1; }
-  __device__ static float dot(const float* q, const float* row, int d) {
-    float s = 0.f;
-    for (int i = 0; i < d; ++i) s = fmaf(q[i], row[i], s);
-    return s;
+  // s[u] = q . row[u]
+  template <int NU> __device__ static void dots(const float* q, const float* const (&row)[4], int d, float* s) {
+#pragma unroll
+    for (int u = 0; u < NU; ++u) s[u] = 0.f;
+#pragma unroll 8
+    for (int i = 0; i < d; ++i) {
+      const float v = q[i];
+#pragma unroll
+      for (int u = 0; u < NU; ++u) s[u] = fmaf(v, row[u][i], s[u]);
+    }
   }
   // the two feature indices a lane owns
   __device__ static int dim0(int lane) { return lane; }
@@ -29,20 +45,23 @@ template <> struct Row<float> {
     b = (lane + 32 < d) ? row[lane + 32] : 0.f;
   }
   __device__ static void fill(float* row, const float* src, int d, int lane) {
-    for (int i = lane; i < d; i += 32) row[i] = src[i];
+    for (int i = lane; i < d; i += 32) copy4_async(row + i, src + i);
   }
 };
 template <> struct Row<bf16> {
   __device__ static int stride(int d) { return d + 2; }
-  __device__ static float dot(const float* q, const bf16* row, int d) {
-    const __nv_bfloat162* r2 = reinterpret_cast<const __nv_bfloat162*>(row);
-    float s = 0.f;
+  template <int NU> __device__ static void dots(const float* q, const bf16* const (&row)[4], int d, float* s) {
+#pragma unroll
+    for (int u = 0; u < NU; ++u) s[u] = 0.f;
+#pragma unroll 4
     for (int i = 0; i < d / 2; ++i) {
-      float2 v = __bfloat1622float2(r2[i]);
-      s = fmaf(q[2 * i], v.x, s);
-      s = fmaf(q[2 * i + 1], v.y, s);
+#pragma unroll
+      for (int u = 0; u < NU; ++u) {
+        const float2 v = __bfloat1622float2(reinterpret_cast<const __nv_bfloat162*>(row[u])[i]);
+        s[u] = fmaf(q[2 * i], v.x, s[u]);
+        s[u] = fmaf(q[2 * i + 1], v.y, s[u]);
+      }
     }
-    return s;
   }
   __device__ static int dim0(int lane) { return 2 * lane; }
   __device__ static int dim1(int lane) { return 2 * lane + 1; }
@@ -53,10 +72,23 @@ template <> struct Row<bf16> {
     } else { a = 0.f; b = 0.f; }
   }
   __device__ static void fill(bf16* row, const bf16* src, int d, int lane) {
-    for (int i = lane; i < d / 2; i += 32)
-      reinterpret_cast<__nv_bfloat162*>(row)[i] = reinterpret_cast<const __nv_bfloat162*>(src)[i];
+    for (int i = lane; i < d / 2; i += 32) copy4_async(row + 2 * i, src + 2 * i);
   }
 };
+
+// Dot products of a vector with rows j, j + 32, ... (as many as lie below `rows` for the warp's first lane, whose j is `first`; at
+// most four), each in order along d, side by side.  A lane whose row lies beyond reads the last one instead; that result is not used.
+template <typename T>
+__device__ __forceinline__ void row_dots(const float* q, const T* mat, int rs, int j, int first, int rows, int d, float (&s)[4]) {
+  const int nu = min(4, (rows - first + 31) >> 5);
+  const T* row[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) row[u] = mat + (size_t)min(j + 32 * u, rows - 1) * rs;
+  if (nu == 1) Row<T>::template dots<1>(q, row, d, s);
+  else if (nu == 2) Row<T>::template dots<2>(q, row, d, s);
+  else if (nu == 3) Row<T>::template dots<3>(q, row, d, s);
+  else Row<T>::template dots<4>(q, row, d, s);
+}
 
 // Copies [T, d] rows of one (image, head, which) slice of qkv (or of a [B, T, H*d] tensor) into padded smem rows.
 template <typename T>
@@ -86,6 +118,7 @@ attn_fwd_kernel(const T* __restrict__ qkv, T* __restrict__ out, float* __restric
   const T* base = qkv + (size_t)b * T_ * tok_stride + (size_t)h * d;
   stage_rows<T>(Ks, base + (size_t)H * d, tok_stride, T_, d);
   stage_rows<T>(Vs, base + 2 * (size_t)H * d, tok_stride, T_, d);
+  copies_done();
   __syncthreads();
   float scale = rsqrtf((float)d);
   float* P = Ps + (size_t)warp * T_;
@@ -95,10 +128,14 @@ attn_fwd_kernel(const T* __restrict__ qkv, T* __restrict__ out, float* __restric
     for (int dd = lane; dd < d; dd += 32) q[dd] = to_f(qrow[dd]) * scale;
     __syncwarp();
     float mx = -INFINITY;
-    for (int j = lane; j < T_; j += 32) {
-      float s = Row<T>::dot(q, Ks + (size_t)j * rs, d);
-      P[j] = s;
-      mx = fmaxf(mx, s);
+    for (int j0 = 0; j0 < T_; j0 += 128) {
+      float s[4];
+      row_dots(q, Ks, rs, j0 + lane, j0, T_, d, s);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int j = j0 + lane + 32 * u;
+        if (j < T_) { P[j] = s[u]; mx = fmaxf(mx, s[u]); }
+      }
     }
     mx = warp_max(mx);
     float sum = 0.f;
@@ -111,6 +148,7 @@ attn_fwd_kernel(const T* __restrict__ qkv, T* __restrict__ out, float* __restric
     float inv = 1.0f / sum;
     __syncwarp();
     float o0 = 0.f, o1 = 0.f;
+#pragma unroll 8
     for (int j = 0; j < T_; ++j) {
       float a, c2;
       Row<T>::pair(Vs + (size_t)j * rs, lane, d, a, c2);
@@ -154,6 +192,7 @@ attn_bwd_dq_kernel(const T* __restrict__ qkv, const T* __restrict__ dout, const 
   const T* base = qkv + (size_t)b * T_ * tok_stride + (size_t)h * d;
   stage_rows<T>(Ks, base + (size_t)H * d, tok_stride, T_, d);
   stage_rows<T>(Vs, base + 2 * (size_t)H * d, tok_stride, T_, d);
+  copies_done();
   __syncthreads();
   float scale = rsqrtf((float)d);
   float invH = 1.0f / (float)H;
@@ -167,22 +206,42 @@ attn_bwd_dq_kernel(const T* __restrict__ qkv, const T* __restrict__ dout, const 
     __syncwarp();
     float l = lse[((size_t)b * H + h) * T_ + i];
     float dl = 0.f;
-    for (int j = lane; j < T_; j += 32) {
-      float p = expf(Row<T>::dot(q, Ks + (size_t)j * rs, d) - l);
-      float dp = Row<T>::dot(g, Vs + (size_t)j * rs, d);
-      if (cls_extra != nullptr && i == 0 && j > 0) dp += cls_extra[(size_t)b * (T_ - 1) + (j - 1)] * invH;
-      dl += p * dp;
-      P[j] = p;
-      // dS needs delta: keep dP in the upper half of the pass by recomputing below
+    float dps[4] = {0.f, 0.f, 0.f, 0.f};                   // of the last 128 keys
+    auto value_dots = [&](int j0) {
+      row_dots(g, Vs, rs, j0 + lane, j0, T_, d, dps);
+      if (cls_extra != nullptr && i == 0)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int j = j0 + lane + 32 * u;
+          if (j > 0 && j < T_) dps[u] += cls_extra[(size_t)b * (T_ - 1) + (j - 1)] * invH;
+        }
+    };
+    for (int j0 = 0; j0 < T_; j0 += 128) {
+      float s[4];
+      row_dots(q, Ks, rs, j0 + lane, j0, T_, d, s);
+      value_dots(j0);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int j = j0 + lane + 32 * u;
+        if (j < T_) {
+          const float p = expf(s[u] - l);
+          dl += p * dps[u];
+          P[j] = p;
+        }
+      }
     }
     dl = warp_sum(dl);
-    for (int j = lane; j < T_; j += 32) {
-      float dp = Row<T>::dot(g, Vs + (size_t)j * rs, d);
-      if (cls_extra != nullptr && i == 0 && j > 0) dp += cls_extra[(size_t)b * (T_ - 1) + (j - 1)] * invH;
-      P[j] = P[j] * (dp - dl);
+    for (int j0 = (T_ - 1) / 128 * 128; j0 >= 0; j0 -= 128) {      // dS needs delta; beyond 128 keys dP is formed again
+      if (j0 + 128 < T_) value_dots(j0);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int j = j0 + lane + 32 * u;
+        if (j < T_) P[j] = P[j] * (dps[u] - dl);
+      }
     }
     __syncwarp();
     float a0 = 0.f, a1 = 0.f;
+#pragma unroll 8
     for (int j = 0; j < T_; ++j) {
       float x0, x1;
       Row<T>::pair(Ks + (size_t)j * rs, lane, d, x0, x1);
@@ -227,6 +286,7 @@ attn_bwd_dkv_kernel(const T* __restrict__ qkv, const T* __restrict__ dout, const
     Ls[i] = lse[((size_t)b * H + h) * T_ + i];
     Ds[i] = delta[((size_t)b * H + h) * T_ + i];
   }
+  copies_done();
   __syncthreads();
   float scale = rsqrtf((float)d);
   float invH = 1.0f / (float)H;
@@ -239,15 +299,23 @@ attn_bwd_dkv_kernel(const T* __restrict__ qkv, const T* __restrict__ dout, const
     const T* vrow = krow + (size_t)H * d;
     for (int dd = lane; dd < d; dd += 32) { kk[dd] = to_f(krow[dd]) * scale; vv[dd] = to_f(vrow[dd]); }
     __syncwarp();
-    for (int i = lane; i < T_; i += 32) {
-      float p = expf(Row<T>::dot(kk, Qs + (size_t)i * rs, d) - Ls[i]);
-      float dp = Row<T>::dot(vv, Gs + (size_t)i * rs, d);
-      if (cls_extra != nullptr && i == 0 && j > 0) dp += cls_extra[(size_t)b * (T_ - 1) + (j - 1)] * invH;
-      P[i] = p;
-      dS[i] = p * (dp - Ds[i]);
+    for (int i0 = 0; i0 < T_; i0 += 128) {
+      float s[4], dp[4];
+      row_dots(kk, Qs, rs, i0 + lane, i0, T_, d, s);
+      row_dots(vv, Gs, rs, i0 + lane, i0, T_, d, dp);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int i = i0 + lane + 32 * u;
+        if (i >= T_) continue;
+        if (cls_extra != nullptr && i == 0 && j > 0) dp[u] += cls_extra[(size_t)b * (T_ - 1) + (j - 1)] * invH;
+        const float p = expf(s[u] - Ls[i]);
+        P[i] = p;
+        dS[i] = p * (dp[u] - Ds[i]);
+      }
     }
     __syncwarp();
     float v0 = 0.f, v1 = 0.f, k0 = 0.f, k1 = 0.f;
+#pragma unroll 4
     for (int i = 0; i < T_; ++i) {
       float g0, g1, q0, q1;
       Row<T>::pair(Gs + (size_t)i * rs, lane, d, g0, g1);
