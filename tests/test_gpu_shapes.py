@@ -393,6 +393,22 @@ def test_selection_compaction_and_layernorm_in_one_launch(dtype, grid, keep, fus
         P.compare_step(cfg, images, labels, task_ids, params, gpu, P.BF16_TOL, P.BF16_EXACT_MARGIN, P.BF16_SCORE_TOL)
 
 
+@pytest.mark.parametrize("T", [1, 5, 16, 33, 64, 65, 128, 129, 160, 161, 192, 193, 224, 256])
+def test_attention_forward_of_an_image_does_not_depend_on_the_batch(T):
+    """One image's tiles fit the SMs at once, those of 300 images do not: two kernels, the same bits."""
+    import torch
+    from paper_2405_10951_b200 import binding as Bd
+    g = torch.Generator(device="cuda").manual_seed(T)
+    qkv = torch.randn(300, T, 3, 2, 64, generator=g, device="cuda").bfloat16()
+    many = Bd.bsr_attention_forward(qkv, 2, use_tensor_cores=True, want_lse=True)
+    one = Bd.bsr_attention_forward(qkv[:1].contiguous(), 2, use_tensor_cores=True, want_lse=True)
+    for a, b in zip(one, many):
+        assert torch.equal(a[:1], b[:1])
+    o = torch.nn.functional.scaled_dot_product_attention(*qkv[:1].double().permute(2, 0, 3, 1, 4)).transpose(1, 2).reshape(1, T, 128)
+    # P and the output are rounded to bf16 (2^-9 each), the rest is 32-bit
+    assert float((one[0].double() - o).norm() / o.norm()) < 6e-3
+
+
 @pytest.mark.parametrize("m,n,k", [(1, 4, 4), (31, 36, 60), (32, 32, 64), (33, 68, 260), (100, 192, 516), (7, 200, 2052), (9000, 512, 512)])
 def test_fp32_products_in_small_tiles(m, n, k):
     """Edges of the 32 x 32 tiles and 64-deep slabs, one to eight parts of k, and the number of tiles beyond which tiles of 64 take over; sums of at
