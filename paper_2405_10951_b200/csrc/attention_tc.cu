@@ -1300,6 +1300,282 @@ attn_bwd_tc256_kernel(const __grid_constant__ CUtensorMap map_qkv, const __grid_
 }
 
 // ------------------------------------------------------------------------------------------------
+// The same range where two CTAs per (image, head) fit the SMs at once: a cluster of two CTAs of 256 threads, each with one tile of 128 keys
+// and both tiles of queries.  delta_i = sum_j P_ij dP_ij and dQ_i = sum_j dS_ij K_j run
+// over both CTAs' keys, which exchange their parts through distributed shared memory.  All scores of a CTA fit tensor memory at
+// once (S and dP of two query tiles: 512 columns), so they are formed once: P stays in registers (128 values a thread) between the sum
+// for delta and dS, dP in tensor memory, and the accumulators take the columns of S.
+//   S, dP -> P (bf16 tiles in shared memory, dV = P^T dO under way) -> delta exchanged -> dS over the tiles of P -> dQ, dK -> the part of the
+//   other CTA's query tile sent to it -> dQ, dK, dV of 128 rows each out.
+// No step leaves early: after a wait that expired the remaining steps only keep the barriers in step.
+// us of a launch in a row of launches, attn_bwd_tc256_kernel / this, 12 heads, 197 tokens: 1 image 19.5 / 11.4, 4 images 19.6 / 12.8, and beyond one
+// wave 8 images 20.5 / 25.1, 128 images 229 / 270 (140 tokens: 15.8 / 10.5, 15.9 / 12.4, 16.9 / 24.4, 185 / 248).
+// ------------------------------------------------------------------------------------------------
+__global__ void __launch_bounds__(256, 1)
+attn_bwd_pair_kernel(const __grid_constant__ CUtensorMap map_qkv, const __grid_constant__ CUtensorMap map_do,
+                     const float* __restrict__ lse, const float* __restrict__ cls_extra, bf16* __restrict__ dqkv,
+                     int T, int H, int* status) {
+  extern __shared__ unsigned char smem_dyn[];
+  __shared__ __align__(8) unsigned long long bar_mem[4];
+  __shared__ float red[2][256];                          // the halves' shares of delta of every query row, over this CTA's keys
+  __shared__ float part[2][256];                         // ... summed, by key tile
+  __shared__ float exs[AT_QROWS];                        // classification-row score gradients of this CTA's keys / H
+  __shared__ uint32_t tmem_slot;
+  __shared__ int abort_flag;
+  const uint32_t base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
+  unsigned char* base_ptr = smem_dyn + (base - smem_u32(smem_dyn));
+  constexpr uint32_t TILE = 2 * AT_BOX_BYTES;            // 128 rows x 128 bytes
+  constexpr uint32_t CH = TILE;                          // one 64-key chunk of a P / dS tile: 128 query rows x 128 bytes
+  const uint32_t sQ = base, sG = sQ + 2 * TILE, sK = sG + 2 * TILE, sV = sK + TILE, sP = sV + TILE, recv = sP + 4 * TILE;
+  unsigned char* pP = base_ptr + (sP - base);
+  const int tid = threadIdx.x, warp = tid >> 5, rowl = tid & 127, half = tid >> 7, quarter = warp & 3;
+  const int bh = blockIdx.x >> 1, j = blockIdx.x & 1, b = bh / H, h = bh - b * H;
+  const uint32_t bars = smem_u32(bar_mem), tma_bar = bars, s_bar = bars + 8, v_bar = bars + 16, m_bar = bars + 24;
+  if (tid == 0) {
+    abort_flag = 0;
+    mbar_init(tma_bar, 1); mbar_init(s_bar, 1); mbar_init(v_bar, 1); mbar_init(m_bar, 2);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    prefetch_map(&map_qkv);
+    prefetch_map(&map_do);
+  }
+  if (warp == 0) {
+    tmem_alloc(smem_u32(&tmem_slot), 512);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  cluster_arrive();                        // this CTA has started: the other may write to its shared memory
+  const uint32_t tmem = tmem_slot;
+  if (leaves_sms_idle()) release_dependents();
+  await_inputs();
+  constexpr uint32_t C_S = 0, C_DP = 256, C_DV = 0, C_DQ = 64, C_DK = 192;       // S, dP, dQ: one tile of queries after the other
+  volatile int* abortp = &abort_flag;
+  const int tpad = (T + 15) & ~15, row0 = b * T, kbase = 128 * j;
+  const int kvalid = min(128, T - kbase), kpad = min(128, tpad - kbase);
+  bool ok = true;
+  if (tid == 0) {
+    mbar_expect_tx(tma_bar, 6 * TILE);
+    for (int q = 0; q < 2; ++q) {                        // rows past the image: the next image's, or zero fill; never used
+      tma_load_2d(sK + q * AT_BOX_BYTES, &map_qkv, tma_bar, (H + h) * AT_D, row0 + kbase + q * AT_BOX);
+      tma_load_2d(sV + q * AT_BOX_BYTES, &map_qkv, tma_bar, (2 * H + h) * AT_D, row0 + kbase + q * AT_BOX);
+    }
+    for (int q = 0; q < 4; ++q) {
+      tma_load_2d(sQ + q * AT_BOX_BYTES, &map_qkv, tma_bar, h * AT_D, row0 + q * AT_BOX);
+      tma_load_2d(sG + q * AT_BOX_BYTES, &map_do, tma_bar, h * AT_D, row0 + q * AT_BOX);
+    }
+  }
+  const bool has_extra = cls_extra != nullptr;
+  float l2[2];
+#pragma unroll
+  for (int i = 0; i < 2; ++i) l2[i] = i * 128 + rowl < T ? lse[(size_t)bh * T + i * 128 + rowl] * 1.4426950408889634f : 0.f;
+  if (tid < 128) exs[tid] = has_extra && kbase + tid >= 1 && tid < kvalid ? cls_extra[(size_t)b * (T - 1) + kbase + tid - 1] * (1.0f / (float)H) : 0.f;
+  __syncthreads();
+  if (tid == 0) {
+    ok = mbar_wait(tma_bar, 0, abortp);
+    if (ok) {
+      tc_fence_after();
+      const uint32_t idesc = make_idesc_mn(AT_QROWS, kpad, false, false);
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+#pragma unroll
+        for (int k = 0; k < AT_D / 16; ++k)
+          umma_bf16(tmem + C_S + 128 * i, make_desc(sQ + i * TILE + k * 32, 16, 1024), make_desc(sK + k * 32, 16, 1024), idesc, k > 0 ? 1u : 0u);
+#pragma unroll
+        for (int k = 0; k < AT_D / 16; ++k)
+          umma_bf16(tmem + C_DP + 128 * i, make_desc(sG + i * TILE + k * 32, 16, 1024), make_desc(sV + k * 32, 16, 1024), idesc, k > 0 ? 1u : 0u);
+      }
+      umma_commit(s_bar);
+    }
+  }
+  __syncwarp();
+  ok = mbar_wait_q(s_bar, 0, abortp) && ok;
+  ok = __all_sync(0xffffffffu, ok);
+  tc_fence_after();
+  const float c = 0.125f * 1.4426950408889634f;
+  const uint32_t trow = tmem + ((uint32_t)(quarter * 32) << 16);
+  const int qpad1 = tpad - 128;                          // rows of the second query tile that enter products (the first: all)
+
+  // 16-byte units of a P / dS tile: values of keys 8 g .. 8 g + 7 of this thread's row
+  auto put = [&](int i, int kk, const float* v) {
+#pragma unroll
+    for (int g = 0; g < 2; ++g) {
+      uint4 x;
+      __nv_bfloat162* hx = reinterpret_cast<__nv_bfloat162*>(&x);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) hx[e] = __floats2bfloat162_rn(v[g * 8 + 2 * e], v[g * 8 + 2 * e + 1]);
+      const int key8 = kk * 2 + g;
+      *reinterpret_cast<uint4*>(pP + i * 2 * TILE + (uint32_t)(key8 >> 3) * CH + (uint32_t)rowl * 128u + (uint32_t)(((key8 & 7) ^ (rowl & 7)) << 4)) = x;
+    }
+  };
+  // this thread's 64 keys in four groups of 16, of both query tiles; groups past kpad and rows past the tile's padding enter no product
+  float p[2][4][16];
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const int row = i * 128 + rowl;
+    const bool extra_row = row == 0 && has_extra;
+    const bool enters = i == 0 || quarter * 32 < qpad1;
+    float dacc = 0.f;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int kk = 4 * half + q;
+#pragma unroll
+      for (int e = 0; e < 16; ++e) p[i][q][e] = 0.f;
+      if (!ok || !enters || kk * 16 >= kpad) continue;
+      uint32_t rs[16], rp[16];
+      tmem_ld16(trow + C_S + 128 * i + kk * 16, rs);
+      tmem_ld16(trow + C_DP + 128 * i + kk * 16, rp);
+      tmem_ld_wait();
+      if (row < T) {
+        float d0 = 0.f, d1 = 0.f;
+#pragma unroll
+        for (int e = 0; e < 16; e += 2) {
+          const int key = kk * 16 + e;
+          const float p0 = key < kvalid ? ex2_fast(fmaf(__uint_as_float(rs[e]), c, -l2[i])) : 0.f;
+          const float p1 = key + 1 < kvalid ? ex2_fast(fmaf(__uint_as_float(rs[e + 1]), c, -l2[i])) : 0.f;
+          float e0 = __uint_as_float(rp[e]), e1 = __uint_as_float(rp[e + 1]);
+          if (extra_row) { e0 += exs[key]; e1 += exs[key + 1]; }
+          d0 = key < kvalid ? fmaf(p0, e0, d0) : d0;
+          d1 = key + 1 < kvalid ? fmaf(p1, e1, d1) : d1;
+          p[i][q][e] = p0;
+          p[i][q][e + 1] = p1;
+        }
+        dacc += d0 + d1;
+      }
+      put(i, kk, p[i][q]);
+    }
+    red[half][row] = dacc;
+  }
+  fence_async_smem();
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t id_t = make_idesc_mn(AT_QROWS, AT_D, true, true);
+  // dV = P^T dO (over S, which every thread has read), and dK = dS^T Q: both operands read with queries as the reduction index
+  auto by_queries = [&](uint32_t col, uint32_t sb) {
+    for (int i = 0; i < 2; ++i)
+      for (int k = 0; k < (i == 0 ? 128 : qpad1) / 16; ++k)
+        umma_bf16(tmem + col, make_desc(sP + i * 2 * TILE + k * 2048, CH, 1024), make_desc(sb + i * TILE + k * 2048, 8192, 1024), id_t, (i > 0 || k > 0) ? 1u : 0u);
+  };
+  if (tid == 0 && ok && !abort_flag) {
+    by_queries(C_DV, sG);
+    umma_commit(v_bar);
+  }
+  __syncwarp();
+  // delta: this CTA's part of every query row to both
+  cluster_wait();
+  {
+    const float mine = red[0][tid] + red[1][tid];
+    part[j][tid] = mine;
+    st_cluster(peer_addr(smem_u32(&part[j][tid]), j ^ 1), mine);
+  }
+  cluster_arrive();
+  cluster_wait();
+  ok = mbar_wait_q(v_bar, 0, abortp) && ok;              // P has been read: dS takes its place
+  ok = __all_sync(0xffffffffu, ok);
+  tc_fence_after();
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const int row = i * 128 + rowl;
+    const bool extra_row = row == 0 && has_extra;
+    const bool enters = i == 0 || quarter * 32 < qpad1;
+    const float delta = part[0][row] + part[1][row];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int kk = 4 * half + q;
+      if (!ok || !enters || kk * 16 >= kpad) continue;
+      uint32_t rp[16];
+      tmem_ld16(trow + C_DP + 128 * i + kk * 16, rp);
+      tmem_ld_wait();
+      float ds[16];
+#pragma unroll
+      for (int e = 0; e < 16; ++e) {
+        float dp = __uint_as_float(rp[e]);
+        if (extra_row) dp += exs[kk * 16 + e];
+        ds[e] = row < T && kk * 16 + e < kvalid ? p[i][q][e] * (dp - delta) * 0.125f : 0.f;
+      }
+      put(i, kk, ds);
+    }
+  }
+  fence_async_smem();
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if ((tid & 31) == 0 && warp < 2 && ok && !abort_flag) {
+    if (warp == 0) {
+      // dQ_i = dS_i K: A = dS (contiguous along keys), B = K read with keys as the reduction index
+      const uint32_t id_q = make_idesc_mn(AT_QROWS, AT_D, false, true);
+      for (int i = 0; i < 2; ++i)
+        for (int k = 0; k < kpad / 16; ++k)
+          umma_bf16(tmem + C_DQ + 64 * i, make_desc(sP + i * 2 * TILE + (k >> 2) * CH + (k & 3) * 32, 16, 1024), make_desc(sK + k * 2048, 8192, 1024), id_q,
+                    k > 0 ? 1u : 0u);
+    } else {
+      by_queries(C_DK, sQ);
+    }
+    umma_commit(m_bar);
+  }
+  __syncwarp();
+  ok = mbar_wait_q(m_bar, 0, abortp) && ok;
+  ok = __all_sync(0xffffffffu, ok);
+  tc_fence_after();
+  // the other CTA's query tile: this CTA's part of its dQ, rows of 256 bytes, 16-byte units permuted by the row
+  const int other = j ^ 1;
+  if (ok && other * 128 + quarter * 32 < T) {
+    uint32_t r[32];
+    tmem_ld32(trow + C_DQ + 64 * other + half * 32, r);
+    tmem_ld_wait();
+    const uint32_t dst = peer_addr(recv + (uint32_t)rowl * 256u, other);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) send16(dst + (((half * 8 + u) ^ (rowl & 7)) << 4), r + 4 * u);
+  }
+  __syncwarp();
+  cluster_arrive();
+  const size_t pitch = (size_t)3 * H * AT_D;
+  bf16* rows_out = dqkv + ((size_t)b * T + kbase) * pitch + (size_t)h * AT_D;      // rows of this CTA's tile, Q's columns
+  if (ok) {
+    stage_half_row(pP, trow + C_DK, rowl, half);
+    stage_half_row(pP + TILE, trow + C_DV, rowl, half);
+  }
+  __syncthreads();
+  if (ok) {
+    write_rows(pP, rows_out + (size_t)H * AT_D, pitch, kvalid);
+    write_rows(pP + TILE, rows_out + 2 * (size_t)H * AT_D, pitch, kvalid);
+  }
+  __syncwarp();
+  cluster_wait();
+  if (ok && quarter * 32 < kvalid) {
+    uint32_t r[32];
+    tmem_ld32(trow + C_DQ + 64 * j + half * 32, r);
+    tmem_ld_wait();
+    const unsigned char* got = base_ptr + (recv - base) + (uint32_t)rowl * 256u;
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+      float v[8];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const float4 x = *reinterpret_cast<const float4*>(got + (((half * 8 + g * 2 + u) ^ (rowl & 7)) << 4));
+        v[u * 4 + 0] = __uint_as_float(r[g * 8 + u * 4 + 0]) + x.x; v[u * 4 + 1] = __uint_as_float(r[g * 8 + u * 4 + 1]) + x.y;
+        v[u * 4 + 2] = __uint_as_float(r[g * 8 + u * 4 + 2]) + x.z; v[u * 4 + 3] = __uint_as_float(r[g * 8 + u * 4 + 3]) + x.w;
+      }
+      store16(reinterpret_cast<bf16*>(pP + 2 * TILE + rowl * 128 + (((half * 4 + g) ^ (rowl & 7)) << 4)), v);
+    }
+  }
+  __syncthreads();
+  if (ok) write_rows(pP + 2 * TILE, rows_out, pitch, kvalid);
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 0) {
+    tc_fence_after();
+    tmem_dealloc(tmem, 512);
+  }
+  if (tid == 0 && abort_flag) {
+    unsigned long long t0 = global_ns();   // copies already issued still land in shared memory
+    while (global_ns() - t0 < 1000000ull) {}
+    if (status != nullptr) atomicOr(status, STATUS_TIMEOUT);
+  }
+}
+
+// ------------------------------------------------------------------------------------------------
 // Backward for longer sequences, in two launches of one kernel.  A CTA owns 128 rows of the attention map and walks the
 // other side in blocks of BL_COLS:
 //   KV = false: rows are queries.  S = Q K_j^T and dP = dO V_j^T; a first walk only accumulates delta_i = sum_j P_ij dP_ij
@@ -1601,6 +1877,15 @@ int attention_bwd_tc(const Ctx& c, const void* qkv, const void* dout, const floa
     note_launch(2);
     launch_k(attn_bwd_long_kernel<false>, grid, 256, smem_l, c.stream, mq, mg, lse, delta, cls_extra, (bf16*)dqkv, B, T, H, c.status);
     launch_k(attn_bwd_long_kernel<true>, grid, 256, smem_l, c.stream, mq, mg, lse, delta, cls_extra, (bf16*)dqkv, B, T, H, c.status);
+    return 0;
+  }
+  const int sms = c.sm_count > 0 ? c.sm_count : B200_SMS;
+  if (T > AT_QROWS && 2l * B * H <= sms) { // a CTA per tile of keys
+    const size_t smem_p = 1024 + 12 * 2 * (size_t)AT_BOX_BYTES;
+    static SmemLimit lim_p;
+    if (!ensure_smem(lim_p, attn_bwd_pair_kernel, smem_p)) return -3;
+    note_launch(1);
+    launch_cluster(attn_bwd_pair_kernel, dim3(2 * B * H), 256, smem_p, c.stream, dim3(2, 1, 1), mq, mg, lse, cls_extra, (bf16*)dqkv, T, H, c.status);
     return 0;
   }
   if (T > AT_QROWS) {                      // two tiles of queries and keys

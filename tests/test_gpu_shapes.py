@@ -424,3 +424,19 @@ def test_fp32_products_in_small_tiles(m, n, k):
     assert rel(Bd.bsr_linear_forward(x, w, bias, act_gelu=True), torch.nn.functional.gelu(z)) < 2e-6
     dx, dw = Bd.bsr_linear_backward(x, w, dy)
     assert rel(dx, dy.double() @ w.double()) < 2e-6 and rel(dw, dy.double().T @ x.double()) < 2e-6
+
+
+@pytest.mark.parametrize("with_score_grad", [False, True])
+@pytest.mark.parametrize("T", [129, 143, 144, 145, 160, 192, 193, 255, 256])
+def test_attention_backward_of_few_and_of_many_pairs(T, with_score_grad):
+    """Two CTAs a pair, as long as all fit the SMs, against one: the same sums, parts of delta and dQ added up in another order in 32 bits, so
+    that after rounding to bf16 values differ by a unit of their last place at most now and then."""
+    import torch
+    from paper_2405_10951_b200 import binding as Bd
+    g = torch.Generator(device="cuda").manual_seed(T)
+    qkv, do = torch.randn(80, T, 3, 1, 64, generator=g, device="cuda").bfloat16(), torch.randn(80, T, 64, generator=g, device="cuda").bfloat16()
+    sg = torch.randn(80, T - 1, generator=g, device="cuda") if with_score_grad else None
+    _, _, lse = Bd.bsr_attention_forward(qkv, 1, use_tensor_cores=True, want_lse=True)
+    many = Bd.bsr_attention_backward(qkv, do, lse, sg, use_tensor_cores=True).float()
+    few = Bd.bsr_attention_backward(qkv[:3].contiguous(), do[:3].contiguous(), lse[:3].contiguous(), None if sg is None else sg[:3].contiguous(), use_tensor_cores=True).float()
+    assert float((few - many[:3]).norm() / many[:3].norm()) < 1e-3
