@@ -825,7 +825,8 @@ __device__ __forceinline__ void write_rows(const unsigned char* tile, bf16* dst,
 //   dQ = dS K;  dK = dS^T Q;  dV = P^T dO                      (chain rule through Eq. 1, cf. Eq. 3)
 // S and dP are two MMA groups into tensor memory; each thread owns one query row and writes P and dS as
 // bf16 operand tiles into shared memory; the three products then read those tiles K-major (dQ) or through
-// transposing descriptors (dK, dV), so nothing is transposed by hand.  A gradient arriving at the head-mean
+// transposing descriptors (dK, dV), so nothing is transposed by hand.  P stays in registers between the sum for delta and dS (formed again
+// from S it took 51.6 instead of 50.0 us at 100 tokens, batch 128, 12 heads, 7.8 instead of 6.9 with 4 images).  A gradient arriving at the head-mean
 // score of token j (cls_extra[b, j-1], from the fused token) is added to dP of the classification row.
 // ------------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256, 2)
@@ -917,51 +918,55 @@ attn_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_qkv, const __grid_con
   const bool extra_row = (row == 0 && has_extra);
   float delta = 0.f;
   // tcgen05.ld is warp-collective: every lane issues it, rows past T only skip the arithmetic.  Keys are taken 16 at
-  // a time (two loads of 16 columns) to keep the live registers of a step few.
-  if (ok) {
-    for (int kk = 4 * half; kk < 4 * half + 4 && kk * 16 < T; ++kk) {
-      uint32_t rs[16], rp[16];
-      tmem_ld16(trow + C_S + kk * 16, rs);
-      tmem_ld16(trow + C_DP + kk * 16, rp);
-      tmem_ld_wait();
-      if (valid_row) {
-        float d0 = 0.f, d1 = 0.f;
+  // a time (two loads of 16 columns); the probabilities of this thread's 64 keys stay in registers for dS.
+  float p[4][16];
 #pragma unroll
-        for (int j = 0; j < 16; j += 2) {
-          int key = kk * 16 + j;
-          float p0 = key < T ? ex2_fast(fmaf(__uint_as_float(rs[j]), c, -l2)) : 0.f;
-          float p1 = key + 1 < T ? ex2_fast(fmaf(__uint_as_float(rs[j + 1]), c, -l2)) : 0.f;
-          float e0 = __uint_as_float(rp[j]), e1 = __uint_as_float(rp[j + 1]);
-          if (extra_row) { e0 += exs[key]; e1 += exs[key + 1]; }
-          d0 = fmaf(p0, e0, d0);
-          d1 = fmaf(p1, e1, d1);
-        }
-        delta += d0 + d1;
+  for (int q = 0; q < 4; ++q) {
+    const int kk = 4 * half + q;
+#pragma unroll
+    for (int j = 0; j < 16; ++j) p[q][j] = 0.f;
+    if (!ok || kk * 16 >= T) continue;
+    uint32_t rs[16], rp[16];
+    tmem_ld16(trow + C_S + kk * 16, rs);
+    tmem_ld16(trow + C_DP + kk * 16, rp);
+    tmem_ld_wait();
+    if (valid_row) {
+      float d0 = 0.f, d1 = 0.f;
+#pragma unroll
+      for (int j = 0; j < 16; j += 2) {
+        int key = kk * 16 + j;
+        float p0 = key < T ? ex2_fast(fmaf(__uint_as_float(rs[j]), c, -l2)) : 0.f;
+        float p1 = key + 1 < T ? ex2_fast(fmaf(__uint_as_float(rs[j + 1]), c, -l2)) : 0.f;
+        float e0 = __uint_as_float(rp[j]), e1 = __uint_as_float(rp[j + 1]);
+        if (extra_row) { e0 += exs[key]; e1 += exs[key + 1]; }
+        d0 = fmaf(p0, e0, d0);
+        d1 = fmaf(p1, e1, d1);
+        p[q][j] = p0;
+        p[q][j + 1] = p1;
       }
+      delta += d0 + d1;
     }
   }
   red[half * AT_QROWS + row] = delta;          // every thread reaches this barrier, whatever the waits returned
   __syncthreads();
   delta = red[row] + red[AT_QROWS + row];
   if (ok) {
-    for (int kk = 4 * half; kk < 4 * half + 4; ++kk) {
-      float p[16], ds[16];
 #pragma unroll
-      for (int j = 0; j < 16; ++j) { p[j] = 0.f; ds[j] = 0.f; }
+    for (int q = 0; q < 4; ++q) {
+      const int kk = 4 * half + q;
+      float ds[16];
+#pragma unroll
+      for (int j = 0; j < 16; ++j) ds[j] = 0.f;
       if (kk * 16 < T) {
-        uint32_t rs[16], rp[16];
-        tmem_ld16(trow + C_S + kk * 16, rs);
+        uint32_t rp[16];
         tmem_ld16(trow + C_DP + kk * 16, rp);
         tmem_ld_wait();
         if (valid_row) {
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
-            int key = kk * 16 + j;
-            float pv = key < T ? ex2_fast(fmaf(__uint_as_float(rs[j]), c, -l2)) : 0.f;
             float dp = __uint_as_float(rp[j]);
-            if (extra_row) dp += exs[key];
-            p[j] = pv;
-            ds[j] = pv * (dp - delta) * 0.125f;
+            if (extra_row) dp += exs[kk * 16 + j];
+            ds[j] = p[q][j] * (dp - delta) * 0.125f;
           }
         }
       }
@@ -972,7 +977,7 @@ attn_bwd_tc_kernel(const __grid_constant__ CUtensorMap map_qkv, const __grid_con
         __nv_bfloat162* hs = reinterpret_cast<__nv_bfloat162*>(&vs);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-          hp[i] = __floats2bfloat162_rn(p[g * 8 + 2 * i], p[g * 8 + 2 * i + 1]);
+          hp[i] = __floats2bfloat162_rn(p[q][g * 8 + 2 * i], p[q][g * 8 + 2 * i + 1]);
           hs[i] = __floats2bfloat162_rn(ds[g * 8 + 2 * i], ds[g * 8 + 2 * i + 1]);
         }
         if (row < tpad) {
