@@ -279,8 +279,7 @@ template <bool A_K, bool B_K>
 __global__ void __launch_bounds__(SS_THREADS)
 gemm_simt_small_kernel(const float* __restrict__ A, long lda, const float* __restrict__ B, long ldb, int K, int k_per_split, SimtEpi<float, float> epi) {
   extern __shared__ __align__(16) float ss[];
-  if (leaves_sms_idle()) release_dependents();
-  await_inputs();
+  dependent_sync();                                          // (small CTAs, three to an SM: the next kernel may always be scheduled; 382 -> 377 us a step at batch 8)
   const int tid = threadIdx.x, grp = tid >> 6, ty = (tid & 63) >> 3, tx = tid & 7;
   const int m0 = blockIdx.y * SS_BM, n0 = blockIdx.x * SS_BN;
   const int splits = gridDim.z, rank = blockIdx.z;
