@@ -374,7 +374,7 @@ size_t plan(bsr_handle* h) {
   for (int l = h->t0; l < d.depth; ++l) {
     BlockBufs& bb = h->bufs_train[l];
     size_t Ma = (size_t)Bm * s.ta[l], Mf = (size_t)Bm * s.tf[l];
-    bool drop = s.k[l] >= 0 && s.tf[l] != s.ta[l];
+    bool drop = s.k[l] >= 0 && s.k[l] < s.ta[l] - 1;
     size_t block0 = b.off;
     bb.x_in = (l == h->t0) ? b.take(Ma * D * 4) : next_in;       // residual stream: float
     // A trainable block keeps the input of every linear layer (Eq. 4: its weight gradient needs it); a frozen block
@@ -557,7 +557,7 @@ int block_forward(bsr_handle* h, const Ctx& c, int l, int B, const BlockBufs& bb
   int Ta = s.ta[l], Tf = s.tf[l], k = s.k[l];
   int Ma = B * Ta, Mf = B * Tf;
   bool is_drop = k >= 0;
-  bool shrinks = is_drop && Tf != Ta;
+  bool shrinks = is_drop && k < Ta - 1;       // (with a fused token the length may stay: all but one kept)
   // gradient-free prefix with 8-bit operands: the LayerNorm output leaves as E4M3 rows and meets the E4M3 weight copy
   const bool fp8 = !save && l < h->t0 && h->cfg.frozen_fp8 && h->q_qkv[l] != 0 && c.use_tc;
   GemmEpilogue e1;
@@ -753,7 +753,7 @@ int block_backward(bsr_handle* h, const Ctx& c, int l, int B, GradStream dxo, Gr
   int D = d.dim, F = d.mlp_hidden, H = d.heads, hd = D / H;
   int Ta = s.ta[l], Tf = s.tf[l], k = s.k[l];
   int Ma = B * Ta, Mf = B * Tf;
-  bool shrinks = k >= 0 && Tf != Ta;
+  bool shrinks = k >= 0 && k < Ta - 1;
   const int* kept = h->at<int>(h->off_kept_all) + kept_before(h, B, l);
   bool bf = d.dtype == BSR_DTYPE_BF16;
   bool tail = cls_tail(h, l);

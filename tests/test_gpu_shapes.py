@@ -440,3 +440,14 @@ def test_attention_backward_of_few_and_of_many_pairs(T, with_score_grad):
     many = Bd.bsr_attention_backward(qkv, do, lse, sg, use_tensor_cores=True).float()
     few = Bd.bsr_attention_backward(qkv[:3].contiguous(), do[:3].contiguous(), lse[:3].contiguous(), None if sg is None else sg[:3].contiguous(), use_tensor_cores=True).float()
     assert float((few - many[:3]).norm() / many[:3].norm()) < 1e-3
+
+
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+def test_drop_location_that_keeps_all_but_one_token_fuses_it(dtype):
+    """Nine patches, one kept and one fused; two tokens, one of them kept: the sequence keeps its length, but its last token is the fused one."""
+    cfg = Config("mini_last_token", 12, 4, 128, 2, 3, 256, (10,), 5, (1, 2), (0, 1), 1, 9, dtype=dtype, seed=2)
+    images, labels, task_ids, params = synth.make_workload(cfg, peaked=dtype == "fp32")
+    gpu = P.run_gpu_step(cfg, images, labels, task_ids, params)
+    tol = P.FP32_TOL if dtype == "fp32" else P.BF16_TOL
+    P.compare_step(cfg, images, labels, task_ids, params, gpu, tol, P.EXACT_MARGIN if dtype == "fp32" else P.BF16_EXACT_MARGIN,
+                   P.FP32_TOL if dtype == "fp32" else P.BF16_SCORE_TOL)
