@@ -1,3 +1,4 @@
+import gc
 import os
 import sys
 
@@ -32,4 +33,11 @@ def native_library():
     from paper_2405_10951_b200 import binding, build
     if not os.path.exists(binding.LIB_PATH):
         build.build()
+    yield
+
+
+@pytest.fixture(scope="module", autouse=True)
+def earlier_modules_collected():
+    """Device tensors in reference cycles (a caught exception's frames) go now, not in the middle of a test that watches the allocator."""
+    gc.collect()
     yield
