@@ -228,17 +228,17 @@ __device__ __forceinline__ uint64_t simt_fma2(uint64_t a, uint64_t b, uint64_t c
 // Rows of a slab lie where quarter-warps read them without bank conflicts: [row][64 + 4] where the operand is
 // contiguous along k (fragments of four k), [k][32 + 4] where along its own index.
 constexpr int SS_BM = 32, SS_BN = 32, SS_BK = 64, SS_THREADS = 256, SS_GROUPS = 4, SS_STAGES = 4;
-constexpr long SS_MANY = 8192;
 constexpr int SS_KLD = SS_BK + 4, SS_MLD = SS_BM + 4;
 constexpr int SS_OPERAND = SS_BK * SS_MLD;                    // floats of a slab of one operand, either layout (32 x 68 or 64 x 36)
 static_assert(SS_OPERAND >= SS_BM * SS_KLD, "either layout fits");
 constexpr size_t SS_SMEM = (size_t)SS_STAGES * 2 * SS_OPERAND * sizeof(float);
 
-// Slab k0 .. k0 + 63 of rows r0 .. r0 + 31; what lies beyond R rows or K columns becomes zero.  Base and row pitch are multiples of 16 bytes.
-template <bool KMAJOR>
+// Slab k0 .. k0 + 63 of ROWS rows from r0 on; what lies beyond R rows or K columns becomes zero.  Base and row pitch are multiples of 16 bytes.
+template <bool KMAJOR, int ROWS = SS_BM>
 __device__ __forceinline__ void ss_load(const float* __restrict__ P, long ld, int r0, int k0, int R, int K, float* S) {
+  static_assert(KMAJOR || ROWS == SS_BM, "tiles of 64 are built for operands contiguous along k");
 #pragma unroll
-  for (int q = 0; q < 2; ++q) {
+  for (int q = 0; q < ROWS / 16; ++q) {
     const int i = q * SS_THREADS + threadIdx.x;
     int left;
     const float* src;
@@ -397,21 +397,138 @@ gemm_simt_small_kernel(const float* __restrict__ A, long lda, const float* __res
   cluster.sync();                                             // no CTA leaves while another may still read its tile
 }
 
-// Splits of the reduction: by its length alone for a layer's output or input gradient, so that an image's result does not
-// depend on the batch; weight gradients by what fills the SMs.  Non-zero: not a product for this kernel.
+// Tiles of 64 x 64 for many rows, both operands contiguous along k: 8 x 8 products a thread read shared memory half as often for a
+// multiply-add, and that is what bounds the small tiles once nothing is idle.  The sum of an output is the one that
+// gemm_simt_small_kernel forms, addition by addition -- four groups with even and odd k apart over each part of k, the groups in
+// order, then the parts -- so the choice between the two may depend on the number of rows, and a row's result still does not.
+// A CTA takes the parts of k one after the other; the next part's slabs arrive while this one's groups are added up, in memory of
+// their own.  One CTA an SM: 255 registers a thread.
+constexpr int SW_BM = 64, SW_BN = 64, SW_TLD = SW_BN + 4;
+constexpr int SW_OPERAND = SW_BM * SS_KLD;
+constexpr size_t SW_SMEM = ((size_t)SS_STAGES * 2 * SW_OPERAND + (size_t)SS_GROUPS * SW_BM * SW_TLD) * sizeof(float);
+
+__global__ void __launch_bounds__(SS_THREADS, 1)
+gemm_simt_wide_kernel(const float* __restrict__ A, long lda, const float* __restrict__ B, long ldb, int K, int k_per_split, SimtEpi<float, float> epi) {
+  extern __shared__ __align__(16) float ss[];
+  if (leaves_sms_idle()) release_dependents();
+  await_inputs();
+  const int tid = threadIdx.x, grp = tid >> 6, ty = (tid & 63) >> 3, tx = tid & 7;
+  const int m0 = blockIdx.y * SW_BM, n0 = blockIdx.x * SW_BN;
+  const int slabs = (K + SS_BK - 1) / SS_BK, per = k_per_split / SS_BK;      // per: slabs of a part
+  float* tiles = ss + SS_STAGES * 2 * SW_OPERAND;
+  auto stage = [&](int i) {
+    if (i < slabs) {
+      float* S = ss + (i % SS_STAGES) * 2 * SW_OPERAND;
+      ss_load<true, SW_BM>(A, lda, m0, i * SS_BK, epi.M, K, S);
+      ss_load<true, SW_BN>(B, ldb, n0, i * SS_BK, epi.N, K, S + SW_OPERAND);
+    }
+    copies_commit();
+  };
+#pragma unroll
+  for (int i = 0; i < SS_STAGES - 1; ++i) stage(i);
+  constexpr int MINE = SW_BM * SW_BN / 4 / SS_THREADS;       // of the finished tile: four columns of a row each
+  uint64_t acc[8][8];
+  float total[MINE][4];
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int j = 0; j < 8; ++j) acc[i][j] = 0ull;
+  int in_part = 0;
+  bool first = true;
+  for (int s = 0; s < slabs; ++s) {
+    copies_wait<SS_STAGES - 2>();
+    __syncthreads();
+    stage(s + SS_STAGES - 1);                                 // into the slab that every thread left before this barrier
+    const float* As = ss + (s % SS_STAGES) * 2 * SW_OPERAND;
+    const float* Bs = As + SW_OPERAND;
+#pragma unroll
+    for (int kk = 0; kk < SS_BK / SS_GROUPS; kk += 4) {
+      const int k = grp * (SS_BK / SS_GROUPS) + kk;
+      float b[8][4];
+#pragma unroll
+      for (int n = 0; n < 8; ++n) load16(Bs + (tx + n * 8) * SS_KLD + k, b[n]);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        float a[4];
+        load16(As + (ty + i * 8) * SS_KLD + k, a);
+#pragma unroll
+        for (int j = 0; j < 4; j += 2)
+#pragma unroll
+          for (int n = 0; n < 8; ++n) acc[i][n] = simt_fma2(simt_pack2(a[j], a[j + 1]), simt_pack2(b[n][j], b[n][j + 1]), acc[i][n]);
+      }
+    }
+    if (++in_part < per && s + 1 < slabs) continue;
+    // end of a part of k: its groups' tiles [4][64][64 + 4], added in order (the part before has been read: a slab's barrier lies between)
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+      for (int n = 0; n < 8; ++n) {
+        float even, odd;
+        simt_unpack2(acc[i][n], even, odd);
+        tiles[(grp * SW_BM + ty + i * 8) * SW_TLD + tx + n * 8] = even + odd;
+        acc[i][n] = 0ull;
+      }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < MINE; ++q) {
+      const int u = q * SS_THREADS + tid, r = u >> 4, c4 = (u & 15) * 4;
+      float v[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+      for (int g = 0; g < SS_GROUPS; ++g) {
+        float t[4];
+        load16(tiles + (g * SW_BM + r) * SW_TLD + c4, t);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) v[j] += t[j];
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) total[q][j] = first ? v[j] : total[q][j] + v[j];
+    }
+    in_part = 0;
+    first = false;
+  }
+  copies_wait<0>();
+#pragma unroll
+  for (int q = 0; q < MINE; ++q) {
+    const int u = q * SS_THREADS + tid;
+    epi(m0 + (u >> 4), n0 + (u & 15) * 4, total[q]);
+  }
+}
+
+// Wide tiles from the second part of k on (one part alone gains nothing: 25216 x 768 x 192 273 / 274 us) and where they fill at least two
+// thirds of the waves they take.  us of a launch in a row of launches, small / wide:
+//   520 x 768 x 768 (108 tiles on 148 SMs)   34.3 / 30.1   1576 x 768 x 768     89.6 / 85.8   788 x 1152 x 384  37.0 / 32.4
+//   788 x 768 x 768 (156)                    48.0 / 57.3   6304 x 768 x 768     335  / 254    1576 x 384 x 1536 92.1 / 110
+//   1576 x 768 x 3072 (300)                  331  / 317    2364 x 768 x 3072    486  / 321    3152 x 384 x 384  46.7 / 47.8
+//   197 x 2304 x 768 (144)                   41.0 / 30.2   25216 x 768 x 768    1322 / 913    3152 x 384 x 1536 177  / 165
+//   197 x 3072 x 768 (192)                   52.7 / 57.1   25216 x 768 x 3072   5110 / 3398   25216 x 384 x 384 338  / 257
+// gemm_simt_kernel's tiles of 64, with sums in another order: 25216 x 768 x 768 1066, 25216 x 768 x 3072 4027, and, where the wide tiles' third
+// wave is nearly empty, faster: 1576 x 768 x 3072 289.  An image's fp32 logits would then depend on the others of its batch.
+static bool wide_tiles(int m, int n, int k, int sms) {
+  const long tiles = (long)ceil_div(m, SW_BM) * ceil_div(n, SW_BN);
+  return k > 256 && 3 * tiles >= 2 * ceil_div(tiles, sms) * (long)sms;
+}
+
+// Parts of the reduction: by its length alone for a layer's output or input gradient, so that an image's result does not
+// depend on the batch; weight gradients by what fills the SMs.  Non-zero: not a product for these kernels -- by alignment, and more
+// rows than a grid of small tiles has where the operands are not both contiguous along k.
 static int launch_simt_small(const Ctx& c, const float* A, long lda, bool ak, const float* B, long ldb, bool bk, int m, int n, int k,
                              const SimtEpi<float, float>& epi) {
   if (lda % 4 != 0 || ldb % 4 != 0 || (uintptr_t)A % 16 != 0 || (uintptr_t)B % 16 != 0) return -1;
   const int sms = c.sm_count > 0 ? c.sm_count : B200_SMS;
   const long tiles = (long)ceil_div(m, SS_BM) * ceil_div(n, SS_BN);
-  if (ceil_div(m, SS_BM) > 65535) return -1;
+  const bool tall = ceil_div(m, SS_BM) > 65535;
   int splits = ceil_div(k, 256) < SG_MAXSPLIT ? ceil_div(k, 256) : SG_MAXSPLIT;
   if (!ak)
     while (splits > 1 && tiles * splits > 4l * sms) --splits;
   const int per = ceil_div(ceil_div(k, splits), SS_BK) * SS_BK;
   splits = ceil_div(k, per) < 1 ? 1 : ceil_div(k, per);
-  // many tiles along k on both sides: nothing is idle, and tiles of 64 read shared memory less often
-  if (ak && bk && tiles * splits > SS_MANY) return -1;
+  if (ak && bk && (tall || wide_tiles(m, n, k, sms))) {
+    static SmemLimit lim;
+    if (!ensure_smem(lim, gemm_simt_wide_kernel, SW_SMEM)) return -3;
+    launch_k(gemm_simt_wide_kernel, dim3(ceil_div(n, SW_BN), ceil_div(m, SW_BM)), SS_THREADS, SW_SMEM, c.stream, A, lda, B, ldb, k, per, epi);
+    return 0;
+  }
+  if (tall) return -1;
   auto go = [&](auto kern, SmemLimit& lim) {
     if (!ensure_smem(lim, kern, SS_SMEM)) return -3;
     launch_cluster(kern, dim3(ceil_div(n, SS_BN), ceil_div(m, SS_BM), splits), SS_THREADS, SS_SMEM, c.stream, dim3(1, 1, splits), A, lda, B, ldb, k, per, epi);

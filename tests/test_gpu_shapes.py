@@ -451,3 +451,36 @@ def test_drop_location_that_keeps_all_but_one_token_fuses_it(dtype):
     tol = P.FP32_TOL if dtype == "fp32" else P.BF16_TOL
     P.compare_step(cfg, images, labels, task_ids, params, gpu, tol, P.EXACT_MARGIN if dtype == "fp32" else P.BF16_EXACT_MARGIN,
                    P.FP32_TOL if dtype == "fp32" else P.BF16_SCORE_TOL)
+
+
+@pytest.mark.parametrize("n,k,rows", [(1536, 384, 4000), (192, 768, 13000), (768, 260, 3000), (4, 8, 2097121 + 40)])
+def test_fp32_rows_do_not_depend_on_how_many_others_there_are(n, k, rows):
+    """Small and wide tiles, and more rows than a grid of small ones has: one sum for an output, bit for bit."""
+    import torch
+    from paper_2405_10951_b200 import binding as Bd
+    g = torch.Generator(device="cuda").manual_seed(n)
+    x, w, bias = (torch.randn(s, generator=g, device="cuda") for s in ((rows, k), (n, k), (n,)))
+    for gelu in (False, True):
+        many = Bd.bsr_linear_forward(x, w, bias, act_gelu=gelu)
+        for m in (1, 33, 65, 520, 788, 1576):
+            assert torch.equal(Bd.bsr_linear_forward(x[:m], w, bias, act_gelu=gelu), many[:m])
+            assert torch.equal(Bd.bsr_linear_forward(x[-m:], w, bias, act_gelu=gelu), many[-m:])
+
+
+@pytest.mark.parametrize("grid,fuse", [(8, 0), (8, 1), (8, 2), (17, 1), (17, 2)])
+def test_fp32_logits_of_an_image_do_not_depend_on_its_batch(grid, fuse):
+    """64 and 289 patches, drop locations in one launch and in three, products in small and in wide tiles."""
+    import torch
+    from paper_2405_10951_b200 import binding as Bd
+    cfg = Config("mini_alone", 4 * grid, 4, 384, 6, 3, 1536, (10,), 50, (2,), (0, 1), 1, 2, dtype="fp32", fuse_mode=fuse, seed=grid)
+    images, _, _, params = synth.make_workload(cfg, peaked=True)
+    eng = Bd.Engine(cfg)
+    eng.set_params(params)
+    img = eng.images_to_device(images)
+    many, kept = eng.eval_forward(img)
+    for part in (slice(0, 1), slice(49, 50), slice(0, 9), slice(0, 32), slice(17, 50), slice(1, 50)):
+        logits, k = eng.eval_forward(img[part].contiguous())
+        assert torch.equal(logits, many[part])
+        assert all(torch.equal(a, b[part]) for a, b in zip(k, kept))
+    eng.sync_status()
+    eng.close()
