@@ -262,7 +262,7 @@ void head_chain(const Ctx& c, const HeadDesc& h, const HeadRow& io, const EvalIo
 //   dW_t[c, d] = sum_b [task(b) = t] dlogits[b, c] xn[b, d],   db_t[c] = sum_b [..] dlogits[b, c]  (lanes stride the images)
 //   dgamma[d] = sum_b dxn[b, d] xhat[b, d],   dbeta[d] = sum_b dxn[b, d]  (four warps stride the images), the mean loss (lanes stride them).
 // A block forms 16 classes x 128 columns of one task, 4 x 4 sums a thread, the loads of eight images in flight (27 us for 128 images,
-// 100 classes x 768, with a thread per element); blocks of the last row of the grid form the rest.
+// 100 classes x 768, with a thread per element); the last blocks along the classes form the rest.
 constexpr int HG_CLS = 16, HG_COLS = 128, HG_THREADS = 128;
 
 __global__ void __launch_bounds__(HG_THREADS)
@@ -271,9 +271,9 @@ head_grads_kernel(HeadDev h, HeadRow io, const int* __restrict__ task_ids, float
   dependent_sync();
   __shared__ float sm[2][HG_THREADS / 32][HG_COLS];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, D = h.D, t = blockIdx.z;
-  const int col = blockIdx.x * HG_COLS + lane * 4, colr = col < D ? col : 0;
-  if (blockIdx.y + 1 < gridDim.y) {
-    const int n = h.ncls[t], c0 = blockIdx.y * HG_CLS + warp * 4;
+  const int col = blockIdx.y * HG_COLS + lane * 4, colr = col < D ? col : 0;
+  if (blockIdx.x + 1 < gridDim.x) {
+    const int n = h.ncls[t], c0 = blockIdx.x * HG_CLS + warp * 4;
     if (c0 >= n) return;
     float acc[4][4] = {};
 #pragma unroll 8
@@ -292,7 +292,7 @@ head_grads_kernel(HeadDev h, HeadRow io, const int* __restrict__ task_ids, float
     for (int i = 0; i < 4; ++i) {
       if (c0 + i >= n) break;
       if (col < D) store16(h.dw[t] + (size_t)(c0 + i) * D + col, acc[i]);
-      if (blockIdx.x == 0) {
+      if (blockIdx.y == 0) {
         float s = 0.f;
         for (int b = lane; b < B; b += 32) s += task_ids == nullptr || task_ids[b] == t ? io.dlogits[(size_t)b * h.cmax + c0 + i] : 0.f;
         s = warp_sum(s);
@@ -314,7 +314,7 @@ head_grads_kernel(HeadDev h, HeadRow io, const int* __restrict__ task_ids, float
 #pragma unroll
   for (int j = 0; j < 4; ++j) { sm[0][warp][lane * 4 + j] = sg[j]; sm[1][warp][lane * 4 + j] = sb[j]; }
   __syncthreads();
-  const int out = blockIdx.x * HG_COLS + threadIdx.x;
+  const int out = blockIdx.y * HG_COLS + threadIdx.x;
   if (out < D) {
     float a = 0.f, s = 0.f;
 #pragma unroll
@@ -322,7 +322,7 @@ head_grads_kernel(HeadDev h, HeadRow io, const int* __restrict__ task_ids, float
     dgamma[out] = a;
     dbeta[out] = s;
   }
-  if (blockIdx.x == 0 && warp == 0) {
+  if (blockIdx.y == 0 && warp == 0) {
     float s = 0.f;
     for (int b = lane; b < B; b += 32) s += io.per_image[b];
     s = warp_sum(s);
@@ -337,7 +337,7 @@ head_grads_kernel(HeadDev h, HeadRow io, const int* __restrict__ task_ids, float
 
 void head_grads(const Ctx& c, const HeadDesc& h, const HeadRow& io, const int* task_ids, float* dgamma, float* dbeta, float* loss, float* loss_copy, int B) {
   note_launch(1);
-  launch_k(head_grads_kernel, dim3(ceil_div(h.D, HG_COLS), ceil_div(h.cmax, HG_CLS) + 1, h.num_tasks), HG_THREADS, 0, c.stream, to_dev(h), io, task_ids,
+  launch_k(head_grads_kernel, dim3(ceil_div(h.cmax, HG_CLS) + 1, ceil_div(h.D, HG_COLS), h.num_tasks), HG_THREADS, 0, c.stream, to_dev(h), io, task_ids,
            dgamma, dbeta, loss, loss_copy, B, c.status);
 }
 

@@ -484,3 +484,36 @@ def test_fp32_logits_of_an_image_do_not_depend_on_its_batch(grid, fuse):
         assert all(torch.equal(a, b[part]) for a, b in zip(k, kept))
     eng.sync_status()
     eng.close()
+
+
+def test_head_of_more_classes_than_a_grid_has_rows_of_sixteen():
+    """1048560 classes and more are beyond 65535 groups of 16: loss, logits and the gradients of the head against 64 bits."""
+    import torch
+    from paper_2405_10951_b200 import binding as Bd
+    n = 16 * 65535 + 21
+    cfg = Config("mini_million", 8, 4, 8, 1, 1, 16, (n,), 2, (), (), 1, 2, dtype="fp32")
+    g = torch.Generator(device="cuda").manual_seed(5)
+    eng = Bd.Engine(cfg)
+    params = {}
+    for name, shape in synth.param_shapes(cfg).items():
+        params[name] = torch.randn(shape, generator=g, device="cuda") * (0.02 if "norm" not in name else 1.0)
+        eng.set_param(name, params[name])
+    images = torch.randn(2, 3, 8, 8, generator=g, device="cuda")
+    labels = torch.tensor([3, n - 1], dtype=torch.int32, device="cuda")
+    loss = eng.forward_backward(images, labels, want_kept=False)[0]
+    logits = eng.get_tensor("logits", (2, n)).double()
+    dw, db, dbeta = (eng.get_tensor("grad/" + name, params[name].shape).double() for name in ("head.0.weight", "head.0.bias", "norm.bias"))
+    eng.sync_status()
+    assert torch.equal(eng.eval_forward(images, want_kept=False)[0].double(), logits)
+    eng.close()
+    w = params["head.0.weight"].double()
+    xn = torch.linalg.solve(w.T @ w, w.T @ (logits - params["head.0.bias"].double()).T).T        # the normalised rows, from a million logits
+    rel = lambda a, b: float((a - b).norm() / b.norm())
+    assert rel(xn @ w.T + params["head.0.bias"].double(), logits) < 1e-6
+    want = torch.nn.functional.cross_entropy(logits, labels.long())
+    d = torch.softmax(logits, 1)
+    d[torch.arange(2), labels.long()] -= 1
+    d /= 2
+    # sums of eight products and of a million terms in at most a few thousand fp32 additions in a row
+    assert abs(float(loss[0]) - float(want)) < 1e-5 * float(want)
+    assert rel(db, d.sum(0)) < 1e-5 and rel(dw, d.T @ xn) < 1e-5 and rel(dbeta, (d @ w).sum(0)) < 1e-4
