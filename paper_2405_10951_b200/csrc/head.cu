@@ -44,8 +44,8 @@ __device__ __forceinline__ float hc_block(float v, float* red) {
 
 // Everything between the last block's output and the gradient of it, one image per cluster: LayerNorm of the classification row,
 // logits, loss and its gradient, back through the head's weights and the LayerNorm.  What bounds it is latency (100 classes x 768 are
-// 154 KB that every image reads from L2), so an image's classes are split over the CTAs of a cluster (`ranks`, by
-// the number of classes alone), which exchange the softmax's maximum and sum and their parts of the gradient through distributed
+// 154 KB that every image reads from L2), so an image's classes are split over the CTAs of a cluster (`ranks`, in
+// training by the number of classes alone), which exchange the softmax's maximum and sum and their parts of the gradient through distributed
 // shared memory in rank order.  Only what sums over images is left to head_grads_kernel, which runs beside the blocks' backward pass.
 // In place of seven launches, and of the copies and zeroed tensors around the last block's classification rows, us a step:
 //   DeiT-S, 1 / 8 images 659 -> 647 / 785 -> 772   ViT-B, 1 image 934 -> 920   ViT-B/384, 7 images 1719 -> 1691   two tasks, 4 images 1229 -> 1206
@@ -240,19 +240,25 @@ head_chain_kernel(HeadDev h, HeadRow io, const EvalIo* __restrict__ eval, const 
   }
 }
 
-// An image's CTAs: at least 16 classes each (10 classes 1, 40 classes 2, 100 classes 4, from 128 classes on 8).
-static int head_ranks(int cmax) {
+// An image's CTAs: at least 16 classes each (10 classes 1, 40 classes 2, 100 classes 4, from 128 classes on 8, the most a cluster
+// has).  In inference the CTAs exchange nothing and need no cluster: many classes of few images spread as far as eight CTAs fit an SM.  us of
+// DeiT-S inference (two blocks), a cluster an image / so: 1000 classes, 1 / 64 images 86.1 / 80.6, 215 / 208; 10000 classes 144 / 82.7,
+// 353 / 272; 21841 classes 219 / 84.6, 535 / 356 (to two CTAs an SM 91.0 and 516, to sixteen 84.6 and 351).
+static int head_ranks(const Ctx& c, int cmax, int B, bool train) {
   int r = 1;
   while (r < HC_MAXRANKS && cmax >= r * 2 * 16) r *= 2;
-  return r;
+  if (train || r < HC_MAXRANKS) return r;
+  const int fill = 8 * (c.sm_count > 0 ? c.sm_count : B200_SMS) / B, most = ceil_div(cmax, 16);
+  const int wide = fill < most ? fill : most;
+  return wide > r ? wide : r;
 }
 
 void head_chain(const Ctx& c, const HeadDesc& h, const HeadRow& io, const EvalIo* eval, const int* labels, const int* task_ids, void* dx_copy, int B) {
   note_launch(1);
-  const int ranks = head_ranks(h.cmax);
   const bool train = labels != nullptr;
+  const int ranks = head_ranks(c, h.cmax, B, train);
   auto go = [&](auto kern, auto* copy) {
-    launch_cluster(kern, dim3(B * ranks), HC_THREADS, 0, c.stream, dim3(ranks, 1, 1), to_dev(h), io, eval, labels, task_ids, copy, ranks, B, c.status);
+    launch_cluster(kern, dim3(B * ranks), HC_THREADS, 0, c.stream, dim3(train ? ranks : 1, 1, 1), to_dev(h), io, eval, labels, task_ids, copy, ranks, B, c.status);
   };
   if (c.dtype == 0) train ? go(head_chain_kernel<float, true>, (float*)nullptr) : go(head_chain_kernel<float, false>, (float*)nullptr);
   else train ? go(head_chain_kernel<bf16, true>, (bf16*)dx_copy) : go(head_chain_kernel<bf16, false>, (bf16*)nullptr);

@@ -517,3 +517,24 @@ def test_head_of_more_classes_than_a_grid_has_rows_of_sixteen():
     # sums of eight products and of a million terms in at most a few thousand fp32 additions in a row
     assert abs(float(loss[0]) - float(want)) < 1e-5 * float(want)
     assert rel(db, d.sum(0)) < 1e-5 and rel(dw, d.T @ xn) < 1e-5 and rel(dbeta, (d @ w).sum(0)) < 1e-4
+
+
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+@pytest.mark.parametrize("classes", [(127,), (128,), (1000, 40), (9001,), (21841,)])
+def test_logits_of_inference_are_those_of_training(classes, dtype):
+    """Inference spreads an image's classes over more CTAs than a cluster has, as far as the SMs have room; the sums stay the same."""
+    import torch
+    from paper_2405_10951_b200 import binding as Bd
+    cfg = Config("mini_many_classes", 16, 4, 64, 1, 2, 128, classes, 70, (1,), (0,), 1, 2, dtype=dtype, seed=3)
+    images, labels, task_ids, params = synth.make_workload(cfg, peaked=False)
+    eng = Bd.Engine(cfg)
+    eng.set_params(params)
+    img, lab = eng.images_to_device(images), torch.as_tensor(labels.astype(np.int32)).cuda()
+    tid = torch.as_tensor(task_ids.astype(np.int32)).cuda() if len(classes) > 1 else None
+    for B in (1, 7, 18, 70):
+        part = lambda t: None if t is None else t[:B].contiguous()
+        eng.forward_backward(part(img), part(lab), part(tid))
+        logits = eng.get_tensor("logits", (70, max(classes)))[:B]
+        assert torch.equal(eng.eval_forward(part(img), part(tid))[0], logits)
+    eng.sync_status()
+    eng.close()
