@@ -283,9 +283,11 @@ void gather_fuse(const Ctx& c, const void* x, int B, int M, int D, int k, const 
 //   kept rows    : a warp a row, taken from a counter; the row is in registers, so its LayerNorm costs no second pass.
 // Scores, kept and dropped lists are those of token_select, ties at the K-th key going to the lower index.
 // us a step, three launches -> one: ViT-B, 1 / 8 / 32 images 920 -> 884 / 1210 -> 1170 / 1951 -> 1916, DeiT-S, 8 / 24 images 772 -> 756 /
-// 971 -> 956, ViT-B/384, 7 images 1691 -> 1666.  Images that fill the SMs by themselves gain nothing from it and the selection is made eight
-// times over (DeiT-S, 64 images 1493 -> 1499; ViT-B, 128 images 5836 -> 5852): beyond SGA_MAXIMAGES the three launches stay.
-constexpr int SGA_MAXIMAGES = 48;
+// 971 -> 956, ViT-B/384, 7 images 1691 -> 1666.  33 clusters are on the SMs at once (two of these CTAs on each; 119 registers a thread); more images
+// wait for a second round, which costs more than the launches.  us of inference, three launches / one, around that: DeiT-S, 30 / 32 / 34 / 40
+// images 630 / 623, 671 / 664, 673 / 680, 711 / 719; ViT-B, 32 / 34 / 40 images 1121 / 1110, 1134 / 1138, 1206 / 1215; 577 tokens, where rows outweigh
+// launches, 32 / 34 / 64 images 2509 / 2484, 2748 / 2752, 4738 / 4761.
+constexpr int SGA_MAXIMAGES = 32;
 constexpr int SGA_THREADS = 256, SGA_RANKS = 8, SGA_MAXM = 1023;   // three counts of up to 1023 share one warp reduction
 constexpr int SGA_MAXD = 1024;
 // Kept rows are shared out over as many clusters an image as the SMs have room for; the first has the dropped ones.
