@@ -297,7 +297,7 @@ template <int IPT, typename TY>
 __global__ void __launch_bounds__(SGA_THREADS)
 select_gather_kernel(const float* __restrict__ p, const float* __restrict__ x, int clusters, int H, int M, int D, int k, int fuse, float* __restrict__ scores,
                      int* __restrict__ kept, int* __restrict__ dropped, KeptCopy copy, float* __restrict__ out, const float* __restrict__ g,
-                     const float* __restrict__ be, TY* __restrict__ y, float* __restrict__ mean, float* __restrict__ rstd, float eps) {
+                     const float* __restrict__ be, TY* __restrict__ y, float* __restrict__ mean, float* __restrict__ rstd, float eps, int* status) {
   dependent_sync();
   __shared__ float sc[SGA_MAXM + 1];
   __shared__ int list[SGA_MAXM + 1];                      // kept positions, then dropped ones, each ascending
@@ -390,6 +390,7 @@ select_gather_kernel(const float* __restrict__ p, const float* __restrict__ x, i
     const uint32_t keep_mask = __ballot_sync(0xffffffffu, keep);
     if (j >= M) continue;
     const int n = __popc(keep_mask & lt_mask), at = keep ? at_kept[w] + n : at_drop[w] + lane - n;
+    if (!BSR_CHECK(keep ? at >= 0 && at < k : at >= k && at < M, status)) continue;
     list[at] = j;
     if (lead) {
       if (keep) {
@@ -410,10 +411,11 @@ select_gather_kernel(const float* __restrict__ p, const float* __restrict__ x, i
       float v[8][4];
 #pragma unroll
       for (int u = 0; u < 8; ++u)
-        if (i0 + u * SGA_RANKS < nd) load16(xb + (size_t)(1 + list[k + i0 + u * SGA_RANKS]) * D + col, v[u]);
+        if (i0 + u * SGA_RANKS < nd && BSR_CHECK(list[k + i0 + u * SGA_RANKS] >= 0 && list[k + i0 + u * SGA_RANKS] < M, status))
+          load16(xb + (size_t)(1 + list[k + i0 + u * SGA_RANKS]) * D + col, v[u]);
 #pragma unroll
       for (int u = 0; u < 8; ++u)
-        if (i0 + u * SGA_RANKS < nd) {
+        if (i0 + u * SGA_RANKS < nd && BSR_CHECK(list[k + i0 + u * SGA_RANKS] >= 0 && list[k + i0 + u * SGA_RANKS] < M, status)) {
           const float w = sc[list[k + i0 + u * SGA_RANKS]];
 #pragma unroll
           for (int e = 0; e < 4; ++e) acc[e] += w * v[u][e];
@@ -436,7 +438,9 @@ select_gather_kernel(const float* __restrict__ p, const float* __restrict__ x, i
     if (lane == 0) r = atomicAdd(&next_row, clusters * SGA_RANKS);
     r = __shfl_sync(0xffffffffu, r, 0);
     if (r > k) break;
-    finish_row(r, r == 0 ? xb : xb + (size_t)(1 + list[r - 1]) * D);
+    const int src = r == 0 ? 0 : 1 + list[r - 1];
+    if (!BSR_CHECK(src >= 0 && src <= M, status)) continue;
+    finish_row(r, xb + (size_t)src * D);
   }
   if (!fuse || !first) return;
   cluster.sync();
@@ -455,7 +459,8 @@ select_gather_kernel(const float* __restrict__ p, const float* __restrict__ x, i
   if (rank == 0 && warp == 0) {
     if (fuse == 2) {                                       // weighted mean: by the sum of the dropped tokens' weights, in a fixed order
       float ws = 0.f;
-      for (int i = lane; i < nd; i += 32) ws += sc[list[k + i]];
+      for (int i = lane; i < nd; i += 32)
+        if (BSR_CHECK(list[k + i] >= 0 && list[k + i] < M, status)) ws += sc[list[k + i]];
       ws = warp_sum(ws);
       for (int c = lane; c < D; c += 32) part[c] = part[c] / ws;
       __syncwarp();
@@ -473,7 +478,7 @@ int select_gather(const Ctx& c, const float* p, const float* x, int B, int H, in
   clusters = clusters < 1 ? 1 : clusters > SGA_MAXCLUSTERS ? SGA_MAXCLUSTERS : clusters;
   auto go = [&](auto kern, auto* yt) {
     launch_cluster(kern, dim3(B * clusters * SGA_RANKS), SGA_THREADS, 0, c.stream, dim3(SGA_RANKS, 1, 1), p, x, clusters, H, M, D, k, fuse, scores, kept, dropped, copy, out, g, b,
-                   yt, mean, rstd, eps);
+                   yt, mean, rstd, eps, c.status);
   };
   auto pick = [&](auto* yt) {
     using TY = std::remove_pointer_t<decltype(yt)>;
