@@ -135,7 +135,8 @@ static inline void note_launch(int n = 1) { g_kernel_launches += n; }
 // It saves launch latency and prologue: a DeiT-S step of one image (199 launches) 746 -> 659 us, of 64 images 1572 -> 1492 us.
 // Kernels that fill the SMs with one large CTA each (GEMM, attention) do not release: the next kernel's CTAs would pile up on
 // the SMs whose CTA leaves first instead of spreading over all of them (ViT-B at batch 128: 5336 us without, 5341 us so,
-// 5534 us with a release at their start).  On at most half of the SMs they do: the next kernel finds the others idle.
+// 5534 us with a release at their start).  On at most half of the SMs they do: the next kernel finds the others idle.  A product whose
+// successor is another one does on any number below all (launch in gemm_tc.cu).
 constexpr int B200_SMS = 148;
 __device__ __forceinline__ bool leaves_sms_idle() { return 2u * gridDim.x * gridDim.y * gridDim.z <= (unsigned)B200_SMS; }
 __device__ __forceinline__ void release_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

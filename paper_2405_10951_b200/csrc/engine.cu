@@ -619,6 +619,7 @@ int block_forward(bsr_handle* h, const Ctx& c, int l, int B, const BlockBufs& bb
     GemmEpilogue q3;
     q3.bias = (const float*)h->wb(l, "mlp.fc1.bias");
     q3.act = 1;
+    q3.product_next = true;
     if (gemm_tc_e4m3(c, h->base + h->off_yq, h->at<float>(h->off_yq_s), h->base + h->q_fc1[l], h->at<float>(h->q_fc1_s[l]),
                      h->base + bb.hh, Mf, F, D, q3) != 0)
       return set_err(h->err, BSR_ERR_CUDA, "8-bit GEMM set-up failed");
@@ -661,6 +662,7 @@ int block_forward(bsr_handle* h, const Ctx& c, int l, int B, const BlockBufs& bb
   GemmEpilogue e3;
   e3.bias = (const float*)h->wb(l, "mlp.fc1.bias");
   e3.act = 1;
+  e3.product_next = true;
   e3.aux_out = save ? h->base + bb.z : nullptr;
   gemm(c, h->base + bb.y2, D, 1, h->wb(l, "mlp.fc1.weight"), D, 1, h->base + bb.hh, 0, Mf, F, D, e3);
   GemmEpilogue e4;
@@ -819,6 +821,7 @@ int block_backward(bsr_handle* h, const Ctx& c, int l, int B, GradStream dxo, Gr
   // FFN second layer: dz = (dxo W2) * GELU'(z); dW2 = dxo^T h; db2 = column sums of dxo
   GemmEpilogue eg;
   eg.act = 2;
+  eg.product_next = true;
   eg.aux_in = h->base + bb.z;
   if (pg) eg.aux_out = h->base + bb.hh;       // GELU(z) again, into scratch, for the weight gradient below
   gemm(c, op(dxo), D, 1, h->wb(l, "mlp.fc2.weight"), 1, F, dz, 0, Mf, F, D, eg);

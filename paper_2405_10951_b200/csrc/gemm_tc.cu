@@ -410,11 +410,11 @@ static int launch(const Ctx& c, const CUtensorMap& ma, const CUtensorMap& mb, vo
   int sms = c.sm_count > 0 ? c.sm_count : 148;
   int grid = work < sms ? work : sms;
   note_launch(1);
-  // The next kernel may be scheduled early where this one leaves half of the SMs idle -- or any, where it is another product (one follows an
-  // activation, in the FFN): one CTA an SM.  Before attention, several of whose CTAs fit an SM, that is wrong: they pile up on the idle ones
-  // (every product below 148 CTAs: ViT-B/384, 7 images 1663 -> 1726 us a step, DeiT-S, 8 images 740 -> 715).
+  // The next kernel may be scheduled early where this one leaves half of the SMs idle -- or any, where the caller says that it is another
+  // product: one CTA an SM (two of gemm_tc_small_kernel).  Before attention, several of whose CTAs fit an SM, that is wrong: they pile up
+  // on the idle ones (every product below 148 CTAs: ViT-B/384, 7 images 1663 -> 1726 us a step, DeiT-S, 8 images 740 -> 715).
   Epi epi = ep;
-  epi.release = 2 * grid <= sms || (ep.act != 0 && grp.mode == 0 && grid < sms);
+  epi.release = 2 * grid <= sms || (ep.release && grid < sms);
   launch_k(kern, grid, THREADS, SMEM_BYTES, c.stream, ma, mb, (TOut*)C, m, n, k, epi, tiles_m, tiles_n, splits, kb_per_split, grp.mode == 2 ? 1 << 20 : sum_slabs(k), grp, c.status);
   return 0;
 }
@@ -462,6 +462,7 @@ int gemm_tc_strided(const Ctx& c, const void* A, long a_rs, long a_cs, const voi
   const int kb_per_split = ceil_div(total_kb, cut.splits), splits = ceil_div(total_kb, kb_per_split);
   Epi ep;
   ep.bias = e.bias; ep.residual = e.residual; ep.res_ld = (int)(e.residual_ld ? e.residual_ld : n); ep.aux_out = e.aux_out; ep.aux_in = e.aux_in; ep.act = e.act;
+  ep.release = e.product_next;
   const bool exact = !a_mn && e.act != 0 && exact_gelu(m, k);       // (tiles of 64 or 128 columns up to 9472 of them)
   void* dst = (splits > 1) ? (void*)split_ws : C;
   if (splits > 1) side_join(c, 2);         // the previous split sum has read the workspace
@@ -551,6 +552,7 @@ int gemm_tc_e4m3(const Ctx& c, const void* Aq, const float* a_scale, const void*
   if (!make_map_u8(&ma, Aq, (uint64_t)k, (uint64_t)m, (uint64_t)k, BM) || !make_map_u8(&mb, Bq, (uint64_t)k, (uint64_t)n, (uint64_t)k, bn)) return -2;
   Epi ep;
   ep.bias = e.bias; ep.aux_out = e.aux_out; ep.act = e.act; ep.row_scale = a_scale; ep.col_scale = b_scale;
+  ep.release = e.product_next;
   int tiles_m = ceil_div(m, BM), tiles_n = ceil_div(n, bn);
   int total_kb = ceil_div(k, 2 * BK);
   GemmGroup gg;

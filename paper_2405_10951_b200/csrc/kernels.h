@@ -130,6 +130,7 @@ struct GemmEpilogue {
   int act = 0;                      // 0 none, 1 GELU (pre-activation optionally stored), 2 multiply by GELU'(aux_in)
   void* aux_out = nullptr;          // act 1: pre-activation [m, n], output type; act 2 (optional): GELU(aux_in) [m, n], storage type
   const void* aux_in = nullptr;     // act 2: pre-activation [m, n], storage type
+  bool product_next = false;        // the next launch on the stream is another of these products: it may be scheduled early
 };
 void gemm(const Ctx& c, const void* A, long a_rs, long a_cs, const void* B, long b_rs, long b_cs, void* C,
           int out_is_float, int m, int n, int k, const GemmEpilogue& e);

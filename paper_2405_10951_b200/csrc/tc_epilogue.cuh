@@ -16,7 +16,7 @@ struct Epi {
   void* aux_out = nullptr;
   const void* aux_in = nullptr;
   int act = 0;
-  bool release = false;             // the next kernel may be scheduled while this one runs
+  bool release = false;             // the next kernel may be scheduled while this one runs (set up: GemmEpilogue's product_next)
   // operands quantised with one scale per row of A and per row of B (8-bit floating point): the accumulator of
   // (row, col) is multiplied by row_scale[row] * col_scale[col] before the bias
   const float* row_scale = nullptr;
