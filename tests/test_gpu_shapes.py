@@ -395,15 +395,17 @@ def test_selection_compaction_and_layernorm_in_one_launch(dtype, grid, keep, fus
 
 @pytest.mark.parametrize("T", [1, 5, 16, 33, 64, 65, 128, 129, 160, 161, 192, 193, 224, 256])
 def test_attention_forward_of_an_image_does_not_depend_on_the_batch(T):
-    """One image's tiles fit the SMs at once, those of 300 images do not: two kernels, the same bits."""
+    """One image's tiles fit the SMs at once, those of 300 images do not: two kernels, the same bits, whichever turn of its CTA an image is."""
     import torch
     from paper_2405_10951_b200 import binding as Bd
     g = torch.Generator(device="cuda").manual_seed(T)
     qkv = torch.randn(300, T, 3, 2, 64, generator=g, device="cuda").bfloat16()
     many = Bd.bsr_attention_forward(qkv, 2, use_tensor_cores=True, want_lse=True)
-    one = Bd.bsr_attention_forward(qkv[:1].contiguous(), 2, use_tensor_cores=True, want_lse=True)
-    for a, b in zip(one, many):
-        assert torch.equal(a[:1], b[:1])
+    assert len(many) == 3                                            # output, classification row, log-sum-exp
+    for i in (299, 150, 77, 1, 0):
+        one = Bd.bsr_attention_forward(qkv[i: i + 1].contiguous(), 2, use_tensor_cores=True, want_lse=True)
+        for a, b in zip(one, many):
+            assert torch.equal(a, b[i: i + 1])
     o = torch.nn.functional.scaled_dot_product_attention(*qkv[:1].double().permute(2, 0, 3, 1, 4)).transpose(1, 2).reshape(1, T, 128)
     # P and the output are rounded to bf16 (2^-9 each), the rest is 32-bit
     assert float((one[0].double() - o).norm() / o.norm()) < 6e-3
@@ -426,20 +428,23 @@ def test_fp32_products_in_small_tiles(m, n, k):
     assert rel(dx, dy.double() @ w.double()) < 2e-6 and rel(dw, dy.double().T @ x.double()) < 2e-6
 
 
+@pytest.mark.parametrize("H", [1, 3])
 @pytest.mark.parametrize("with_score_grad", [False, True])
 @pytest.mark.parametrize("T", [129, 143, 144, 145, 160, 192, 193, 255, 256])
-def test_attention_backward_of_few_and_of_many_pairs(T, with_score_grad):
+def test_attention_backward_of_few_and_of_many_pairs(T, with_score_grad, H):
     """Two CTAs a pair, as long as all fit the SMs, against one: the same sums, parts of delta and dQ added up in another order in 32 bits, so
     that after rounding to bf16 values differ by a unit of their last place at most now and then."""
     import torch
     from paper_2405_10951_b200 import binding as Bd
     g = torch.Generator(device="cuda").manual_seed(T)
-    qkv, do = torch.randn(80, T, 3, 1, 64, generator=g, device="cuda").bfloat16(), torch.randn(80, T, 64, generator=g, device="cuda").bfloat16()
+    qkv, do = torch.randn(80, T, 3, H, 64, generator=g, device="cuda").bfloat16(), torch.randn(80, T, H * 64, generator=g, device="cuda").bfloat16()
     sg = torch.randn(80, T - 1, generator=g, device="cuda") if with_score_grad else None
-    _, _, lse = Bd.bsr_attention_forward(qkv, 1, use_tensor_cores=True, want_lse=True)
+    _, _, lse = Bd.bsr_attention_forward(qkv, H, use_tensor_cores=True, want_lse=True)
     many = Bd.bsr_attention_backward(qkv, do, lse, sg, use_tensor_cores=True).float()
-    few = Bd.bsr_attention_backward(qkv[:3].contiguous(), do[:3].contiguous(), lse[:3].contiguous(), None if sg is None else sg[:3].contiguous(), use_tensor_cores=True).float()
-    assert float((few - many[:3]).norm() / many[:3].norm()) < 1e-3
+    for part in (slice(0, 3), slice(77, 80)):
+        few = Bd.bsr_attention_backward(qkv[part].contiguous(), do[part].contiguous(), lse[part].contiguous(), None if sg is None else sg[part].contiguous(),
+                                        use_tensor_cores=True).float()
+        assert float((few - many[part]).norm() / many[part].norm()) < 1e-3
 
 
 @pytest.mark.parametrize("dtype", ["fp32", "bf16"])
