@@ -1,6 +1,8 @@
-// FP32-FMA dense contraction with arbitrary operand strides.  It is the contraction of the fp32
-// configuration (TF32 tensor-core math cannot hold a 1e-4 relative tolerance; gemm_simt_small_kernel wherever rows are aligned) and the
-// fall-back for bf16 problems the tcgen05 kernel does not take (tiny or unaligned shapes).
+// FP32-FMA dense contraction with arbitrary operand strides: the contraction of the fp32 configuration (TF32 tensor-core math
+// cannot hold a 1e-4 relative tolerance) and the fall-back for bf16 problems the tcgen05 kernels do not take.  Three kernels:
+//   gemm_simt_small_kernel  float, rows aligned: tiles of 32 x 32;
+//   gemm_simt_wide_kernel   the same sums in tiles of 64 x 64, many rows of a layer;
+//   gemm_simt_kernel        bf16, and float with unaligned rows.
 #include <cooperative_groups.h>
 
 #include <type_traits>
@@ -14,11 +16,11 @@ namespace cg = cooperative_groups;
 
 // A CTA of 128 threads forms a 64 x 64 tile, 8 x 4 outputs per thread: per k step a warp reads 2 + 1 wavefronts of shared
 // memory for 1024 multiply-adds, so the FMA pipe is the limit.  Slabs of 32 along k go through registers into two shared
-// buffers, the loads of the next slab in flight during the arithmetic of this one.  The products of this configuration are
-// small (520 x 576 x 192: 81 tiles on 148 SMs), so a tile's k range is split over the CTAs of a cluster (up to 8), whose
+// buffers, the loads of the next slab in flight during the arithmetic of this one.  Products of few tiles (520 x 576 x 192: 81 tiles
+// on 148 SMs) leave SMs idle, so a tile's k range is split over the CTAs of a cluster (up to 8), whose
 // partial tiles are summed through distributed shared memory in rank order before the epilogue: no second kernel, no
-// workspace, the result does not depend on scheduling.  The step of the fp32 configuration at batch 8 (41 products) took
-// 1310 us with 4 x 4 outputs per thread, no split and no loads in flight, 800 us so.
+// workspace, the result does not depend on scheduling.  A step of 41 such products took 1310 us with 4 x 4 outputs per thread, no
+// split and no loads in flight, 800 us so.
 constexpr int SG_BM = 64, SG_BN = 64, SG_BK = 32, SG_THREADS = 128, SG_LD = SG_BM + 4, SG_MAXSPLIT = 8;
 
 // One thread's share (16 values) of a 64 x 32 operand slab: contiguous along k (row r = t % 64, 16 k values) or along its

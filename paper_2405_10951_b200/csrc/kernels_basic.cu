@@ -1,5 +1,5 @@
 // Bandwidth-bound kernels of the BSR step: patch extraction, token assembly, LayerNorm forward and
-// backward, column sums, head/loss, AdamW, conversions.  All reductions run in a fixed order.
+// backward, column sums, AdamW, conversions.  All reductions run in a fixed order.
 #include "common.cuh"
 #include "kernels.h"
 #include "layernorm.cuh"
