@@ -138,7 +138,10 @@ head_chain_kernel(HeadDev h, HeadRow io, const EvalIo* __restrict__ eval, const 
     float mx = -INFINITY, se = 0.f;
     for (int c = c0 + tid; c < cn; c += HC_THREADS) mx = fmaxf(mx, lg[c - c0]);
     mx = hc_block<true>(mx, red);
-    for (int c = c0 + tid; c < cn; c += HC_THREADS) se += expf(lg[c - c0] - mx);
+    for (int c = c0 + tid; c < cn; c += HC_THREADS) {          // (a masked class adds nothing, even where all of this CTA's are masked)
+      const float l = lg[c - c0];
+      se += l == -INFINITY ? 0.f : expf(l - mx);
+    }
     se = hc_block<false>(se, red);
     if (ranks > 1) {
       if (tid == 0) { ex[0] = mx; ex[1] = se; }

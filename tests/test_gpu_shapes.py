@@ -543,3 +543,30 @@ def test_logits_of_inference_are_those_of_training(classes, dtype):
         assert torch.equal(eng.eval_forward(part(img), part(tid))[0], logits)
     eng.sync_status()
     eng.close()
+
+
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+@pytest.mark.parametrize("classes,masked", [(100, (20, 80)), (128, (0, 16)), (1000, (100, 1000)), (10, (3, 9))])
+def test_classes_masked_by_a_bias_of_minus_infinity(classes, masked, dtype):
+    """A CTA all of whose classes are masked has the maximum -inf and adds nothing to the softmax's sum; masked classes get no gradient."""
+    import torch
+    from paper_2405_10951_b200 import binding as Bd
+    cfg = Config("mini_masked", 16, 4, 64, 1, 2, 128, (classes,), 5, (1,), (0,), 1, 2, dtype=dtype, seed=3)
+    images, _, _, params = synth.make_workload(cfg, peaked=False)
+    a, b = masked
+    params["head.0.bias"][a:b] = -np.inf
+    eng = Bd.Engine(cfg)
+    eng.set_params(params)
+    labels = torch.tensor([c for c in range(classes) if not a <= c < b][:5] * 5, dtype=torch.int32, device="cuda")[:5].contiguous()
+    loss = eng.train_step(eng.images_to_device(images), labels, want_kept=False)[0]
+    eng.sync_status()
+    logits = eng.get_tensor("logits", (5, classes)).double()
+    assert bool((logits[:, a:b] == -float("inf")).all())
+    want = torch.nn.functional.cross_entropy(logits, labels.long())
+    assert abs(float(loss[0]) - float(want)) < 1e-5 * float(want)
+    d = torch.softmax(logits, 1)
+    d[torch.arange(5), labels.long()] -= 1
+    db = eng.get_tensor("grad/head.0.bias", (classes,)).double()
+    assert float((db - d.sum(0) / 5).norm() / d.sum(0).norm()) < 1e-5 and not bool(db[a:b].any())
+    assert bool(eng.grad_buffer().isfinite().all())
+    eng.close()
