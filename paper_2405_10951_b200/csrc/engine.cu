@@ -1226,6 +1226,15 @@ int32_t bsr_set_step(bsr_handle* h, int64_t steps_done) {
   return BSR_OK;
 }
 
+// Whether the kernels may write to a caller's pointer themselves.  Others (memory of another device, pinned memory, anything else) are left
+// to a copy, which knows how to reach them or refuses.
+static bool kernels_can_write(const void* p) {
+  cudaPointerAttributes a;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaPointerGetAttributes(&a, p) != cudaSuccess) { cudaGetLastError(); return false; }
+  return (a.type == cudaMemoryTypeDevice && a.device == dev) || a.type == cudaMemoryTypeManaged;
+}
+
 // Enqueues every kernel of one step on `stream` (forward, loss, backward, AdamW reading its scalars from device memory).
 // loss_out may be null (the multi-step loop writes the loss itself); img_offset as in forward_all.
 static int enqueue_step_kernels(bsr_handle* h, const Ctx& c, const void* images, const int32_t* labels, const int32_t* task_ids, int32_t batch,
@@ -1236,9 +1245,12 @@ static int enqueue_step_kernels(bsr_handle* h, const Ctx& c, const void* images,
   size_t es = dtype_size(d.dtype);
   size_t x_last = 0;
   KeptCopy kept_copy;
-  kept_copy.dst = kept_out;
+  const bool copy_kept = kept_out != nullptr && !kernels_can_write(kept_out), copy_loss = loss_out != nullptr && !kernels_can_write(loss_out);
+  kept_copy.dst = copy_kept ? nullptr : kept_out;
   rc = forward_all(h, c, images, B, true, &x_last, task_ids, kept_copy, img_offset);
   if (rc != BSR_OK) return rc;
+  if (copy_kept && kept_total(h, B) > 0)
+    cudaMemcpyAsync(kept_out, h->base + h->off_kept_all, kept_total(h, B) * 4, cudaMemcpyDeviceToDevice, c.stream);
   // head, loss and final LayerNorm forward and backward in one launch; what they sum over the images beside the blocks' backward pass
   HeadDesc hd = head_desc(h);
   HeadRow row = head_row(h, x_last);
@@ -1255,7 +1267,8 @@ static int enqueue_step_kernels(bsr_handle* h, const Ctx& c, const void* images,
   {
     Ctx w = c;
     w.stream = side_begin(cl);
-    head_grads(w, hd, row, task_ids, h->gradp("norm.weight"), h->gradp("norm.bias"), h->at<float>(h->off_loss), loss_out, B);
+    head_grads(w, hd, row, task_ids, h->gradp("norm.weight"), h->gradp("norm.bias"), h->at<float>(h->off_loss), copy_loss ? nullptr : loss_out, B);
+    if (copy_loss) cudaMemcpyAsync(loss_out, h->at<float>(h->off_loss), 4, cudaMemcpyDeviceToDevice, w.stream);
     side_end(cl, 3);
   }
   // backward through the trainable blocks in reverse, nothing before the earliest one

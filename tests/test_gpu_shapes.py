@@ -570,3 +570,51 @@ def test_classes_masked_by_a_bias_of_minus_infinity(classes, masked, dtype):
     assert float((db - d.sum(0) / 5).norm() / d.sum(0).norm()) < 1e-5 and not bool(db[a:b].any())
     assert bool(eng.grad_buffer().isfinite().all())
     eng.close()
+
+
+@pytest.mark.parametrize("graph", [False, True])
+def test_step_outputs_in_pinned_memory(graph):
+    """Loss and kept positions go where a copy can take them, not only where a kernel can write: pinned host memory as device memory."""
+    import torch
+    from paper_2405_10951_b200 import binding as Bd
+    cfg = MINI.with_(optimizer="sgd", lr=0.0, weight_decay=0.0)
+    images, labels, _, params = synth.make_workload(cfg, peaked=True)
+    eng = Bd.Engine(cfg)
+    eng.set_params(params)
+    with torch.cuda.stream(torch.cuda.Stream()):
+        eng.set_graph_mode(graph)
+        img, lab = eng.images_to_device(images), torch.as_tensor(labels).cuda()
+        loss, kept = eng.train_step(img, lab)
+        out = torch.zeros(1).pin_memory(), torch.full((sum(k.numel() for k in kept),), -1, dtype=torch.int32).pin_memory()
+        for call in (eng.train_step, eng.train_step, eng.train_step, eng.forward_backward):
+            out[0].zero_(), out[1].fill_(-1)
+            call(img, lab, out=out)
+            torch.cuda.current_stream().synchronize()
+            assert torch.equal(out[0], loss.cpu()) and torch.equal(out[1], torch.cat([k.flatten() for k in kept]).cpu())
+        eng.sync_status()
+    eng.close()
+
+
+def test_step_in_a_graph_of_the_callers():
+    """A caller may capture the step into a graph of its own (in the strictest capture mode); replays equal calls."""
+    import torch
+    from paper_2405_10951_b200 import binding as Bd
+    cfg = MINI.with_(optimizer="sgd", lr=0.0, weight_decay=0.0)
+    images, labels, _, params = synth.make_workload(cfg, peaked=True)
+    eng = Bd.Engine(cfg)
+    eng.set_params(params)
+    img, lab = eng.images_to_device(images), torch.as_tensor(labels).cuda()
+    loss, kept = eng.train_step(img, lab)
+    want = [loss.clone(), torch.cat([k.flatten() for k in kept]), eng.grad_buffer().clone()]
+    out = torch.zeros(1, device="cuda"), torch.full_like(want[1], -1)
+    graph = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph, capture_error_mode="global"):
+        eng.train_step(img, lab, out=out)
+    for _ in range(2):
+        out[0].zero_(), out[1].fill_(-1), eng.grad_buffer().zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert all(torch.equal(a, b) for a, b in zip(want, [*out, eng.grad_buffer()]))
+    eng.sync_status()
+    eng.close()
